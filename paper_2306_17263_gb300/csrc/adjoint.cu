@@ -144,7 +144,7 @@ void taylor_h64_T(ms_grid* g, const double* lhx, const double* lhy, double* out,
 }
 
 // One transposed step on the adjoint state adj[0..2] = (l_E, l_Hx, l_Hy), in place.
-// Scratch: adj[3..5] and the FP64 solve's s64[3], s64[4].
+// Scratch: adj[3..5] and the solves' s64[0..4].
 void adjoint_step64(ms_grid* g) {
   const int N = g->N;
   int nl = 0;
@@ -152,8 +152,8 @@ void adjoint_step64(ms_grid* g) {
   double *e = g->adj[3], *x = g->adj[4], *y = g->adj[5];
   const double s_eh = g->kappa2 / (g->Z * g->h), s_he = g->kappa2 * g->Z / g->h;
   // S2^T: u_H = P1_H^{-1} l_H; v = (kappa^2/Z)(delta_x^T u_y - delta_y^T u_x); l_E += h_tau F_E v
-  p1_solve64(g, HX, lHx, x, nullptr, 0.0, &nl);
-  p1_solve64(g, HY, lHy, y, nullptr, 0.0, &nl);
+  double* const buf[2][2] = {{g->s64[0], g->s64[1]}, {g->s64[2], g->s64[3]}};
+  p1_solve64_h(g, lHx, lHy, x, y, nullptr, nullptr, 0.0, buf, &nl);
   const PadeTable& tn = g->padeT[NODE_TO_HALF];
   launch_pade64(0, y, e, N + 1, N, N + 1, N + 1, 0, 1, N, tn, s_eh, 0, g->stream);
   launch_pade64(1, x, e, N + 1, N + 1, N + 1, N + 1, 0, 1, N, tn, -s_eh, 1, g->stream);

@@ -15,6 +15,7 @@
 #include "grid3d.cuh"
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
+#include "k_rec64.cuh"
 #include "k_src3.cuh"
 #include "k_tiled.cuh"
 #include "k_tracked32.cuh"
@@ -58,8 +59,6 @@ ms_status dalloc(T** p, size_t n) {
   return MS_OK;
 }
 
-double omega_of(double c1h2) { return 2.0 / (2.0 * c1h2 + 16.0 / 3.0); }
-
 // ---------------------------------------------------------------------------------------
 // FP64 operator building blocks on arbitrary device arrays.
 
@@ -92,22 +91,25 @@ void curl_eh64(ms_grid* g, const double* GE, double* Rx, double* Ry, int* nl) {
 }  // namespace
 
 namespace ms {
-// x = P1^{-1} b by Richardson sweeps; the last sweep writes `out` and, if upd != nullptr,
-// adds upd_scale * x to upd (the state update E += h_tau E*).
 void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl) {
   const Shape& s = g->sh[f];
-  const double c1h2 = g->c1 * g->h * g->h, om = omega_of(c1h2), h2 = g->h * g->h;
-  const int S = g->p1_sweeps;
-  double* buf[2] = {g->s64[3], g->s64[4]};
-  const double* xin = nullptr;
-  for (int k = 0; k < S; ++k) {
-    const bool last = (k == S - 1);
-    double* xo = last ? out : buf[k & 1];
-    launch_p1_sweep64(b, xin, xo, s, c1h2, om, h2, k == 0, last ? upd : nullptr, upd_scale, g->stream);
-    prof_mark(g, KK_P1SWEEP64, 8.0 * (double)s.size() * ((k == 0 ? 2 : 3) + (last && upd ? 2 : 0)));
-    xin = xo;
+  if (b == out) {  // a block's halo would read points that another block has overwritten
+    cudaMemcpyAsync(g->s64[5], b, s.size() * sizeof(double), cudaMemcpyDeviceToDevice, g->stream);
+    b = g->s64[5];
   }
-  *nl += S;
+  const Cheb2dField F{b, out, upd, s};
+  double* const buf[1][2] = {{g->s64[3], g->s64[4]}};
+  launch_cheb2d64(&F, 1, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
+  prof_mark(g, KK_P1SWEEP64, 8.0 * (double)s.size() * (1.0 + (out ? 1.0 : 0.0) + (upd ? 2.0 : 0.0)));
+  *nl += 1;
+}
+
+void p1_solve64_h(ms_grid* g, const double* bx, const double* by, double* outx, double* outy, double* updx, double* updy,
+                  double upd_scale, double* const (*buf)[2], int* nl) {
+  const Cheb2dField F[2] = {{bx, outx, updx, g->sh[HX]}, {by, outy, updy, g->sh[HY]}};
+  launch_cheb2d64(F, 2, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
+  prof_mark(g, KK_P1SWEEP64, 16.0 * (double)g->sh[HX].size() * (1.0 + (outx ? 1.0 : 0.0) + (updx ? 2.0 : 0.0)));
+  *nl += 1;
 }
 }  // namespace ms
 
@@ -138,8 +140,8 @@ void h_increment64(ms_grid* g, const double* ez, double* hxs, double* hys, doubl
     prof_mark(g, KK_SRC, 8.0 * 8.0 * g->N);
     *nl += 1;
   }
-  p1_solve64(g, HX, Rx, hxs, hx_upd, g->ht, nl);
-  p1_solve64(g, HY, Ry, hys, hy_upd, g->ht, nl);
+  double* const buf[2][2] = {{g->s64[0], g->s64[3]}, {g->s64[4], g->s64[5]}};
+  p1_solve64_h(g, Rx, Ry, hxs, hys, hx_upd, hy_upd, g->ht, buf, nl);
 }
 
 // The step as printed in Sec. 3.4 (MS_SCHEME_C4_DE): Step 1 as in step64, then DE advanced by
@@ -150,11 +152,9 @@ ms_status step64_tracked(ms_grid* g) {
   double* Gx = g->s64[0];
   double* Gy = g->s64[1];
   double* R = g->s64[2];
-  launch_filter64(hx, Gx, g->sh[HX], g->beta, g->stream);
-  prof_mark(g, KK_FILTER64, 16.0 * (double)g->sh[HX].size());
-  launch_filter64(hy, Gy, g->sh[HY], g->beta, g->stream);
-  prof_mark(g, KK_FILTER64, 16.0 * (double)g->sh[HY].size());
-  nl += 2;
+  launch_filter64x2(hx, Gx, g->sh[HX], hy, Gy, g->sh[HY], g->beta, g->stream);
+  prof_mark(g, KK_FILTER64, 32.0 * (double)g->sh[HX].size());
+  nl += 1;
   curl_he64(g, Gx, Gy, R, &nl);
   p1_solve64(g, EZ, R, g->s64[5], ez, g->ht, &nl);  // E* in s64[5], E += h_tau E*
   curl_he64(g, hx, hy, g->s64[0], &nl);              // kappa^2 Z curl_h H (unfiltered)
@@ -165,8 +165,8 @@ ms_status step64_tracked(ms_grid* g) {
   double* Rx = g->s64[0];
   double* Ry = g->s64[2];
   curl_eh64(g, GE, Rx, Ry, &nl);
-  p1_solve64(g, HX, Rx, g->s64[5], hx, g->ht, &nl);
-  p1_solve64(g, HY, Ry, g->s64[5], hy, g->ht, &nl);
+  double* const buf[2][2] = {{g->s64[1], g->s64[3]}, {g->s64[4], g->s64[5]}};
+  p1_solve64_h(g, Rx, Ry, nullptr, nullptr, hx, hy, g->ht, buf, &nl);
   g->launches_per_step = nl;
   return check_launch("fp64 tracked step");
 }
@@ -197,11 +197,9 @@ ms_status step64(ms_grid* g) {
   double* Gx = g->s64[0];
   double* Gy = g->s64[1];
   double* R = g->s64[2];
-  launch_filter64(hx, Gx, g->sh[HX], g->beta, g->stream);
-  prof_mark(g, KK_FILTER64, 16.0 * (double)g->sh[HX].size());
-  launch_filter64(hy, Gy, g->sh[HY], g->beta, g->stream);
-  prof_mark(g, KK_FILTER64, 16.0 * (double)g->sh[HY].size());
-  nl += 2;
+  launch_filter64x2(hx, Gx, g->sh[HX], hy, Gy, g->sh[HY], g->beta, g->stream);
+  prof_mark(g, KK_FILTER64, 32.0 * (double)g->sh[HX].size());
+  nl += 1;
   if (g->src_wall) {  // the inhomogeneous ghosts of H^{n+1/2} in the filter
     launch_wall_hfilter64(g, Gx, Gy);
     prof_mark(g, KK_SRC, 8.0 * 8.0 * g->N);
@@ -215,10 +213,9 @@ ms_status step64(ms_grid* g) {
     prof_mark(g, KK_SRC, 16.0 * (double)g->sh[EZ].size());
     nl += 2;
   }
-  // the solve's result lands in s64[5]; the last sweep also performs E += h_tau E*
-  p1_solve64(g, EZ, R, g->s64[5], ez, g->ht, &nl);
+  p1_solve64(g, EZ, R, nullptr, ez, g->ht, &nl);  // E += h_tau E*
   // Step 2 on E^{n+1}
-  h_increment64(g, ez, g->s64[5], g->s64[5], hx, hy, &nl, true);
+  h_increment64(g, ez, nullptr, nullptr, hx, hy, &nl, true);
   if (g->nsrc) {
     launch_tick(g);
     prof_mark(g, KK_SRC, 0.0);
@@ -596,8 +593,9 @@ static ms_status create_grid_impl(const ms_grid_desc* d, double* const* shared64
       return cleanup(fail(MS_ECUDA, "copy of Pade tables failed"));
   }
   if (compact) {
-    ms_status sw = ms_solver_sweeps(2, d->r, MS_FP64, 1e-17, &g->p1_sweeps);
-    if (sw != MS_OK) return cleanup(sw);
+    // 6 h^2 P1 = D - T, T in [4, 36] (k_rec64.cu)
+    if (!cheb_coefs(6.0 * g->c1 * g->h * g->h + 36.0, 20.0, 16.0, 1e-17, &g->cheb64))
+      return cleanup(fail(MS_ENOTCONV, "the FP64 solve polynomial needs too high a degree"));
   }
   const size_t nmax = (size_t)(g->N + 1) * (g->N + 1);
   ms_status s = MS_OK;

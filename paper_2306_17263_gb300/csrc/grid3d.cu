@@ -23,6 +23,8 @@
 
 #include "grid3d.cuh"
 #include "k_fp64.cuh"
+#include "k_pdl.cuh"
+#include "k_rec64.cuh"
 #include "k_tiled.cuh"
 #include "k_src3.cuh"
 #include "k_transform.cuh"
@@ -44,7 +46,7 @@ struct Grid3D {
   double* f64[6] = {};
   float* hi[6] = {};
   float* lo[6] = {};
-  double* s64[7] = {};  // FP64: G[3], R, sweep ping-pong [2], solve output; FP32 grids use [0], [1]
+  double* s64[9] = {};  // FP64: G[3], R[3], and, with G again, the work planes of the solves; FP32 grids use [0], [1]
   float* s32[4] = {};   // FP32: differences, R, sweep ping-pong [2]
   float* gh[3] = {};    // FP32: filtered components G~ (hi, lo) of one half-step, slot c % 3
   float* gl[3] = {};
@@ -91,20 +93,30 @@ dim3 grid3(const Shape3& s, dim3 blk) {
 // ---------------------------------------------------------------------------------------
 // FP64 kernels
 
-// G = beta u + (1/12) L u, L = h^2 Delta_h (7 points), 0 at wall points.
-__global__ void k_filter3d64(const double* __restrict__ u, double* __restrict__ G, Shape3 s, double beta) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
-  if (i >= s.n[0] || j >= s.n[1]) return;
+// G = beta u + (1/12) L u, L = h^2 Delta_h (7 points), 0 at wall points; three components per launch.
+struct Filter3d64Args {
+  const double* u[3];
+  double* G[3];
+  Shape3 s[3];
+  int nz;  // planes of the largest component
+};
+__global__ void k_filter3d64(Filter3d64Args A, double c0) {
+  pdl_trigger();
+  pdl_wait();
+  const int f = blockIdx.z / A.nz, k = blockIdx.z - f * A.nz;
+  const Shape3& s = A.s[f];
+  const double* __restrict__ u = A.u[f];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= s.n[0] || j >= s.n[1] || k >= s.n[2]) return;
   const size_t p = at3(s, i, j, k);
   if (!unk3(s, i, j, k)) {
-    G[p] = 0.0;
+    A.G[f][p] = 0.0;
     return;
   }
-  const double c = u[p];
-  const double lap = (u[at3(s, clampi(i - 1, s.n[0]), j, k)] + u[at3(s, clampi(i + 1, s.n[0]), j, k)]) +
-                     (u[at3(s, i, clampi(j - 1, s.n[1]), k)] + u[at3(s, i, clampi(j + 1, s.n[1]), k)]) +
-                     (u[at3(s, i, j, clampi(k - 1, s.n[2]))] + u[at3(s, i, j, clampi(k + 1, s.n[2]))]) - 6.0 * c;
-  G[p] = beta * c + lap * (1.0 / 12.0);
+  const double nb = (u[at3(s, clampi(i - 1, s.n[0]), j, k)] + u[at3(s, clampi(i + 1, s.n[0]), j, k)]) +
+                    (u[at3(s, i, clampi(j - 1, s.n[1]), k)] + u[at3(s, i, clampi(j + 1, s.n[1]), k)]) +
+                    (u[at3(s, i, j, clampi(k - 1, s.n[2]))] + u[at3(s, i, j, clampi(k + 1, s.n[2]))]);
+  A.G[f][p] = fma(c0, u[p], nb * (1.0 / 12.0));  // c0 = beta - 6/12
 }
 
 // Pade band along AXIS (App. A.1): out[o] (+)= scale * sum_t W(r, t) in[r - left + t], r = o - out_off,
@@ -141,41 +153,6 @@ __global__ void k_pade3d64(const double* __restrict__ in, double* __restrict__ o
     v *= scale;
   }
   out[po] = accumulate ? out[po] + v : v;
-}
-
-// One Richardson sweep for P~ x = bscale b, P~ = h^2 P1 = c1h2 - (Lx + Ly + Lz) - (1/6)(LxLy + LyLz + LzLx)
-// (19 points); first != 0: x_in = 0.  upd != nullptr: upd += upd_scale * x_out.
-__global__ void k_sweep3d64(const double* __restrict__ b, const double* __restrict__ xin, double* __restrict__ xout,
-                            Shape3 s, double c1h2, double omega, double bscale, int first, double* __restrict__ upd,
-                            double upd_scale) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
-  if (i >= s.n[0] || j >= s.n[1]) return;
-  const size_t p = at3(s, i, j, k);
-  if (!unk3(s, i, j, k)) {
-    xout[p] = 0.0;
-    return;
-  }
-  double x;
-  if (first) {
-    x = omega * bscale * b[p];
-  } else {
-    const int im = clampi(i - 1, s.n[0]), ip = clampi(i + 1, s.n[0]);
-    const int jm = clampi(j - 1, s.n[1]), jp = clampi(j + 1, s.n[1]);
-    const int km = clampi(k - 1, s.n[2]), kp = clampi(k + 1, s.n[2]);
-    auto X = [&](int a, int bb, int c) { return xin[at3(s, a, bb, c)]; };
-    auto LX = [&](int bb, int c) { return X(im, bb, c) - 2.0 * X(i, bb, c) + X(ip, bb, c); };
-    auto LY = [&](int a, int c) { return X(a, jm, c) - 2.0 * X(a, j, c) + X(a, jp, c); };
-    const double c0 = X(i, j, k);
-    const double lx = LX(j, k), ly = LY(i, k);
-    const double lz = X(i, j, km) - 2.0 * c0 + X(i, j, kp);
-    const double lxly = LX(jm, k) - 2.0 * lx + LX(jp, k);
-    const double lxlz = LX(j, km) - 2.0 * lx + LX(j, kp);
-    const double lylz = LY(i, km) - 2.0 * ly + LY(i, kp);
-    const double px = c1h2 * c0 - (lx + ly + lz) - (lxly + lylz + lxlz) * (1.0 / 6.0);
-    x = c0 + omega * (bscale * b[p] - px);
-  }
-  xout[p] = x;
-  if (upd) upd[p] += upd_scale * x;
 }
 
 __global__ void k_zero_walls3d64(double* __restrict__ u, Shape3 s) {
@@ -871,90 +848,171 @@ __global__ void k_join3(const float* __restrict__ hi, const float* __restrict__ 
 
 const dim3 kBlk(32, 8, 1);
 
-void filter3d64(ms_grid* g, int c, const double* u, double* G) {
-  const Shape3& s = g->g3->sh[c];
-  k_filter3d64<<<grid3(s, kBlk), kBlk, 0, g->stream>>>(u, G, s, g->beta);
-  prof_mark(g, KK_FILTER3D64, 16.0 * (double)s.size());
-}
-
-// out (+)= scale * delta_axis(in), in of component cs, out of component cd
-void pade3d64(ms_grid* g, int axis, int cs, int cd, const double* in, double* out, double scale, int accumulate) {
-  const Shape3& si = g->g3->sh[cs];
-  const Shape3& so = g->g3->sh[cd];
-  const int kind = (si.bc[axis] == NEU) ? HALF_TO_NODE : NODE_TO_HALF;
-  const PadeTable& t = g->pade[kind];
-  const int off = (kind == HALF_TO_NODE) ? 1 : 0;
-  const dim3 grd = grid3(so, kBlk);
-  if (axis == 0)
-    k_pade3d64<0><<<grd, kBlk, 0, g->stream>>>(in, out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                                t.all_explicit, off, scale, accumulate);
-  else if (axis == 1)
-    k_pade3d64<1><<<grd, kBlk, 0, g->stream>>>(in, out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                                t.all_explicit, off, scale, accumulate);
-  else
-    k_pade3d64<2><<<grd, kBlk, 0, g->stream>>>(in, out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                                t.all_explicit, off, scale, accumulate);
-  prof_mark(g, KK_PADE3D64, 8.0 * ((double)si.size() + (accumulate ? 2.0 : 1.0) * (double)so.size()));
-}
-
-// x = P1^{-1} b for component c; the last sweep adds upd_scale * x to upd.
-void solve3d64(ms_grid* g, int c, const double* b, double* upd, double upd_scale, int* nl) {
-  const Shape3& s = g->g3->sh[c];
-  const double c1h2 = g->c1 * g->h * g->h, om = 2.0 / (2.0 * c1h2 + 16.0 / 3.0), h2 = g->h * g->h;
-  double* buf[2] = {g->g3->s64[4], g->g3->s64[5]};
-  const double* xin = nullptr;
-  for (int k = 0; k < g->p1_sweeps; ++k) {
-    const bool last = (k == g->p1_sweeps - 1);
-    double* xo = last ? g->g3->s64[6] : buf[k & 1];
-    k_sweep3d64<<<grid3(s, kBlk), kBlk, 0, g->stream>>>(b, xin, xo, s, c1h2, om, h2, k == 0, last ? upd : nullptr,
-                                                         upd_scale);
-    prof_mark(g, KK_SWEEP3D64, 8.0 * (double)s.size() * ((k == 0 ? 2 : 3) + (last ? 2 : 0)));
-    xin = xo;
+// G[c] = filtered u[c] for the components c0 .. c0 + 2.
+void filter3d64(ms_grid* g, int c0, double* const* u, double* const* G) {
+  Filter3d64Args A;
+  A.nz = 0;
+  double pts = 0.0;
+  int nx = 0, ny = 0;
+  for (int c = 0; c < 3; ++c) {
+    const Shape3& s = g->g3->sh[c0 + c];
+    A.u[c] = u[c];
+    A.G[c] = G[c];
+    A.s[c] = s;
+    A.nz = s.n[2] > A.nz ? s.n[2] : A.nz;
+    nx = s.n[0] > nx ? s.n[0] : nx;
+    ny = s.n[1] > ny ? s.n[1] : ny;
+    pts += (double)s.size();
   }
-  *nl += g->p1_sweeps;
+  launch_pdl(k_filter3d64, dim3((nx + 31) / 32, (ny + 7) / 8, 3 * A.nz), kBlk, 0, g->stream, A, g->beta - 0.5);
+  prof_mark(g, KK_FILTER3D64, 16.0 * pts);
+}
+
+// out (+)= scale * delta_axis(in), in of component shape si, out of shape so
+struct Pade3d64 {
+  int axis;
+  Shape3 si, so;
+  const double* in;
+  double* out;
+  double scale;
+  int accumulate;
+};
+
+LineArgs line_of(const Pade3d64& q, const PadeTable& t) {
+  const int P = q.axis == 0 ? 1 : 0, Q = q.axis == 2 ? 1 : 2;  // the two other axes
+  auto stride = [](const Shape3& s, int a) { return a == 0 ? (size_t)1 : (a == 1 ? (size_t)s.n[0] : (size_t)s.n[0] * s.n[1]); };
+  LineArgs a{};
+  a.in = q.in;
+  a.out = q.out;
+  a.M = t.M;
+  a.out_len = q.so.n[q.axis];
+  a.out_off = q.si.bc[q.axis] == NEU && q.so.bc[q.axis] == DIR ? 1 : 0;
+  a.n0 = q.so.n[P];
+  a.n1 = q.so.n[Q];
+  a.lo = 0;
+  a.hi = a.n0;
+  a.in_sa = stride(q.si, q.axis);
+  a.in_s0 = stride(q.si, P);
+  a.in_s1 = stride(q.si, Q);
+  a.out_sa = stride(q.so, q.axis);
+  a.out_s0 = stride(q.so, P);
+  a.out_s1 = stride(q.so, Q);
+  a.scale = q.scale;
+  a.accumulate = q.accumulate;
+  return a;
+}
+
+// Up to three independent derivatives of one kind (all with axis 0 or none), in one launch; lines
+// shorter than kRecMinLine take the band kernel, one launch each.  Returns the number of launches.
+int pade3d64(ms_grid* g, const Pade3d64* q, int count) {
+  const PadeTable& t = g->pade[q[0].si.bc[q[0].axis] == NEU ? HALF_TO_NODE : NODE_TO_HALF];
+  auto bytes = [&](int k) {
+    return 8.0 * ((double)q[k].si.size() + (q[k].accumulate ? 2.0 : 1.0) * (double)q[k].so.size());
+  };
+  if (t.M >= kRecMinLine) {
+    LineArgs a[kLineBatch];
+    double b = 0.0;
+    for (int k = 0; k < count; ++k) {
+      a[k] = line_of(q[k], t);
+      b += bytes(k);
+    }
+    launch_line64(a, count, t.ends, false, g->stream);
+    prof_mark(g, KK_PADE3D64, b);
+    return 1;
+  }
+  for (int k = 0; k < count; ++k) {
+    const LineArgs a = line_of(q[k], t);
+    const Shape3 &so = q[k].so, &si = q[k].si;
+    const dim3 grd = grid3(so, kBlk);
+    if (q[k].axis == 0)
+      k_pade3d64<0><<<grd, kBlk, 0, g->stream>>>(q[k].in, q[k].out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
+                                                  t.all_explicit, a.out_off, q[k].scale, q[k].accumulate);
+    else if (q[k].axis == 1)
+      k_pade3d64<1><<<grd, kBlk, 0, g->stream>>>(q[k].in, q[k].out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
+                                                  t.all_explicit, a.out_off, q[k].scale, q[k].accumulate);
+    else
+      k_pade3d64<2><<<grd, kBlk, 0, g->stream>>>(q[k].in, q[k].out, so, si, t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
+                                                  t.all_explicit, a.out_off, q[k].scale, q[k].accumulate);
+    prof_mark(g, KK_PADE3D64, bytes(k));
+  }
+  return count;
+}
+
+// R[c] = s (d_{c+1} G_{c+2} - d_{c+2} G_{c+1}) on the components cd0 + c, G of the components cs0 + c.
+// The first launch writes with axes across x only (the terms of axis 1, 2, 1), then the term of axis 2
+// and the two of axis 0 add to it.
+int curl3d64(ms_grid* g, int cs0, int cd0, double* const* G, double* const* R, double s) {
+  Grid3D* G3 = g->g3;
+  auto term = [&](int c, int axis, int acc) {
+    const int p1 = (c + 1) % 3, p2 = (c + 2) % 3;
+    const int src = axis == p1 ? p2 : p1;
+    return Pade3d64{axis, G3->sh[cs0 + src], G3->sh[cd0 + c], G[src], R[c], axis == p1 ? s : -s, acc};
+  };
+  const Pade3d64 first[3] = {term(0, 1, 0), term(1, 2, 0), term(2, 1, 0)};
+  const Pade3d64 second[1] = {term(0, 2, 1)};
+  const Pade3d64 third[2] = {term(1, 0, 1), term(2, 0, 1)};
+  return pade3d64(g, first, 3) + pade3d64(g, second, 1) + pade3d64(g, third, 2);
+}
+
+// x = P1^{-1} b for the components c0 .. c0 + 2; upd[c] += upd_scale x, and, if out is set, out[c] is the
+// work plane that holds x (its wall points are not written).
+void solve3d64(ms_grid* g, int c0, double* const* b, double* const* upd, double upd_scale, const double** out, int* nl) {
+  Grid3D* G3 = g->g3;
+  Cheb3dField f[3];
+  double* buf[3][2];
+  double pts = 0.0;
+  const int m = g->cheb64.m;
+  for (int c = 0; c < 3; ++c) {
+    const Shape3& s = G3->sh[c0 + c];
+    buf[c][0] = G3->s64[c];
+    buf[c][1] = G3->s64[6 + c];
+    f[c].b = b[c];
+    f[c].out = nullptr;
+    f[c].upd = upd ? upd[c] : nullptr;
+    if (out) {
+      f[c].out = buf[c][m & 1];
+      out[c] = f[c].out;
+    }
+    for (int a = 0; a < 3; ++a) {
+      f[c].n[a] = s.n[a];
+      f[c].bc[a] = s.bc[a];
+    }
+    pts += (double)s.size();
+  }
+  launch_cheb3d64(f, buf, 3, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
+  prof_mark(g, KK_SWEEP3D64, 8.0 * pts * (3.0 * (m - 1) + (upd ? 1.0 : 0.0)));
+  *nl += m - 1;
 }
 
 ms_status step3d64(ms_grid* g) {
   Grid3D* G3 = g->g3;
   int nl = 0;
-  double** G = G3->s64;  // G[0..2]
-  double* R = G3->s64[3];
+  double** G = G3->s64;      // G[0..2]
+  double** R = G3->s64 + 3;  // R[0..2]
   const double s_he = g->kappa2 * g->Z / g->h, s_eh = g->kappa2 / (g->Z * g->h);
   if (g->src3) {  // time factors of this step's source terms
     src3_time(g);
     prof_mark(g, KK_SRC, 0.0);
     nl += 1;
   }
+  auto add_src = [&](int c0) {
+    if (!g->src3) return;
+    for (int c = 0; c < 3; ++c) {
+      src3_add(g, c0 + c, R[c]);
+      prof_mark(g, KK_SRC, 16.0 * (double)G3->sh[c0 + c].size());
+      nl += 1;
+    }
+  };
   // Step 1: R_e = kappa^2 Z (d_{e+1} G_{e+2} - d_{e+2} G_{e+1}) on E_e, P1 E* = R, E += h_tau E*
-  for (int c = 0; c < 3; ++c) filter3d64(g, 3 + c, G3->f64[3 + c], G[c]);
-  nl += 3;
-  for (int e = 0; e < 3; ++e) {
-    const int p1 = (e + 1) % 3, p2 = (e + 2) % 3;
-    pade3d64(g, p1, 3 + p2, e, G[p2], R, s_he, 0);
-    pade3d64(g, p2, 3 + p1, e, G[p1], R, -s_he, 1);
-    nl += 2;
-    if (g->src3) {
-      src3_add(g, e, R);
-      prof_mark(g, KK_SRC, 16.0 * (double)G3->sh[e].size());
-      nl += 1;
-    }
-    solve3d64(g, e, R, G3->f64[e], g->ht, &nl);
-  }
+  filter3d64(g, 3, G3->f64 + 3, G);
+  nl += 1 + curl3d64(g, 3, 0, G, R, s_he);
+  add_src(0);
+  solve3d64(g, 0, R, G3->f64, g->ht, nullptr, &nl);
   // Step 2: R_h = -(kappa^2/Z)(d_{h+1} G_{E,h+2} - d_{h+2} G_{E,h+1}) on H_h
-  for (int c = 0; c < 3; ++c) filter3d64(g, c, G3->f64[c], G[c]);
-  nl += 3;
-  for (int hc = 0; hc < 3; ++hc) {
-    const int p1 = (hc + 1) % 3, p2 = (hc + 2) % 3;
-    pade3d64(g, p1, p2, 3 + hc, G[p2], R, -s_eh, 0);
-    pade3d64(g, p2, p1, 3 + hc, G[p1], R, s_eh, 1);
-    nl += 2;
-    if (g->src3) {
-      src3_add(g, 3 + hc, R);
-      prof_mark(g, KK_SRC, 16.0 * (double)G3->sh[3 + hc].size());
-      nl += 1;
-    }
-    solve3d64(g, 3 + hc, R, G3->f64[3 + hc], g->ht, &nl);
-  }
+  filter3d64(g, 0, G3->f64, G);
+  nl += 1 + curl3d64(g, 0, 3, G, R, -s_eh);
+  add_src(3);
+  solve3d64(g, 3, R, G3->f64 + 3, g->ht, nullptr, &nl);
   if (g->src3) {  // the device step index advances with the step
     launch_tick(g);
     prof_mark(g, KK_SRC, 0.0);
@@ -1184,6 +1242,13 @@ int upload_band_row() {
   return 0;
 }
 
+// The polynomial of the FP64 solves: 6 h^2 P1 = D - T, T in [-8, 24] (k_rec64.cu).
+ms_status cheb3d64(ms_grid* g) {
+  if (!cheb_coefs(6.0 * g->c1 * g->h * g->h + 24.0, 8.0, 16.0, 1e-17, &g->cheb64))
+    return fail3(MS_ENOTCONV, "the FP64 solve polynomial needs too high a degree");
+  return MS_OK;
+}
+
 template <typename T>
 ms_status alloc3(T** p, size_t n) {
   cudaError_t e = dev_malloc((void**)p, n * sizeof(T) + 256);
@@ -1397,9 +1462,9 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
       if (s == MS_OK && cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
         s = fail3(MS_ECUDA, "copy of Pade tables failed");
     }
-    if (s == MS_OK) s = ms_solver_sweeps(3, d->r, MS_FP64, 1e-17, &g->p1_sweeps);
+    if (s == MS_OK) s = cheb3d64(g);
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->f64[c], G3->sh[c].size());
-    for (int k = 0; k < 7 && s == MS_OK; ++k) s = alloc3(&G3->s64[k], G3->nmax);
+    for (int k = 0; k < 9 && s == MS_OK; ++k) s = alloc3(&G3->s64[k], G3->nmax);
   } else {
     for (int kind = 0; kind < 2 && s == MS_OK; ++kind) {
       const int M = (kind == HALF_TO_NODE) ? g->N - 1 : g->N;
@@ -1440,7 +1505,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
     if (G3->hi[c]) cudaMemsetAsync(G3->hi[c], 0, n * sizeof(float), g->stream);
     if (G3->lo[c]) cudaMemsetAsync(G3->lo[c], 0, n * sizeof(float), g->stream);
   }
-  for (int k = 0; k < 7; ++k)
+  for (int k = 0; k < 9; ++k)
     if (G3->s64[k]) cudaMemsetAsync(G3->s64[k], 0, G3->nmax * sizeof(double), g->stream);
   for (int k = 0; k < 4; ++k)
     if (G3->s32[k]) cudaMemsetAsync(G3->s32[k], 0, G3->nmax * sizeof(float), g->stream);
@@ -1520,7 +1585,7 @@ void destroy_grid3d(ms_grid* g) {
     dev_free(G3->lo[c]);
     dev_free(G3->dview[c]);
   }
-  for (int k = 0; k < 7; ++k) dev_free(G3->s64[k]);
+  for (int k = 0; k < 9; ++k) dev_free(G3->s64[k]);
   for (int k = 0; k < 4; ++k) dev_free(G3->s32[k]);
   for (int k = 0; k < 3; ++k) {
     dev_free(G3->gh[k]);
@@ -1607,8 +1672,8 @@ ms_status diag_view3d(ms_grid* g, double** f) {
     if (cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail3(MS_ECUDA, "copy of Pade tables failed");
   }
-  if (!g->p1_sweeps) MS3_TRY(ms_solver_sweeps(3, g->desc.r, MS_FP64, 1e-17, &g->p1_sweeps));
-  for (int k = 0; k < 7; ++k)
+  if (!g->cheb64.m) MS3_TRY(cheb3d64(g));
+  for (int k = 0; k < 9; ++k)
     if (!G3->s64[k]) MS3_TRY(alloc3(&G3->s64[k], G3->nmax));
   for (int c = 0; c < 6; ++c) {
     const size_t n = G3->sh[c].size();
@@ -1627,24 +1692,26 @@ ms_status energy3d(ms_grid* g, double* W) {
   double* f[6];
   MS3_TRY(diag_view3d(g, f));
   double** G = G3->s64;  // G[0..2]: filtered E
-  double* R = G3->s64[3];
-  const double* X = G3->s64[6];  // the last sweep's iterate
+  double** R = G3->s64 + 3;
+  const double* X[3];  // the increments
   const double s_eh = g->kappa2 / (g->Z * g->h);
   int nl = 0;
+  filter3d64(g, 0, f, G);
   for (int c = 0; c < 3; ++c) {
-    filter3d64(g, c, f[c], G[c]);
     const size_t n = G3->sh[c].size();
     launch_dot(f[c], f[c], n, g->d_partial, reduce_blocks(n), g->d_result, 0, c > 0, g->stream);
   }
+  curl3d64(g, 0, 3, G, R, -s_eh);
+  for (int c = 0; c < 3; ++c) {  // walls of the work planes, which the solve does not write
+    MS3_CUDA(cudaMemsetAsync(G3->s64[c], 0, G3->nmax * sizeof(double), g->stream));
+    MS3_CUDA(cudaMemsetAsync(G3->s64[6 + c], 0, G3->nmax * sizeof(double), g->stream));
+  }
+  solve3d64(g, 3, R, nullptr, 0.0, X, &nl);
   for (int hc = 0; hc < 3; ++hc) {
-    const int p1 = (hc + 1) % 3, p2 = (hc + 2) % 3;
-    pade3d64(g, p1, p2, 3 + hc, G[p2], R, -s_eh, 0);
-    pade3d64(g, p2, p1, 3 + hc, G[p1], R, s_eh, 1);
-    solve3d64(g, 3 + hc, R, nullptr, 0.0, &nl);
     const size_t n = G3->sh[3 + hc].size();
     const double* Hc = f[3 + hc];
     launch_dot(Hc, Hc, n, g->d_partial, reduce_blocks(n), g->d_result, 1, hc > 0, g->stream);
-    launch_dot(X, Hc, n, g->d_partial, reduce_blocks(n), g->d_result, 2, hc > 0, g->stream);
+    launch_dot(X[hc], Hc, n, g->d_partial, reduce_blocks(n), g->d_result, 2, hc > 0, g->stream);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail3(MS_ECUDA, std::string("3D energy: ") + cudaGetErrorString(e));
@@ -1668,15 +1735,11 @@ ms_status divergence3d(ms_grid* g, double* norm) {
     sc.bc[a] = NEU;
   }
   double* div = G3->s64[0];
-  const PadeTable& t = g->pade[NODE_TO_HALF];
-  const dim3 grd = grid3(sc, kBlk);
   const double sc_h = 1.0 / g->h;
-  k_pade3d64<0><<<grd, kBlk, 0, g->stream>>>(f[3], div, sc, G3->sh[3], t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                              t.all_explicit, 0, sc_h, 0);
-  k_pade3d64<1><<<grd, kBlk, 0, g->stream>>>(f[4], div, sc, G3->sh[4], t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                              t.all_explicit, 0, sc_h, 1);
-  k_pade3d64<2><<<grd, kBlk, 0, g->stream>>>(f[5], div, sc, G3->sh[5], t.d_w, t.rows, t.n_in, t.left, t.K, t.B,
-                                              t.all_explicit, 0, sc_h, 1);
+  for (int a = 0; a < 3; ++a) {
+    const Pade3d64 q{a, G3->sh[3 + a], sc, f[3 + a], div, sc_h, a > 0};
+    pade3d64(g, &q, 1);
+  }
   const size_t n = sc.size();
   launch_dot(div, div, n, g->d_partial, reduce_blocks(n), g->d_result, 0, 0, g->stream);
   cudaError_t e = cudaGetLastError();

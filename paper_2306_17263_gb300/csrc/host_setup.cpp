@@ -10,6 +10,7 @@
 #include <cstring>
 
 #include "k_fp64.cuh"
+#include "k_rec64.cuh"
 
 namespace ms {
 
@@ -156,6 +157,9 @@ int build_pade_table(int M, int closure, int kind, double tol, PadeTable* t, std
   t->rows = M;
   t->n_in = M + 1;
   t->left = K;
+  t->transposed = false;
+  line_ends(closure, kind, false, &t->ends);
+  line_ends(closure, kind, true, &t->ends_T);
   t->all_explicit = (2 * B >= M);
   if (t->all_explicit) B = M;
   t->B = B;
@@ -199,6 +203,8 @@ void build_pade_table_T(const PadeTable& f, PadeTable* t) {
   t->rows = R;
   t->n_in = M;
   t->left = K + 1;
+  t->transposed = true;
+  t->ends = f.ends_T;
   t->all_explicit = f.all_explicit || 2 * B >= R;
   if (t->all_explicit) B = R;
   t->B = B;

@@ -1,9 +1,12 @@
-// FP64 kernels of the compact scheme (MS_FP64): one operator per launch.
+// FP64 kernels of the compact scheme (MS_FP64).
 //
 // GB300 runs FP64 at about 1/60 of its FP32 rate, so this path is bound by the FP64 pipe,
-// not by HBM; it exists as the full-precision form of the step.  Every kernel is an
-// independent-output stencil over a 2D field with coalesced x-fastest access.
+// not by HBM; it exists as the full-precision form of the step.  The kernels here are
+// independent-output stencils over a 2D field with coalesced x-fastest access; the Pade derivatives
+// of all but the shortest lines and the P1 solves of the step are in k_rec64.cu.
 #include "k_fp64.cuh"
+#include "k_pdl.cuh"
+#include "k_rec64.cuh"
 
 namespace ms {
 
@@ -11,21 +14,31 @@ namespace ms {
 // Right-hand-side filter of Eq. "eq:ell": G = beta u + (1/12) L u with L = h^2 Delta_h,
 // Dirichlet boundary points (stored zeros) and even Neumann ghosts (index clamping,
 // Corollary "cor:ghost_cor").  G = 0 on Dirichlet boundary points.
-__global__ void k_filter64(const double* __restrict__ u, double* __restrict__ G, int nx, int ny, int bcx, int bcy,
-                           double beta) {
+// One or two fields per launch (blockIdx.z); five FP64 operations per point.
+struct Filter64Args {
+  const double* u[2];
+  double* G[2];
+  Shape s[2];
+};
+__global__ void k_filter64(Filter64Args A, double c0) {
+  pdl_trigger();
+  pdl_wait();
+  const int f = blockIdx.z;
+  const Shape& s = A.s[f];
+  const double* __restrict__ u = A.u[f];
+  double* __restrict__ G = A.G[f];
+  const int nx = s.nx, ny = s.ny;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= nx || j >= ny) return;
   const size_t p = (size_t)j * nx + i;
-  if (!interior(bcx, i, nx) || !interior(bcy, j, ny)) {
+  if (!interior(s.bcx, i, nx) || !interior(s.bcy, j, ny)) {
     G[p] = 0.0;
     return;
   }
   const int im = clampi(i - 1, nx), ip = clampi(i + 1, nx), jm = clampi(j - 1, ny), jp = clampi(j + 1, ny);
-  const double c = u[p];
-  const double lap = u[(size_t)j * nx + im] + u[(size_t)j * nx + ip] + u[(size_t)jm * nx + i] +
-                     u[(size_t)jp * nx + i] - 4.0 * c;
-  G[p] = beta * c + lap * (1.0 / 12.0);
+  const double nb = (u[(size_t)j * nx + im] + u[(size_t)j * nx + ip]) + (u[(size_t)jm * nx + i] + u[(size_t)jp * nx + i]);
+  G[p] = fma(c0, u[p], nb * (1.0 / 12.0));  // c0 = beta - 4/12
 }
 
 // ---------------------------------------------------------------------------------------
@@ -33,7 +46,8 @@ __global__ void k_filter64(const double* __restrict__ u, double* __restrict__ G,
 // (or of its transpose W^T in the reverse pass):
 //   out[line, o] (+)= scale * sum_{t} W(i, t) in[line, i - left + t],  o = i + out_off,
 // for the M output rows i of the table and inputs 0 .. n_in - 1.
-// AXIS 0: lines are rows (x contiguous); AXIS 1: lines are columns.  Every point of the
+// AXIS 0: lines are rows (x contiguous); AXIS 1: lines are columns.  It serves lines shorter than
+// kRecMinLine, where both ends shape every row; longer ones take the recurrences of k_rec64.cu.  Every point of the
 // output array is written: outputs outside [out_off, out_off + M) or lines outside
 // [line_lo, line_hi) receive 0 (or are left unchanged when accumulating).
 template <int AXIS>
@@ -71,10 +85,9 @@ __global__ void k_pade64(const double* __restrict__ in, double* __restrict__ out
 // One Richardson sweep for P~ x = b~, P~ = h^2 P1 = c1h2 - Lx - Ly - (1/6) Lx Ly (Def.
 // "def:operatorsP" with L = h^2 D_2 per axis, Dirichlet zeros and even Neumann ghosts):
 //   x_out = x_in + omega (bscale * b - P~ x_in),  omega = 2 / (lambda_min + lambda_max).
-// first != 0: x_in is taken as 0 (x_in not read).  upd != nullptr: upd += upd_scale * x_out.
+// first != 0: x_in is taken as 0 (x_in not read).  Used by the allocation-free solve (k_static.cu).
 __global__ void k_p1_sweep64(const double* __restrict__ b, const double* __restrict__ xin, double* __restrict__ xout,
-                             int nx, int ny, int bcx, int bcy, double c1h2, double omega, double bscale, int first,
-                             double* __restrict__ upd, double upd_scale) {
+                             int nx, int ny, int bcx, int bcy, double c1h2, double omega, double bscale, int first) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= nx || j >= ny) return;
@@ -102,7 +115,6 @@ __global__ void k_p1_sweep64(const double* __restrict__ b, const double* __restr
     x = c + omega * (bscale * b[p] - px);
   }
   xout[p] = x;
-  if (upd) upd[p] += upd_scale * x;
 }
 
 // P~ x (the matrix-free operator alone), scaled by out_scale.
@@ -157,14 +169,44 @@ __global__ void k_yee_h64(const double* __restrict__ ez, double* __restrict__ hx
 
 static inline dim3 grid2(int nx, int ny, dim3 blk) { return dim3((nx + blk.x - 1) / blk.x, (ny + blk.y - 1) / blk.y); }
 
+void launch_filter64x2(const double* u0, double* G0, const Shape& s0, const double* u1, double* G1, const Shape& s1,
+                       double beta, cudaStream_t st) {
+  const dim3 blk(32, 8);
+  const Filter64Args A{{u0, u1}, {G0, G1}, {s0, s1}};
+  dim3 grd = grid2(s0.nx > s1.nx ? s0.nx : s1.nx, s0.ny > s1.ny ? s0.ny : s1.ny, blk);
+  grd.z = 2;
+  launch_pdl(k_filter64, grd, blk, 0, st, A, beta - 4.0 / 12.0);
+}
+
 void launch_filter64(const double* u, double* G, const Shape& s, double beta, cudaStream_t st) {
-  dim3 blk(32, 8);
-  k_filter64<<<grid2(s.nx, s.ny, blk), blk, 0, st>>>(u, G, s.nx, s.ny, s.bcx, s.bcy, beta);
+  const dim3 blk(32, 8);
+  const Filter64Args A{{u, u}, {G, G}, {s, s}};
+  launch_pdl(k_filter64, grid2(s.nx, s.ny, blk), blk, 0, st, A, beta - 4.0 / 12.0);
 }
 
 void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_ld, int out_len, int out_ld,
                    int out_off, int line_lo, int line_hi, const PadeTable& t, double scale, int accumulate,
                    cudaStream_t st) {
+  if (t.M >= kRecMinLine) {
+    LineArgs a{};
+    a.in = in;
+    a.out = out;
+    a.M = t.M;
+    a.out_len = out_len;
+    a.out_off = out_off;
+    a.n0 = n_lines;
+    a.n1 = 1;
+    a.lo = line_lo;
+    a.hi = line_hi;
+    a.in_sa = axis == 0 ? 1 : in_ld;
+    a.in_s0 = axis == 0 ? in_ld : 1;
+    a.out_sa = axis == 0 ? 1 : out_ld;
+    a.out_s0 = axis == 0 ? out_ld : 1;
+    a.scale = scale;
+    a.accumulate = accumulate;
+    launch_line64(&a, 1, t.ends, t.transposed, st);
+    return;
+  }
   dim3 blk(32, 8);
   if (axis == 0) {
     k_pade64<0><<<grid2(out_len, n_lines, blk), blk, 0, st>>>(in, out, n_lines, t.rows, in_ld, out_len, out_ld,
@@ -178,10 +220,10 @@ void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_
 }
 
 void launch_p1_sweep64(const double* b, const double* xin, double* xout, const Shape& s, double c1h2, double omega,
-                       double bscale, int first, double* upd, double upd_scale, cudaStream_t st) {
+                       double bscale, int first, cudaStream_t st) {
   dim3 blk(32, 8);
   k_p1_sweep64<<<grid2(s.nx, s.ny, blk), blk, 0, st>>>(b, xin, xout, s.nx, s.ny, s.bcx, s.bcy, c1h2, omega, bscale,
-                                                        first, upd, upd_scale);
+                                                        first);
 }
 
 void launch_p1_apply64(const double* x, double* out, const Shape& s, double c1h2, double out_scale, cudaStream_t st) {

@@ -24,11 +24,13 @@ __host__ __device__ __forceinline__ const T* pade_row_ptr(const T* tab, int i, i
 }
 
 void launch_filter64(const double* u, double* G, const Shape& s, double beta, cudaStream_t st);
+void launch_filter64x2(const double* u0, double* G0, const Shape& s0, const double* u1, double* G1, const Shape& s1,
+                       double beta, cudaStream_t st);
 void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_ld, int out_len, int out_ld,
                    int out_off, int line_lo, int line_hi, const PadeTable& t, double scale, int accumulate,
                    cudaStream_t st);
 void launch_p1_sweep64(const double* b, const double* xin, double* xout, const Shape& s, double c1h2, double omega,
-                       double bscale, int first, double* upd, double upd_scale, cudaStream_t st);
+                       double bscale, int first, cudaStream_t st);
 void launch_p1_apply64(const double* x, double* out, const Shape& s, double c1h2, double out_scale, cudaStream_t st);
 void launch_yee_e64(double* ez, const double* hx, const double* hy, int N, double c_e, cudaStream_t st);
 void launch_yee_h64(const double* ez, double* hx, double* hy, int N, double c_h, cudaStream_t st);
@@ -69,9 +71,12 @@ void launch_wall_hsolve64(ms_grid* g, double* Rx, double* Ry);
 void launch_nc_e64(double* ez, const double* hx, const double* hy, int N, double c_e, cudaStream_t st);
 void launch_nc_h64(const double* ez, double* hx, double* hy, int N, double c_h, cudaStream_t st);
 
-// x = P1^{-1} b for field f by the FP64 Richardson sweeps (scratch planes s64[3], s64[4]); the
-// last sweep writes `out` and, when upd != nullptr, adds upd_scale * x to upd (capi.cu).
+// x = P1^{-1} b for field f (k_rec64.cu): writes `out` (if not nullptr; it may be b, then s64[5] is
+// scratch) and, when upd != nullptr, adds upd_scale * x to upd; work planes s64[3], s64[4].  The second
+// form solves both H fields with the work planes given (capi.cu).
 void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl);
+void p1_solve64_h(ms_grid* g, const double* bx, const double* by, double* outx, double* outy, double* updx, double* updy,
+                  double upd_scale, double* const (*buf)[2], int* nl);
 // Reverse pass (adjoint.cu): releases the transposed tables, adjoint planes and graphs.
 void adjoint_teardown(ms_grid* g);
 

@@ -55,7 +55,7 @@ extern "C" ms_status ms_p1_solve_static(int n, double r, int field, const double
   }
   const ms::Shape s = ms::field_shape(n, field);
   // P~ = h^2 P1 = c1h2 - Lx - Ly - (1/6) Lx Ly, c1h2 = (24/r^2)(1 + 2/r^2), spectrum in
-  // [c1h2, c1h2 + 16/3]; the same sweep count, relaxation and kernel as the grid's FP64 solve.
+  // [c1h2, c1h2 + 16/3]; Richardson sweeps to the tolerance of the grid's FP64 solve.
   const double c1h2 = (24.0 / (r * r)) * (1.0 + 2.0 / (r * r));
   const double rho = (16.0 / 3.0) / (2.0 * c1h2 + 16.0 / 3.0);
   int S = (int)std::ceil(std::log(1e-17) / std::log(rho));
@@ -67,7 +67,7 @@ extern "C" ms_status ms_p1_solve_static(int n, double r, int field, const double
   const double* xin = nullptr;
   for (int k = 0; k < S; ++k) {
     double* xo = (k == S - 1) ? x : buf[k & 1];
-    ms::launch_p1_sweep64(b, xin, xo, s, c1h2, omega, h2, k == 0, nullptr, 0.0, st);
+    ms::launch_p1_sweep64(b, xin, xo, s, c1h2, omega, h2, k == 0, st);
     xin = xo;
   }
   cudaError_t e = cudaGetLastError();

@@ -21,6 +21,24 @@ struct Shape {
 };
 Shape field_shape(int N, int f);
 
+// rho^kRecWarm < 1.6e-19: a recurrence started that many rows outside a segment has forgotten its start.
+constexpr int kRecWarm = 14;
+// End rows of A^{-1} (or of its transpose) on a line of M rows.  With Y the solution of the infinite
+// Toeplitz line for the zero-extended right-hand side, the solution with the closure's end rows is
+// Y_i + v_i (g_0 Y_0 + .. + g_3 Y_3) at the first end, and its mirror image at the last.
+struct LineEnds {
+  double v[kRecWarm];
+  double g[4];
+};
+
+// Polynomial solve of P1 (k_rec64.cu): y <- b + q[k] T y for k = m-1 .. 1, x = p0 y.
+constexpr int kChebMax = 12;
+struct Cheb {
+  int m = 0;
+  double q[kChebMax + 1] = {};
+  double p0 = 0;
+};
+
 // Explicit banded form of the Pade derivative W = A^{-1} D1~ of one line type (App. A.1,
 // Eq. "eq:lhs"), D1~ the plain two-point difference (M x (M+1)), so that delta f = (1/h) W f.
 // Output i uses inputs i-K .. i+K+1.  Rows [0, B) and [M-B, M) are stored explicitly, the
@@ -32,6 +50,8 @@ struct PadeTable {
   // reading inputs i - left .. i - left + 2K + 1.  Forward tables: rows = M, n_in = M + 1,
   // left = K.  Transposed tables (W^T, the reverse pass): rows = M + 1, n_in = M, left = K + 1.
   int rows = 0, n_in = 0, left = 0;
+  bool transposed = false;
+  LineEnds ends, ends_T;             // end corrections of the recurrences of this table, of its transpose
   std::vector<double> w;             // (2B + 1) rows x (2K + 2)
   double* d_w = nullptr;             // device copy (FP64)
   float* d_whi = nullptr;            // device FP32 split: w = whi + wlo exactly to ~2^-48
@@ -106,7 +126,7 @@ struct ms_grid {
 
   // Pade tables: [0] half->node (M = N-1), [1] node->half (M = N)
   ms::PadeTable pade[2];
-  int p1_sweeps = 0;  // Richardson sweeps for the FP64 solve
+  ms::Cheb cheb64;  // polynomial of the FP64 solve
   // FP32 path: tables truncated for FP32 and split hi/lo; Richardson sweeps for FP32
   ms::PadeTable pade32[2];
   int p1_sweeps32 = 0;
