@@ -1,7 +1,7 @@
 // Reverse (adjoint) pass of the FP32_REFINED step in FP32 arithmetic with a float-float adjoint
 // state.
 //
-// The FP32_REFINED forward step, in the units of its tile kernels (k_tiled.cu, k_mixed.cu), is
+// The FP32_REFINED forward step, in the units of k_mixed.cu, is
 //   S1: E   += sE P~_E^{-1} (Y_x F~ H_y - Y_y F~ H_x),
 //   S2: H_x += sH P~_Hx^{-1} (-Y_y F~ E),   H_y += sH P~_Hy^{-1} (Y_x F~ E),
 // with P~ = 6 h^2 P1 (Def. "def:operatorsP"), F~ = 12 beta + L the filter of Eq. "eq:ell" on the
@@ -27,7 +27,7 @@
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
-#include "k_tiled.cuh"
+#include "k_walk.cuh"
 
 namespace ms {
 
@@ -133,7 +133,7 @@ __device__ __forceinline__ void ff_fma_acc(float& sh, float& sl, float w, float 
 // past the line) are staged once in shared memory with coalesced loads; outputs whose window lies
 // in the interior rows of the table read the one interior row.
 constexpr int BT_THREADS = 256;
-constexpr int BT_KMAX = kTiledKMax;
+constexpr int BT_KMAX = kBand32Max;
 template <int AXIS>
 struct BandTile {
   static constexpr int LINES = AXIS == 0 ? 8 : 32;

@@ -17,7 +17,7 @@
 #include "k_mixed.cuh"
 #include "k_rec64.cuh"
 #include "k_src3.cuh"
-#include "k_tiled.cuh"
+#include "k_walk.cuh"
 #include "k_tracked32.cuh"
 
 using namespace ms;
@@ -343,7 +343,7 @@ ms_status state64(ms_grid* g, double* dst[3], const double* view[3]) {
     if (g->desc.precision == MS_FP64) {
       view[f] = g->f64[f];
     } else {
-      launch_join(g->hi[f], g->lo[f], dst[f], g->sh[f].size(), g->stream);
+      launch_join2d(g->hi[f], g->lo[f], g->ld32, dst[f], g->sh[f], g->stream);
       view[f] = dst[f];
     }
   }
@@ -358,11 +358,7 @@ ms_status store_state(ms_grid* g, const double* const* src) {
         MS_CUDA(cudaMemcpyAsync(g->f64[f], src[f], n * sizeof(double), cudaMemcpyDeviceToDevice, g->stream));
       launch_zero_dirichlet64(g->f64[f], g->sh[f], g->stream);
     } else {
-      // zero the Dirichlet entries in a scratch copy, then split
-      double* tmp = g->s64[0];
-      MS_CUDA(cudaMemcpyAsync(tmp, src[f], n * sizeof(double), cudaMemcpyDeviceToDevice, g->stream));
-      launch_zero_dirichlet64(tmp, g->sh[f], g->stream);
-      launch_split(tmp, g->hi[f], g->lo[f], n, g->stream);
+      launch_split2d(src[f], g->hi[f], g->lo[f], g->ld32, g->sh[f], g->stream);  // zero on Dirichlet walls
     }
   }
   return check_launch("store state");
@@ -481,7 +477,7 @@ ms_status ms_stability_limit(int dim, double* rmax) {
 // Largest Richardson sweep count the solve kernels of a precision hold.
 static int max_sweeps(int dim, int precision) {
   if (precision == MS_FP64) return 64;
-  return dim == 2 ? kTiledMaxSweeps : kMaxSweeps3d32;
+  return dim == 2 ? kMaxSweeps32 : kMaxSweeps3d32;
 }
 
 ms_status ms_solver_sweeps(int dim, double r, int precision, double tol, int* sweeps) {
@@ -613,8 +609,6 @@ static ms_status create_grid_impl(const ms_grid_desc* d, double* const* shared64
       if (s == MS_OK) cudaMemsetAsync(g->de64, 0, g->sh[EZ].size() * sizeof(double), g->stream);
     }
   } else {
-    for (int f = 0; f < 3 && s == MS_OK; ++f) s = dalloc(&g->hi[f], g->sh[f].size());
-    for (int f = 0; f < 3 && s == MS_OK; ++f) s = dalloc(&g->lo[f], g->sh[f].size());
     if (s == MS_OK) {
       s = mixed_setup(g);
       if (s != MS_OK) fail(s, mixed_last_error());
@@ -629,8 +623,6 @@ static ms_status create_grid_impl(const ms_grid_desc* d, double* const* shared64
   if (s != MS_OK) return cleanup(s);
   for (int f = 0; f < 3; ++f) {
     if (g->f64[f]) cudaMemsetAsync(g->f64[f], 0, g->sh[f].size() * sizeof(double), g->stream);
-    if (g->hi[f]) cudaMemsetAsync(g->hi[f], 0, g->sh[f].size() * sizeof(float), g->stream);
-    if (g->lo[f]) cudaMemsetAsync(g->lo[f], 0, g->sh[f].size() * sizeof(float), g->stream);
   }
   for (int k = 0; k < 6 && !g->shared64; ++k)
     if (g->s64[k]) cudaMemsetAsync(g->s64[k], 0, nmax * sizeof(double), g->stream);
@@ -655,8 +647,6 @@ ms_status ms_destroy(ms_grid* g) {
   }
   for (int f = 0; f < 3; ++f) {
     dev_free(g->f64[f]);
-    dev_free(g->hi[f]);
-    dev_free(g->lo[f]);
   }
   dev_free(g->de64);
   tracked32_teardown(g);
@@ -668,7 +658,6 @@ ms_status ms_destroy(ms_grid* g) {
   dev_free(g->d_wresp);
   dev_free(g->d_step);
   for (int k = 0; k < 6 && !g->shared64; ++k) dev_free(g->s64[k]);
-  for (int k = 0; k < 8; ++k) dev_free(g->s32[k]);
   mixed_teardown(g);
   dev_free(g->d_partial);
   dev_free(g->d_result);
@@ -713,7 +702,7 @@ ms_status ms_set_fields_device(ms_grid* g, const double* const* comps, long step
   MS_TRY(store_state(g, comps));
   if (g->de64) launch_lap_e64(g->f64[EZ], g->de64, g->N, g->h, g->stream);  // DE^0 = Delta_h E^0
   if (g->de_hi) {  // DE^0 = Delta_h E^0 of the stored (wall-zeroed) E
-    launch_join(g->hi[EZ], g->lo[EZ], g->s64[1], g->sh[EZ].size(), g->stream);
+    launch_join2d(g->hi[EZ], g->lo[EZ], g->ld32, g->s64[1], g->sh[EZ], g->stream);
     launch_lap_e64(g->s64[1], g->s64[0], g->N, g->h, g->stream);
     tracked32_set_de(g, g->s64[0]);
   }
@@ -731,7 +720,7 @@ ms_status ms_get_fields_device(ms_grid* g, double* const* comps) {
     if (g->desc.precision == MS_FP64)
       MS_CUDA(cudaMemcpyAsync(comps[f], g->f64[f], n * sizeof(double), cudaMemcpyDeviceToDevice, g->stream));
     else
-      launch_join(g->hi[f], g->lo[f], comps[f], n, g->stream);
+      launch_join2d(g->hi[f], g->lo[f], g->ld32, comps[f], g->sh[f], g->stream);
   }
   return check_launch("get fields");
 }
@@ -751,7 +740,7 @@ ms_status ms_set_fields(ms_grid* g, const double* const* comps, long step) {
   MS_TRY(store_state(g, dst));
   if (g->de64) launch_lap_e64(g->f64[EZ], g->de64, g->N, g->h, g->stream);  // DE^0 = Delta_h E^0
   if (g->de_hi) {  // DE^0 = Delta_h E^0 of the stored (wall-zeroed) E
-    launch_join(g->hi[EZ], g->lo[EZ], g->s64[1], g->sh[EZ].size(), g->stream);
+    launch_join2d(g->hi[EZ], g->lo[EZ], g->ld32, g->s64[1], g->sh[EZ], g->stream);
     launch_lap_e64(g->s64[1], g->s64[0], g->N, g->h, g->stream);
     tracked32_set_de(g, g->s64[0]);
   }
@@ -1167,7 +1156,7 @@ struct ms_batch {
   ms_grid_desc desc{};
   std::vector<ms_grid*> cav;
   double* s64[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  ms::TiledBatch tb;
+  ms::WalkBatch tb;
   ms::Graph graph1, graphk;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -1188,7 +1177,7 @@ ms_status batch_cavity(ms_batch* b, int cavity, ms_grid** g) {
 }
 
 ms_status batch_step_launch(ms_batch* b) {
-  tiled_batch_step(b->tb, b->stream, b->plan[2]);
+  walk_batch_step(b->tb, b->stream, b->plan[2]);
   return check_launch("batch step");
 }
 
@@ -1196,9 +1185,9 @@ ms_status batch_step_launch(ms_batch* b) {
 ms_status batch_apply_plan(ms_batch* b, const int* plan) {
   if (plan[0] != b->plan[0]) {
     MS_CUDA(cudaStreamSynchronize(b->stream));
-    tiled_batch_free(&b->tb);
+    walk_batch_free(&b->tb);
     std::string err;
-    if (tiled_batch_build(b->cav.data(), (int)b->cav.size(), plan[0], &b->tb, &err) != 0) return fail(MS_ENOMEM, err);
+    if (walk_batch_build(b->cav.data(), (int)b->cav.size(), plan[0], &b->tb, &err) != 0) return fail(MS_ENOMEM, err);
   }
   free_graph(&b->graph1);
   free_graph(&b->graphk);
@@ -1292,7 +1281,7 @@ ms_status ms_batch_destroy(ms_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   free_graph(&b->graph1);
   free_graph(&b->graphk);
-  tiled_batch_free(&b->tb);
+  walk_batch_free(&b->tb);
   for (ms_grid* g : b->cav) ms_destroy(g);
   for (int k = 0; k < 6; ++k) dev_free(b->s64[k]);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -1344,7 +1333,7 @@ ms_status ms_create_batch(const ms_grid_desc* d, const int* n, int count, ms_bat
     b->cells += (long long)n[c] * n[c];
   }
   std::string err;
-  if (tiled_batch_build(b->cav.data(), count, b->plan[0], &b->tb, &err) != 0) return cleanup(fail(MS_ENOMEM, err));
+  if (walk_batch_build(b->cav.data(), count, b->plan[0], &b->tb, &err) != 0) return cleanup(fail(MS_ENOMEM, err));
   *out = b;
   return MS_OK;
 }

@@ -30,23 +30,41 @@ struct Hdr {
   long long step;
 };
 
+// FP32 planes of pitch ld floats hold rows of w; 3D arrays are one row.
+struct Rows {
+  size_t w, ld;
+};
+
 // Device arrays of the state (2D: E_z, H_x, H_y [+ Delta E_z]; 3D: six components).
-int state_arrays(ms_grid* g, double** f64, float** hi, float** lo, size_t* n) {
-  if (g->g3) return state_arrays3d(g, f64, hi, lo, n);
+int state_arrays(ms_grid* g, double** f64, float** hi, float** lo, size_t* n, Rows* rows) {
+  if (g->g3) {
+    const int nc = state_arrays3d(g, f64, hi, lo, n);
+    for (int c = 0; c < nc; ++c) rows[c] = Rows{n[c], n[c]};
+    return nc;
+  }
   for (int f = 0; f < 3; ++f) {
     f64[f] = g->f64[f];
     hi[f] = g->hi[f];
     lo[f] = g->lo[f];
     n[f] = g->sh[f].size();
+    rows[f] = Rows{(size_t)g->sh[f].nx, (size_t)g->ld32};
   }
   if (g->de64 || g->de_hi) {
     f64[3] = g->de64;
     hi[3] = g->de_hi;
     lo[3] = g->de_lo;
     n[3] = g->sh[EZ].size();
+    rows[3] = rows[EZ];
     return 4;
   }
   return 3;
+}
+
+// n floats between a packed host array and a device plane.
+cudaError_t copy_plane(float* dst, const float* src, size_t n, const Rows& r, cudaMemcpyKind kind) {
+  const bool out = kind == cudaMemcpyDeviceToHost;
+  return cudaMemcpy2D(dst, (out ? r.w : r.ld) * sizeof(float), src, (out ? r.ld : r.w) * sizeof(float),
+                      r.w * sizeof(float), n / r.w, kind);
 }
 
 }  // namespace
@@ -62,7 +80,8 @@ ms_status ms_save(ms_grid* g, const char* path) {
   float* hi[7];
   float* lo[7];
   size_t n[7];
-  const int nc = state_arrays(g, f64, hi, lo, n);
+  Rows rows[7];
+  const int nc = state_arrays(g, f64, hi, lo, n, rows);
   if (cudaStreamSynchronize(g->stream) != cudaSuccess) return cfail(MS_ECUDA, "stream synchronisation failed");
   FILE* fp = std::fopen(path, "wb");
   if (!fp) return cfail(MS_EINVAL, std::string("cannot open ") + path + " for writing");
@@ -83,7 +102,7 @@ ms_status ms_save(ms_grid* g, const char* path) {
     } else {
       std::vector<float> buf(n[c]);
       for (float* arr : {hi[c], lo[c]}) {
-        ok = ok && cudaMemcpy(buf.data(), arr, n[c] * sizeof(float), cudaMemcpyDeviceToHost) == cudaSuccess;
+        ok = ok && copy_plane(buf.data(), arr, n[c], rows[c], cudaMemcpyDeviceToHost) == cudaSuccess;
         ok = ok && std::fwrite(buf.data(), sizeof(float), n[c], fp) == n[c];
       }
     }
@@ -98,7 +117,8 @@ ms_status ms_load(ms_grid* g, const char* path) {
   float* hi[7];
   float* lo[7];
   size_t n[7];
-  const int nc = state_arrays(g, f64, hi, lo, n);
+  Rows rows[7];
+  const int nc = state_arrays(g, f64, hi, lo, n, rows);
   FILE* fp = std::fopen(path, "rb");
   if (!fp) return cfail(MS_EINVAL, std::string("cannot open ") + path);
   char magic[8];
@@ -150,8 +170,8 @@ ms_status ms_load(ms_grid* g, const char* path) {
     if (f64[c]) {
       cp = cudaMemcpy(f64[c], b64[c].data(), n[c] * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
     } else {
-      cp = cudaMemcpy(hi[c], b32[2 * c].data(), n[c] * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
-           cudaMemcpy(lo[c], b32[2 * c + 1].data(), n[c] * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+      cp = copy_plane(hi[c], b32[2 * c].data(), n[c], rows[c], cudaMemcpyHostToDevice) == cudaSuccess &&
+           copy_plane(lo[c], b32[2 * c + 1].data(), n[c], rows[c], cudaMemcpyHostToDevice) == cudaSuccess;
     }
     if (!cp) return cfail(MS_ECUDA, "copying the checkpoint to the device failed");
   }

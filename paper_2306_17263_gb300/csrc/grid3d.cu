@@ -25,7 +25,7 @@
 #include "k_fp64.cuh"
 #include "k_pdl.cuh"
 #include "k_rec64.cuh"
-#include "k_tiled.cuh"
+#include "k_walk.cuh"
 #include "k_src3.cuh"
 #include "k_transform.cuh"
 
@@ -101,7 +101,6 @@ struct Filter3d64Args {
   int nz;  // planes of the largest component
 };
 __global__ void k_filter3d64(Filter3d64Args A, double c0) {
-  pdl_trigger();
   pdl_wait();
   const int f = blockIdx.z / A.nz, k = blockIdx.z - f * A.nz;
   const Shape3& s = A.s[f];

@@ -135,6 +135,34 @@ void launch_join(const float* hi, const float* lo, double* v, size_t n, cudaStre
   k_join<<<reduce_blocks(n), kRedThreads, 0, st>>>(hi, lo, v, n);
 }
 
+// The same between a dense FP64 field and pitched FP32 planes; the split stores 0 on Dirichlet walls.
+__global__ void k_split2d(const double* __restrict__ v, float* __restrict__ hi, float* __restrict__ lo, int ld, int nx,
+                          int ny, int bcx, int bcy) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= nx || j >= ny) return;
+  const double x = interior(bcx, i, nx) && interior(bcy, j, ny) ? v[(size_t)j * nx + i] : 0.0;
+  const float h = (float)x;
+  hi[(size_t)j * ld + i] = h;
+  lo[(size_t)j * ld + i] = (float)(x - (double)h);
+}
+
+__global__ void k_join2d(const float* __restrict__ hi, const float* __restrict__ lo, int ld, double* __restrict__ v,
+                         int nx, int ny) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= nx || j >= ny) return;
+  v[(size_t)j * nx + i] = (double)hi[(size_t)j * ld + i] + (double)lo[(size_t)j * ld + i];
+}
+
+void launch_split2d(const double* v, float* hi, float* lo, int ld, const Shape& s, cudaStream_t st) {
+  const dim3 blk(32, 8), grd((s.nx + 31) / 32, (s.ny + 7) / 8);
+  k_split2d<<<grd, blk, 0, st>>>(v, hi, lo, ld, s.nx, s.ny, s.bcx, s.bcy);
+}
+
+void launch_join2d(const float* hi, const float* lo, int ld, double* v, const Shape& s, cudaStream_t st) {
+  const dim3 blk(32, 8), grd((s.nx + 31) / 32, (s.ny + 7) / 8);
+  k_join2d<<<grd, blk, 0, st>>>(hi, lo, ld, v, s.nx, s.ny);
+}
+
 __global__ void k_zero_dirichlet64(double* __restrict__ u, int nx, int ny, int bcx, int bcy) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;

@@ -21,7 +21,6 @@ struct Filter64Args {
   Shape s[2];
 };
 __global__ void k_filter64(Filter64Args A, double c0) {
-  pdl_trigger();
   pdl_wait();
   const int f = blockIdx.z;
   const Shape& s = A.s[f];

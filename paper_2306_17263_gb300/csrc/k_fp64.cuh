@@ -54,8 +54,9 @@ size_t src_factor_bytes();
 void launch_src_time(ms_grid* g, double scale_e, double scale_h);
 void launch_src_e64(ms_grid* g, double* R);
 void launch_src_h64(ms_grid* g, double* Rx, double* Ry);
-void launch_src_e32(ms_grid* g, float* R, double scale_e);
-void launch_src_h32(ms_grid* g, float* Rx, float* Ry, double scale_h);
+// FP32 planes of pitch ld
+void launch_src_e32(ms_grid* g, float* R, int ld, double scale_e);
+void launch_src_h32(ms_grid* g, float* Rx, float* Ry, int ld, double scale_h);
 // FP32 wall terms: the wall data of a step (launched after launch_src_time) and, on the host, the
 // Pade responses to the end values of a line.
 void launch_wall_data(ms_grid* g);
@@ -93,6 +94,8 @@ void launch_dot(const double* a, const double* b, size_t n, double* partial, int
 // FP32 hi/lo <-> FP64 conversion
 void launch_split(const double* v, float* hi, float* lo, size_t n, cudaStream_t st);
 void launch_join(const float* hi, const float* lo, double* v, size_t n, cudaStream_t st);
+void launch_split2d(const double* v, float* hi, float* lo, int ld, const Shape& s, cudaStream_t st);
+void launch_join2d(const float* hi, const float* lo, int ld, double* v, const Shape& s, cudaStream_t st);
 void launch_zero_dirichlet64(double* u, const Shape& s, cudaStream_t st);
 int reduce_blocks(size_t n);
 

@@ -16,19 +16,19 @@
 // values (|D1 G| ~ theta |G|, theta = pi k h), so an FP32 rounding of G at the level of |G|
 // would be amplified by 1/theta in every step.  The kernels therefore take the first
 // differences of the float-float state, (hi_{m+1} - hi_m) + (lo_{m+1} - lo_m), filter the
-// differences (the filter commutes with D1~), and only then apply the well-conditioned A^{-1}
-// band.  The Richardson residual forms the dominant diagonal product exactly (FMA), and
-// the last correction is added to the state separately so the iteration cannot stall into a
-// coherent bias.  The state is a float-float pair updated with error-free transformations.
+// differences (the filter commutes with D1~), and only then apply the well-conditioned A^{-1}.
+// The last correction of the solve is added to the state separately, so that no rounding of the
+// solution itself shrinks every increment the same way.  The state is a float-float pair updated with
+// error-free transformations.
 //
-// Kernels (k_tiled.cu): one right-hand-side tile kernel and one solve-and-update tile kernel
-// per half-step, i.e. four launches per time step.
+// Kernels (k_walk.cu): the derivatives along both axes, then the solve and the update, per half-step,
+// i.e. four launches per time step.
 #include <cmath>
 #include <string>
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
-#include "k_tiled.cuh"
+#include "k_walk.cuh"
 
 namespace ms {
 
@@ -71,18 +71,18 @@ MixedConsts mixed_consts(const ms_grid* g) {
 ms_status step_mixed(ms_grid* g, int* nl) {
   const double N1 = g->N + 1.0, Nd = g->N;
   const double ne = N1 * N1, nh = Nd * N1;  // points of E_z and of each H component
-  const MixedConsts k = mixed_consts(g);
-  // Step 1: b = A^{-1} D1 G~_y (along x) - A^{-1} D1 G~_x (along y) on E_z, then the E solve
-  float* bE = g->s32[4];
-  tiled_curl(g, 0, k.cb_hi, k.cb_lo, bE, nullptr);
+  // Step 1: b on E_z in two planes, then the E solve and update
+  walk_d(g, 0);
   // recorded bytes: the state each launch must touch (8 B per point per float-float read or
   // write), the algorithmic bytes of a step being 48 B per cell (each component read and written
-  // once); the right-hand-side planes b are intermediates and are not counted
-  prof_mark(g, KK_CURL32, 8.0 * 2.0 * nh);                   // H_x, H_y (hi, lo) read
-  // sources in the units of b: 6 h^2 P1 x = b with E += (12 Z / r) x, so b = (h^3 r^2 / (2 Z)) R
-  const double hr2 = g->h * g->h * g->h * g->desc.r * g->desc.r;
-  if (g->nsrc) {  // H += (12 / (r Z)) x, so b = (h^3 r^2 Z / 2) R on the H side
-    launch_src_time(g, hr2 / (2.0 * g->Z), hr2 * g->Z / 2.0);
+  // once); the right-hand-side planes are intermediates and are not counted
+  prof_mark(g, KK_CURL32, 16.0 * nh);                        // H_x, H_y (hi, lo) read
+  // sources in the units of b: 6 h^2 P1 x = (1 - rho)^2 b with E += (12 Z / r) x, so
+  // b = (h^3 r^2 / (2 Z)) R / (1 - rho)^2; H += (12 / (r Z)) x, b = (h^3 r^2 Z / 2) R / (1 - rho)^2
+  const double hr2 = g->h * g->h * g->h * g->desc.r * g->desc.r / walk_rhs_scale();
+  const double scale_e = hr2 / (2.0 * g->Z), scale_h = hr2 * g->Z / 2.0;
+  if (g->nsrc) {
+    launch_src_time(g, scale_e, scale_h);
     prof_mark(g, KK_SRC, 0.0);
     *nl += 1;
     if (g->d_walldata) {
@@ -90,27 +90,21 @@ ms_status step_mixed(ms_grid* g, int* nl) {
       prof_mark(g, KK_SRC, 8.0 * 12.0 * N1);
       *nl += 1;
     }
-    launch_src_e32(g, bE, hr2 / (2.0 * g->Z));
+    launch_src_e32(g, g->s32[4], g->ld32, scale_e);
     prof_mark(g, KK_SRC, 8.0 * ne);
     *nl += 1;
   }
-  const int fe[1] = {EZ};
-  const float* be[1] = {bE};
-  tiled_solve(g, 1, fe, be, k.S, k.d_hi, k.d_lo, k.omega, k.sE_hi, k.sE_lo);
-  prof_mark(g, KK_SOLVE32, 16.0 * ne);                       // E (hi, lo) read and written
-  // Step 2: b_x = -A^{-1} D1 G~_E (along y), b_y = +A^{-1} D1 G~_E (along x), then both H solves
-  float* bx = g->s32[2];
-  float* by = g->s32[3];
-  tiled_curl(g, 1, k.cb_hi, k.cb_lo, bx, by);
-  prof_mark(g, KK_CURL32, 8.0 * ne);                         // E (hi, lo) read
+  walk_s(g, 0);
+  prof_mark(g, KK_SOLVE32, 16.0 * ne);                       // E_z (hi, lo) read and written
+  // Step 2: b_x and b_y, then both H solves and updates
+  walk_d(g, 1);
+  prof_mark(g, KK_CURL32, 8.0 * ne);                         // E_z (hi, lo) read
   if (g->nsrc) {
-    launch_src_h32(g, bx, by, hr2 * g->Z / 2.0);
+    launch_src_h32(g, g->s32[2], g->s32[3], g->ld32, scale_h);
     prof_mark(g, KK_SRC, 16.0 * nh);
     *nl += 1;
   }
-  const int fh[2] = {HX, HY};
-  const float* bh[2] = {bx, by};
-  tiled_solve(g, 2, fh, bh, k.S, k.d_hi, k.d_lo, k.omega, k.sH_hi, k.sH_lo);
+  walk_s(g, 1);
   prof_mark(g, KK_SOLVE32, 16.0 * 2.0 * nh);                 // H_x, H_y (hi, lo) read and written
   if (g->nsrc) {
     launch_tick(g);
@@ -130,9 +124,9 @@ ms_status mixed_setup(ms_grid* g) {
       g_mixed_err = err;
       return MS_EINVAL;
     }
-    // the explicit rows of the tile kernels hold half-widths up to kTiledKMax
-    if (t.K > kTiledKMax) {
-      g_mixed_err = "FP32 Pade band half-width outside the range the tile kernels hold";
+    // the band kernels (tracked form, reverse pass) hold half-widths up to kBand32Max
+    if (t.K > kBand32Max) {
+      g_mixed_err = "FP32 Pade band half-width outside the range the kernels hold";
       return MS_EUNSUPPORTED;
     }
     std::vector<float> whi(t.w.size()), wlo(t.w.size());
@@ -152,25 +146,35 @@ ms_status mixed_setup(ms_grid* g) {
       return MS_ECUDA;
     }
   }
-  // Richardson sweeps to 1e-10 (below the FP32 rounding noise, which is not coherent)
+  // Richardson sweeps of the reverse pass to 1e-10 (below the FP32 rounding noise, which is not coherent)
   const ms_status sw = ms_solver_sweeps(2, g->desc.r, MS_FP32_REFINED, 1e-10, &g->p1_sweeps32);
   if (sw != MS_OK) {
-    g_mixed_err = "too many Richardson sweeps for the FP32 tile solve";
+    g_mixed_err = "too many Richardson sweeps for the FP32 solve";
     return sw;
   }
-  if (tiled_configure() != 0) {
-    g_mixed_err = "cannot configure shared memory of the tile kernels";
+  const ms_status wk = walk_setup(g);
+  if (wk != MS_OK) {
+    g_mixed_err = "the FP32 solve polynomial needs too high a degree";
+    return wk;
+  }
+  // state and right-hand-side planes in one allocation
+  const size_t pl = plane_floats(g->N);
+  if (dev_malloc(&g->slab32, 10 * pl * sizeof(float)) != cudaSuccess) {
+    g_mixed_err = "cudaMalloc of the FP32 planes failed";
+    return MS_ENOMEM;
+  }
+  if (cudaMemsetAsync(g->slab32, 0, 10 * pl * sizeof(float), g->stream) != cudaSuccess) {
+    g_mixed_err = "clearing the FP32 planes failed";
     return MS_ECUDA;
   }
-  // right-hand-side planes of the tile kernels: s32[4] (E_z), s32[2] (H_x), s32[3] (H_y)
-  const size_t nmax = (size_t)(g->N + 1) * (g->N + 1);
-  for (int k = 2; k < 5; ++k) {
-    if (dev_malloc(&g->s32[k], nmax * sizeof(float) + 256) != cudaSuccess) {
-      g_mixed_err = "cudaMalloc of FP32 scratch failed";
-      return MS_ENOMEM;
-    }
-    cudaMemset(g->s32[k], 0, nmax * sizeof(float));
+  for (int f = 0; f < 3; ++f) {
+    g->hi[f] = g->slab32 + f * pl + plane_origin(f);
+    g->lo[f] = g->slab32 + (3 + f) * pl + plane_origin(f);
   }
+  g->s32[2] = g->slab32 + 6 * pl + plane_origin(HX);
+  g->s32[3] = g->slab32 + 7 * pl + plane_origin(HY);
+  g->s32[4] = g->slab32 + 8 * pl + plane_origin(EZ);
+  g->s32[1] = g->slab32 + 9 * pl + plane_origin(EZ);
   return MS_OK;
 }
 
@@ -180,6 +184,8 @@ void mixed_teardown(ms_grid* g) {
     dev_free(g->pade32[k].d_wlo);
     g->pade32[k].d_whi = g->pade32[k].d_wlo = nullptr;
   }
+  dev_free(g->slab32);
+  g->slab32 = nullptr;
 }
 
 }  // namespace ms

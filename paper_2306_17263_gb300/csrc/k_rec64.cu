@@ -72,14 +72,14 @@ void line_ends(int closure, int kind, bool transposed, LineEnds* e) {
   e->g[1] = e->g[2] = e->g[3] = 0.0;
 }
 
-bool cheb_coefs(double D, double c, double s, double tol, Cheb* p) {
+bool cheb_coefs(double D, double c, double s, double tol, Cheb* p, int mmin) {
   // T_m((t - c) / s) as a polynomial in t, and its value at D
   const int n = kChebMax + 1;
   long double a[kChebMax + 2] = {1.0L}, b[kChebMax + 2] = {-(long double)c / s, 1.0L / (long double)s};
   const long double x = ((long double)D - c) / s;
   long double va = 1.0L, vb = x;
   int m = 1;
-  while (m < 2 || 1.0L / vb > tol) {
+  while (m < mmin || 1.0L / vb > tol) {
     if (++m > kChebMax) return false;
     long double t[kChebMax + 2] = {};
     for (int k = 0; k < n; ++k) t[k] = 2.0L * (-(long double)c / s * b[k] + (k ? b[k - 1] / s : 0.0L)) - a[k];
@@ -184,7 +184,6 @@ constexpr double kOneMinusRhoSq = 1.093172397520265540654504;  // (1 - rho)^2 = 
 // one before it stops there), so both ends and the rows they correct sit at fixed places of a segment.
 template <int L, bool TRANS>
 __global__ void __launch_bounds__(32 * LW) k_line_walk64(LineBatch b) {
-  pdl_trigger();
   pdl_wait();
   const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
   const LineArgs& a = b.a[which];
@@ -229,7 +228,6 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
   constexpr int OUTS = LW * L, PW = OUTS + 2 * kRecWarm + 3;  // odd
   static_assert(PW % 2 == 1, "odd row pitch");
   __shared__ double sm[32 * PW];
-  pdl_trigger();
   pdl_wait();
   const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
   const LineArgs& a = b.a[which];
@@ -350,7 +348,6 @@ static_assert(3 * 8 * (16 + 2 * (kChebMax - 1)) * (16 + 2 * (kChebMax - 1)) <= 4
 // Neumann wall the ghost equals its mirror, the point itself.
 __global__ void __launch_bounds__(C2T) k_cheb2d64(Cheb2dArgs A) {
   extern __shared__ double sm64[];
-  pdl_trigger();
   pdl_wait();
   const Cheb2dField& F = A.f[blockIdx.z];
   const int nx = F.s.nx, ny = F.s.ny;
@@ -422,7 +419,6 @@ struct Cheb2dLevel {
 };
 template <bool LAST>
 __global__ void __launch_bounds__(128) k_cheb2d64_level(Cheb2dLevel A) {
-  pdl_trigger();
   pdl_wait();
   const int fi = blockIdx.z;
   const Cheb2dField& F = A.f[fi];
@@ -536,7 +532,6 @@ struct Cheb3dArgs {
 
 template <bool LAST>
 __global__ void __launch_bounds__(C3T) k_cheb3d64(Cheb3dArgs A) {
-  pdl_trigger();
   pdl_wait();
   const int which = blockIdx.y / A.nz, kz = blockIdx.y - which * A.nz;
   const Cheb3dField& F = A.f[which];

@@ -16,7 +16,8 @@ void line_ends(int closure, int kind, bool transposed, LineEnds* e);
 // x = scale * y, y the polynomial p(T) b / p_0 in Horner form, y <- b + q[k] T y for k = m-1 .. 1,
 // p(t) ~ 1 / (D - t) with the relative error of the Chebyshev polynomial of degree m on the spectrum
 // [c - s, c + s] of T: 1 / T_m((D - c) / s) <= tol.
-bool cheb_coefs(double D, double c, double s, double tol, Cheb* p);
+// At least degree mmin; false if kChebMax is not enough.
+bool cheb_coefs(double D, double c, double s, double tol, Cheb* p, int mmin = 2);
 
 // out (+)= scale * delta in along a line (App. A.1), or its transpose: `axis_stride_*` between points
 // of a line, n0 lines apart by s0_*, n1 apart by s1_*.  Output r (0 .. rows-1) goes to point r + out_off

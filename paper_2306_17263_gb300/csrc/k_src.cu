@@ -18,8 +18,8 @@
 //     next to the wall; in the H solves of Step 2 (data of H* = (H^{n+3/2} - H^{n+1/2}) / h_tau)
 //     the right-hand side loses P1 applied to the ghosts alone, which is nonzero next to the wall;
 //   - G_E on the boundary nodes is (h^2/12) Delta E_z = (h^2/12) Z d_t J_z at t^{n+1}.
-// The FP64 step applies them with k_wall_hfilter64 / k_wall_ge64 / k_wall_hsolve64.  The FP32 tile
-// curl never forms G, so there the filter's ghost terms and G_E on the walls enter b as their Pade
+// The FP64 step applies them with k_wall_hfilter64 / k_wall_ge64 / k_wall_hsolve64.  The FP32 walk
+// never forms G, so there the filter's ghost terms and G_E on the walls enter b as their Pade
 // responses (the curl is linear in G), added by the FP32 source kernels with the ghost part of P1.
 #include <cmath>
 #include <cstring>
@@ -40,7 +40,7 @@ struct SrcDev {
 // The time factors are the same at every point: a one-block kernel at the start of each step
 // forms them (k_src_time), and the point kernels read them.  FP64: v = sum_q (ce_q sin(w_q t))
 // X_q(i) Y_q(j), the product taken in the order of the plain definition.  FP32 (right-hand sides of
-// the tile solve): the factors are scaled to the tile's units and rounded to float, and the sum is
+// k_walk.cu): the factors are scaled to their units and rounded to float, and the sum is
 // taken in float from the float copy of the tables.
 constexpr int kMaxSrc = 64;
 struct SrcFac {
@@ -97,7 +97,7 @@ constexpr int kSrcRows = 8;
 //   kappa^2 Z / h (W_{i-1,0} (-g^y_lo(j) / 12) + W_{i-1,N-1} g^y_hi(j) / 12
 //                  - W_{j-1,0} (-g^x_lo(i) / 12) - W_{j-1,N-1} g^x_hi(i) / 12)   (W = A^{-1} D1 per line).
 template <typename T>
-__global__ void __launch_bounds__(32 * kSrcBy) k_src_e(T* __restrict__ R, int N, int nsrc, const double* __restrict__ tab,
+__global__ void __launch_bounds__(32 * kSrcBy) k_src_e(T* __restrict__ R, int ld, int N, int nsrc, const double* __restrict__ tab,
                                                        const float* __restrict__ tab32, const SrcFac* __restrict__ fac,
                                                        WallView wv, float cE) {
   const int i = blockIdx.x * 32 + threadIdx.x;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_e(T* __restrict__ R, int N,
 #pragma unroll
   for (int r = 0; r < kSrcRows; ++r) {
     const int j = j0 + r * kSrcBy;
-    old[r] = (j >= 1 && j < N) ? R[(size_t)j * (N + 1) + i] : (T)0;
+    old[r] = (j >= 1 && j < N) ? R[(size_t)j * ld + i] : (T)0;
     v[r] = (T)0;
   }
   for (int q = 0; q < nsrc; ++q) {
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_e(T* __restrict__ R, int N,
         v[r] = fmaf(cE * (1.0f / 12.0f), ax - ay, v[r]);
       }
     }
-    R[(size_t)j * (N + 1) + i] = old[r] + v[r];
+    R[(size_t)j * ld + i] = old[r] + v[r];
   }
 }
 
@@ -159,7 +159,8 @@ __device__ __forceinline__ double ghost_p1(const double* g, int k) {
 // +cH (W_{i,0} v(0, j) + W_{i,N} v(N, j)) on R_y (cH = scale kappa^2 / (Z h)), minus the ghost part of
 // P1 with the data of H* next to the walls (times sP = scale / h^2).
 template <typename T>
-__global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __restrict__ Ry, int N, int nsrc,
+__global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __restrict__ Ry, int ldx, int ldy,
+                                                       int N, int nsrc,
                                                        const double* __restrict__ tab, const float* __restrict__ tab32,
                                                        const SrcFac* __restrict__ fac, WallView wv, float cH, double sP) {
   const int i = blockIdx.x * 32 + threadIdx.x;
@@ -172,8 +173,8 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __
 #pragma unroll
   for (int r = 0; r < kSrcRows; ++r) {
     const int j = j0 + r * kSrcBy;
-    ox[r] = (ix && j < N) ? Rx[(size_t)j * (N + 1) + i] : (T)0;
-    oy[r] = (iy && j >= 1 && j < N) ? Ry[(size_t)j * N + i] : (T)0;
+    ox[r] = (ix && j < N) ? Rx[(size_t)j * ldx + i] : (T)0;
+    oy[r] = (iy && j >= 1 && j < N) ? Ry[(size_t)j * ldy + i] : (T)0;
     vx[r] = (T)0;
     vy[r] = (T)0;
   }
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __
           if (j == N - 1) vx[r] += (float)(sP * ghost_p1(wd + WD_SX_HI * L, i));
         }
       }
-      Rx[(size_t)j * (N + 1) + i] = ox[r] + vx[r];
+      Rx[(size_t)j * ldx + i] = ox[r] + vx[r];
     }
     if (iy && j >= 1 && j < N) {
       if constexpr (sizeof(T) == 4) {
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __
           if (i == N - 1) vy[r] -= (float)(sP * ghost_p1(wd + WD_SY_HI * L, j));
         }
       }
-      Ry[(size_t)j * N + i] = oy[r] - vy[r];
+      Ry[(size_t)j * ldy + i] = oy[r] - vy[r];
     }
   }
 }
@@ -408,26 +409,26 @@ static dim3 src_grid(int N) { return dim3((N + 1 + 31) / 32, (N + 1 + kSrcBy * k
 
 void launch_src_e64(ms_grid* g, double* R) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
-  k_src_e<double><<<grd, blk, 0, g->stream>>>(R, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  k_src_e<double><<<grd, blk, 0, g->stream>>>(R, g->N + 1, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                                (const SrcFac*)g->d_srcfac, WallView{}, 0.0f);
 }
 void launch_src_h64(ms_grid* g, double* Rx, double* Ry) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
-  k_src_h<double><<<grd, blk, 0, g->stream>>>(Rx, Ry, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  k_src_h<double><<<grd, blk, 0, g->stream>>>(Rx, Ry, g->N + 1, g->N, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                                (const SrcFac*)g->d_srcfac, WallView{}, 0.0f, 0.0);
 }
-void launch_src_e32(ms_grid* g, float* R, double scale_e) {
+void launch_src_e32(ms_grid* g, float* R, int ld, double scale_e) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
   const WallView wv = g->d_walldata ? wall_view(g->d_walldata, g->d_wresp, g->N) : WallView{};
   const float cE = (float)(scale_e * g->kappa2 * g->Z / g->h);
-  k_src_e<float><<<grd, blk, 0, g->stream>>>(R, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  k_src_e<float><<<grd, blk, 0, g->stream>>>(R, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                               (const SrcFac*)g->d_srcfac, wv, cE);
 }
-void launch_src_h32(ms_grid* g, float* Rx, float* Ry, double scale_h) {
+void launch_src_h32(ms_grid* g, float* Rx, float* Ry, int ld, double scale_h) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
   const WallView wv = g->d_walldata ? wall_view(g->d_walldata, g->d_wresp, g->N) : WallView{};
   const float cH = (float)(scale_h * g->kappa2 / (g->Z * g->h));
-  k_src_h<float><<<grd, blk, 0, g->stream>>>(Rx, Ry, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  k_src_h<float><<<grd, blk, 0, g->stream>>>(Rx, Ry, ld, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                               (const SrcFac*)g->d_srcfac, wv, cH, scale_h / (g->h * g->h));
 }
 void launch_wall_data(ms_grid* g) {

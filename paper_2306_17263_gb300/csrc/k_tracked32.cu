@@ -10,11 +10,11 @@
 // the Pade derivative of the unfiltered H (App. A.1) taken on exact first differences (two-sum of
 // the hi parts plus the difference of the lo parts) through a band whose central taps are summed
 // in float-float (exact two-products) and whose far taps, below 1.2e-4 of the centre, in FP32.
-// Step 2 then runs the tile curl of the FP32 step on G~_E with its filter switched off.
+// Step 2 then runs the walks of the FP32 step on G~_E with their filter switched off.
 #include <cmath>
 
 #include "k_fp64.cuh"
-#include "k_tiled.cuh"
+#include "k_walk.cuh"
 #include "k_tracked32.cuh"
 
 namespace ms {
@@ -69,7 +69,7 @@ struct BandF {
 // are columns): 32 lines x 32 outputs, lanes across the lines.  The differences a tile reads (its
 // outputs widened by the band's reach, zero past the line) are staged once in shared memory.
 constexpr int BF_THREADS = 256;
-constexpr int BF_KMAX = kTiledKMax;
+constexpr int BF_KMAX = kBand32Max;
 template <int AXIS>
 struct BandFTile {
   static constexpr int LINES = AXIS == 0 ? 8 : 32;
@@ -166,12 +166,12 @@ __global__ void k_de_combine32(const float* __restrict__ eh, const float* __rest
                                const float* __restrict__ oh, const float* __restrict__ ol,
                                const float* __restrict__ xh, const float* __restrict__ xl,
                                const float* __restrict__ yh, const float* __restrict__ yl, float* __restrict__ dh,
-                               float* __restrict__ dl, float* __restrict__ gh, float* __restrict__ gl, int n,
+                               float* __restrict__ dl, float* __restrict__ gh, float* __restrict__ gl, int n, int ld,
                                float k2_hi, float k2_lo, float cz_hi, float cz_lo, float cb_hi, float cb_lo,
                                float h2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= n || j >= n) return;
-  const size_t p = (size_t)j * n + i;
+  const size_t p = (size_t)j * ld + i;
   if (i == 0 || j == 0 || i == n - 1 || j == n - 1) {
     dh[p] = dl[p] = gh[p] = gl[p] = 0.0f;
     return;
@@ -222,28 +222,23 @@ Split2 split2(double v) {
 }  // namespace
 
 ms_status tracked32_setup(ms_grid* g) {
-  const size_t n = g->sh[EZ].size();
-  float** planes[] = {&g->de_hi, &g->de_lo, &g->t32[0], &g->t32[1], &g->t32[2], &g->t32[3],
-                      &g->t32[4], &g->t32[5], &g->t32[6], &g->t32[7]};
-  for (float** q : planes) {
-    if (dev_malloc(q, n * sizeof(float) + 256) != cudaSuccess) return MS_ENOMEM;
-    if (cudaMemsetAsync(*q, 0, n * sizeof(float) + 256, g->stream) != cudaSuccess) return MS_ECUDA;
-  }
+  const size_t pl = plane_floats(g->N);
+  float** planes[10] = {&g->de_hi, &g->de_lo, &g->t32[0], &g->t32[1], &g->t32[2], &g->t32[3],
+                        &g->t32[4], &g->t32[5], &g->t32[6], &g->t32[7]};
+  if (dev_malloc(&g->slab_de, 10 * pl * sizeof(float)) != cudaSuccess) return MS_ENOMEM;
+  if (cudaMemsetAsync(g->slab_de, 0, 10 * pl * sizeof(float), g->stream) != cudaSuccess) return MS_ECUDA;
+  for (int k = 0; k < 10; ++k) *planes[k] = g->slab_de + k * pl + plane_origin(EZ);
   return MS_OK;
 }
 
 void tracked32_teardown(ms_grid* g) {
-  dev_free(g->de_hi);
-  dev_free(g->de_lo);
-  g->de_hi = g->de_lo = nullptr;
-  for (int k = 0; k < 8; ++k) {
-    dev_free(g->t32[k]);
-    g->t32[k] = nullptr;
-  }
+  dev_free(g->slab_de);
+  g->slab_de = g->de_hi = g->de_lo = nullptr;
+  for (int k = 0; k < 8; ++k) g->t32[k] = nullptr;
 }
 
 void tracked32_set_de(ms_grid* g, const double* de) {
-  launch_split(de, g->de_hi, g->de_lo, g->sh[EZ].size(), g->stream);
+  launch_split2d(de, g->de_hi, g->de_lo, g->ld32, g->sh[EZ], g->stream);
 }
 
 ms_status step_mixed_tracked(ms_grid* g, int* nl) {
@@ -251,18 +246,16 @@ ms_status step_mixed_tracked(ms_grid* g, int* nl) {
   const double N1 = N + 1.0, Nd = N;
   const double ne = N1 * N1, nh = Nd * N1;
   const MixedConsts k = mixed_consts(g);
-  const size_t nE = g->sh[EZ].size();
+  const size_t nE = plane_floats(N) - plane_origin(EZ);  // a plane from its point (0, 0) on
+  const int ld = g->ld32;
   // Step 1 as in the FP32 step, keeping E^n for the increment
   if (cudaMemcpyAsync(g->t32[0], g->hi[EZ], nE * sizeof(float), cudaMemcpyDeviceToDevice, g->stream) != cudaSuccess ||
       cudaMemcpyAsync(g->t32[1], g->lo[EZ], nE * sizeof(float), cudaMemcpyDeviceToDevice, g->stream) != cudaSuccess)
     return MS_ECUDA;
   prof_mark(g, KK_TRACKED32, 16.0 * ne);
-  float* bE = g->s32[4];
-  tiled_curl(g, 0, k.cb_hi, k.cb_lo, bE, nullptr);
-  prof_mark(g, KK_CURL32, 8.0 * 2.0 * nh);
-  const int fe[1] = {EZ};
-  const float* be[1] = {bE};
-  tiled_solve(g, 1, fe, be, k.S, k.d_hi, k.d_lo, k.omega, k.sE_hi, k.sE_lo);
+  walk_d(g, 0);
+  prof_mark(g, KK_CURL32, 16.0 * nh);
+  walk_s(g, 0);
   prof_mark(g, KK_SOLVE32, 16.0 * ne);
   // the unfiltered Pade curl of H in float-float: y_x = W delta_x H_y, y_y = W delta_y H_x
   const PadeTable& t = g->pade32[HALF_TO_NODE];
@@ -272,9 +265,9 @@ ms_status step_mixed_tracked(ms_grid* g, int* nl) {
   bx.yh = g->t32[2];
   bx.yl_ = g->t32[3];
   bx.ua = 1;
-  bx.ul = g->sh[HY].nx;  // H_y rows: N half-node values, N + 1 rows
+  bx.ul = ld;  // H_y rows: N half-node values, N + 1 rows
   bx.ya = 1;
-  bx.yl = N + 1;
+  bx.yl = ld;
   bx.nlines = N + 1;
   bx.whi = t.d_whi;
   bx.wlo = t.d_wlo;
@@ -287,9 +280,9 @@ ms_status step_mixed_tracked(ms_grid* g, int* nl) {
   by.ul_ = g->lo[HX];
   by.yh = g->t32[4];
   by.yl_ = g->t32[5];
-  by.ua = g->sh[HX].nx;  // H_x columns: N + 1 columns of N half-node values
+  by.ua = ld;  // H_x columns: N + 1 columns of N half-node values
   by.ul = 1;
-  by.ya = N + 1;
+  by.ya = ld;
   by.yl = 1;
   {
     using T0 = BandFTile<0>;
@@ -307,18 +300,14 @@ ms_status step_mixed_tracked(ms_grid* g, int* nl) {
     const Split2 k2 = split2(g->kappa2), cz = split2(24.0 * g->Z / (ht * h));
     const dim3 blk(32, 8), grd((N + 1 + 31) / 32, (N + 1 + 7) / 8);
     k_de_combine32<<<grd, blk, 0, g->stream>>>(g->hi[EZ], g->lo[EZ], g->t32[0], g->t32[1], g->t32[2], g->t32[3],
-                                               g->t32[4], g->t32[5], g->de_hi, g->de_lo, g->t32[6], g->t32[7], N + 1,
+                                               g->t32[4], g->t32[5], g->de_hi, g->de_lo, g->t32[6], g->t32[7], N + 1, ld,
                                                k2.hi, k2.lo, cz.hi, cz.lo, k.cb_hi, k.cb_lo, (float)(h * h));
     prof_mark(g, KK_TRACKED32, 4.0 * 12.0 * ne);
   }
-  // Step 2 on G~_E with the filter off, then both H solves
-  float* bxp = g->s32[2];
-  float* byp = g->s32[3];
-  tiled_curl_unfiltered(g, g->t32[6], g->t32[7], bxp, byp);
+  // Step 2 on G~_E with the filter off
+  walk_d(g, 1, g->t32[6], g->t32[7]);
   prof_mark(g, KK_CURL32, 8.0 * ne);
-  const int fh[2] = {HX, HY};
-  const float* bh[2] = {bxp, byp};
-  tiled_solve(g, 2, fh, bh, k.S, k.d_hi, k.d_lo, k.omega, k.sH_hi, k.sH_lo);
+  walk_s(g, 1);
   prof_mark(g, KK_SOLVE32, 16.0 * 2.0 * nh);
   *nl += 9;
   const cudaError_t e = cudaGetLastError();

@@ -1,0 +1,1004 @@
+// FP32_REFINED step of 2D grids.  Two launches per half-step, both made of warps that walk along y with
+// everything they carry in registers: no shared memory, no barriers.
+//
+//   walk_d : the Pade derivatives (App. A.1, Eq. "eq:lhs") of the filtered source into right-hand-side
+//            planes, one plane per axis.  Along y a lane takes one column (30 of 32 lanes write, the
+//            outer two hold the neighbour columns of the filter) and walks down its segment of the line.
+//            Along x a lane takes four adjacent columns of a row (a warp 128, of which it writes 112)
+//            and walks down a block of rows, carrying the differences of the rows above and below.
+//   walk_s : the solve of P1 (Def. "def:operatorsP") and the float-float update E += h_tau E* /
+//            H += h_tau H*.  A lane takes four adjacent columns (a warp 128, of which it writes 120)
+//            and walks down a block of rows; the levels of the solve follow one another a row apart,
+//            so no iterate is stored and the state is read and written once.
+//
+// Differences are taken on the float-float state, delta_m = (hi_{m+1} - hi_m) + (lo_{m+1} - lo_m), and
+// filtered, d = 12 beta delta + L delta (the filter of Eq. "eq:ell" commutes with the difference: D1
+// (12 beta + L) u = (12 beta + L') D1 u with the ghost rules below).  A^{-1} d is the two first-order
+// recurrences A factors into, z_i = d_i + rho z_{i-1} and y_i = z_i + rho y_{i+1}, up to the factor (1 -
+// rho)^2 that the increment scales carry, each z and y rounded once.  Along y the forward one follows the
+// walk and the backward one runs over groups of eight rows from seven rows beyond (|rho|^8 = 2e-11);
+// along x a lane runs both over its four columns and takes the carries of two lanes on either side.  The closure's end rows
+// change the solution by a multiple of the decaying vector rho^i (LineEnds), added to the first and the
+// last eight rows of a line.
+//
+// Ghost rules of the difference along a line: a source that is Neumann along it (H_y along x, H_x along
+// y; even ghost u(-1) = u(0), Cor. "cor:ghost_cor") has zero differences beyond the ends; one that is
+// Dirichlet (E_z, zero at the wall, filter zero there) even ones (delta_{-1} = delta_0).  Across the line
+// every source is Dirichlet with stored zeros.
+//
+// The solve is the Chebyshev polynomial of k_rec64.cu, 6 h^2 P1 = D - T with T = (L_x + 6)(L_y + 6), in
+// Horner form y <- b + q T y to a relative error of 1e-10: five operations per point and level.  T y is
+// 7e-3 of D y at most, so an FP32 level rounds the increment at 1e-9 of itself, and the last level's
+// q T y enters the state apart from b, never rounded into it.
+//
+// Why walks: both kernels of the tile form this replaces (64 x 64 tiles in shared memory) were bound by
+// instruction issue, 140-150 warp instructions per 32 points and field.  Derivative along x and solve in
+// one walk (no plane between them) was tried: 146 registers leave 12 warps per SM, and with a chain of
+// eight shuffles per row it ran 66 us for E_z at 2048^2.
+#include <algorithm>
+#include <cmath>
+#include <string>
+#include <vector>
+
+#include "k_fp64.cuh"
+#include "k_pdl.cuh"
+#include "k_rec64.cuh"
+#include "k_walk.cuh"
+
+namespace ms {
+
+constexpr int kEnd = 8;  // rows of a line the end correction reaches
+
+// Arguments of a derivative along y: lines are the columns 1 .. ncol-2 of the source.
+struct YArgs {
+  const float* sh;  // source, point (0, 0)
+  const float* sl;
+  float* b;         // destination plane, row of output 0, column 0
+  int ld, ncol, M, even;
+  float cb_hi, cb_lo;  // 12 beta - 4: coefficient of delta beside the sum of its four neighbours
+  float g[4], v[kEnd];
+  int nstrip, nseg, chunk, rb;  // column strips; segments of `chunk` rows, the last one [rb, M)
+  // grids of at most kTinyN cells: explicit rows of A^{-1}, every derivative of the half-step
+  int tiny, step, N;
+  const float *th[2], *tl[2];  // sources: Step 1 H_y, H_x; Step 2 E_z
+  float* tb[2];
+  const float *whi, *wlo;
+  int K;
+  float tcb_hi, tcb_lo;  // 12 beta
+  int filter;
+};
+
+// Arguments of a derivative along x; pointers at column m = 0 (the first unknown one) of row 0.
+struct XArgs {
+  const float* sh;  // source
+  const float* sl;
+  float* b;         // destination plane
+  int ld, M;        // outputs 0 .. M-1 of every row
+  int u0, u1;       // rows u0 .. u1-1
+  float cb_hi, cb_lo;
+  float g[4], v[kEnd];
+  int nstrip, nblk, rows;
+};
+
+// Arguments of walk_s for one field; pointers at the first unknown column of row 0.
+struct SArgs {
+  const float* p1;  // right-hand side; of E_z the sum of two planes
+  const float* p2;
+  float* hi;
+  float* lo;
+  int ld, M;        // unknown columns 0 .. M-1
+  int u0, u1;       // unknown rows u0 .. u1-1
+  int kind;         // KIND_*
+  float q[4];          // level l + 1 of the solve
+  float s_hi, s_lo;    // increment scale
+  int nstrip, nblk, rows;
+};
+
+namespace {
+
+constexpr float kRhoF = -0.045548850f;  // rounds to the FP32 root
+constexpr float kR2 = kRhoF * kRhoF, kR4 = kR2 * kR2;
+constexpr int WPB = 4;      // warps per block
+constexpr int YOUT = 30;    // columns a walk_y warp writes
+constexpr int XOUT = 112;   // columns a warp writes along x
+constexpr int XHALO = 8;
+constexpr int SOUT = 120;   // columns a walk_s warp writes
+constexpr int SHALO = 4;
+constexpr unsigned kFull = 0xffffffffu;
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// Paired FP32 instructions (two correctly rounded operations each, bitwise those of the scalar ones): the
+// walks are bound by instruction issue.  a - b as one FMA with -1, which rounds the same.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
+
+// Rows come through a ring in shared memory that each warp fills for itself with cp.async, kAhead rows
+// ahead: the walk of a row is shorter than a memory round trip, and the registers are taken.  A slot is
+// refilled one row after it was read.
+constexpr int kAhead = 3, kRing = kAhead + 1;
+__device__ __forceinline__ void cp16(float4* dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// ---- derivative along y --------------------------------------------------------------------------------
+
+// One segment of 32 columns.  Rows m = r0 - 9 .. are pushed through the recurrences in groups of eight;
+// the y of a group lags its last row by seven, so the first two groups only warm up.  EDGE: rows of the
+// walk may lie beyond the line's ends.
+template <bool FILTER, bool EDGE>
+__device__ __forceinline__ void y_segment(const YArgs& A, int strip, int seg) {
+  const int lane = threadIdx.x & 31;
+  const int col = YOUT * strip + lane;
+  const bool live = lane >= 1 && lane <= YOUT && col <= A.ncol - 2;
+  const bool last = seg == A.nseg - 1;
+  const int r0 = last ? A.rb : seg * A.chunk, r1 = last ? A.M : min(r0 + A.chunk, A.rb);
+  const size_t ld = A.ld;
+  const int cc = min(col, A.ncol - 1);
+  const float* ph = A.sh + cc;
+  const float* pl = A.sl + cc;
+  auto row = [&](int r) { return EDGE ? (size_t)min(max(r, 0), A.M) * ld : (size_t)r * ld; };
+  const int ms = r0 - 9;
+  // u at rows ms - 1, ms, ms + 1 -> delta_{ms-1}, delta_ms
+  float h1 = ph[row(ms + 1)], l1 = pl[row(ms + 1)];
+  float dm, d0;
+  {
+    const float hm = ph[row(ms - 1)], lm = pl[row(ms - 1)], h0 = ph[row(ms)], l0 = pl[row(ms)];
+    dm = (h0 - hm) + (l0 - lm);
+    d0 = (h1 - h0) + (l1 - l0);
+  }
+  float z = 0.0f, zp[7] = {};  // z of the last row; of the seven rows before a group
+  float nh[8], nl[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    nh[t] = ph[row(ms + 2 + t)];
+    nl[t] = pl[row(ms + 2 + t)];
+  }
+  float* bp = A.b + (size_t)r0 * ld + col;
+  const int ngrp = 2 + (r1 - r0 + 7) / 8;
+  for (int gidx = 0; gidx < ngrp; ++gidx) {
+    const int m0 = ms + 8 * gidx;
+    float ch[8], cl[8], zc[8], y[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      ch[t] = nh[t];
+      cl[t] = nl[t];
+    }
+    if (gidx + 1 < ngrp) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        nh[t] = ph[row(m0 + 10 + t)];
+        nl[t] = pl[row(m0 + 10 + t)];
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int m = m0 + t;
+      float dp = (ch[t] - h1) + (cl[t] - l1);  // delta_{m+1}
+      h1 = ch[t];
+      l1 = cl[t];
+      float d;
+      if (FILTER) {
+        const float a = __shfl_up_sync(kFull, d0, 1), b = __shfl_down_sync(kFull, d0, 1);
+        float um = dm, up = dp;
+        if (EDGE && A.even) {
+          um = m == 0 ? d0 : um;
+          up = m == A.M - 1 ? d0 : up;
+        }
+        d = fmaf(A.cb_hi, d0, fmaf(A.cb_lo, d0, (a + b) + (um + up)));
+      } else {
+        d = d0;
+      }
+      if (EDGE) d = (m >= 0 && m < A.M) ? d : 0.0f;
+      dm = d0;
+      d0 = dp;
+      z = fmaf(kRhoF, z, d);
+      zc[t] = z;
+    }
+    // backward from the group's last row: seven rows of warm-up, then the rows r0 + 8 (gidx - 2) .. + 7
+    float acc = zc[7];
+#pragma unroll
+    for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
+    y[7] = acc = fmaf(kRhoF, acc, zc[0]);
+#pragma unroll
+    for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRhoF, acc, zp[t]);
+#pragma unroll
+    for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
+    if (gidx < 2) continue;
+    if (EDGE) {
+      if (seg == 0 && gidx == 2) {
+        const float phi = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
+#pragma unroll
+        for (int t = 0; t < kEnd; ++t) y[t] = fmaf(A.v[t], phi, y[t]);
+      }
+      if (last && gidx == ngrp - 1) {
+        const float phi = fmaf(A.g[0], y[7], fmaf(A.g[1], y[6], fmaf(A.g[2], y[5], A.g[3] * y[4])));
+#pragma unroll
+        for (int t = 0; t < kEnd; ++t) y[7 - t] = fmaf(A.v[t], phi, y[7 - t]);
+      }
+    }
+    if (live) {
+      const int left = r1 - (r0 + 8 * (gidx - 2));
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t < left) bp[(size_t)t * ld] = -y[t];
+    }
+    bp += 8 * ld;
+  }
+}
+
+// Lines of fewer than 16 rows: every output from the explicit rows of A^{-1}, a point per lane.
+__device__ __forceinline__ void tiny_curl(const YArgs& A) {
+  const int lane = threadIdx.x & 31, N = A.N, K = A.K, rs = 2 * K + 2;
+  auto u = [&](const float* h, const float* l, int j, int i, int j2, int i2) {
+    return (h[(size_t)j2 * A.ld + i2] - h[(size_t)j * A.ld + i]) + (l[(size_t)j2 * A.ld + i2] - l[(size_t)j * A.ld + i]);
+  };
+  // y of line c at row r: axis 0 lines are rows of the source, 1 columns
+  auto term = [&](int s, int axis, int c, int r) {
+    const int M = A.M;
+    const float *h = A.th[s], *l = A.tl[s];
+    auto delta = [&](int cc, int m) -> float {
+      if (m < 0 || m >= M) {
+        if (!A.even || m < -1 || m > M) return 0.0f;
+        m = m < 0 ? 0 : M - 1;
+      }
+      return axis == 0 ? u(h, l, cc, m, cc, m + 1) : u(h, l, m, cc, m + 1, cc);
+    };
+    float hi = 0.0f, lo = 0.0f;
+    for (int t = 0; t < rs; ++t) {
+      const int m = r - K + t;
+      if (m < 0 || m >= M) continue;
+      const float x = delta(c, m);
+      float d = x;
+      if (A.filter) {
+        const float lap = ((delta(c, m - 1) - x) + (delta(c, m + 1) - x)) + ((delta(c - 1, m) - x) + (delta(c + 1, m) - x));
+        d = fmaf(A.tcb_hi, x, fmaf(A.tcb_lo, x, lap));
+      }
+      hi = fmaf(A.whi[r * rs + t], d, hi);
+      lo = fmaf(A.wlo[r * rs + t], d, lo);
+    }
+    return hi + lo;
+  };
+  // the planes hold right-hand sides over (1 - rho)^2
+  constexpr float inv = 1.0f / ((1.0f - kRhoF) * (1.0f - kRhoF));
+  if (A.step == 0) {
+    for (int p = lane; p < (N - 1) * (N - 1); p += 32) {
+      const int j = 1 + p / (N - 1), i = 1 + p % (N - 1);
+      A.tb[0][(size_t)j * A.ld + i] = inv * (term(0, 0, j, i - 1) - term(1, 1, i, j - 1));
+    }
+  } else {
+    for (int p = lane; p < N * (N - 1); p += 32) {
+      const int j = p / (N - 1), i = 1 + p % (N - 1);
+      A.tb[0][(size_t)j * A.ld + i] = -inv * term(0, 1, i, j);
+      A.tb[1][(size_t)i * A.ld + j] = inv * term(0, 0, i, j);
+    }
+  }
+}
+
+template <bool FILTER>
+__device__ __forceinline__ void y_item(const YArgs& A, int item) {
+  if (A.tiny) {
+    if (item == 0) tiny_curl(A);
+    return;
+  }
+  if (item >= A.nstrip * A.nseg) return;
+  const int seg = item / A.nstrip, strip = item - seg * A.nstrip;
+  const int r0 = seg == A.nseg - 1 ? A.rb : seg * A.chunk;
+  const int r1 = seg == A.nseg - 1 ? A.M : min(r0 + A.chunk, A.rb);
+  // rows the walk touches: r0 - 10 .. the end of its last group and of the next one's loads
+  if (r0 >= 10 && r1 + 18 <= A.M) y_segment<FILTER, false>(A, strip, seg);
+  else y_segment<FILTER, true>(A, strip, seg);
+}
+
+// ---- derivative along x --------------------------------------------------------------------
+
+// One block of rows of one 128-column strip.  SE: the source is E_z (delta_m ends at its column m, even
+// beyond the ends).  EDGE: the strip sees an end of the lines; lanes beyond it hold zeros.
+template <bool SE, bool FILTER, bool EDGE>
+__device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip, int blk) {
+  const int lane = threadIdx.x & 31;
+  const int m_s = XOUT * strip - XHALO, m0 = m_s + 4 * lane;
+  const int M = A.M;
+  const int j0 = A.u0 + blk * A.rows, j1 = min(j0 + A.rows, A.u1);
+  const size_t ld = A.ld;
+  const bool ok = !EDGE || (m0 >= -4 && m0 + 8 <= A.ld);  // the lane's columns lie in the row
+  const bool out = lane >= XHALO / 4 && lane < (XHALO + XOUT) / 4 && (!EDGE || (m0 < M && m0 >= 0));
+  const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  auto load = [&](const float* p, int row) { return ok ? ld4(p + (size_t)row * ld + m0) : zero4; };
+  // edge strips: masks, and the end corrections' coefficients at the lane's columns
+  bool in[4] = {true, true, true, true}, first[4] = {}, lastc[4] = {};
+  float vl[4] = {}, vr[4] = {}, gr[4] = {};
+  int la = 0, lb = 0;
+  bool right = false;
+  if (EDGE) {
+    right = M - 1 <= m_s + 127;
+    la = (M - 1 - m_s) >> 2;
+    lb = (M - 4 - m_s) >> 2;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int m = m0 + k, e = M - 1 - m;
+      in[k] = m >= 0 && m < M;
+      first[k] = m == 0;
+      lastc[k] = e == 0;
+      vl[k] = (strip == 0 && m >= 0 && m < kEnd) ? A.v[m & 7] : 0.0f;
+      vr[k] = (right && e >= 0 && e < kEnd) ? A.v[e & 7] : 0.0f;
+      gr[k] = (right && e >= 0 && e < 4) ? A.g[e & 3] : 0.0f;
+    }
+  }
+  // differences of one source row
+  auto diff = [&](const float4& h, const float4& l, float(&d)[4]) {
+    if (SE) {
+      const float hp = __shfl_up_sync(kFull, h.w, 1), lp = __shfl_up_sync(kFull, l.w, 1);
+      d[0] = (h.x - hp) + (l.x - lp);
+      d[1] = (h.y - h.x) + (l.y - l.x);
+      d[2] = (h.z - h.y) + (l.z - l.y);
+      d[3] = (h.w - h.z) + (l.w - l.z);
+    } else {
+      const float hn = __shfl_down_sync(kFull, h.x, 1), ln = __shfl_down_sync(kFull, l.x, 1);
+      d[0] = (h.y - h.x) + (l.y - l.x);
+      d[1] = (h.z - h.y) + (l.z - l.y);
+      d[2] = (h.w - h.z) + (l.w - l.z);
+      d[3] = (hn - h.w) + (ln - l.w);
+    }
+  };
+  // ring: [slot][hi, lo of row jj + 1][lane]
+  const size_t off = ok ? m0 : 0;
+  const float* fh = A.sh + (size_t)(j0 + 1) * ld + off;
+  const float* fl = A.sl + (size_t)(j0 + 1) * ld + off;
+  int left = j1 - j0;  // rows to fetch (the last is row j1 <= u1)
+  auto fetch = [&](int slot) {
+    if (left > 0) {
+      cp16(ring + (2 * slot) * 32 + lane, fh, ok);
+      cp16(ring + (2 * slot + 1) * 32 + lane, fl, ok);
+    }
+    cp_commit();
+    fh += ld;
+    fl += ld;
+    --left;
+  };
+#pragma unroll
+  for (int t = 0; t < kAhead; ++t) fetch(t);
+  float dm[4], d0[4];
+  {
+    const float4 ah = load(A.sh, j0 - 1), al = load(A.sl, j0 - 1), bh = load(A.sh, j0), bl = load(A.sl, j0);
+    diff(ah, al, dm);
+    diff(bh, bl, d0);
+  }
+  float* bp = A.b + (size_t)j0 * ld + m0;
+  int rd = 0, wr = kAhead;  // slots of rows jj + 1 and jj + 1 + kAhead
+  for (int jj = j0; jj < j1; ++jj, bp += ld) {
+    float dp[4], d[4], y[4];
+    cp_wait<kAhead - 1>();
+    const float4 ch = ring[(2 * rd) * 32 + lane], cl = ring[(2 * rd + 1) * 32 + lane];
+    fetch(wr);
+    rd = rd == kRing - 1 ? 0 : rd + 1;
+    wr = wr == kRing - 1 ? 0 : wr + 1;
+    diff(ch, cl, dp);
+    if (FILTER) {
+      const float a = __shfl_up_sync(kFull, d0[3], 1), e = __shfl_down_sync(kFull, d0[0], 1);
+      float l[4] = {a, d0[0], d0[1], d0[2]}, r[4] = {d0[1], d0[2], d0[3], e};
+      if (EDGE) {  // zero differences beyond the ends of a Neumann source, even ones of E_z
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          l[k] = first[k] ? (SE ? d0[k] : 0.0f) : l[k];
+          r[k] = lastc[k] ? (SE ? d0[k] : 0.0f) : r[k];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k += 2) {
+        const float2 x = make_float2(d0[k], d0[k + 1]);
+        const float2 nb = add2(make_float2(l[k] + r[k], l[k + 1] + r[k + 1]),
+                               add2(make_float2(dm[k], dm[k + 1]), make_float2(dp[k], dp[k + 1])));
+        const float2 v = fma2(bc2(A.cb_hi), x, fma2(bc2(A.cb_lo), x, nb));
+        d[k] = v.x;
+        d[k + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) d[k] = d0[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (EDGE) d[k] = in[k] ? d[k] : 0.0f;
+      dm[k] = d0[k];
+      d0[k] = dp[k];
+    }
+    // forward: the carry of the two lanes before (eight terms) from their local chains, then the chain with
+    // it, so that every z is rounded once at its own size; backward the same
+    float t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[0], d[1]), d[2]), d[3]);
+    float c1 = __shfl_up_sync(kFull, t, 1), c2 = __shfl_up_sync(kFull, t, 2);
+    if (EDGE) {
+      c1 = lane < 1 ? 0.0f : c1;
+      c2 = lane < 2 ? 0.0f : c2;
+    }
+    float c = fmaf(kR4, c2, c1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c = d[k] = fmaf(kRhoF, c, d[k]);
+    t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[3], d[2]), d[1]), d[0]);
+    c1 = __shfl_down_sync(kFull, t, 1);
+    c2 = __shfl_down_sync(kFull, t, 2);
+    if (EDGE) {
+      c1 = lane > 30 ? 0.0f : c1;
+      c2 = lane > 29 ? 0.0f : c2;
+    }
+    c = fmaf(kR4, c2, c1);
+#pragma unroll
+    for (int k = 3; k >= 0; --k) c = y[k] = fmaf(kRhoF, c, d[k]);
+    if (EDGE) {
+      if (strip == 0) {  // columns 0 .. 3 are lane 2's
+        const float part = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
+        const float phi = __shfl_sync(kFull, part, XHALO / 4);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) y[k] = fmaf(vl[k], phi, y[k]);
+      }
+      if (right) {
+        const float part = fmaf(gr[0], y[0], fmaf(gr[1], y[1], fmaf(gr[2], y[2], gr[3] * y[3])));
+        const float pa = __shfl_sync(kFull, part, la), pb = __shfl_sync(kFull, part, lb);
+        const float phi = la == lb ? pa : pa + pb;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) y[k] = fmaf(vr[k], phi, y[k]);
+      }
+    }
+    if (out) *reinterpret_cast<float4*>(bp) = make_float4(y[0], y[1], y[2], y[3]);  // (pads: never read unmasked)
+  }
+}
+
+template <bool SE, bool FILTER>
+__device__ __forceinline__ void x_item(const XArgs& A, float4* ring, int item) {
+  if (item >= A.nstrip * A.nblk) return;
+  const int blk = item / A.nstrip, strip = item - blk * A.nstrip;
+  if (strip == 0 || A.M - 1 <= XOUT * strip - XHALO + 127) x_block<SE, FILTER, true>(A, ring, strip, blk);
+  else x_block<SE, FILTER, false>(A, ring, strip, blk);
+}
+
+// The two derivatives of a half-step: blocks [0, nyb) along y, the others along x.
+template <bool SE, bool FILTER>
+__global__ void __launch_bounds__(32 * WPB) k_walk_d(const __grid_constant__ YArgs Y, const __grid_constant__ XArgs X,
+                                                     int nyb) {
+  __shared__ float4 ring[WPB][2 * kRing * 32];
+  pdl_wait();
+  const int w = threadIdx.x >> 5, b = blockIdx.x;
+  if (b < nyb) y_item<FILTER>(Y, b * WPB + w);
+  else x_item<SE, FILTER>(X, ring[w], (b - nyb) * WPB + w);
+}
+
+// ---- solve and update ----------------------------------------------------------------------
+
+// (hi, lo) += (s_hi + s_lo)(b + c), |c| <= 8e-3 |b|: an exact two-product of s_hi b with the other
+// products in its error term, and a two-sum into the pair.
+__device__ __forceinline__ void ff_add_scaled(float2& hi, float2& lo, float2 b, float2 c, float2 s_hi, float2 n_hi,
+                                              float2 s_lo) {
+  const float2 np = mul2(n_hi, b);  // -p, p = fl(s_hi b)
+  float2 e = fma2(s_hi, b, np);
+  e = fma2(s_lo, b, e);
+  e = fma2(s_hi, c, e);
+  const float2 u = sub2(hi, np);
+  const float2 bb = sub2(u, hi);
+  const float2 err = sub2(sub2(hi, sub2(u, bb)), add2(np, bb));
+  const float2 l = add2(lo, add2(err, e));
+  const float2 h2 = add2(u, l);
+  lo = sub2(l, sub2(h2, u));
+  hi = h2;
+}
+
+// The kinds of field: right-hand side in two planes (E_z), Neumann along y (H_x), along x (H_y).
+enum { KIND_E = 0, KIND_HX = 1, KIND_HY = 2 };
+
+// One block of rows of one 128-column strip; P levels.  EDGE: lanes beyond the field hold zeros.
+template <int P, int KIND, bool EDGE>
+__device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip, int blk) {
+  constexpr bool TWO = KIND == KIND_E;
+  const int lane = threadIdx.x & 31;
+  const int m0 = SOUT * strip - SHALO + 4 * lane;
+  const int M = A.M, u0 = A.u0, u1 = A.u1;
+  const int j0 = u0 + blk * A.rows, j1 = min(j0 + A.rows, u1);
+  const size_t ld = A.ld;
+  const bool ok = !EDGE || (m0 >= 0 && m0 < M);
+  const bool out = lane >= SHALO / 4 && lane < (SHALO + SOUT) / 4 && ok;
+  bool in[4] = {true, true, true, true}, first = false, lastc[4] = {};
+  if (EDGE) {
+    first = KIND == KIND_HY && m0 == 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      in[k] = m0 + k >= 0 && m0 + k < M;
+      lastc[k] = KIND == KIND_HY && m0 + k == M - 1;
+    }
+  }
+  auto mask = [&](float2(&y)[2]) {
+    if (EDGE) {
+      y[0].x = in[0] ? y[0].x : 0.0f;
+      y[0].y = in[1] ? y[0].y : 0.0f;
+      y[1].x = in[2] ? y[1].x : 0.0f;
+      y[1].y = in[3] ? y[1].y : 0.0f;
+    }
+  };
+  const float2 four = bc2(4.0f);
+  // w = 4 y + left + right
+  auto wsum = [&](const float2(&y)[2], float2(&w)[2]) {
+    float a = __shfl_up_sync(kFull, y[1].y, 1), b = __shfl_down_sync(kFull, y[0].x, 1);
+    float r0 = y[0].y, r1 = y[1].x, r2 = y[1].y;
+    if (EDGE && KIND == KIND_HY) {
+      a = first ? y[0].x : a;
+      r0 = lastc[0] ? y[0].x : r0;
+      r1 = lastc[1] ? y[0].y : r1;
+      r2 = lastc[2] ? y[1].x : r2;
+      b = lastc[3] ? y[1].y : b;
+    }
+    w[0] = fma2(four, y[0], make_float2(a + r0, y[0].x + r1));
+    w[1] = fma2(four, y[1], make_float2(y[0].y + r2, y[1].x + b));
+  };
+  const int js = max(j0 - P, u0);
+  // ring: [slot][p1, p2 of row jj, hi, lo of row jj - P][lane]
+  const size_t off = ok ? m0 : 0;
+  const float* f1 = A.p1 + (size_t)js * ld + off;  // row jj of the planes, row jj - P of the state
+  const float* f2 = TWO ? A.p2 + (size_t)js * ld + off : nullptr;
+  const float* fh = A.hi + off + ((ptrdiff_t)js - P) * (ptrdiff_t)ld;
+  const float* fl = A.lo + off + ((ptrdiff_t)js - P) * (ptrdiff_t)ld;
+  const int jb = min(j1 + P, u1);  // rows of b
+  int jf = js;                     // next row to fetch
+  auto fetch = [&](int slot) {
+    float4* r = ring + 4 * slot * 32 + lane;
+    if (jf < jb) {
+      cp16(r, f1, ok);
+      if (TWO) cp16(r + 32, f2, ok);
+    }
+    if (out && jf >= j0 + P && jf < j1 + P) {
+      cp16(r + 64, fh, true);
+      cp16(r + 96, fl, true);
+    }
+    cp_commit();
+    f1 += ld;
+    if (TWO) f2 += ld;
+    fh += ld;
+    fl += ld;
+    ++jf;
+  };
+#pragma unroll
+  for (int t = 0; t < kAhead; ++t) fetch(t);
+  int rd = 0, wr = kAhead;
+  const float2 z2 = bc2(0.0f);
+  float2 b[P + 1][2], w[P][2][2];  // b[l]: row jj - l; w[l][1]: level l at row jj - l - 1, w[l][0] above it
+#pragma unroll
+  for (int l = 0; l <= P; ++l) b[l][0] = b[l][1] = z2;
+#pragma unroll
+  for (int l = 0; l < P; ++l) w[l][0][0] = w[l][0][1] = w[l][1][0] = w[l][1][1] = z2;
+  const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo);
+  float* ph = A.hi + off + (size_t)j0 * ld;
+  float* pl = A.lo + off + (size_t)j0 * ld;
+  const int jend = j1 + P;
+#pragma unroll 1
+  for (int jj = js; jj < jend; ++jj) {
+    cp_wait<kAhead - 1>();
+    const float4* r = ring + 4 * rd * 32 + lane;
+    fetch(wr);
+    rd = rd == kRing - 1 ? 0 : rd + 1;
+    wr = wr == kRing - 1 ? 0 : wr + 1;
+    float2 wn[2];
+#pragma unroll
+    for (int l = P; l > 0; --l)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) b[l][k] = b[l - 1][k];
+    if (jj < u1) {  // b of row jj
+      const float4 c = r[0];
+      b[0][0] = make_float2(c.x, c.y);
+      b[0][1] = make_float2(c.z, c.w);
+      if (TWO) {
+        const float4 e = r[32];
+        b[0][0] = add2(b[0][0], make_float2(e.x, e.y));
+        b[0][1] = add2(b[0][1], make_float2(e.z, e.w));
+      }
+      mask(b[0]);
+      wsum(b[0], wn);
+    } else {
+      b[0][0] = b[0][1] = wn[0] = wn[1] = z2;
+    }
+    // level l + 1 at row t = jj - l - 1 from w of level l at rows t - 1, t, t + 1
+#pragma unroll
+    for (int l = 0; l < P; ++l) {
+      const int t = jj - l - 1;
+      float2 tt[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float2 ud = add2(w[l][0][k], wn[k]);
+        if (KIND == KIND_HX && (t == u0 || t == u1 - 1))  // the ghost row equals the wall row
+          ud = add2(w[l][1][k], t == u0 ? wn[k] : w[l][0][k]);
+        tt[k] = fma2(four, w[l][1][k], ud);
+        w[l][0][k] = w[l][1][k];
+        w[l][1][k] = wn[k];
+      }
+      if (l < P - 1) {
+        if ((unsigned)(t - u0) < (unsigned)(u1 - u0)) {
+          float2 y[2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) y[k] = fma2(bc2(A.q[l]), tt[k], b[l + 1][k]);
+          mask(y);
+          wsum(y, wn);
+        } else {
+          wn[0] = wn[1] = z2;
+        }
+      } else if (t >= j0) {
+        if (out) {
+          const float4 sh = r[64], sl = r[96];
+          float2 h[2] = {make_float2(sh.x, sh.y), make_float2(sh.z, sh.w)};
+          float2 o[2] = {make_float2(sl.x, sl.y), make_float2(sl.z, sl.w)};
+#pragma unroll
+          for (int k = 0; k < 2; ++k) ff_add_scaled(h[k], o[k], b[P][k], mul2(bc2(A.q[P - 1]), tt[k]), s_hi, n_hi, s_lo);
+          if (!EDGE || m0 + 4 <= M) {
+            *reinterpret_cast<float4*>(ph) = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+            *reinterpret_cast<float4*>(pl) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+          } else {
+            const float hv[3] = {h[0].x, h[0].y, h[1].x}, ov[3] = {o[0].x, o[0].y, o[1].x};
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+              if (in[k]) {
+                ph[k] = hv[k];
+                pl[k] = ov[k];
+              }
+          }
+        }
+        ph += ld;
+        pl += ld;
+      }
+    }
+  }
+}
+
+template <int P>
+__device__ __forceinline__ void s_item(const SArgs& A, float4* ring, int item) {
+  if (item >= A.nstrip * A.nblk) return;
+  const int blk = item / A.nstrip, strip = item - blk * A.nstrip;
+  const bool edge = strip == 0 || A.M - 1 < SOUT * strip - SHALO + 127;
+  if (A.kind == KIND_E) {
+    if (edge) s_block<P, KIND_E, true>(A, ring, strip, blk);
+    else s_block<P, KIND_E, false>(A, ring, strip, blk);
+  } else if (A.kind == KIND_HX) {
+    if (edge) s_block<P, KIND_HX, true>(A, ring, strip, blk);
+    else s_block<P, KIND_HX, false>(A, ring, strip, blk);
+  } else {
+    if (edge) s_block<P, KIND_HY, true>(A, ring, strip, blk);
+    else s_block<P, KIND_HY, false>(A, ring, strip, blk);
+  }
+}
+
+// One or two fields: blocks [0, na) solve the first.
+template <int P>
+__global__ void __launch_bounds__(32 * WPB, P <= 3 ? 5 : 4) k_walk_s(const __grid_constant__ SArgs A, const __grid_constant__ SArgs B,
+                                                     int na) {
+  __shared__ float4 ring[WPB][4 * kRing * 32];
+  pdl_wait();
+  const int w = threadIdx.x >> 5, b = blockIdx.x;
+  if (b < na) s_item<P>(A, ring[w], b * WPB + w);
+  else s_item<P>(B, ring[w], (b - na) * WPB + w);
+}
+
+// ---- batches -------------------------------------------------------------------------------
+
+template <typename T>
+__device__ __forceinline__ void copy_args(T* dst, const T* src) {
+  static_assert(sizeof(T) % 4 == 0, "argument structs are made of 4-byte words");
+  const int* s = reinterpret_cast<const int*>(src);
+  int* d = reinterpret_cast<int*>(dst);
+  for (int k = threadIdx.x; k < (int)(sizeof(T) / 4); k += 32 * WPB) d[k] = s[k];
+  __syncthreads();
+}
+
+// Entry e of a work list: argument work[2 e], its items work[2 e + 1] .. + WPB - 1 on the warps of a block.
+// Derivatives: arguments below ny are walks along y, the others along x (ny is that of both half-steps'
+// lists).
+template <bool SE>
+__global__ void __launch_bounds__(32 * WPB) k_batch_d(const YArgs* __restrict__ ya, const XArgs* __restrict__ xa, int ny,
+                                                      const int* __restrict__ work, int n) {
+  __shared__ union {
+    YArgs y;
+    XArgs x;
+  } sA;
+  __shared__ float4 ring[WPB][2 * kRing * 32];
+  pdl_wait();
+  for (int e = blockIdx.x; e < n; e += gridDim.x) {
+    const int arg = work[2 * e], item = work[2 * e + 1] + (threadIdx.x >> 5);
+    if (arg < ny) {
+      copy_args(&sA.y, ya + arg);
+      y_item<true>(sA.y, item);
+    } else {
+      copy_args(&sA.x, xa + (arg - ny));
+      x_item<SE, true>(sA.x, ring[threadIdx.x >> 5], item);
+    }
+    __syncthreads();
+  }
+}
+
+template <int P>
+__global__ void __launch_bounds__(32 * WPB, P <= 3 ? 5 : 4) k_batch_s(const SArgs* __restrict__ args, const int* __restrict__ work, int n) {
+  __shared__ SArgs sA;
+  __shared__ float4 ring[WPB][4 * kRing * 32];
+  pdl_wait();
+  for (int e = blockIdx.x; e < n; e += gridDim.x) {
+    copy_args(&sA, args + work[2 * e]);
+    s_item<P>(sA, ring[threadIdx.x >> 5], work[2 * e + 1] + (threadIdx.x >> 5));
+    __syncthreads();
+  }
+}
+
+// ---- host ----------------------------------------------------------------------------------
+
+struct Split {
+  float hi, lo;
+};
+Split split(double v) {
+  Split s;
+  s.hi = (float)v;
+  s.lo = (float)(v - (double)s.hi);
+  return s;
+}
+
+// Segments of the y lines: about `rows` rows each, the last one a multiple of 8 rows that ends with the
+// line, every other one ending at least 8 rows before the line's end.
+void y_segments(YArgs* a, int rows) {
+  const int M = a->M;
+  int K = (M + rows - 1) / rows;
+  if (K < 2) K = 2;
+  const int lastr = std::max(8, M / (8 * K) * 8);
+  a->rb = M - lastr;
+  a->chunk = std::max(8, ((a->rb + K - 2) / (K - 1) + 7) / 8 * 8);
+  a->nseg = (a->rb + a->chunk - 1) / a->chunk + 1;
+}
+
+YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const float* src_hi, const float* src_lo) {
+  YArgs a{};
+  const int N = g->N;
+  const int src = step == 0 ? HX : EZ;
+  const int kind = step == 0 ? HALF_TO_NODE : NODE_TO_HALF;
+  a.sh = src_hi ? src_hi : g->hi[src];
+  a.sl = src_hi ? src_lo : g->lo[src];
+  a.ld = g->ld32;
+  a.b = plane0 + (step == 0 ? a.ld : 0);  // output r at row r + 1 (E_z), r (H_x)
+  a.ncol = N + 1;
+  a.M = step == 0 ? N - 1 : N;
+  a.even = step == 1;
+  const Split c = split(12.0 * g->beta - 4.0), t = split(12.0 * g->beta);
+  a.cb_hi = c.hi;
+  a.cb_lo = c.lo;
+  for (int k = 0; k < 4; ++k) a.g[k] = (float)g->walk.ends[kind].g[k];
+  for (int k = 0; k < kEnd; ++k) a.v[k] = (float)g->walk.ends[kind].v[k];
+  a.nstrip = (N - 1 + YOUT - 1) / YOUT;
+  // Rows per segment: 16 more warm up its recurrences, so long segments do less work, but a grid wants
+  // about ten warps per SM, and small grids short walks.  The choice depends on N alone: a cavity of a batch takes the segments of a
+  // single grid, and with them its rounding.
+  y_segments(&a, a.nstrip * (a.M / 64) >= 1500 ? 64 : (N > 320 ? 32 : 16));
+  a.tiny = N <= kTinyN;
+  a.step = step;
+  a.N = N;
+  if (a.tiny) {
+    a.th[0] = step == 0 ? g->hi[HY] : a.sh;
+    a.tl[0] = step == 0 ? g->lo[HY] : a.sl;
+    a.th[1] = a.sh;
+    a.tl[1] = a.sl;
+    a.tb[0] = plane0;
+    a.tb[1] = plane1;
+    a.whi = g->pade32[kind].d_whi;
+    a.wlo = g->pade32[kind].d_wlo;
+    a.K = g->pade32[kind].K;
+    a.tcb_hi = t.hi;
+    a.tcb_lo = t.lo;
+    a.nstrip = a.nseg = 1;
+  }
+  a.filter = src_hi == nullptr;
+  return a;
+}
+
+// The derivative along x of a half-step: into E_z (step 0), H_y (step 1).
+XArgs make_x(const ms_grid* g, int step, float* plane, const float* src_hi, const float* src_lo) {
+  XArgs a{};
+  const int N = g->N;
+  const int ms = step == 0 ? 0 : 1, md = step == 0 ? 1 : 0;  // column of m = 0 in source and destination
+  const int src = step == 0 ? HY : EZ;
+  a.ld = g->ld32;
+  a.sh = (src_hi ? src_hi : g->hi[src]) + ms;
+  a.sl = (src_hi ? src_lo : g->lo[src]) + ms;
+  a.b = plane ? plane + md : nullptr;
+  a.M = step == 0 ? N - 1 : N;
+  a.u0 = 1;
+  a.u1 = N;
+  const Split c = split(12.0 * g->beta - 4.0);
+  a.cb_hi = c.hi;
+  a.cb_lo = c.lo;
+  const LineEnds& e = g->walk.ends[step == 0 ? HALF_TO_NODE : NODE_TO_HALF];
+  for (int k = 0; k < 4; ++k) a.g[k] = (float)e.g[k];
+  for (int k = 0; k < kEnd; ++k) a.v[k] = (float)e.v[k];
+  a.nstrip = N <= kTinyN ? 0 : (a.M + XOUT - 1) / XOUT;
+  const int rows = a.nstrip * (N / 8) < 1216 ? 4 : 8;  // as in make_s
+  a.nblk = (N - 1 + rows - 1) / rows;
+  a.rows = (N - 1 + a.nblk - 1) / a.nblk;
+  return a;
+}
+
+SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfields) {
+  SArgs a{};
+  const int N = g->N;
+  const int mc = f == HY ? 0 : 1;  // column of m = 0
+  a.ld = g->ld32;
+  a.hi = g->hi[f] + mc;
+  a.lo = g->lo[f] + mc;
+  a.p1 = p1 + mc;
+  a.p2 = p2 ? p2 + mc : nullptr;
+  a.M = f == HY ? N : N - 1;
+  a.u0 = f == HX ? 0 : 1;
+  a.u1 = N;
+  a.kind = f == EZ ? KIND_E : (f == HX ? KIND_HX : KIND_HY);
+  const Cheb& p = g->walk.cheb;
+  for (int l = 0; l < p.m - 1; ++l) a.q[l] = (float)p.q[p.m - 1 - l];
+  const Split sp = split((f == EZ ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0 * walk_rhs_scale());
+  a.s_hi = sp.hi;
+  a.s_lo = sp.lo;
+  a.nstrip = (a.M + SOUT - 1) / SOUT;
+  // Rows per block: P rows above and below are computed twice, but a grid wants about thirteen warps per
+  // SM; small grids are bound by the length of one walk.
+  const int nr = a.u1 - a.u0;
+  int rows = 32;
+  while (rows > 8 && nfields * a.nstrip * ((nr + rows - 1) / rows) < 2000) rows /= 2;
+  if (rows == 8 && nfields * a.nstrip * ((nr + 7) / 8) < 608) rows = 4;
+  a.nblk = (nr + rows - 1) / rows;
+  a.rows = (nr + a.nblk - 1) / a.nblk;
+  return a;
+}
+
+int blocks_of(int items) { return (items + WPB - 1) / WPB; }
+
+}  // namespace
+
+double walk_rhs_scale() { return (1.0 - (double)kRhoF) * (1.0 - (double)kRhoF); }
+
+int walk_ld(int N) { return (N + 8 + 31) / 32 * 32; }
+size_t plane_floats(int N) { return (size_t)(N + 1) * walk_ld(N) + 64; }
+size_t plane_origin(int f) { return 32 + (f == HY ? 4 : 3); }
+
+ms_status walk_setup(ms_grid* g) {
+  g->ld32 = walk_ld(g->N);
+  line_ends(g->desc.closure, HALF_TO_NODE, false, &g->walk.ends[HALF_TO_NODE]);
+  line_ends(g->desc.closure, NODE_TO_HALF, false, &g->walk.ends[NODE_TO_HALF]);
+  // D as in k_rec64.cu; at least two levels, at most four (every stable r needs m <= 5)
+  if (!cheb_coefs(6.0 * g->c1 * g->h * g->h + 36.0, 20.0, 16.0, 1e-10, &g->walk.cheb, 3) || g->walk.cheb.m > 5)
+    return MS_ENOTCONV;
+  return MS_OK;
+}
+
+void walk_d(ms_grid* g, int step, const float* src_hi, const float* src_lo) {
+  // Step 1: along y into s32[4], along x into s32[1]; Step 2: s32[2] (H_x), s32[3] (H_y)
+  const YArgs y = make_y(g, step, step == 0 ? g->s32[4] : g->s32[2], step == 0 ? nullptr : g->s32[3], src_hi, src_lo);
+  const XArgs x = make_x(g, step, step == 0 ? g->s32[1] : g->s32[3], src_hi, src_lo);
+  const int nyb = blocks_of(y.nstrip * y.nseg);
+  const dim3 grd(nyb + blocks_of(x.nstrip * x.nblk)), blk(32 * WPB);
+  if (step == 0) launch_pdl(k_walk_d<false, true>, grd, blk, 0, g->stream, y, x, nyb);
+  else if (src_hi) launch_pdl(k_walk_d<true, false>, grd, blk, 0, g->stream, y, x, nyb);
+  else launch_pdl(k_walk_d<true, true>, grd, blk, 0, g->stream, y, x, nyb);
+}
+
+void walk_s(ms_grid* g, int step) {
+  const int P = g->walk.cheb.m - 1;
+  SArgs a, b;
+  int na, nb = 0;
+  if (step == 0) {
+    a = b = make_s(g, EZ, g->s32[4], g->s32[1], 1);
+    na = blocks_of(a.nstrip * a.nblk);
+  } else {
+    a = make_s(g, HX, g->s32[2], nullptr, 2);
+    b = make_s(g, HY, g->s32[3], nullptr, 2);
+    na = blocks_of(a.nstrip * a.nblk);
+    nb = blocks_of(b.nstrip * b.nblk);
+  }
+  const dim3 grd(na + nb), blk(32 * WPB);
+  if (P == 2) launch_pdl(k_walk_s<2>, grd, blk, 0, g->stream, a, b, na);
+  else if (P == 3) launch_pdl(k_walk_s<3>, grd, blk, 0, g->stream, a, b, na);
+  else launch_pdl(k_walk_s<4>, grd, blk, 0, g->stream, a, b, na);
+}
+
+int walk_batch_build(ms_grid* const* cav, int count, int order, WalkBatch* wb, std::string* err) {
+  std::vector<YArgs> ya(2 * (size_t)count);
+  std::vector<XArgs> xa(2 * (size_t)count);
+  std::vector<SArgs> sa(3 * (size_t)count);
+  std::vector<int> seq(count);
+  for (int c = 0; c < count; ++c) seq[c] = c;
+  if (order == 2) std::stable_sort(seq.begin(), seq.end(), [&](int a, int b) { return cav[a]->N > cav[b]->N; });
+  wb->P = cav[0]->walk.cheb.m - 1;
+  wb->ny = 2 * count;
+  for (int c = 0; c < count; ++c) {
+    const ms_grid* g = cav[c];
+    ya[c] = make_y(g, 0, g->s32[4], nullptr, nullptr, nullptr);
+    ya[count + c] = make_y(g, 1, g->s32[2], g->s32[3], nullptr, nullptr);
+    xa[c] = make_x(g, 0, g->s32[1], nullptr, nullptr);
+    xa[count + c] = make_x(g, 1, g->s32[3], nullptr, nullptr);
+    sa[c] = make_s(g, EZ, g->s32[4], g->s32[1], 1);
+    sa[count + c] = make_s(g, HX, g->s32[2], nullptr, 2);
+    sa[2 * count + c] = make_s(g, HY, g->s32[3], nullptr, 2);
+    for (int k = 0; k < 3; ++k) {  // the batch fills the GPU, whatever its cavities' sizes: long blocks
+      SArgs& a = sa[(size_t)k * count + c];
+      const int nr = a.u1 - a.u0;
+      a.nblk = (nr + 31) / 32;
+      a.rows = (nr + a.nblk - 1) / a.nblk;
+    }
+  }
+  std::vector<int> list[4];
+  auto add = [&](std::vector<int>& l, int arg, int items) {
+    for (int i = 0; i < items; i += WPB) l.insert(l.end(), {arg, i});
+  };
+  // order 1: the cavities one strip wide (nothing but walls) ahead of the others
+  for (int pass = 0; pass < (order == 1 ? 2 : 1); ++pass)
+    for (int c : seq) {
+      if (order == 1 && (sa[c].nstrip == 1) != (pass == 0)) continue;
+      for (int k = 0; k < 2; ++k) {
+        const YArgs& y = ya[(size_t)k * count + c];
+        const XArgs& x = xa[(size_t)k * count + c];
+        add(list[2 * k], k * count + c, y.nstrip * y.nseg);
+        add(list[2 * k], wb->ny + k * count + c, x.nstrip * x.nblk);
+      }
+      add(list[1], c, sa[c].nstrip * sa[c].nblk);
+      for (int k = 1; k < 3; ++k) add(list[3], k * count + c, sa[(size_t)k * count + c].nstrip * sa[(size_t)k * count + c].nblk);
+    }
+  std::vector<int> work;
+  for (int k = 0; k < 4; ++k) {
+    wb->off[k] = work.size();
+    wb->n[k] = (int)(list[k].size() / 2);
+    work.insert(work.end(), list[k].begin(), list[k].end());
+  }
+  if (dev_malloc(&wb->d_y, ya.size() * sizeof(YArgs)) != cudaSuccess ||
+      dev_malloc(&wb->d_x, xa.size() * sizeof(XArgs)) != cudaSuccess ||
+      dev_malloc(&wb->d_s, sa.size() * sizeof(SArgs)) != cudaSuccess ||
+      dev_malloc(&wb->d_work, work.size() * sizeof(int)) != cudaSuccess) {
+    *err = "cudaMalloc of the batch work lists failed";
+    return -1;
+  }
+  if (cudaMemcpy(wb->d_y, ya.data(), ya.size() * sizeof(YArgs), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(wb->d_x, xa.data(), xa.size() * sizeof(XArgs), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(wb->d_s, sa.data(), sa.size() * sizeof(SArgs), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(wb->d_work, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
+    *err = "copy of the batch work lists failed";
+    return -1;
+  }
+  // blocks resident on the device at once (persistent launches)
+  int dev = 0, sms = 0, pd = 0, ps = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pd, k_batch_d<true>, 32 * WPB, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_batch_s<4>, 32 * WPB, 0);
+  wb->resident_d = sms * pd;
+  wb->resident_s = sms * ps;
+  return 0;
+}
+
+void walk_batch_step(const WalkBatch& wb, cudaStream_t st, int persistent) {
+  const dim3 blk(32 * WPB);
+  auto blocks = [&](int n, int resident) { return dim3((persistent && resident > 0 && resident < n) ? resident : n); };
+  const YArgs* y = wb.d_y;
+  const XArgs* x = wb.d_x;
+  const SArgs* s = wb.d_s;
+  for (int k = 0; k < 4; ++k) {
+    const int* w = wb.d_work + wb.off[k];
+    const int n = wb.n[k];
+    const dim3 gd = blocks(n, wb.resident_d), gs = blocks(n, wb.resident_s);
+    if (k == 0) launch_pdl(k_batch_d<false>, gd, blk, 0, st, y, x, wb.ny, w, n);
+    else if (k == 2) launch_pdl(k_batch_d<true>, gd, blk, 0, st, y, x, wb.ny, w, n);
+    else if (wb.P == 2) launch_pdl(k_batch_s<2>, gs, blk, 0, st, s, w, n);
+    else if (wb.P == 3) launch_pdl(k_batch_s<3>, gs, blk, 0, st, s, w, n);
+    else launch_pdl(k_batch_s<4>, gs, blk, 0, st, s, w, n);
+  }
+}
+
+void walk_batch_free(WalkBatch* wb) {
+  dev_free(wb->d_y);
+  dev_free(wb->d_x);
+  dev_free(wb->d_s);
+  dev_free(wb->d_work);
+  *wb = WalkBatch{};
+}
+
+}  // namespace ms

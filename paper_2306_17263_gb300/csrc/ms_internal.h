@@ -130,6 +130,12 @@ struct ms_grid {
   // FP32 path: tables truncated for FP32 and split hi/lo; Richardson sweeps for FP32
   ms::PadeTable pade32[2];
   int p1_sweeps32 = 0;
+  int ld32 = 0;            // row pitch of the 2D FP32 planes
+  float* slab32 = nullptr;  // their storage: hi[3], lo[3], s32[1..4]
+  struct {
+    ms::LineEnds ends[2];  // by PadeKind
+    ms::Cheb cheb;
+  } walk;  // constants of the 2D FP32 step (k_walk.cu)
 
   // FP64 state and scratch
   double* f64[3] = {nullptr, nullptr, nullptr};   // E_z, H_x, H_y
@@ -137,12 +143,13 @@ struct ms_grid {
   float* de_hi = nullptr;                          // the same in MS_FP32_REFINED (float-float)
   float* de_lo = nullptr;
   float* t32[8] = {};                              // its scratch: E^n, y_x, y_y, G~_E (hi, lo each)
+  float* slab_de = nullptr;                        // storage of de_hi, de_lo, t32 (E_z planes)
   double* s64[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   bool shared64 = false;  // s64 planes belong to a batch
   // FP32 hi/lo state (MS_FP32_REFINED)
   float* hi[3] = {nullptr, nullptr, nullptr};
   float* lo[3] = {nullptr, nullptr, nullptr};
-  float* s32[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  float* s32[5] = {};  // 2D FP32 right-hand-side planes: [2] H_x, [3] H_y, [4] and [1] E_z
 
   // reductions and diagnostics
   double* d_partial = nullptr;  // per-block partial sums
