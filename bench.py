@@ -167,11 +167,11 @@ def bf16_peak():
 # source files that define each kernel kind reported by ms_step_profiled
 KIND_SOURCES = {
     "curl32": ["k_tiled.cu", "k_tiled.cuh"], "solve32": ["k_tiled.cu", "k_tiled.cuh"],
-    "filter64": ["k_fp64.cu", "k_fp64.cuh"], "pade64": ["k_fp64.cu", "k_fp64.cuh"],
+    "filter64": ["k_fp64.cu", "k_fp64.cuh"], "pade64": ["k_rec64.cu", "k_rec64.cuh"],
     "filt3d32": ["grid3d.cu", "grid3d.cuh"], "band3d32": ["grid3d.cu", "grid3d.cuh"],
     "term3d32": ["grid3d.cu", "grid3d.cuh"], "tsgemm": ["k_transform.cu", "k_transform.cuh"],
     "sweep3d32": ["grid3d.cu", "grid3d.cuh"],
-    "p1sweep64": ["k_fp64.cu", "k_fp64.cuh"], "yee64": ["k_fp64.cu", "k_fp64.cuh"],
+    "p1sweep64": ["k_rec64.cu", "k_rec64.cuh"], "yee64": ["k_fp64.cu", "k_fp64.cuh"],
 }
 
 

@@ -27,7 +27,7 @@
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 
 namespace ms {
 

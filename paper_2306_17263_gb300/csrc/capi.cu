@@ -17,7 +17,7 @@
 #include "k_mixed.cuh"
 #include "k_rec64.cuh"
 #include "k_src3.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 #include "k_tracked32.cuh"
 
 using namespace ms;

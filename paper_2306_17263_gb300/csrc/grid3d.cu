@@ -25,7 +25,7 @@
 #include "k_fp64.cuh"
 #include "k_pdl.cuh"
 #include "k_rec64.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 #include "k_src3.cuh"
 #include "k_transform.cuh"
 

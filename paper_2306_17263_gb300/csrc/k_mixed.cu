@@ -21,14 +21,14 @@
 // solution itself shrinks every increment the same way.  The state is a float-float pair updated with
 // error-free transformations.
 //
-// Kernels (k_walk.cu): the derivatives along both axes, then the solve and the update, per half-step,
+// Kernels (k_tiled.cu): the derivatives along both axes, then the solve and the update, per half-step,
 // i.e. four launches per time step.
 #include <cmath>
 #include <string>
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 
 namespace ms {
 

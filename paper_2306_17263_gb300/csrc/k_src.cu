@@ -40,7 +40,7 @@ struct SrcDev {
 // The time factors are the same at every point: a one-block kernel at the start of each step
 // forms them (k_src_time), and the point kernels read them.  FP64: v = sum_q (ce_q sin(w_q t))
 // X_q(i) Y_q(j), the product taken in the order of the plain definition.  FP32 (right-hand sides of
-// k_walk.cu): the factors are scaled to their units and rounded to float, and the sum is
+// k_tiled.cu): the factors are scaled to their units and rounded to float, and the sum is
 // taken in float from the float copy of the tables.
 constexpr int kMaxSrc = 64;
 struct SrcFac {

@@ -43,7 +43,7 @@
 #include "k_fp64.cuh"
 #include "k_pdl.cuh"
 #include "k_rec64.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 
 namespace ms {
 

@@ -1,4 +1,4 @@
-// FP32_REFINED step of 2D grids (k_walk.cu): warps that walk along y, two launches per half-step.
+// FP32_REFINED step of 2D grids (k_tiled.cu): warps that walk along y, two launches per half-step.
 #pragma once
 
 #include <string>

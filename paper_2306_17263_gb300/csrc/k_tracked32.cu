@@ -14,7 +14,7 @@
 #include <cmath>
 
 #include "k_fp64.cuh"
-#include "k_walk.cuh"
+#include "k_tiled.cuh"
 #include "k_tracked32.cuh"
 
 namespace ms {

@@ -135,7 +135,7 @@ struct ms_grid {
   struct {
     ms::LineEnds ends[2];  // by PadeKind
     ms::Cheb cheb;
-  } walk;  // constants of the 2D FP32 step (k_walk.cu)
+  } walk;  // constants of the 2D FP32 step (k_tiled.cu)
 
   // FP64 state and scratch
   double* f64[3] = {nullptr, nullptr, nullptr};   // E_z, H_x, H_y
