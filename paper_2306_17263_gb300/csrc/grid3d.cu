@@ -6,16 +6,18 @@
 // + D_xx D_yy (Def. "def:operatorsP").  Every component is Dirichlet (stored wall zeros) along
 // the axes on which it sits on nodes and Neumann (even ghosts) along its half-node axes.
 //
-// MS_FP64: one operator per launch in FP64 (filter, Pade band along one axis, Richardson sweep).
+// MS_FP64: filter, Pade recurrences (k_rec64.cu; bands on short lines) and polynomial solves, up to three
+// components per launch.
 // MS_FP32_REFINED: the arithmetic of the 2D FP32 path (k_mixed.cu) carried to 3D: float-float
 // state; each half-step first filters its three source components once into float-float
 // G = 12 beta u + L u (k_ffilt3d32), then per Pade term one tile kernel (k_term3d32) forms the
 // first differences of G along the line (the filter commutes with the difference under the ghost
 // rules) and applies A^{-1} (interior rows by two first-order recurrences, rows near a wall by the
 // explicit band rows, farthest taps first), accumulating the right-hand side (a difference kernel
-// and a band kernel take over for tables wider than the tile holds); the solve
-// (k_sweep3d32) is the Richardson iteration on 6 h^2 P1 with the exact-product residual and
-// the split last correction, each sweep one launch that marches tiles along z.
+// and a band kernel take over for tables wider than the tile holds); the solve (k_lev3d32) is a Chebyshev
+// polynomial in Horner form, one level per launch.  The three components of a half-step share launches
+// (14 per step).  The transform solver (k_transform.cu) is followed by Richardson sweeps (k_sweep3d32).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <string>
@@ -47,7 +49,7 @@ struct Grid3D {
   float* hi[6] = {};
   float* lo[6] = {};
   double* s64[9] = {};  // FP64: G[3], R[3], and, with G again, the work planes of the solves; FP32 grids use [0], [1]
-  float* s32[4] = {};   // FP32: differences, R, sweep ping-pong [2]
+  float* s32[4] = {};   // FP32: differences, R[3]
   float* gh[3] = {};    // FP32: filtered components G~ (hi, lo) of one half-step, slot c % 3
   float* gl[3] = {};
   double* dview[6] = {};  // FP32_REFINED grids: FP64 copy of the state for the diagnostics
@@ -175,20 +177,6 @@ __global__ void k_mode_field3(double* __restrict__ out, Shape3 s, const double* 
 // ---------------------------------------------------------------------------------------
 // FP32_REFINED kernels
 
-// (hi, lo) += (s_hi + s_lo) x with error-free transformations (two-product by FMA, Knuth two-sum).
-__device__ __forceinline__ void ff_add_scaled3(float& hi, float& lo, float x, float s_hi, float s_lo) {
-  const float p = __fmul_rn(s_hi, x);
-  float e = fmaf(s_hi, x, -p);
-  e = fmaf(s_lo, x, e);
-  const float s = __fadd_rn(hi, p);
-  const float bb = __fsub_rn(s, hi);
-  const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  const float l = __fadd_rn(lo, __fadd_rn(err, e));
-  const float h2 = __fadd_rn(s, l);
-  lo = __fsub_rn(l, __fsub_rn(h2, s));
-  hi = h2;
-}
-
 // Interior row of A^{-1} at offsets -KB3 .. KB3+1 (hi) and the lo parts of offsets -1, 0, 1: the
 // same Toeplitz row for every grid, 24 (-rho) rho^|d| / (1 - rho^2), rho = -11 + sqrt(120).
 constexpr int KB3 = 7;
@@ -207,7 +195,8 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
 
-// ff_add_scaled3 on two independent pairs at once.
+// (hi, lo) += (s_hi + s_lo) x with error-free transformations (two-product by FMA, Knuth two-sum), on two
+// independent pairs at once.
 __device__ __forceinline__ void ff_add_scaled3_2(float2& hi, float2& lo, float2 x, float2 s_hi, float2 s_lo) {
   const float2 p = mul2(s_hi, x);
   float2 e = fma2(s_hi, x, neg2(p));
@@ -229,95 +218,115 @@ __device__ __forceinline__ void ff_add_scaled3_2(float2& hi, float2& lo, float2 
 // accuracy), joins the low word, and two-sum renormalises the pair.  The Pade terms below then
 // difference G: D1 G = (12 beta + L') D1 u, the filter commuting with the difference under the
 // ghost rules (zero differences beyond the ends of a Neumann line, even ones on a Dirichlet line).
-// The layout is that of the sweep below: a block of 32 x 8 threads takes a 32 x 16 tile, a thread
-// rows j and j + 8 of one column as a pair (paired FP32 instructions), marching FZ3 planes along
-// z with the planes z-1, z, z+1 (hi and lo, one-point halo in x and y, clamped) in a ring in
-// shared memory; the next plane is fetched into registers while the current one is computed.
-constexpr int FZ3 = 16;
-constexpr int FTX = 32, FTT = 8, FTY = 2 * FTT;
-constexpr int FXP = FTX + 2, FRP = FTT + 2, FN = FRP * FXP;
-static_assert(FN <= 2 * FTX * FTT, "two staged pairs per thread");
-__global__ void __launch_bounds__(FTX * FTT, 6) k_ffilt3d32(const float* __restrict__ hi, const float* __restrict__ lo,
-                                                            Shape3 s, float* __restrict__ gh, float* __restrict__ gl,
-                                                            float cb_hi, float cb_lo) {
-  __shared__ float2 hs[3][FRP][FXP];
-  __shared__ float2 ls[3][FRP][FXP];
+// A thread takes two rows of one column and marches FZ3 planes along z with the planes below and above in
+// registers, the next plane fetched ahead (no shared memory; the neighbour rows and columns come from L1).
+// The tile form before it, 32 x 16 tiles of three planes in shared memory, issued 112 instructions per 32
+// points, 70 us per component at 256^3.
+constexpr int FZ3 = 16, FY3 = 8;
+struct Filter3d32Args {  // the three components of a half-step
+  const float *hi[3], *lo[3];
+  float *gh[3], *gl[3];
+  Shape3 s[3];
+  int nz;  // blocks along z of the largest component
+};
+__global__ void __launch_bounds__(32 * FY3, 4) k_ffilt3d32(const __grid_constant__ Filter3d32Args A, float cb_hi,
+                                                          float cb_lo) {
+  pdl_wait();
+  const int which = blockIdx.z / A.nz, kz = blockIdx.z - which * A.nz;
+  const float* __restrict__ hi = A.hi[which];
+  const float* __restrict__ lo = A.lo[which];
+  float* __restrict__ gh = A.gh[which];
+  float* __restrict__ gl = A.gl[which];
+  const Shape3& s = A.s[which];
   const int n0 = s.n[0], n1 = s.n[1], n2 = s.n[2];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i = blockIdx.x * FTX + tx, j = blockIdx.y * FTY + ty;  // rows j and j + FTT
-  const int k0 = blockIdx.z * FZ3, k1 = min(k0 + FZ3, n2);
-  const bool in0 = i < n0 && j < n1, in1 = i < n0 && j + FTT < n1;
-  const bool ux = i < n0 && interior(s.bc[0], i, n0);
-  const bool unk0 = in0 && ux && interior(s.bc[1], j, n1), unk1 = in1 && ux && interior(s.bc[1], j + FTT, n1);
-  const int sz = n0 * n1;
-  const int t1 = ty * FTX + tx, t2 = t1 + FTX * FTT;
-  const bool has2 = t2 < FN;
-  auto pair_off = [&](int e, int half) {
-    const int row = e / FXP, col = e - row * FXP;
-    return clampi(blockIdx.y * FTY + row - 1 + half * FTT, n1) * n0 + clampi(blockIdx.x * FTX + col - 1, n0);
-  };
-  const int o1a = pair_off(t1, 0), o1b = pair_off(t1, 1);
-  const int o2a = pair_off(has2 ? t2 : t1, 0), o2b = pair_off(has2 ? t2 : t1, 1);
-  float2 ha, la, hb, lb;
-  auto fetch = [&](int kk) {
-    const int q = clampi(kk, n2) * sz;
-    ha = make_float2(hi[q + o1a], hi[q + o1b]);
-    la = make_float2(lo[q + o1a], lo[q + o1b]);
-    if (has2) {
-      hb = make_float2(hi[q + o2a], hi[q + o2b]);
-      lb = make_float2(lo[q + o2a], lo[q + o2b]);
+  const int i = blockIdx.x * 32 + threadIdx.x, j = 2 * (blockIdx.y * FY3 + threadIdx.y);
+  const int k0 = kz * FZ3, k1 = min(k0 + FZ3, n2);
+  if (i >= n0 || j >= n1 || k0 >= k1) return;
+  const bool two = j + 1 < n1, ux = interior(s.bc[0], i, n0);
+  const bool u[2] = {ux && interior(s.bc[1], j, n1), ux && interior(s.bc[1], j + 1, n1)};
+  const unsigned sz = n0 * n1;
+  // rows j - 1 .. j + 2 of the column, and left and right of rows j, j + 1 (clamped: even ghosts; results
+  // on walls are set to 0)
+  unsigned om[4], ol[2], orr[2];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) om[r] = clampi(j - 1 + r, n1) * n0 + i;
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    ol[t] = om[t + 1] - i + clampi(i - 1, n0);
+    orr[t] = om[t + 1] - i + clampi(i + 1, n0);
+  }
+  float hm[4], lm[4], hl[2], hr[2], sl[2];  // one plane: the column (hi, lo), left and right (hi, sum of lo)
+  auto fetch = [&](int k) {
+    const float* __restrict__ ph = hi + (size_t)clampi(k, n2) * sz;
+    const float* __restrict__ pl = lo + (size_t)clampi(k, n2) * sz;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      hm[r] = ph[om[r]];
+      lm[r] = pl[om[r]];
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      hl[t] = ph[ol[t]];
+      hr[t] = ph[orr[t]];
+      sl[t] = pl[ol[t]] + pl[orr[t]];
     }
   };
-  auto stage = [&](int slot) {
-    (&hs[slot][0][0])[t1] = ha;
-    (&ls[slot][0][0])[t1] = la;
-    if (has2) {
-      (&hs[slot][0][0])[t2] = hb;
-      (&ls[slot][0][0])[t2] = lb;
-    }
-  };
+  float hz[2], lz[2];            // plane below
+  float hc[4], lc[4], xl[2], xr[2], xs[2];  // plane k
   fetch(k0 - 1);
-  stage(0);
+  hz[0] = hm[1];
+  hz[1] = hm[2];
+  lz[0] = lm[1];
+  lz[1] = lm[2];
+  auto shift = [&]() {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      hc[r] = hm[r];
+      lc[r] = lm[r];
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      xl[t] = hl[t];
+      xr[t] = hr[t];
+      xs[t] = sl[t];
+    }
+  };
   fetch(k0);
-  stage(1);
+  shift();
   fetch(k0 + 1);
-  int zm = 0, z0 = 1, zp = 2;
-  int p = k0 * sz + j * n0 + i;
-  const int dj = FTT * n0;
-  const int c0 = tx + 1, r0 = ty + 1;
-  const float2 cbh = bc2(cb_hi), cbl = bc2(cb_lo);
-  for (int k = k0; k < k1; ++k, p += sz) {
-    stage(zp);
-    __syncthreads();
-    if (k + 1 < k1) fetch(k + 2);
-    const float2 hc = hs[z0][r0][c0], lc = ls[z0][r0][c0];
-    auto dv = [&](int pl, int rr, int cc) { return add2(sub2(hs[pl][rr][cc], hc), sub2(ls[pl][rr][cc], lc)); };
-    const float2 lap = add2(add2(add2(dv(z0, r0, c0 - 1), dv(z0, r0, c0 + 1)), add2(dv(z0, r0 - 1, c0), dv(z0, r0 + 1, c0))),
-                            add2(dv(zm, r0, c0), dv(zp, r0, c0)));
-    const float2 pr = mul2(cbh, hc);
-    float2 e = fma2(cbh, hc, neg2(pr));
-    e = fma2(cbh, lc, e);
-    e = fma2(cbl, hc, e);
-    const float2 t = add2(e, lap);
-    const float2 g_hi = add2(pr, t);
-    const float2 bb = sub2(g_hi, pr);
-    const float2 g_lo = add2(sub2(pr, sub2(g_hi, bb)), sub2(t, bb));
+  unsigned g[2] = {k0 * sz + om[1], k0 * sz + (two ? om[2] : om[1])};
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
     const bool uz = interior(s.bc[2], k, n2);
-    if (in0) {
-      const bool u = unk0 && uz;
-      gh[p] = u ? g_hi.x : 0.0f;
-      gl[p] = u ? g_lo.x : 0.0f;
+    float G[2], E[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const float c = hc[t + 1], d = lc[t + 1];
+      // first differences of the hi parts; the lo parts as one sum
+      const float lap = (((xl[t] - c) + (xr[t] - c)) + ((hc[t] - c) + (hc[t + 2] - c))) + ((hz[t] - c) + (hm[t + 1] - c));
+      const float lol = fmaf(-6.0f, d, (xs[t] + (lc[t] + lc[t + 2])) + (lz[t] + lm[t + 1]));
+      const float p = __fmul_rn(cb_hi, c);
+      float e = fmaf(cb_hi, c, -p);
+      e = fmaf(cb_hi, d, e);
+      e = fmaf(cb_lo, c, e);
+      const float x = __fadd_rn(e, lap + lol);
+      const float h = __fadd_rn(p, x), bb = __fsub_rn(h, p);
+      const bool live = uz && u[t];
+      G[t] = live ? h : 0.0f;
+      E[t] = live ? __fadd_rn(__fsub_rn(p, __fsub_rn(h, bb)), __fsub_rn(x, bb)) : 0.0f;
+      hz[t] = c;
+      lz[t] = d;
     }
-    if (in1) {
-      const bool u = unk1 && uz;
-      gh[p + dj] = u ? g_hi.y : 0.0f;
-      gl[p + dj] = u ? g_lo.y : 0.0f;
+    shift();
+    if (k + 1 < k1) fetch(k + 2);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      if (t == 0 || two) {
+        gh[g[t]] = G[t];
+        gl[g[t]] = E[t];
+      }
+      g[t] += sz;
     }
-    __syncthreads();  // the slot of plane k - 1 is staged again as plane k + 2
-    const int t0 = zm;
-    zm = z0;
-    z0 = zp;
-    zp = t0;
   }
 }
 
@@ -486,17 +495,35 @@ struct TermGeo {
 };
 constexpr int DP3 = D3L | 1;  // odd row pitch: lanes across the rows are conflict-free
 
+struct TermArgs {
+  const float* gh;
+  const float* gl;
+  float* R;
+  Shape3 ss, sd;
+  float sign;
+  int accumulate;
+};
+struct TermArgs2 {  // the two terms of a half-step along one axis
+  TermArgs t[2];
+  int nq;  // lines along Q of the larger component
+};
 template <int AXIS>
-__global__ void __launch_bounds__(256, AXIS == 0 ? 4 : 5) k_term3d32(const float* __restrict__ gh, const float* __restrict__ gl, Shape3 ss,
-                                                     float* __restrict__ R, Shape3 sd, int out_off, int M,
+__global__ void __launch_bounds__(256, AXIS == 0 ? 4 : 5) k_term3d32(const __grid_constant__ TermArgs2 A, int out_off, int M,
                                                      const float* __restrict__ whi, const float* __restrict__ wlo, int K,
-                                                     int B, int all_explicit, float sign, int accumulate) {
+                                                     int B, int all_explicit) {
   constexpr int P = TermGeo<AXIS>::P, Q = TermGeo<AXIS>::Q;
   __shared__ float dd[32 * DP3];
-  int tr, p0, q;
-  if (AXIS == 0) { tr = blockIdx.x; p0 = blockIdx.y * 32; q = blockIdx.z; }
-  else if (AXIS == 1) { p0 = blockIdx.x * 32; tr = blockIdx.y; q = blockIdx.z; }
-  else { p0 = blockIdx.x * 32; tr = blockIdx.y; q = blockIdx.z; }  // tiles along z a few blocks apart
+  pdl_wait();
+  const int which = blockIdx.z / A.nq, q = blockIdx.z - which * A.nq;
+  const TermArgs& T = A.t[which];
+  const float* __restrict__ gh = T.gh;
+  const float* __restrict__ gl = T.gl;
+  float* __restrict__ R = T.R;
+  const Shape3 &ss = T.ss, &sd = T.sd;
+  const float sign = T.sign;
+  const int accumulate = T.accumulate;
+  if (q >= sd.n[Q]) return;
+  const int tr = AXIS == 0 ? blockIdx.x : blockIdx.y, p0 = 32 * (AXIS == 0 ? blockIdx.y : blockIdx.x);
   const int r0 = tr * T3O;  // first band row of the tile
   const int st[3] = {1, ss.n[0], ss.n[0] * ss.n[1]};
   const int sdt[3] = {1, sd.n[0], sd.n[0] * sd.n[1]};
@@ -662,10 +689,180 @@ __global__ void __launch_bounds__(256, AXIS == 0 ? 4 : 5) k_term3d32(const float
   }
 }
 
+// The solve of a half-step: 6 h^2 P1 = D - T with D = 6 c1 h^2 + 24 and, from the 19-point stencil,
+// T y = 2 e + c + (2 y + e)_{z-1} + (2 y + e)_{z+1}, e and c the sums over the four edge and the four
+// corner neighbours in the plane, spectrum [-8, 24].  The Chebyshev polynomial of k_rec64.cu in Horner
+// form, y <- b + q T y, to a relative error of 1e-10, one level per launch for the three components; T y
+// is 2e-3 of D y at most, so a level rounds the increment at 1e-9 of itself, and the last level's q T y
+// enters the state apart from b.  A thread takes two rows of one column and marches L3Z planes along z
+// with e, c and q = 2 y + e of the planes in registers, the next plane's twelve values fetched ahead: ten
+// operations and six loads (from L1 but for the halo) per point and level, no test in the march, where a Richardson sweep with
+// its residual took 84 instructions on shared-memory tiles.  256^3, three levels of one component: 215 us
+// by the sweeps.
+constexpr int L3Y = 4, L3Z = 16;  // warps (pairs of rows) per block, planes per march
+constexpr int kPre3 = 3;           // planes ahead of the loads that a march asks L2 for
+__device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+struct Lev3d32Args {
+  const float* b[3];
+  const float* y[3];
+  float* out[3];         // iterate (not LAST)
+  float *hi[3], *lo[3];  // state (LAST)
+  Shape3 s[3];
+  float q, s_hi, s_lo;
+  int nz;  // marches along z of the largest component
+};
+
+// (hi, lo) += (s_hi + s_lo)(b + c): an exact two-product of s_hi b with the other products in its error
+// term, and a two-sum into the pair.
+__device__ __forceinline__ void ff_add_scaled_bc(float& hi, float& lo, float b, float c, float s_hi, float s_lo) {
+  const float p = __fmul_rn(s_hi, b);
+  float e = fmaf(s_hi, b, -p);
+  e = fmaf(s_lo, b, e);
+  e = fmaf(s_hi, c, e);
+  const float u = __fadd_rn(hi, p);
+  const float bb = __fsub_rn(u, hi);
+  const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(u, bb)), __fsub_rn(p, bb));
+  const float l = __fadd_rn(lo, __fadd_rn(err, e));
+  const float h2 = __fadd_rn(u, l);
+  lo = __fsub_rn(l, __fsub_rn(h2, u));
+  hi = h2;
+}
+
+template <bool LAST>
+__global__ void __launch_bounds__(32 * L3Y, LAST ? 6 : 8) k_lev3d32(const __grid_constant__ Lev3d32Args A) {
+  pdl_wait();
+  const int which = blockIdx.z / A.nz, kz = blockIdx.z - which * A.nz;
+  const Shape3& s = A.s[which];
+  const int n0 = s.n[0], n1 = s.n[1], n2 = s.n[2];
+  const int d0 = s.bc[0] == DIR, d1 = s.bc[1] == DIR, d2 = s.bc[2] == DIR;
+  const int i = d0 + blockIdx.x * 32 + threadIdx.x, j = d1 + 2 * (blockIdx.y * L3Y + threadIdx.y);
+  const int k0 = d2 + kz * L3Z, k1 = min(k0 + L3Z, n2 - d2);
+  if (i >= n0 - d0 || j >= n1 - d1 || k0 >= k1) return;
+  const bool two = j + 1 < n1 - d1;
+  const unsigned sz = n0 * n1;  // points per component fit 31 bits (n <= 512)
+  const float* __restrict__ y = A.y[which];
+  const float* __restrict__ b = A.b[which];
+  float* __restrict__ out = A.out[which];
+  float* __restrict__ shi = A.hi[which];
+  float* __restrict__ slo = A.lo[which];
+  // offsets in a plane of the rows j - 1 .. j + 2, and of the columns left and right: ghosts of a Neumann
+  // axis mirror, walls of a Dirichlet axis hold zeros (b: the terms write them; y: the level before)
+  unsigned om[4], ol[4], orr[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int row = clampi(j - 1 + r, n1) * n0;
+    om[r] = row + i;
+    ol[r] = row + clampi(i - 1, n0);
+    orr[r] = row + clampi(i + 1, n0);
+  }
+  float m[4], l[4], r[4];  // one plane's values
+  auto fetch = [&](int k) {
+    const float* __restrict__ p = y + (size_t)clampi(k, n2) * sz;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      m[t] = p[om[t]];
+      l[t] = p[ol[t]];
+      r[t] = p[orr[t]];
+    }
+  };
+  float qm[2], q0[2], e0[2], c0[2], qn[2], en[2], cn[2];
+  auto sums = [&](float(&q)[2], float(&e)[2], float(&c)[2]) {
+    float x[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) x[t] = l[t] + r[t];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      e[t] = x[t + 1] + (m[t] + m[t + 2]);
+      c[t] = x[t] + x[t + 2];
+      q[t] = fmaf(2.0f, m[t + 1], e[t]);
+    }
+  };
+  fetch(k0 - 1);
+  sums(qm, e0, c0);
+  fetch(k0);
+  sums(q0, e0, c0);
+  fetch(k0 + 1);
+  unsigned g[2] = {k0 * sz + om[1], k0 * sz + (two ? om[2] : om[1])};
+  float bn[2] = {b[g[0]], b[g[1]]}, hn[2], ln[2];
+  if (LAST) {
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      hn[t] = shi[g[t]];
+      ln[t] = slo[g[t]];
+    }
+  }
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    sums(qn, en, cn);
+    const float bc[2] = {bn[0], bn[1]};
+    float hc[2], lc[2];
+    if (LAST) {
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        hc[t] = hn[t];
+        lc[t] = ln[t];
+      }
+    }
+    const unsigned go[2] = {g[0], g[1]};
+    if (k + 1 < k1) {
+      fetch(k + 2);
+      if (k + 2 + kPre3 <= k1) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          prefetch_l2(y + g[t] + (2 + kPre3) * sz);
+          if (y != b) prefetch_l2(b + g[t] + (1 + kPre3) * sz);
+          if (LAST) {
+            prefetch_l2(shi + g[t] + (1 + kPre3) * sz);
+            prefetch_l2(slo + g[t] + (1 + kPre3) * sz);
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        g[t] += sz;
+        bn[t] = b[g[t]];
+        if (LAST) {
+          hn[t] = shi[g[t]];
+          ln[t] = slo[g[t]];
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const float T = fmaf(2.0f, e0[t], c0[t]) + (qm[t] + qn[t]);
+      if (LAST) {
+        ff_add_scaled_bc(hc[t], lc[t], bc[t], A.q * T, A.s_hi, A.s_lo);
+        if (t == 0 || two) {
+          shi[go[t]] = hc[t];
+          slo[go[t]] = lc[t];
+        }
+      } else if (t == 0 || two) {
+        out[go[t]] = fmaf(A.q, T, bc[t]);
+      }
+      qm[t] = q0[t];
+      q0[t] = qn[t];
+      e0[t] = en[t];
+      c0[t] = cn[t];
+    }
+  }
+  if (!LAST) {
+    // zeros on the walls the next level reads: those next to the thread's points, corners included
+    const int jl = two ? j + 1 : j;
+    const int di0 = d0 && i == 1 ? -1 : 0, di1 = d0 && i == n0 - 2 ? 1 : 0;
+    const int dj0 = d1 && j == 1 ? -1 : 0, dj1 = d1 && jl == n1 - 2 ? 1 : 0;
+    const int dk0 = d2 && k0 == 1 ? -1 : 0, dk1 = d2 && k1 == n2 - 1 ? 1 : 0;
+    if (di0 | di1 | dj0 | dj1 | dk0 | dk1)
+      for (int k = k0 + dk0; k < k1 + dk1; ++k)
+        for (int jj = j + dj0; jj <= jl + dj1; ++jj)
+          for (int ii = i + di0; ii <= i + di1; ++ii)
+            if (k < k0 || k >= k1 || jj < j || jj > jl || ii != i) out[((size_t)k * n1 + jj) * n0 + ii] = 0.0f;
+  }
+}
+
 // One sweep of the FP32 Richardson iteration on 6 h^2 P1 x = b (6h^2 P1 = d - 6(Lx + Ly + Lz)
-// - (LxLy + LyLz + LzLx), d = 6 c1 h^2 as hi + lo), x_{k+1} = x_k + omega (b - 6 h^2 P1 x_k) from
-// x_1 = omega b.  FIRST: the sweep from x_1, read as omega b.  LAST: the state (hi, lo) += s x +
-// s corr (two separate error-free additions) instead of writing x.
+// - (LxLy + LyLz + LzLx), d = 6 c1 h^2 as hi + lo), x_{k+1} = x_k + omega (b - 6 h^2 P1 x_k): the
+// refinement after a transform solve.  LAST: the state (hi, lo) += s x + s corr (two separate
+// error-free additions) instead of writing x.
 // A block of SWX x SWT threads takes a tile of SWX x SWY points and marches SWZ planes along z;
 // a thread takes rows j and j + SWT of one column, and every operation acts on that pair at once
 // (paired FP32 instructions).  The iterate on planes z-1, z, z+1 over the tile with a one-point
@@ -680,7 +877,7 @@ constexpr int SWXP = SWX + 2, SWRP = SWT + 2;  // pair rows of a staged plane
 constexpr int SWN = SWRP * SWXP;               // staged pairs per plane
 static_assert(SWN <= 2 * SWX * SWT, "two staged pairs per thread");
 
-template <bool FIRST, bool LAST>
+template <bool LAST>
 __global__ void __launch_bounds__(SWX * SWT, LAST ? 4 : 5) k_sweep3d32(const float* __restrict__ b, const float* __restrict__ xin,
                                                             float* __restrict__ xout, Shape3 s, float d_hi, float d_lo,
                                                             float omega, float* __restrict__ shi,
@@ -696,7 +893,7 @@ __global__ void __launch_bounds__(SWX * SWT, LAST ? 4 : 5) k_sweep3d32(const flo
   const int k0 = blockIdx.z * SWZ, k1 = min(k0 + SWZ, nu2);
   const bool in0 = iu < nu0 && ju < nu1, in1 = iu < nu0 && ju + SWT < nu1;
   const int sz = n0 * n1;
-  const float* X0 = FIRST ? b : xin;
+  const float* X0 = xin;
   // position q along an axis of n points: false where the value is a wall zero, else the point
   // (even ghosts of a Neumann axis clamped)
   auto place = [](int q, int n, int dir, int* at) {
@@ -732,8 +929,8 @@ __global__ void __launch_bounds__(SWX * SWT, LAST ? 4 : 5) k_sweep3d32(const flo
   const float2 om2 = bc2(omega);
   auto stage = [&](float2(*pl)[SWXP]) {
     float2* f = &pl[0][0];
-    f[t1] = FIRST ? mul2(om2, ra) : ra;
-    if (has2) f[t2] = FIRST ? mul2(om2, rb) : rb;
+    f[t1] = ra;
+    if (has2) f[t2] = rb;
   };
   // per-point operands of the next plane
   float2 bq = make_float2(0.0f, 0.0f), hq = bq, lq = bq;
@@ -809,18 +1006,6 @@ __global__ void __launch_bounds__(SWX * SWT, LAST ? 4 : 5) k_sweep3d32(const flo
     Z0 = Zp;
     Zp = t;
   }
-}
-
-// S = 1: the single iterate x = omega b is the correction, state += s omega b.
-__global__ void k_single3d32(const float* __restrict__ b, Shape3 s, float omega, float* __restrict__ shi,
-                             float* __restrict__ slo, float s_hi, float s_lo) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
-  if (i >= s.n[0] || j >= s.n[1] || !unk3(s, i, j, k)) return;
-  const int p = (k * s.n[1] + j) * s.n[0] + i;
-  float h = shi[p], l = slo[p];
-  ff_add_scaled3(h, l, omega * b[p], s_hi, s_lo);
-  shi[p] = h;
-  slo[p] = l;
 }
 
 dim3 sweep_grid3(const Shape3& s) {  // tiles over the unknowns
@@ -1023,69 +1208,101 @@ ms_status step3d64(ms_grid* g) {
   return MS_OK;
 }
 
-// FP32_REFINED: G (hi, lo) = 12 beta u + L u of component c into the filter buffers of slot c % 3.
-void filter3d32(ms_grid* g, int c, float cb_hi, float cb_lo) {
+// FP32_REFINED: G (hi, lo) = 12 beta u + L u of the components c0 .. c0 + 2 into the filter buffers.
+void filter3d32(ms_grid* g, int c0, float cb_hi, float cb_lo) {
   Grid3D* G3 = g->g3;
-  const Shape3& s = G3->sh[c];
-  const dim3 grd((s.n[0] + FTX - 1) / FTX, (s.n[1] + FTY - 1) / FTY, (s.n[2] + FZ3 - 1) / FZ3), blk(FTX, FTT, 1);
-  k_ffilt3d32<<<grd, blk, 0, g->stream>>>(G3->hi[c], G3->lo[c], s, G3->gh[c % 3], G3->gl[c % 3], cb_hi, cb_lo);
-  // state hi + lo in, G hi + lo out
-  prof_mark(g, KK_FILT3D32, 16.0 * (double)s.size());
+  Filter3d32Args A;
+  int nx = 0, ny = 0;
+  A.nz = 0;
+  double pts = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    const Shape3& s = G3->sh[c0 + c];
+    A.hi[c] = G3->hi[c0 + c];
+    A.lo[c] = G3->lo[c0 + c];
+    A.gh[c] = G3->gh[c];
+    A.gl[c] = G3->gl[c];
+    A.s[c] = s;
+    nx = s.n[0] > nx ? s.n[0] : nx;
+    ny = s.n[1] > ny ? s.n[1] : ny;
+    const int nz = (s.n[2] + FZ3 - 1) / FZ3;
+    A.nz = nz > A.nz ? nz : A.nz;
+    pts += (double)s.size();
+  }
+  launch_pdl(k_ffilt3d32, dim3((nx + 31) / 32, (ny + 2 * FY3 - 1) / (2 * FY3), 3 * A.nz), dim3(32, FY3), 0, g->stream, A,
+             cb_hi, cb_lo);
+  prof_mark(g, KK_FILT3D32, 16.0 * pts);  // state hi + lo in, G hi + lo out
 }
 
-// FP32_REFINED: one Pade term y = A^{-1} D1 G of source component cs (G made by filter3d32) along
-// axis, added with `sign` into R on component cd.  Returns the number of launches issued.
-int term3d32(ms_grid* g, int axis, int cs, int cd, float sign, int accumulate) {
+// FP32_REFINED: one Pade term y = A^{-1} D1 G of source component cs (G made by filter3d32) along an
+// axis, added with `sign` into R of component cd (or written to it).
+struct Term3 {
+  int cs, cd;
+  float sign;
+  int accumulate;
+};
+
+// The two terms of a half-step along one axis in one launch (tables wider than the tile holds: two
+// launches per term).  Returns the number of launches issued.
+int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
   Grid3D* G3 = g->g3;
-  const Shape3& ss = G3->sh[cs];
-  const Shape3& sd = G3->sh[cd];
-  const int kind = (ss.bc[axis] == NEU) ? HALF_TO_NODE : NODE_TO_HALF;
+  const int kind = (G3->sh[q0.cs].bc[axis] == NEU) ? HALF_TO_NODE : NODE_TO_HALF;
   const PadeTable& t = g->pade32[kind];
   const int off = (kind == HALF_TO_NODE) ? 1 : 0;
-  const float* gh = G3->gh[cs % 3];
-  const float* gl = G3->gl[cs % 3];
-  float* R = G3->s32[1];
+  const Term3* q[2] = {&q0, &q1};
   if (t.K + 1 <= K3H) {
-    // differences and band in one tiled kernel
-    const int nt = (t.M + T3O - 1) / T3O;
-    if (axis == 0) {
-      const dim3 grd(nt, (sd.n[1] + 31) / 32, sd.n[2]);
-      k_term3d32<0><<<grd, 256, 0, g->stream>>>(gh, gl, ss, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit,
-                                                 sign, accumulate);
-    } else if (axis == 1) {
-      const dim3 grd((sd.n[0] + 31) / 32, nt, sd.n[2]);
-      k_term3d32<1><<<grd, 256, 0, g->stream>>>(gh, gl, ss, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit,
-                                                 sign, accumulate);
-    } else {
-      const dim3 grd((sd.n[0] + 31) / 32, nt, sd.n[1]);
-      k_term3d32<2><<<grd, 256, 0, g->stream>>>(gh, gl, ss, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit,
-                                                 sign, accumulate);
+    const int P = axis == 0 ? 1 : 0, Q = axis == 2 ? 1 : 2;
+    TermArgs2 A;
+    int np = 0;
+    A.nq = 0;
+    double bytes = 0.0;
+    for (int k = 0; k < 2; ++k) {
+      TermArgs& a = A.t[k];
+      a.gh = G3->gh[q[k]->cs % 3];
+      a.gl = G3->gl[q[k]->cs % 3];
+      a.R = G3->s32[1 + q[k]->cd % 3];
+      a.ss = G3->sh[q[k]->cs];
+      a.sd = G3->sh[q[k]->cd];
+      a.sign = q[k]->sign;
+      a.accumulate = q[k]->accumulate;
+      np = a.sd.n[P] > np ? a.sd.n[P] : np;
+      A.nq = a.sd.n[Q] > A.nq ? a.sd.n[Q] : A.nq;
+      // G hi + lo in, R out (read too when accumulating)
+      bytes += 4.0 * (2.0 * (double)a.ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)a.sd.size());
     }
-    // G hi + lo in, R out (read too when accumulating)
-    prof_mark(g, KK_TERM3D32, 4.0 * (2.0 * (double)ss.size() + (accumulate ? 2.0 : 1.0) * (double)sd.size()));
+    const int nt = (t.M + T3O - 1) / T3O;
+    const dim3 grd = axis == 0 ? dim3(nt, (np + 31) / 32, 2 * A.nq) : dim3((np + 31) / 32, nt, 2 * A.nq), blk(256);
+    auto go = [&](auto kernel) {
+      launch_pdl(kernel, grd, blk, 0, g->stream, A, off, t.M, (const float*)t.d_whi, (const float*)t.d_wlo, t.K, t.B,
+                 (int)t.all_explicit);
+    };
+    if (axis == 0) go(k_term3d32<0>);
+    else if (axis == 1) go(k_term3d32<1>);
+    else go(k_term3d32<2>);
+    prof_mark(g, KK_TERM3D32, bytes);
     return 1;
   }
-  float* d = G3->s32[0];
-  const dim3 grd = grid3(sd, kBlk);
-  if (axis == 0)
-    k_diff3d32<0><<<grd, kBlk, 0, g->stream>>>(gh, gl, ss, d, sd, off, t.M);
-  else if (axis == 1)
-    k_diff3d32<1><<<grd, kBlk, 0, g->stream>>>(gh, gl, ss, d, sd, off, t.M);
-  else
-    k_diff3d32<2><<<grd, kBlk, 0, g->stream>>>(gh, gl, ss, d, sd, off, t.M);
-  if (axis == 0)
-    k_band3d32<0><<<grd, kBlk, 0, g->stream>>>(d, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit, sign,
-                                                accumulate);
-  else if (axis == 1)
-    k_band3d32<1><<<grd, kBlk, 0, g->stream>>>(d, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit, sign,
-                                                accumulate);
-  else
-    k_band3d32<2><<<grd, kBlk, 0, g->stream>>>(d, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit, sign,
-                                                accumulate);
-  // G hi + lo in, d out; d in, R out (read too when accumulating)
-  prof_mark(g, KK_BAND3D32,
-            4.0 * (2.0 * (double)ss.size() + (double)sd.size()) + 4.0 * (double)sd.size() * (accumulate ? 3.0 : 2.0));
-  return 2;
+  for (int k = 0; k < 2; ++k) {
+    const Shape3& ss = G3->sh[q[k]->cs];
+    const Shape3& sd = G3->sh[q[k]->cd];
+    const float* gh = G3->gh[q[k]->cs % 3];
+    const float* gl = G3->gl[q[k]->cs % 3];
+    float* R = G3->s32[1 + q[k]->cd % 3];
+    const float sign = q[k]->sign;
+    const int accumulate = q[k]->accumulate;
+    float* d = G3->s32[0];
+    const dim3 grd = grid3(sd, kBlk);
+    auto go = [&](auto diff, auto band) {
+      diff<<<grd, kBlk, 0, g->stream>>>(gh, gl, ss, d, sd, off, t.M);
+      band<<<grd, kBlk, 0, g->stream>>>(d, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit, sign, accumulate);
+    };
+    if (axis == 0) go(k_diff3d32<0>, k_band3d32<0>);
+    else if (axis == 1) go(k_diff3d32<1>, k_band3d32<1>);
+    else go(k_diff3d32<2>, k_band3d32<2>);
+    // G hi + lo in, d out; d in, R out (read too when accumulating)
+    prof_mark(g, KK_BAND3D32,
+              4.0 * (2.0 * (double)ss.size() + (double)sd.size()) + 4.0 * (double)sd.size() * (accumulate ? 3.0 : 2.0));
+  }
+  return 4;
 }
 
 // Transform solve (tensor cores) of component c followed by ts_sweeps Richardson sweeps with the
@@ -1093,8 +1310,8 @@ int term3d32(ms_grid* g, int axis, int cs, int cd, float sign, int accumulate) {
 void solve3d32_ts(ms_grid* g, int c, float d_hi, float d_lo, float omega, float s_hi, float s_lo, int* nl) {
   Grid3D* G3 = g->g3;
   const Shape3& s = G3->sh[c];
-  const float* b = G3->s32[1];
-  float* buf[2] = {G3->s32[2], G3->s32[3]};
+  const float* b = G3->s32[1 + c % 3];
+  float* buf[2] = {G3->gh[c % 3], G3->gl[c % 3]};  // the filter's planes are free by now
   *nl += ts_solve(*G3->ts, s, b, buf[0], 6.0f * (float)(g->c1 * g->h * g->h), g->stream, g);
   const dim3 grd = sweep_grid3(s), blk(SWX, SWT, 1);
   const int R = G3->ts_sweeps;
@@ -1102,48 +1319,61 @@ void solve3d32_ts(ms_grid* g, int c, float d_hi, float d_lo, float omega, float 
     const float* xin = buf[k & 1];
     float* xo = buf[(k + 1) & 1];
     if (k == R - 1)
-      k_sweep3d32<false, true><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, G3->hi[c], G3->lo[c],
+      k_sweep3d32<true><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, G3->hi[c], G3->lo[c],
                                                            s_hi, s_lo);
     else
-      k_sweep3d32<false, false><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, G3->hi[c], G3->lo[c],
+      k_sweep3d32<false><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, G3->hi[c], G3->lo[c],
                                                             s_hi, s_lo);
     prof_mark(g, KK_SWEEP3D32, 4.0 * (double)s.size() * (2.0 + (k == R - 1 ? 4.0 : 1.0)));
   }
   *nl += R;
 }
 
-void solve3d32(ms_grid* g, int c, float d_hi, float d_lo, float omega, float s_hi, float s_lo, int S, int* nl) {
+// The solves and updates of the components c0 .. c0 + 2 from s32[1..3]; the filter buffers, free by now,
+// hold the iterates.
+void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
   Grid3D* G3 = g->g3;
+  const bool e = c0 == 0;
   if (G3->solver == MS_SOLVER_TRANSFORM_TC) {
-    solve3d32_ts(g, c, d_hi, d_lo, omega, s_hi, s_lo, nl);
+    for (int c = 0; c < 3; ++c)
+      solve3d32_ts(g, c0 + c, k.d_hi, k.d_lo, k.omega, e ? k.sE_hi : k.sH_hi, e ? k.sE_lo : k.sH_lo, nl);
     return;
   }
-  const Shape3& s = G3->sh[c];
-  const float* b = G3->s32[1];
-  float* buf[2] = {G3->s32[2], G3->s32[3]};
-  // launch k (k = 1 .. S-1, or one launch when S = 1) produces iterate k + 1 from iterate k
-  const float* xin = nullptr;
-  const int L = S > 1 ? S - 1 : 1;
-  for (int k = 0; k < L; ++k) {
-    const bool last = (k == L - 1);
-    float* xo = buf[k & 1];
-    const dim3 grd = sweep_grid3(s), blk(SWX, SWT, 1);
-    float* hi = G3->hi[c];
-    float* lo = G3->lo[c];
-    if (S == 1)
-      k_single3d32<<<grid3(s, kBlk), kBlk, 0, g->stream>>>(b, s, omega, hi, lo, s_hi, s_lo);
-    else if (k == 0 && last)
-      k_sweep3d32<true, true><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, hi, lo, s_hi, s_lo);
-    else if (k == 0)
-      k_sweep3d32<true, false><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, hi, lo, s_hi, s_lo);
-    else if (last)
-      k_sweep3d32<false, true><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, hi, lo, s_hi, s_lo);
-    else
-      k_sweep3d32<false, false><<<grd, blk, 0, g->stream>>>(b, xin, xo, s, d_hi, d_lo, omega, hi, lo, s_hi, s_lo);
-    prof_mark(g, KK_SWEEP3D32, 4.0 * (double)s.size() * ((k == 0 ? 1.0 : 2.0) + (last ? 4.0 : 1.0)));
-    xin = xo;
+  const Cheb& p = g->walk.cheb;
+  Lev3d32Args A;
+  int tx = 0, ty = 0;
+  A.nz = 0;
+  double pts = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    const Shape3& s = G3->sh[c0 + c];
+    A.s[c] = s;
+    A.b[c] = G3->s32[1 + c];
+    A.hi[c] = G3->hi[c0 + c];
+    A.lo[c] = G3->lo[c0 + c];
+    int u[3];
+    for (int a = 0; a < 3; ++a) u[a] = s.n[a] - 2 * (s.bc[a] == DIR);
+    tx = std::max(tx, (u[0] + 31) / 32);
+    ty = std::max(ty, (u[1] + 2 * L3Y - 1) / (2 * L3Y));
+    A.nz = std::max(A.nz, (u[2] + L3Z - 1) / L3Z);
+    pts += (double)s.size();
   }
-  *nl += L;
+  const double s = (e ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0;
+  A.s_hi = (float)s;
+  A.s_lo = (float)(s - (double)A.s_hi);
+  const dim3 grd(tx, ty, 3 * A.nz), blk(32, L3Y);
+  for (int l = p.m - 1; l >= 1; --l) {
+    const int step = p.m - 1 - l;
+    A.q = (float)p.q[l];
+    for (int c = 0; c < 3; ++c) {
+      float* buf[2] = {G3->gh[c], G3->gl[c]};
+      A.y[c] = step == 0 ? A.b[c] : buf[(step + 1) & 1];
+      A.out[c] = buf[step & 1];
+    }
+    if (l == 1) launch_pdl(k_lev3d32<true>, grd, blk, 0, g->stream, A);
+    else launch_pdl(k_lev3d32<false>, grd, blk, 0, g->stream, A);
+    prof_mark(g, KK_SWEEP3D32, 4.0 * pts * ((step == 0 ? 1.0 : 2.0) + (l == 1 ? 4.0 : 1.0)));
+  }
+  *nl += p.m - 1;
 }
 
 ms_status step3d32(ms_grid* g) {
@@ -1155,32 +1385,24 @@ ms_status step3d32(ms_grid* g) {
     prof_mark(g, KK_SRC, 0.0);
     nl += 1;
   }
-  auto add_src = [&](int c) {  // source term in the units of b, before the solve of component c
-    if (!g->src3) return;
-    src3_add(g, c, G3->s32[1]);
-    prof_mark(g, KK_SRC, 8.0 * (double)G3->sh[c].size());
+  // c0: first component of the half-step's fields, cs: of its sources; R_c = sign (D_{c+1} G_{c+2} -
+  // D_{c+2} G_{c+1}) axis by axis, source terms in the units of b, the solves
+  auto half = [&](int c0, int cs, float sign) {
+    filter3d32(g, cs, k.cb_hi, k.cb_lo);
     nl += 1;
+    nl += terms3d32(g, 2, Term3{cs + 1, c0 + 0, -sign, 0}, Term3{cs + 0, c0 + 1, sign, 0});
+    nl += terms3d32(g, 1, Term3{cs + 2, c0 + 0, sign, 1}, Term3{cs + 0, c0 + 2, -sign, 0});
+    nl += terms3d32(g, 0, Term3{cs + 2, c0 + 1, -sign, 1}, Term3{cs + 1, c0 + 2, sign, 1});
+    if (g->src3)
+      for (int c = 0; c < 3; ++c) {
+        src3_add(g, c0 + c, G3->s32[1 + c]);
+        prof_mark(g, KK_SRC, 8.0 * (double)G3->sh[c0 + c].size());
+        nl += 1;
+      }
+    solve3d32(g, c0, k, &nl);
   };
-  // Step 1: G~ of H_x, H_y, H_z, then per E component its two Pade terms and its solve
-  for (int c = 3; c < 6; ++c) filter3d32(g, c, k.cb_hi, k.cb_lo);
-  nl += 3;
-  for (int e = 0; e < 3; ++e) {
-    const int p1 = (e + 1) % 3, p2 = (e + 2) % 3;
-    nl += term3d32(g, p1, 3 + p2, e, 1.0f, 0);
-    nl += term3d32(g, p2, 3 + p1, e, -1.0f, 1);
-    add_src(e);
-    solve3d32(g, e, k.d_hi, k.d_lo, k.omega, k.sE_hi, k.sE_lo, k.S, &nl);
-  }
-  // Step 2: G~ of the updated E components, then per H component
-  for (int c = 0; c < 3; ++c) filter3d32(g, c, k.cb_hi, k.cb_lo);
-  nl += 3;
-  for (int hc = 0; hc < 3; ++hc) {
-    const int p1 = (hc + 1) % 3, p2 = (hc + 2) % 3;
-    nl += term3d32(g, p1, p2, 3 + hc, -1.0f, 0);
-    nl += term3d32(g, p2, p1, 3 + hc, 1.0f, 1);
-    add_src(3 + hc);
-    solve3d32(g, 3 + hc, k.d_hi, k.d_lo, k.omega, k.sH_hi, k.sH_lo, k.S, &nl);
-  }
+  half(0, 3, 1.0f);   // Step 1: E from H
+  half(3, 0, -1.0f);  // Step 2: H from the updated E
   if (g->src3) {
     launch_tick(g);
     prof_mark(g, KK_SRC, 0.0);
@@ -1482,8 +1704,9 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
         s = fail3(MS_ECUDA, "copy of FP32 Pade tables failed");
     }
     if (s == MS_OK && upload_band_row() != 0) s = fail3(MS_ECUDA, "cannot upload the interior band row");
-    // Richardson sweeps to 1e-10 (below the FP32 rounding noise, which is not coherent)
-    if (s == MS_OK) s = ms_solver_sweeps(3, d->r, MS_FP32_REFINED, 1e-10, &g->p1_sweeps32);
+    // the solve polynomial to 1e-10 (below the FP32 rounding noise, which is not coherent)
+    if (s == MS_OK && !cheb_coefs(6.0 * g->c1 * g->h * g->h + 24.0, 8.0, 16.0, 1e-10, &g->walk.cheb))
+      s = fail3(MS_ENOTCONV, "the FP32 solve polynomial needs too high a degree");
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->hi[c], G3->sh[c].size());
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->lo[c], G3->sh[c].size());
     for (int k = 0; k < 4 && s == MS_OK; ++k) s = alloc3(&G3->s32[k], G3->nmax);
