@@ -227,10 +227,11 @@ ms_status taylor_init_dev(ms_grid* g, const double* ez0) {
   return ms_set_fields_device(g, comps, 0);
 }
 
-// The reverse pass in FP32 (adjoint32.cu) on FP32_REFINED grids unless FP64 was selected.
+// The reverse pass in FP32 (adjoint32.cu) on FP32_REFINED grids unless FP64 was selected.  Grids of fewer
+// cells than the walks' two end segments take (32) run it in FP64: fewer launches' work there.
 bool use32(const ms_grid* g) {
   const int prec = g->adj_precision < 0 ? g->desc.precision : g->adj_precision;
-  return prec == MS_FP32_REFINED;
+  return prec == MS_FP32_REFINED && g->N >= 32;
 }
 
 // (M^T)^nsteps on adj[0..2] in the selected arithmetic (FP32: through the float-float state).

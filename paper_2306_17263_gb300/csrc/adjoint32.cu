@@ -5,46 +5,50 @@
 //   S1: E   += sE P~_E^{-1} (Y_x F~ H_y - Y_y F~ H_x),
 //   S2: H_x += sH P~_Hx^{-1} (-Y_y F~ E),   H_y += sH P~_Hy^{-1} (Y_x F~ E),
 // with P~ = 6 h^2 P1 (Def. "def:operatorsP"), F~ = 12 beta + L the filter of Eq. "eq:ell" on the
-// source grid, Y = W D the Pade derivative of App. A.1 as a band W of A^{-1} applied to the first
-// differences D of a line, sE = 12 Z / r, sH = 12 / (r Z).  F~ and P~ are symmetric on the unknowns
-// (Dirichlet zeros, even Neumann ghosts), so the transposed step M^T = S1^T S2^T is
+// source grid, Y = A^{-1} D the Pade derivative of App. A.1 (D the first differences of a line),
+// sE = 12 Z / r, sH = 12 / (r Z).  F~ and P~ are symmetric on the unknowns (Dirichlet zeros, even Neumann
+// ghosts), so the transposed step M^T = S1^T S2^T is
 //   S2^T: l_E  += sH F~_E (-Y_y^T P~^{-1} l_Hx + Y_x^T P~^{-1} l_Hy),
 //   S1^T: l_Hy += sE F~_Hy Y_x^T P~_E^{-1} l_E,   l_Hx += -sE F~_Hx Y_y^T P~_E^{-1} l_E,
-// with Y^T = D^T W^T: (Y^T u)_j = v_{j-1} - v_j, v = W^T u, v_{-1} = v_M = 0.
+// with Y^T = D^T A^{-T}: (Y^T u)_j = v_{j-1} - v_j, v = A^{-T} u, v_{-1} = v_M = 0.
 //
 // Precision.  D^T takes the difference of two nearly equal values of a smooth v, which would
-// amplify an FP32 rounding of v by 1 / (pi k h).  So every quantity before that difference is
-// carried with more than FP32 accuracy: the adjoint state l is a float-float pair; the solve
-// u = P~^{-1} l iterates in FP32 against a residual with l's low part and an exact two-product of
-// the diagonal term, and returns the last iterate x and its correction c as a pair (u = x + c to
-// about 31 bits, far below the correction's own size); v = W^T u is accumulated in float-float
-// (exact two-products of the hi parts, the lo parts of W and u folded into the error term); only
-// the difference of v is rounded to FP32.  The filter and the sH / sE scaling act on that
-// difference, a well-conditioned FP32 value, and the result is added to l with error-free
-// transformations.  The step is the exact transpose of the FP32_REFINED forward operator (same
-// truncated band tables) up to this rounding.
+// amplify an FP32 rounding of v by 1 / (pi k h).  A^{-1} and the difference commute on the infinite line,
+// so the difference is taken first, of the float-float u, and A^{-1} is applied to it in FP32: with
+// e_j = u_{j-1} - u_j (u_{-1} = u_M = 0, zero beyond the line) and w the infinite-line solution for e,
+// (Y^T u)_j = w_j + k_j w_0 near the first end and its mirror image at the last (the end rows of A^{-T}
+// change v by a multiple of its first value, and w_0 = (rho - 1) v_0).  u = p_0 (l + c), c the last level
+// of the solve's polynomial applied to l_hi: the pair (l_hi, l_lo + c) holds it to about 31 bits without
+// a new high part.  The filter and the scaling act on the difference, a well-conditioned FP32 value, and
+// the result is added to l with error-free transformations.  The step is the transpose of the
+// FP32_REFINED forward operator up to this rounding.
+//
+// Kernels, six launches per reverse step, the walks of k_tiled.cu turned round: solve (k_solve_pair),
+// both transposed derivatives into planes (k_walk_dT), filter and update (k_filter_update), for the H
+// fields and then for E_z.  The band form before it (separate sweeps, transposed bands in float-float, one
+// kernel per operator, 18 launches) took 165 us per reverse step at 1024^2.
 #include <string>
+#include <vector>
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
+#include "k_rec64.cuh"
 #include "k_tiled.cuh"
+#include "k_walk_dev.cuh"
 
 namespace ms {
 
 struct Adj32 {
+  float* slab = nullptr;
   float* lh[3] = {};  // adjoint state (l_E, l_Hx, l_Hy), hi parts
   float* ll[3] = {};  // lo parts
-  float* ux[2] = {};  // solve results: last iterate ...
-  float* uc[2] = {};  // ... and its correction
-  float* vh[2] = {};  // W^T u, float-float, in the target field's layout
-  float* vl[2] = {};
-  float* sw[2] = {};  // sweep iterates
+  float* uc[3] = {};  // low parts of the solutions u = p_0 (l_hi + uc)
+  float* py[3] = {};  // transposed derivatives along y (E_z, H_x) and ...
+  float* px[3] = {};  // ... along x (E_z, H_y)
   Graph g1, gk;
 };
 
 namespace {
-
-const dim3 kBlk2(32, 8, 1);
 
 ms_status a32fail(ms_status s, const std::string& m) {
   set_last_error(m.c_str());
@@ -57,343 +61,456 @@ void free_graph32(Graph* gr) {
   *gr = Graph{};
 }
 
-dim3 grid2(int nx, int ny) { return dim3((nx + kBlk2.x - 1) / kBlk2.x, (ny + kBlk2.y - 1) / kBlk2.y); }
+constexpr int kEndT = 16;   // rows the end correction reaches (its vector decays from the fourth row on)
+constexpr int TOUT = 104;   // columns a warp writes along x (12 on each side: carries and end rows)
+constexpr int THALO = 12;
 
-// Richardson sweep on 6 h^2 P1 x = b with b = (b_hi, b_lo) (see the tile solve): FIRST reads the
-// first iterate as omega b_hi; LAST writes the iterate and its correction separately.
-template <bool FIRST, bool LAST>
-__global__ void k_sweepT32(const float* __restrict__ bh, const float* __restrict__ bl, const float* __restrict__ xin,
-                           float* __restrict__ xout, float* __restrict__ cout, int nx, int ny, int bcx, int bcy,
-                           float d_hi, float d_lo, float omega) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= nx || j >= ny) return;
-  const size_t p = (size_t)j * nx + i;
-  if (!interior(bcx, i, nx) || !interior(bcy, j, ny)) {
-    xout[p] = 0.0f;
-    if (LAST) cout[p] = 0.0f;
-    return;
+// ---- solve ---------------------------------------------------------------------------------
+
+template <int P>
+__global__ void __launch_bounds__(32 * WPB, P <= 3 ? 5 : 4) k_solve_pair(const __grid_constant__ SArgs A,
+                                                                         const __grid_constant__ SArgs B, int na) {
+  __shared__ float4 ring[WPB][4 * kRing * 32];
+  pdl_wait();
+  const int w = threadIdx.x >> 5, b = blockIdx.x;
+  if (b < na) s_item<P, true>(A, ring[w], b * WPB + w);
+  else s_item<P, true>(B, ring[w], (b - na) * WPB + w);
+}
+
+// ---- transposed derivatives ----------------------------------------------------------------
+
+// Along y: lines are the columns 1 .. ncol-2, inputs u_0 .. u_{M-1}, outputs 0 .. M, written negated.
+struct YTArgs {
+  const float* uh;  // row of u_0, column 0
+  const float* ul;
+  float* b;         // row of output 0
+  int ld, ncol, M;
+  float k[kEndT];
+  int nstrip, nseg, chunk, end;  // segments: 0 down from the first end, 1 up from the last (`end` rows
+                                 // each), the others `chunk` rows down between them
+};
+
+// Along x, rows 1 .. nrows of E_z- or H_y-shaped fields; pointers at column m = 0.
+struct XTArgs {
+  const float* uh;
+  const float* ul;
+  float* b;
+  int ld, M;     // inputs per line
+  int from_h;    // input u_i at column i of H_y, output j at column j - 1 of E_z; else u_i at column i of
+                 // E_z, output j at column j of H_y
+  float k[kEndT];
+  int nrows, nstrip, nblk, rows;
+};
+
+// A segment of 32 columns: y of e = differences of u, groups of eight rows (k_tiled.cu).  UP: the segment
+// walks up from the last end, rows and sign mirrored.  EDGE: rows may lie beyond the line.
+template <bool EDGE>
+__device__ __forceinline__ void yt_segment(const YTArgs& A, int strip, int seg) {
+  const int lane = threadIdx.x & 31;
+  const int col = 1 + 32 * strip + lane;
+  const bool live = col <= A.ncol - 2;
+  const int cc = min(col, A.ncol - 2);
+  const int M = A.M, R = M + 1;
+  const bool up = seg == 1;
+  const int r0 = seg < 2 ? 0 : A.end + (seg - 2) * A.chunk;
+  const int r1 = seg < 2 ? A.end : min(r0 + A.chunk, R - A.end);
+  const ptrdiff_t st = up ? -(ptrdiff_t)A.ld : (ptrdiff_t)A.ld;
+  const float* ph = A.uh + cc + (up ? (size_t)(M - 1) * A.ld : 0);  // logical row i at ph[i * st]
+  const float* pl = A.ul + cc + (up ? (size_t)(M - 1) * A.ld : 0);
+  float* bp = A.b + cc + (up ? (ptrdiff_t)M * A.ld : 0) + (ptrdiff_t)r0 * st;
+  const float sign = up ? 1.0f : -1.0f;  // results are written negated; the mirror changes the sign
+  auto get = [&](const float* p, int i) { return EDGE ? ((i >= 0 && i < M) ? p[i * st] : 0.0f) : p[i * st]; };
+  const int ms = r0 - 9;
+  float h0 = get(ph, ms - 1), l0 = get(pl, ms - 1);  // u_{m-1}
+  float nh[8], nl[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    nh[t] = get(ph, ms + t);
+    nl[t] = get(pl, ms + t);
   }
-  const int im = clampi(i - 1, nx), ip = clampi(i + 1, nx), jm = clampi(j - 1, ny), jp = clampi(j + 1, ny);
-  // iterate on the 3 x 3 neighbourhood (Dirichlet neighbours are stored zeros, Neumann ones clamp)
-  auto X = [&](int jj, int ii) {
-    const size_t q = (size_t)jj * nx + ii;
-    return FIRST ? omega * bh[q] : xin[q];
+  float z = 0.0f, zp[7] = {}, w0 = 0.0f;
+  const int ngrp = 2 + (r1 - r0 + 7) / 8;
+  for (int gi = 0; gi < ngrp; ++gi) {
+    const int m0 = ms + 8 * gi;
+    float ch[8], cl[8], zc[8], y[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      ch[t] = nh[t];
+      cl[t] = nl[t];
+    }
+    if (gi + 1 < ngrp) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        nh[t] = get(ph, m0 + 8 + t);
+        nl[t] = get(pl, m0 + 8 + t);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const float e = (h0 - ch[t]) + (l0 - cl[t]);
+      h0 = ch[t];
+      l0 = cl[t];
+      zc[t] = z = fmaf(kRhoF, z, e);
+    }
+    float acc = zc[7];
+#pragma unroll
+    for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
+    y[7] = acc = fmaf(kRhoF, acc, zc[0]);
+#pragma unroll
+    for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRhoF, acc, zp[t]);
+#pragma unroll
+    for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
+    if (gi < 2) continue;
+    if (EDGE && seg < 2) {  // the first end's rows
+      if (gi == 2) w0 = y[0];
+      if (gi < 2 + kEndT / 8) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) y[t] = fmaf(A.k[8 * (gi - 2) + t], w0, y[t]);
+      }
+    }
+    if (live) {
+      const int left = r1 - (r0 + 8 * (gi - 2));
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t < left) bp[t * st] = sign * y[t];
+    }
+    bp += 8 * st;
+  }
+}
+
+__device__ __forceinline__ void yt_item(const YTArgs& A, int item) {
+  if (item >= A.nstrip * A.nseg) return;
+  const int seg = item / A.nstrip, strip = item - seg * A.nstrip;
+  // rows of u: r0 - 10 .. r1 + 15
+  if (seg >= 2 && A.end + (seg - 2) * A.chunk >= 10 && min(A.end + (seg - 1) * A.chunk, A.M + 1 - A.end) + 15 < A.M)
+    yt_segment<false>(A, strip, seg);
+  else yt_segment<true>(A, strip, seg);
+}
+
+template <bool FROM_H, bool EDGE>
+__device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int strip, int blk) {
+  const int lane = threadIdx.x & 31;
+  const int m_s = TOUT * strip - THALO, m0 = m_s + 4 * lane;
+  const int M = A.M, o = FROM_H ? 1 : 0;  // output index j = column + o
+  const int Mo = M + 1 - 2 * o;           // columns written: the unknown ones of E_z (0 .. M-2), all of H_y
+  const int j0 = 1 + blk * A.rows, j1 = min(j0 + A.rows, 1 + A.nrows);
+  const size_t ld = A.ld;
+  const bool ok = !EDGE || (m0 >= -4 && m0 + 8 <= A.ld);
+  const bool out = lane >= THALO / 4 && lane < (THALO + TOUT) / 4 && (!EDGE || (m0 >= 0 && m0 < Mo));
+  bool inu[4] = {true, true, true, true}, ine[4] = {true, true, true, true};
+  float kl[4] = {}, kr[4] = {};
+  bool left = false, right = false;
+  int ll = 0, el = 0, lr = 0, er = 0;  // lane and element of output 0 and of output M
+  if (EDGE) {
+    left = strip == 0;
+    right = M - o <= m_s + 127;
+    ll = (-o - m_s) >> 2;
+    el = (-o - m_s) & 3;
+    lr = (M - o - m_s) >> 2;
+    er = (M - o - m_s) & 3;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int m = m0 + q, j = m + o, r = M - j;
+      inu[q] = m >= 0 && m < M;
+      ine[q] = j >= 0 && j <= M;
+      kl[q] = (left && j >= 0 && j < kEndT) ? A.k[j & (kEndT - 1)] : 0.0f;
+      kr[q] = (right && r >= 0 && r < kEndT) ? A.k[r & (kEndT - 1)] : 0.0f;
+    }
+  }
+  const size_t off = ok ? m0 : 0;
+  const float* fh = A.uh + (size_t)j0 * ld + off;
+  const float* fl = A.ul + (size_t)j0 * ld + off;
+  int todo = j1 - j0;
+  auto fetch = [&](int slot) {
+    if (todo > 0) {
+      cp16(ring + (2 * slot) * 32 + lane, fh, ok);
+      cp16(ring + (2 * slot + 1) * 32 + lane, fl, ok);
+    }
+    cp_commit();
+    fh += ld;
+    fl += ld;
+    --todo;
   };
-  const float x = X(j, i);
-  const float lx = fmaf(-2.0f, x, X(j, im) + X(j, ip));
-  const float ly = fmaf(-2.0f, x, X(jm, i) + X(jp, i));
-  const float lxm = fmaf(-2.0f, X(jm, i), X(jm, im) + X(jm, ip));
-  const float lxp = fmaf(-2.0f, X(jp, i), X(jp, im) + X(jp, ip));
-  const float lxly = fmaf(-2.0f, lx, lxm + lxp);
-  const float rest = fmaf(-6.0f, lx + ly, -lxly);
-  const float ph = __fmul_rn(d_hi, x);
-  const float pl = fmaf(d_lo, x, fmaf(d_hi, x, -ph));
-  const float res = __fsub_rn(__fsub_rn(__fadd_rn(__fsub_rn(bh[p], ph), bl[p]), pl), rest);
-  const float corr = omega * res;
-  if (LAST) {
-    xout[p] = x;
-    cout[p] = corr;
-  } else {
-    xout[p] = x + corr;
+#pragma unroll
+  for (int t = 0; t < kAhead; ++t) fetch(t);
+  float* bp = A.b + (size_t)j0 * ld + m0;
+  int rd = 0, wr = kAhead;
+  for (int jj = j0; jj < j1; ++jj, bp += ld) {
+    cp_wait<kAhead - 1>();
+    const float4 H = ring[(2 * rd) * 32 + lane], L = ring[(2 * rd + 1) * 32 + lane];
+    fetch(wr);
+    rd = rd == kRing - 1 ? 0 : rd + 1;
+    wr = wr == kRing - 1 ? 0 : wr + 1;
+    float h[4] = {H.x, H.y, H.z, H.w}, l[4] = {L.x, L.y, L.z, L.w}, d[4], y[4];
+    if (EDGE) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        h[q] = inu[q] ? h[q] : 0.0f;
+        l[q] = inu[q] ? l[q] : 0.0f;
+      }
+    }
+    // e of output j = u_{j-1} - u_j
+    if (FROM_H) {  // j = column + 1
+      const float hn = __shfl_down_sync(kFull, h[0], 1), ln = __shfl_down_sync(kFull, l[0], 1);
+      d[0] = (h[0] - h[1]) + (l[0] - l[1]);
+      d[1] = (h[1] - h[2]) + (l[1] - l[2]);
+      d[2] = (h[2] - h[3]) + (l[2] - l[3]);
+      d[3] = (h[3] - hn) + (l[3] - ln);
+    } else {  // j = column
+      const float hp = __shfl_up_sync(kFull, h[3], 1), lp = __shfl_up_sync(kFull, l[3], 1);
+      d[0] = (hp - h[0]) + (lp - l[0]);
+      d[1] = (h[0] - h[1]) + (l[0] - l[1]);
+      d[2] = (h[1] - h[2]) + (l[1] - l[2]);
+      d[3] = (h[2] - h[3]) + (l[2] - l[3]);
+    }
+    if (EDGE) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) d[q] = ine[q] ? d[q] : 0.0f;
+    }
+    float t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[0], d[1]), d[2]), d[3]);
+    float c1 = __shfl_up_sync(kFull, t, 1), c2 = __shfl_up_sync(kFull, t, 2);
+    if (EDGE) {
+      c1 = lane < 1 ? 0.0f : c1;
+      c2 = lane < 2 ? 0.0f : c2;
+    }
+    float c = fmaf(kR4, c2, c1);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c = d[q] = fmaf(kRhoF, c, d[q]);
+    t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[3], d[2]), d[1]), d[0]);
+    c1 = __shfl_down_sync(kFull, t, 1);
+    c2 = __shfl_down_sync(kFull, t, 2);
+    if (EDGE) {
+      c1 = lane > 30 ? 0.0f : c1;
+      c2 = lane > 29 ? 0.0f : c2;
+    }
+    c = fmaf(kR4, c2, c1);
+#pragma unroll
+    for (int q = 3; q >= 0; --q) c = y[q] = fmaf(kRhoF, c, d[q]);
+    if (EDGE) {
+      auto pick = [&](int e) { return e == 0 ? y[0] : (e == 1 ? y[1] : (e == 2 ? y[2] : y[3])); };
+      float wl = 0.0f, wrt = 0.0f;
+      if (left) wl = __shfl_sync(kFull, pick(el), ll);
+      if (right) wrt = __shfl_sync(kFull, pick(er), lr);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] = fmaf(kr[q], wrt, fmaf(kl[q], wl, y[q]));
+    }
+    if (out) *reinterpret_cast<float4*>(bp) = make_float4(y[0], y[1], y[2], y[3]);  // (pads: never read unmasked)
   }
 }
 
-// v = W^T u along lines of one axis, in float-float.  Line l (lines [line_lo, line_hi)) holds the
-// M outputs r of the forward band at u[(r + uoff) * ustride_along + l * ustride_across]; v_m
-// (m = 0..M-1) and v_M = 0 go to v[m * vstride_along + l * vstride_across].
-struct BandT {
-  const float* ux;
-  const float* uc;
-  float* vh;
-  float* vl;
-  int ua, uc_, uoff;  // u strides along / across the line, offset of output 0 along the line
-  int va, vc;         // v strides along / across
-  int line_lo, line_hi;
-  const float* whi;
-  const float* wlo;
-  int M, K, B, all_explicit;
+template <bool FROM_H>
+__device__ __forceinline__ void xt_item(const XTArgs& A, float4* ring, int item) {
+  if (item >= A.nstrip * A.nblk) return;
+  const int blk = item / A.nstrip, strip = item - blk * A.nstrip;
+  if (strip == 0 || A.M <= TOUT * strip - THALO + 128) xt_block<FROM_H, true>(A, ring, strip, blk);
+  else xt_block<FROM_H, false>(A, ring, strip, blk);
+}
+
+template <bool FROM_H>
+__global__ void __launch_bounds__(32 * WPB) k_walk_dT(const __grid_constant__ YTArgs Y, const __grid_constant__ XTArgs X,
+                                                      int nyb) {
+  __shared__ float4 ring[WPB][2 * kRing * 32];
+  pdl_wait();
+  const int w = threadIdx.x >> 5, b = blockIdx.x;
+  if (b < nyb) yt_item(Y, b * WPB + w);
+  else xt_item<FROM_H>(X, ring[w], (b - nyb) * WPB + w);
+}
+
+// ---- filter and update ---------------------------------------------------------------------
+
+// l (hi, lo) += (s_hi + s_lo)(12 beta y + L y) at the unknowns of a field, y = p1 + p2 (or p1) there, 0 on
+// Dirichlet walls, mirrored across Neumann ones.  Bound by memory: a lane takes four columns of a row.
+struct FArgs {
+  const float* p1;  // at column m = 0 of row 0
+  const float* p2;
+  float* lh;
+  float* ll;
+  int ld, M, u0, u1, neu_x, neu_y;
+  float cb_hi, cb_lo, s_hi, s_lo;  // 12 beta - 4
 };
-
-// One term of the float-float sum: (sh, sl) += (w + wl)(a + c), exact product of the hi parts.
-__device__ __forceinline__ void ff_fma_acc(float& sh, float& sl, float w, float wl, float a, float c) {
-  const float prod = __fmul_rn(w, a);
-  float e = fmaf(w, a, -prod);
-  e = fmaf(w, c, e);
-  e = fmaf(wl, a, e);
-  const float s = __fadd_rn(sh, prod);
-  const float bb = __fsub_rn(s, sh);
-  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(prod, bb));
-  sh = s;
-  sl = __fadd_rn(sl, __fadd_rn(err, e));
-}
-
-// Tiles of the transposed band: AXIS 0 (lines are rows): 8 lines x 128 outputs per block, a warp
-// per line and four outputs per lane 32 apart; AXIS 1 (lines are columns): 32 lines x 32 outputs,
-// lanes across the lines.  The inputs a tile reads (its outputs widened by the band's reach, zero
-// past the line) are staged once in shared memory with coalesced loads; outputs whose window lies
-// in the interior rows of the table read the one interior row.
-constexpr int BT_THREADS = 256;
-constexpr int BT_KMAX = kBand32Max;
-template <int AXIS>
-struct BandTile {
-  static constexpr int LINES = AXIS == 0 ? 8 : 32;
-  static constexpr int OUTS = AXIS == 0 ? 128 : 32;
-  static constexpr int WIN = OUTS + 2 * BT_KMAX + 2;  // staged inputs per line
+struct FArgs2 {
+  FArgs f[2];
 };
-
-template <int AXIS>
-__global__ void __launch_bounds__(BT_THREADS) k_bandT32(BandT p) {
-  using T = BandTile<AXIS>;
-  __shared__ float sx[T::LINES][T::WIN + 1];
-  __shared__ float sc[T::LINES][T::WIN + 1];
-  const int tid = threadIdx.x;
-  const int m0 = blockIdx.x * T::OUTS;               // first output of the tile
-  const int l0 = p.line_lo + blockIdx.y * T::LINES;  // first line of the tile
-  const int base = m0 - p.K - 1;                     // input index of slot 0
-  const int win = T::OUTS + 2 * p.K + 2;
-  // stage u on [base, base + win) of every line of the tile
-  if (AXIS == 0) {
-    for (int e = tid; e < T::LINES * win; e += BT_THREADS) {
-      const int ll = e / win, q = e - ll * win, r = base + q, l = l0 + ll;
-      float a = 0.0f, c = 0.0f;
-      if (r >= 0 && r < p.M && l < p.line_hi) {
-        const size_t uo = (size_t)(r + p.uoff) * p.ua + (size_t)l * p.uc_;
-        a = p.ux[uo];
-        c = p.uc[uo];
-      }
-      sx[ll][q] = a;
-      sc[ll][q] = c;
+constexpr int FY = 8;
+__global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant__ FArgs2 A2) {
+  pdl_wait();
+  const FArgs& A = A2.f[blockIdx.z];
+  const int m0 = 4 * (blockIdx.x * 32 + threadIdx.x), j = A.u0 + blockIdx.y * FY + threadIdx.y;
+  if (m0 >= A.M || j >= A.u1) return;
+  const size_t ld = A.ld;
+  const int M = A.M;
+  // rows above and below: 0 beyond a Dirichlet wall, the row itself across a Neumann one
+  const int ja = j > A.u0 ? j - 1 : j, jb = j + 1 < A.u1 ? j + 1 : j;
+  const bool oka = j > A.u0 || A.neu_y, okb = j + 1 < A.u1 || A.neu_y;
+  auto row = [&](int r, bool ok, float(&y)[4]) {
+    if (!ok) {
+      y[0] = y[1] = y[2] = y[3] = 0.0f;
+      return;
     }
-  } else {
-    for (int e = tid; e < T::LINES * win; e += BT_THREADS) {
-      const int q = e / T::LINES, ll = e - q * T::LINES, r = base + q, l = l0 + ll;
-      float a = 0.0f, c = 0.0f;
-      if (r >= 0 && r < p.M && l < p.line_hi) {
-        const size_t uo = (size_t)(r + p.uoff) * p.ua + (size_t)l * p.uc_;
-        a = p.ux[uo];
-        c = p.uc[uo];
-      }
-      sx[ll][q] = a;
-      sc[ll][q] = c;
+    float4 a = ld4(A.p1 + r * ld + m0);
+    if (A.p2) {
+      const float4 b = ld4(A.p2 + r * ld + m0);
+      a = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
     }
-  }
-  // the interior row of the table (taps d = m - r = -K .. K+1 at index d + K)
-  __shared__ float wh_s[2 * BT_KMAX + 2], wl_s[2 * BT_KMAX + 2];
-  const int rs = 2 * p.K + 2;
-  if (!p.all_explicit && tid < rs) {
-    wh_s[tid] = p.whi[(size_t)(2 * p.B) * rs + tid];
-    wl_s[tid] = p.wlo[(size_t)(2 * p.B) * rs + tid];
-  }
-  __syncthreads();
-  constexpr int PER = T::OUTS * T::LINES / BT_THREADS;  // outputs per thread
+    y[0] = a.x;
+    y[1] = a.y;
+    y[2] = a.z;
+    y[3] = a.w;
+  };
+  auto one = [&](int m) { return A.p1[j * ld + m] + (A.p2 ? A.p2[j * ld + m] : 0.0f); };
+  float y[4], a[4], b[4];
+  row(j, true, y);
+  row(ja, oka, a);
+  row(jb, okb, b);
+  // columns beside the four, and those past the field
+  const float yl = m0 > 0 ? one(m0 - 1) : (A.neu_x ? y[0] : 0.0f);
+  float l[4] = {yl, y[0], y[1], y[2]}, r[4] = {y[1], y[2], y[3], m0 + 4 < M ? one(m0 + 4) : 0.0f};
 #pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    int ll, mo;
-    if (AXIS == 0) {
-      ll = tid >> 5;
-      mo = (tid & 31) + 32 * k;
-    } else {
-      ll = tid & 31;
-      mo = (tid >> 5) + 8 * k;
-    }
-    const int m = m0 + mo, l = l0 + ll;
-    if (m > p.M || l >= p.line_hi) continue;
-    const size_t vo = (size_t)m * p.va + (size_t)l * p.vc;
-    if (m == p.M) {
-      p.vh[vo] = 0.0f;
-      p.vl[vo] = 0.0f;
-      continue;
-    }
-    float sh = 0.0f, sl = 0.0f;
-    const int r0 = max(0, m - p.K - 1), r1 = min(p.M - 1, m + p.K);
-    if (!p.all_explicit && r0 >= p.B && r1 < p.M - p.B) {
-      // interior row: taps |m - r| >= 3 are below 1.2e-4 of the centre tap (|rho|^3), so their sum
-      // (below 2e-4 of |v|) is accumulated in plain FP32 (error ~1e-11 |v|, including the dropped
-      // lo parts); the five central taps go through the float-float sum
-      const float* ax = &sx[ll][m - base];  // ax[-d] = u_{m-d}
-      const float* ac = &sc[ll][m - base];
-      float small = 0.0f;
+  for (int q = 0; q < 4; ++q)
+    if (m0 + q == M - 1) r[q] = A.neu_x ? y[q] : 0.0f;
+  float* ph = A.lh + j * ld + m0;
+  float* pl = A.ll + j * ld + m0;
+  const float4 H = ld4(ph), L = ld4(pl);
+  float h[4] = {H.x, H.y, H.z, H.w}, lo[4] = {L.x, L.y, L.z, L.w};
 #pragma unroll
-      for (int d = BT_KMAX + 1; d >= -BT_KMAX; --d) {  // farthest taps first
-        if (d >= -2 && d <= 2) continue;
-        if (d > p.K + 1 || d < -p.K) continue;
-        small = fmaf(wh_s[d + p.K], ax[-d], small);
-      }
-#pragma unroll
-      for (int d = 2; d >= -2; --d) ff_fma_acc(sh, sl, wh_s[d + p.K], wl_s[d + p.K], ax[-d], ac[-d]);
-      sl = __fadd_rn(sl, small);
-    } else {
-      for (int r = r0; r <= r1; ++r) {
-        const int t = m - r + p.K;  // tap of input m in row r
-        const float* wh = pade_row_ptr(p.whi, r, p.M, p.K, p.B, p.all_explicit);
-        const float* wl = pade_row_ptr(p.wlo, r, p.M, p.K, p.B, p.all_explicit);
-        ff_fma_acc(sh, sl, wh[t], wl[t], sx[ll][r - base], sc[ll][r - base]);
-      }
-    }
-    const float h2 = __fadd_rn(sh, sl);
-    p.vh[vo] = h2;
-    p.vl[vo] = __fsub_rn(sl, __fsub_rn(h2, sh));
+  for (int q = 0; q < 4; ++q) {
+    if (m0 + q >= M) continue;  // the pads keep their zeros
+    const float f = fmaf(A.cb_hi, y[q], fmaf(A.cb_lo, y[q], (l[q] + r[q]) + (a[q] + b[q])));
+    const float p = __fmul_rn(A.s_hi, f);
+    float e = fmaf(A.s_hi, f, -p);
+    e = fmaf(A.s_lo, f, e);
+    const float u = __fadd_rn(h[q], p);
+    const float bb = __fsub_rn(u, h[q]);
+    const float err = __fadd_rn(__fsub_rn(h[q], __fsub_rn(u, bb)), __fsub_rn(p, bb));
+    const float l2 = __fadd_rn(lo[q], __fadd_rn(err, e));
+    const float h2 = __fadd_rn(u, l2);
+    lo[q] = __fsub_rn(l2, __fsub_rn(h2, u));
+    h[q] = h2;
+  }
+  *reinterpret_cast<float4*>(ph) = make_float4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<float4*>(pl) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+// ---- host ----------------------------------------------------------------------------------
+
+int blocks_of(int items) { return (items + WPB - 1) / WPB; }
+
+// The end correction of the transposed derivative: v = y + t (y_0) with t the vector of the closure's
+// A^{-T} (LineEnds), t_{-1} = -rho, so k_j = (t_{j-1} - t_j) / (rho - 1) on w_0 = (rho - 1) y_0.
+void end_rows_T(int closure, int kind, float* k) {
+  LineEnds e;
+  line_ends(closure, kind, true, &e);
+  const double rho = (double)kRhoF;
+  double prev = -rho;
+  for (int j = 0; j < kEndT; ++j) {
+    const double t = j < kRecWarm ? e.v[j] : 0.0;
+    k[j] = (float)((prev - t) / (rho - 1.0));
+    prev = t;
   }
 }
 
-// l (hi, lo) += (s_hi + s_lo)(12 beta y + L y) at the unknowns of a field, with
-//   y = sx (v^x_{i-1} - v^x_i) + sy (v^y_{j-1} - v^y_j)  (v_{-1} = 0; sx, sy in {-1, 0, 1}),
-// the differences taken of float-float values; L the 5-point h^2 Delta_h with Dirichlet zeros and
-// even Neumann ghosts.  A 32 x 8 tile of y with a one-point halo is formed in shared memory (0 off
-// the unknowns), then filtered and added to l with error-free transformations.
-constexpr int FT_X = 32, FT_Y = 8;
-__global__ void __launch_bounds__(FT_X * FT_Y) k_combine_filterT32(const float* __restrict__ vxh, const float* __restrict__ vxl,
-                                                                   const float* __restrict__ vyh, const float* __restrict__ vyl,
-                                                                   float* __restrict__ lh, float* __restrict__ ll, int nx,
-                                                                   int ny, int bcx, int bcy, float sx, float sy, float cb_hi,
-                                                                   float cb_lo, float s_hi, float s_lo) {
-  __shared__ float ys[FT_Y + 2][FT_X + 2];
-  const int i0 = blockIdx.x * FT_X - 1, j0 = blockIdx.y * FT_Y - 1;
-  for (int e = threadIdx.y * FT_X + threadIdx.x; e < (FT_X + 2) * (FT_Y + 2); e += FT_X * FT_Y) {
-    const int a = e / (FT_X + 2), b = e - a * (FT_X + 2);
-    // ghost positions take the clamped point (even ghosts of a Neumann axis; a Dirichlet axis has
-    // its stored zero wall there, whose y is 0 below)
-    const int i = clampi(i0 + b, nx), j = clampi(j0 + a, ny);
-    float v = 0.0f;
-    if (interior(bcx, i, nx) && interior(bcy, j, ny)) {
-      const size_t p = (size_t)j * nx + i;
-      if (sx != 0.0f) {
-        const float h0 = i > 0 ? vxh[p - 1] : 0.0f, l0 = i > 0 ? vxl[p - 1] : 0.0f;
-        v = sx * (__fsub_rn(h0, vxh[p]) + __fsub_rn(l0, vxl[p]));
-      }
-      if (sy != 0.0f) {
-        const float h0 = j > 0 ? vyh[p - nx] : 0.0f, l0 = j > 0 ? vyl[p - nx] : 0.0f;
-        v = fmaf(sy, __fsub_rn(h0, vyh[p]) + __fsub_rn(l0, vyl[p]), v);
-      }
-    }
-    ys[a][b] = v;
-  }
-  __syncthreads();
-  const int i = blockIdx.x * FT_X + threadIdx.x, j = blockIdx.y * FT_Y + threadIdx.y;
-  if (i >= nx || j >= ny || !interior(bcx, i, nx) || !interior(bcy, j, ny)) return;
-  const int a = threadIdx.y + 1, b = threadIdx.x + 1;
-  const float c = ys[a][b];
-  const float lap = fmaf(-4.0f, c, (ys[a][b - 1] + ys[a][b + 1]) + (ys[a - 1][b] + ys[a + 1][b]));
-  const float f = fmaf(cb_hi, c, fmaf(cb_lo, c, lap));
-  const size_t p = (size_t)j * nx + i;
-  float h = lh[p], l = ll[p];
-  const float prod = __fmul_rn(s_hi, f);
-  float e = fmaf(s_hi, f, -prod);
-  e = fmaf(s_lo, f, e);
-  const float s2 = __fadd_rn(h, prod);
-  const float bb = __fsub_rn(s2, h);
-  const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s2, bb)), __fsub_rn(prod, bb));
-  const float l2 = __fadd_rn(l, __fadd_rn(err, e));
-  const float h2 = __fadd_rn(s2, l2);
-  ll[p] = __fsub_rn(l2, __fsub_rn(h2, s2));
-  lh[p] = h2;
-}
-
-// u = P~^{-1} l for field f: pair (ux[slot], uc[slot]).
-void solveT32(ms_grid* g, int f, int slot, const MixedConsts& k) {
+// H (from_h: solutions of H_x and H_y into the E_z planes) or E_z (into the H_x and H_y planes).
+void derivatives_T(ms_grid* g, bool from_h) {
   Adj32* A = g->adj32;
-  const Shape& s = g->sh[f];
-  const dim3 grd = grid2(s.nx, s.ny);
-  const float* bh = A->lh[f];
-  const float* bl = A->ll[f];
-  // sweeps k = 1 .. S-1 (x_1 = omega b is read inside the first); the last writes the pair
-  const int L = k.S - 1;
-  const float* xin = nullptr;
-  for (int q = 0; q < L; ++q) {
-    const bool first = q == 0, last = q == L - 1;
-    float* xo = last ? A->ux[slot] : A->sw[q & 1];
-    float* co = A->uc[slot];
-    if (first && last)
-      k_sweepT32<true, true><<<grd, kBlk2, 0, g->stream>>>(bh, bl, xin, xo, co, s.nx, s.ny, s.bcx, s.bcy, k.d_hi, k.d_lo,
-                                                          k.omega);
-    else if (first)
-      k_sweepT32<true, false><<<grd, kBlk2, 0, g->stream>>>(bh, bl, xin, xo, co, s.nx, s.ny, s.bcx, s.bcy, k.d_hi,
-                                                           k.d_lo, k.omega);
-    else if (last)
-      k_sweepT32<false, true><<<grd, kBlk2, 0, g->stream>>>(bh, bl, xin, xo, co, s.nx, s.ny, s.bcx, s.bcy, k.d_hi,
-                                                           k.d_lo, k.omega);
-    else
-      k_sweepT32<false, false><<<grd, kBlk2, 0, g->stream>>>(bh, bl, xin, xo, co, s.nx, s.ny, s.bcx, s.bcy, k.d_hi,
-                                                            k.d_lo, k.omega);
-    xin = xo;
-  }
+  const int N = g->N;
+  const int kind = from_h ? NODE_TO_HALF : HALF_TO_NODE;
+  YTArgs y{};
+  XTArgs x{};
+  const int ys = from_h ? HX : EZ, yd = from_h ? EZ : HX, xs = from_h ? HY : EZ, xd = from_h ? EZ : HY;
+  y.ld = x.ld = g->ld32;
+  y.M = x.M = from_h ? N : N - 1;
+  const size_t row1 = from_h ? 0 : y.ld;  // E_z: u_0 at row 1
+  y.uh = A->lh[ys] + row1;
+  y.ul = A->uc[ys] + row1;
+  y.b = A->py[yd];
+  y.ncol = N + 1;
+  end_rows_T(g->desc.closure, kind, y.k);
+  for (int j = 0; j < kEndT; ++j) x.k[j] = y.k[j];
+  y.nstrip = (N - 1 + 31) / 32;
+  const int R = y.M + 1;
+  const int rows = y.nstrip * (R / 64) >= 1500 ? 64 : 32;
+  y.end = R >= 4 * rows ? rows : 16;
+  const int mid = R - 2 * y.end;
+  const int K = mid > 0 ? (mid + rows - 1) / rows : 0;
+  y.chunk = K ? ((mid + K - 1) / K + 7) / 8 * 8 : 8;
+  y.nseg = 2 + (mid > 0 ? (mid + y.chunk - 1) / y.chunk : 0);
+  x.from_h = from_h;
+  x.uh = A->lh[xs] + (from_h ? 0 : 1);
+  x.ul = A->uc[xs] + (from_h ? 0 : 1);
+  x.b = A->px[xd] + (from_h ? 1 : 0);
+  x.nrows = N - 1;
+  const int Mo = from_h ? N - 1 : N;
+  x.nstrip = (Mo + TOUT - 1) / TOUT;
+  const int br = x.nstrip * (N / 8) < 1216 ? 4 : 8;
+  x.nblk = (x.nrows + br - 1) / br;
+  x.rows = (x.nrows + x.nblk - 1) / x.nblk;
+  const int nyb = blocks_of(y.nstrip * y.nseg);
+  const dim3 grd(nyb + blocks_of(x.nstrip * x.nblk)), blk(32 * WPB);
+  if (from_h) launch_pdl(k_walk_dT<true>, grd, blk, 0, g->stream, y, x, nyb);
+  else launch_pdl(k_walk_dT<false>, grd, blk, 0, g->stream, y, x, nyb);
 }
 
-// v = W^T u (one transposed band) into pair slot vs.  axis 0: lines are rows (along x), axis 1:
-// columns.  u: pair slot us of field fu; the target field ft gives v's layout; uoff: offset of the
-// band's output 0 in u along the line; lines [1, n - 1) of the target.
-void bandT32(ms_grid* g, int axis, int kind, int us, int fu, int ft, int uoff, int vs) {
+// u = P~^{-1} l over p_0 for the H fields or E_z: uc.
+void solve_pair(ms_grid* g, bool of_h) {
   Adj32* A = g->adj32;
-  const PadeTable& t = g->pade32[kind];
-  const Shape& su = g->sh[fu];
-  const Shape& st = g->sh[ft];
-  BandT p;
-  p.ux = A->ux[us];
-  p.uc = A->uc[us];
-  p.vh = A->vh[vs];
-  p.vl = A->vl[vs];
-  p.uoff = uoff;
-  if (axis == 0) {
-    p.ua = 1;
-    p.uc_ = su.nx;
-    p.va = 1;
-    p.vc = st.nx;
-    p.line_lo = 1;
-    p.line_hi = st.ny - 1;
-  } else {
-    p.ua = su.nx;
-    p.uc_ = 1;
-    p.va = st.nx;
-    p.vc = 1;
-    p.line_lo = 1;
-    p.line_hi = st.nx - 1;
+  SArgs a[2];
+  int nb[2] = {0, 0};
+  const int nf = of_h ? 2 : 1;
+  for (int k = 0; k < nf; ++k) {
+    const int f = of_h ? (k ? HY : HX) : EZ, mc = f == HY ? 0 : 1;
+    a[k] = make_s(g, f, A->lh[f], nullptr, nf);
+    a[k].hi = nullptr;
+    a[k].lo = A->ll[f] + mc;
+    a[k].out = A->uc[f] + mc;
+    nb[k] = blocks_of(a[k].nstrip * a[k].nblk);
   }
-  p.whi = t.d_whi;
-  p.wlo = t.d_wlo;
-  p.M = t.M;
-  p.K = t.K;
-  p.B = t.B;
-  p.all_explicit = t.all_explicit;
-  const int nl = p.line_hi - p.line_lo;
-  if (axis == 0) {
-    using T = BandTile<0>;
-    k_bandT32<0><<<dim3((t.M + 1 + T::OUTS - 1) / T::OUTS, (nl + T::LINES - 1) / T::LINES), BT_THREADS, 0,
-                   g->stream>>>(p);
-  } else {
-    using T = BandTile<1>;
-    k_bandT32<1><<<dim3((t.M + 1 + T::OUTS - 1) / T::OUTS, (nl + T::LINES - 1) / T::LINES), BT_THREADS, 0,
-                   g->stream>>>(p);
-  }
+  if (nf == 1) a[1] = a[0];
+  const dim3 grd(nb[0] + nb[1]), blk(32 * WPB);
+  const int P = g->walk.cheb.m - 1;
+  if (P == 2) launch_pdl(k_solve_pair<2>, grd, blk, 0, g->stream, a[0], a[1], nb[0]);
+  else if (P == 3) launch_pdl(k_solve_pair<3>, grd, blk, 0, g->stream, a[0], a[1], nb[0]);
+  else launch_pdl(k_solve_pair<4>, grd, blk, 0, g->stream, a[0], a[1], nb[0]);
 }
 
-// l_f += s F~ (sx Y^T along x + sy Y^T along y) from the v pairs vx, vy (slots, -1: none).
-void combine_filterT32(ms_grid* g, int f, int vx, float sx, int vy, float sy, const MixedConsts& k, float s_hi,
-                       float s_lo) {
+FArgs filter_args(ms_grid* g, int f) {
   Adj32* A = g->adj32;
-  const Shape& s = g->sh[f];
-  const dim3 blk(FT_X, FT_Y, 1), grd((s.nx + FT_X - 1) / FT_X, (s.ny + FT_Y - 1) / FT_Y);
-  k_combine_filterT32<<<grd, blk, 0, g->stream>>>(
-      vx >= 0 ? A->vh[vx] : nullptr, vx >= 0 ? A->vl[vx] : nullptr, vy >= 0 ? A->vh[vy] : nullptr,
-      vy >= 0 ? A->vl[vy] : nullptr, A->lh[f], A->ll[f], s.nx, s.ny, s.bcx, s.bcy, sx, sy, k.cb_hi, k.cb_lo, s_hi,
-      s_lo);
+  const int N = g->N, mc = f == HY ? 0 : 1;
+  FArgs a{};
+  a.p1 = (f == HX ? A->py[HX] : A->px[f]) + mc;
+  a.p2 = f == EZ ? A->py[EZ] + mc : nullptr;
+  a.lh = A->lh[f] + mc;
+  a.ll = A->ll[f] + mc;
+  a.ld = g->ld32;
+  a.M = f == HY ? N : N - 1;
+  a.u0 = f == HX ? 0 : 1;
+  a.u1 = N;
+  a.neu_x = f == HY;
+  a.neu_y = f == HX;
+  const double cb = 12.0 * g->beta - 4.0;
+  a.cb_hi = (float)cb;
+  a.cb_lo = (float)(cb - (double)a.cb_hi);
+  const double s = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * g->walk.cheb.p0 * walk_rhs_scale();
+  a.s_hi = (float)s;
+  a.s_lo = (float)(s - (double)a.s_hi);
+  return a;
+}
+
+void filter_update(ms_grid* g, bool of_h) {
+  FArgs2 A;
+  A.f[0] = filter_args(g, of_h ? HX : EZ);
+  A.f[1] = filter_args(g, of_h ? HY : EZ);
+  const dim3 grd((g->N + 127) / 128, (g->N + FY - 1) / FY, of_h ? 2 : 1), blk(32, FY);
+  launch_pdl(k_filter_update, grd, blk, 0, g->stream, A);
 }
 
 // One transposed step on the float-float adjoint state.
 void adjoint_step32(ms_grid* g) {
-  const MixedConsts k = mixed_consts(g);
-  // S2^T: u_H = P~^{-1} l_H; y_E = Y_x^T u_Hy - Y_y^T u_Hx (node-to-half bands); l_E += sH F~ y_E
-  solveT32(g, HX, 0, k);
-  solveT32(g, HY, 1, k);
-  bandT32(g, 1, NODE_TO_HALF, 0, HX, EZ, 0, 0);  // columns of H_x -> columns of E
-  bandT32(g, 0, NODE_TO_HALF, 1, HY, EZ, 0, 1);  // rows of H_y -> rows of E
-  combine_filterT32(g, EZ, 1, 1.0f, 0, -1.0f, k, k.sH_hi, k.sH_lo);
-  // S1^T: u_E = P~^{-1} l_E; y_Hy = Y_x^T u_E, y_Hx = -Y_y^T u_E (half-to-node bands, output r at
-  // node r + 1); l_H += sE F~ y_H
-  solveT32(g, EZ, 0, k);
-  bandT32(g, 0, HALF_TO_NODE, 0, EZ, HY, 1, 1);  // rows of E -> rows of H_y
-  bandT32(g, 1, HALF_TO_NODE, 0, EZ, HX, 1, 0);  // columns of E -> columns of H_x
-  combine_filterT32(g, HY, 1, 1.0f, -1, 0.0f, k, k.sE_hi, k.sE_lo);
-  combine_filterT32(g, HX, -1, 0.0f, 0, -1.0f, k, k.sE_hi, k.sE_lo);
+  solve_pair(g, true);       // S2^T: u_H = P~^{-1} l_H; y_E = Y_x^T u_Hy - Y_y^T u_Hx; l_E += sH F~ y_E
+  derivatives_T(g, true);
+  filter_update(g, false);
+  solve_pair(g, false);      // S1^T: u_E = P~^{-1} l_E; y_Hy = Y_x^T u_E, y_Hx = -Y_y^T u_E; l_H += sE F~ y_H
+  derivatives_T(g, false);
+  filter_update(g, true);
 }
 
 ms_status capture32(ms_grid* g, Graph* gr, int steps) {
@@ -420,19 +537,31 @@ ms_status adjoint32_setup(ms_grid* g) {
   if (g->adj32) return MS_OK;
   Adj32* A = new Adj32();
   g->adj32 = A;
-  const size_t n = (size_t)(g->N + 1) * (g->N + 1);
-  float** planes[] = {&A->lh[0], &A->lh[1], &A->lh[2], &A->ll[0], &A->ll[1], &A->ll[2], &A->ux[0], &A->ux[1],
-                      &A->uc[0], &A->uc[1], &A->vh[0], &A->vh[1], &A->vl[0], &A->vl[1], &A->sw[0], &A->sw[1]};
-  for (float** p : planes) {
-    if (dev_malloc((void**)p, n * sizeof(float) + 256) != cudaSuccess) {
-      adjoint32_teardown(g);
-      return a32fail(MS_ENOMEM, "cudaMalloc of the FP32 adjoint planes failed");
-    }
-    if (cudaMemsetAsync(*p, 0, n * sizeof(float) + 256, g->stream) != cudaSuccess) {
-      adjoint32_teardown(g);
-      return a32fail(MS_ECUDA, "clearing the FP32 adjoint planes failed");
-    }
+  const size_t pl = plane_floats(g->N);
+  constexpr int kPlanes = 13;
+  if (dev_malloc(&A->slab, kPlanes * pl * sizeof(float)) != cudaSuccess) {
+    adjoint32_teardown(g);
+    return a32fail(MS_ENOMEM, "cudaMalloc of the FP32 adjoint planes failed");
   }
+  if (cudaMemsetAsync(A->slab, 0, kPlanes * pl * sizeof(float), g->stream) != cudaSuccess) {
+    adjoint32_teardown(g);
+    return a32fail(MS_ECUDA, "clearing the FP32 adjoint planes failed");
+  }
+  float* next = A->slab;
+  auto plane = [&](int f) {
+    float* p = next + plane_origin(f);
+    next += pl;
+    return p;
+  };
+  for (int f = 0; f < 3; ++f) {
+    A->lh[f] = plane(f);
+    A->ll[f] = plane(f);
+    A->uc[f] = plane(f);
+  }
+  A->py[EZ] = plane(EZ);
+  A->px[EZ] = plane(EZ);
+  A->py[HX] = plane(HX);
+  A->px[HY] = plane(HY);
   return MS_OK;
 }
 
@@ -441,19 +570,17 @@ void adjoint32_teardown(ms_grid* g) {
   if (!A) return;
   free_graph32(&A->g1);
   free_graph32(&A->gk);
-  float* all[] = {A->lh[0], A->lh[1], A->lh[2], A->ll[0], A->ll[1], A->ll[2], A->ux[0], A->ux[1], A->uc[0],
-                  A->uc[1], A->vh[0], A->vh[1], A->vl[0], A->vl[1], A->sw[0], A->sw[1]};
-  for (float* p : all) dev_free(p);
+  dev_free(A->slab);
   delete A;
   g->adj32 = nullptr;
 }
 
 // The adjoint state from / to FP64 arrays (device), three fields.
 void adjoint32_load(ms_grid* g, const double* const* l) {
-  for (int f = 0; f < 3; ++f) launch_split(l[f], g->adj32->lh[f], g->adj32->ll[f], g->sh[f].size(), g->stream);
+  for (int f = 0; f < 3; ++f) launch_split2d(l[f], g->adj32->lh[f], g->adj32->ll[f], g->ld32, g->sh[f], g->stream);
 }
 void adjoint32_store(ms_grid* g, double* const* l) {
-  for (int f = 0; f < 3; ++f) launch_join(g->adj32->lh[f], g->adj32->ll[f], l[f], g->sh[f].size(), g->stream);
+  for (int f = 0; f < 3; ++f) launch_join2d(g->adj32->lh[f], g->adj32->ll[f], g->ld32, l[f], g->sh[f], g->stream);
 }
 
 // (M^T)^nsteps on the float-float adjoint state, replaying captured chunks of 16 steps.

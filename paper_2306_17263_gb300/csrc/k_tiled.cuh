@@ -40,10 +40,14 @@ void walk_d(ms_grid* g, int step, const float* src_hi = nullptr, const float* sr
 void walk_s(ms_grid* g, int step);
 constexpr int kTinyN = 16;
 
+// Arguments of the solve of field f on its own (k_walk_dev.cuh), with the row blocks of a launch over
+// nfields fields.
+struct SArgs;
+SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfields);
+
 // One launch per kernel for many cavities: per-cavity arguments and (cavity, item) work lists.
 struct YArgs;
 struct XArgs;
-struct SArgs;
 struct WalkBatch {
   YArgs* d_y = nullptr;    // [Step 1 of every cavity][Step 2]
   XArgs* d_x = nullptr;    // the same

@@ -1,0 +1,278 @@
+// Device code shared by the FP32 walks of the step (k_tiled.cu) and of the reverse pass (adjoint32.cu):
+// constants, paired arithmetic, the row ring and the solve.
+#pragma once
+
+#include "k_fp64.cuh"
+#include "k_pdl.cuh"
+
+namespace ms {
+
+// Arguments of walk_s for one field; pointers at the first unknown column of row 0.
+struct SArgs {
+  const float* p1;  // right-hand side; of E_z the sum of two planes
+  const float* p2;
+  float* hi;
+  float* lo;
+  float* out;       // reverse pass: low part of the solution
+  int ld, M;        // unknown columns 0 .. M-1
+  int u0, u1;       // unknown rows u0 .. u1-1
+  int kind;         // KIND_*
+  float q[4];          // level l + 1 of the solve
+  float s_hi, s_lo;    // increment scale
+  int nstrip, nblk, rows;
+};
+
+namespace {
+
+constexpr float kRhoF = -0.045548850f;  // rounds to the FP32 root
+constexpr float kR2 = kRhoF * kRhoF, kR4 = kR2 * kR2;
+constexpr int WPB = 4;      // warps per block
+constexpr int YOUT = 30;    // columns a walk_y warp writes
+constexpr int XOUT = 112;   // columns a warp writes along x
+constexpr int XHALO = 8;
+constexpr int SOUT = 120;   // columns a walk_s warp writes
+constexpr int SHALO = 4;
+constexpr unsigned kFull = 0xffffffffu;
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// Paired FP32 instructions (two correctly rounded operations each, bitwise those of the scalar ones): the
+// walks are bound by instruction issue.  a - b as one FMA with -1, which rounds the same.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
+
+// Rows come through a ring in shared memory that each warp fills for itself with cp.async, kAhead rows
+// ahead: the walk of a row is shorter than a memory round trip, and the registers are taken.  A slot is
+// refilled one row after it was read.
+constexpr int kAhead = 3, kRing = kAhead + 1;
+__device__ __forceinline__ void cp16(float4* dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// ---- solve and update ----------------------------------------------------------------------
+
+// (hi, lo) += (s_hi + s_lo)(b + c), |c| <= 8e-3 |b|: an exact two-product of s_hi b with the other
+// products in its error term, and a two-sum into the pair.
+__device__ __forceinline__ void ff_add_scaled(float2& hi, float2& lo, float2 b, float2 c, float2 s_hi, float2 n_hi,
+                                              float2 s_lo) {
+  const float2 np = mul2(n_hi, b);  // -p, p = fl(s_hi b)
+  float2 e = fma2(s_hi, b, np);
+  e = fma2(s_lo, b, e);
+  e = fma2(s_hi, c, e);
+  const float2 u = sub2(hi, np);
+  const float2 bb = sub2(u, hi);
+  const float2 err = sub2(sub2(hi, sub2(u, bb)), add2(np, bb));
+  const float2 l = add2(lo, add2(err, e));
+  const float2 h2 = add2(u, l);
+  lo = sub2(l, sub2(h2, u));
+  hi = h2;
+}
+
+// The kinds of field: right-hand side in two planes (E_z), Neumann along y (H_x), along x (H_y).
+enum { KIND_E = 0, KIND_HX = 1, KIND_HY = 2 };
+
+// One block of rows of one 128-column strip; P levels.  EDGE: lanes beyond the field hold zeros.  PAIR (the
+// reverse pass): the right-hand side is the float-float field (p1, lo) and the solution over p_0 is left as
+// the pair (p1, out), out = lo + q T y.
+template <int P, int KIND, bool EDGE, bool PAIR>
+__device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip, int blk) {
+  constexpr bool TWO = KIND == KIND_E && !PAIR;
+  const int lane = threadIdx.x & 31;
+  const int m0 = SOUT * strip - SHALO + 4 * lane;
+  const int M = A.M, u0 = A.u0, u1 = A.u1;
+  const int j0 = u0 + blk * A.rows, j1 = min(j0 + A.rows, u1);
+  const size_t ld = A.ld;
+  const bool ok = !EDGE || (m0 >= 0 && m0 < M);
+  const bool out = lane >= SHALO / 4 && lane < (SHALO + SOUT) / 4 && ok;
+  bool in[4] = {true, true, true, true}, first = false, lastc[4] = {};
+  if (EDGE) {
+    first = KIND == KIND_HY && m0 == 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      in[k] = m0 + k >= 0 && m0 + k < M;
+      lastc[k] = KIND == KIND_HY && m0 + k == M - 1;
+    }
+  }
+  auto mask = [&](float2(&y)[2]) {
+    if (EDGE) {
+      y[0].x = in[0] ? y[0].x : 0.0f;
+      y[0].y = in[1] ? y[0].y : 0.0f;
+      y[1].x = in[2] ? y[1].x : 0.0f;
+      y[1].y = in[3] ? y[1].y : 0.0f;
+    }
+  };
+  const float2 four = bc2(4.0f);
+  // w = 4 y + left + right
+  auto wsum = [&](const float2(&y)[2], float2(&w)[2]) {
+    float a = __shfl_up_sync(kFull, y[1].y, 1), b = __shfl_down_sync(kFull, y[0].x, 1);
+    float r0 = y[0].y, r1 = y[1].x, r2 = y[1].y;
+    if (EDGE && KIND == KIND_HY) {
+      a = first ? y[0].x : a;
+      r0 = lastc[0] ? y[0].x : r0;
+      r1 = lastc[1] ? y[0].y : r1;
+      r2 = lastc[2] ? y[1].x : r2;
+      b = lastc[3] ? y[1].y : b;
+    }
+    w[0] = fma2(four, y[0], make_float2(a + r0, y[0].x + r1));
+    w[1] = fma2(four, y[1], make_float2(y[0].y + r2, y[1].x + b));
+  };
+  const int js = max(j0 - P, u0);
+  // ring: [slot][p1, p2 of row jj, hi, lo of row jj - P][lane]
+  const size_t off = ok ? m0 : 0;
+  const float* f1 = A.p1 + (size_t)js * ld + off;  // row jj of the planes, row jj - P of the state
+  const float* f2 = TWO ? A.p2 + (size_t)js * ld + off : nullptr;
+  const float* fh = A.hi + off + ((ptrdiff_t)js - P) * (ptrdiff_t)ld;
+  const float* fl = A.lo + off + ((ptrdiff_t)js - P) * (ptrdiff_t)ld;
+  const int jb = min(j1 + P, u1);  // rows of b
+  int jf = js;                     // next row to fetch
+  auto fetch = [&](int slot) {
+    float4* r = ring + 4 * slot * 32 + lane;
+    if (jf < jb) {
+      cp16(r, f1, ok);
+      if (TWO) cp16(r + 32, f2, ok);
+    }
+    if (out && jf >= j0 + P && jf < j1 + P) {
+      if (!PAIR) cp16(r + 64, fh, true);
+      cp16(r + 96, fl, true);
+    }
+    cp_commit();
+    f1 += ld;
+    if (TWO) f2 += ld;
+    fh += ld;
+    fl += ld;
+    ++jf;
+  };
+#pragma unroll
+  for (int t = 0; t < kAhead; ++t) fetch(t);
+  int rd = 0, wr = kAhead;
+  const float2 z2 = bc2(0.0f);
+  float2 b[P + 1][2], w[P][2][2];  // b[l]: row jj - l; w[l][1]: level l at row jj - l - 1, w[l][0] above it
+#pragma unroll
+  for (int l = 0; l <= P; ++l) b[l][0] = b[l][1] = z2;
+#pragma unroll
+  for (int l = 0; l < P; ++l) w[l][0][0] = w[l][0][1] = w[l][1][0] = w[l][1][1] = z2;
+  const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo);
+  float* ph = (PAIR ? A.out : A.hi) + off + (size_t)j0 * ld;
+  float* pl = A.lo + off + (size_t)j0 * ld;
+  const int jend = j1 + P;
+#pragma unroll 1
+  for (int jj = js; jj < jend; ++jj) {
+    cp_wait<kAhead - 1>();
+    const float4* r = ring + 4 * rd * 32 + lane;
+    fetch(wr);
+    rd = rd == kRing - 1 ? 0 : rd + 1;
+    wr = wr == kRing - 1 ? 0 : wr + 1;
+    float2 wn[2];
+#pragma unroll
+    for (int l = P; l > 0; --l)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) b[l][k] = b[l - 1][k];
+    if (jj < u1) {  // b of row jj
+      const float4 c = r[0];
+      b[0][0] = make_float2(c.x, c.y);
+      b[0][1] = make_float2(c.z, c.w);
+      if (TWO) {
+        const float4 e = r[32];
+        b[0][0] = add2(b[0][0], make_float2(e.x, e.y));
+        b[0][1] = add2(b[0][1], make_float2(e.z, e.w));
+      }
+      mask(b[0]);
+      wsum(b[0], wn);
+    } else {
+      b[0][0] = b[0][1] = wn[0] = wn[1] = z2;
+    }
+    // level l + 1 at row t = jj - l - 1 from w of level l at rows t - 1, t, t + 1
+#pragma unroll
+    for (int l = 0; l < P; ++l) {
+      const int t = jj - l - 1;
+      float2 tt[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float2 ud = add2(w[l][0][k], wn[k]);
+        if (KIND == KIND_HX && (t == u0 || t == u1 - 1))  // the ghost row equals the wall row
+          ud = add2(w[l][1][k], t == u0 ? wn[k] : w[l][0][k]);
+        tt[k] = fma2(four, w[l][1][k], ud);
+        w[l][0][k] = w[l][1][k];
+        w[l][1][k] = wn[k];
+      }
+      if (l < P - 1) {
+        if ((unsigned)(t - u0) < (unsigned)(u1 - u0)) {
+          float2 y[2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) y[k] = fma2(bc2(A.q[l]), tt[k], b[l + 1][k]);
+          mask(y);
+          wsum(y, wn);
+        } else {
+          wn[0] = wn[1] = z2;
+        }
+      } else if (t >= j0) {
+        if (out) {
+          const float4 sl = r[96];
+          float2 o[2] = {make_float2(sl.x, sl.y), make_float2(sl.z, sl.w)};
+          if (PAIR) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) o[k] = fma2(bc2(A.q[P - 1]), tt[k], o[k]);
+            if (!EDGE || m0 + 4 <= M) {
+              *reinterpret_cast<float4*>(ph) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+            } else {
+              const float ov[3] = {o[0].x, o[0].y, o[1].x};
+#pragma unroll
+              for (int k = 0; k < 3; ++k)
+                if (in[k]) ph[k] = ov[k];
+            }
+          } else {
+            const float4 sh = r[64];
+            float2 h[2] = {make_float2(sh.x, sh.y), make_float2(sh.z, sh.w)};
+#pragma unroll
+            for (int k = 0; k < 2; ++k) ff_add_scaled(h[k], o[k], b[P][k], mul2(bc2(A.q[P - 1]), tt[k]), s_hi, n_hi, s_lo);
+            if (!EDGE || m0 + 4 <= M) {
+              *reinterpret_cast<float4*>(ph) = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+              *reinterpret_cast<float4*>(pl) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+            } else {
+              const float hv[3] = {h[0].x, h[0].y, h[1].x}, ov[3] = {o[0].x, o[0].y, o[1].x};
+#pragma unroll
+              for (int k = 0; k < 3; ++k)
+                if (in[k]) {
+                  ph[k] = hv[k];
+                  pl[k] = ov[k];
+                }
+            }
+          }
+        }
+        ph += ld;
+        pl += ld;
+      }
+    }
+  }
+}
+
+template <int P, bool PAIR = false>
+__device__ __forceinline__ void s_item(const SArgs& A, float4* ring, int item) {
+  if (item >= A.nstrip * A.nblk) return;
+  const int blk = item / A.nstrip, strip = item - blk * A.nstrip;
+  const bool edge = strip == 0 || A.M - 1 < SOUT * strip - SHALO + 127;
+  if (A.kind == KIND_E) {
+    if (edge) s_block<P, KIND_E, true, PAIR>(A, ring, strip, blk);
+    else s_block<P, KIND_E, false, PAIR>(A, ring, strip, blk);
+  } else if (A.kind == KIND_HX) {
+    if (edge) s_block<P, KIND_HX, true, PAIR>(A, ring, strip, blk);
+    else s_block<P, KIND_HX, false, PAIR>(A, ring, strip, blk);
+  } else {
+    if (edge) s_block<P, KIND_HY, true, PAIR>(A, ring, strip, blk);
+    else s_block<P, KIND_HY, false, PAIR>(A, ring, strip, blk);
+  }
+}
+
+}  // namespace
+
+}  // namespace ms

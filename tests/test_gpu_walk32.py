@@ -67,3 +67,20 @@ def test_batch_cavities_equal_single_grids():
             g.run(3)
             for a, e in zip(fields, g.get_fields()):
                 assert np.array_equal(a, e)
+
+
+@pytest.mark.parametrize("closure", [pkg.CLOSURE_PAPER, pkg.CLOSURE_REFLECT])
+@pytest.mark.parametrize("n", [5, 31, 32, 33, 34, 47, 64, 65, 103, 104, 105, 116, 117, 118, 127, 128, 129, 130, 209,
+                               233, 260])
+def test_reverse_steps_match_oracle(n, closure):
+    """The walking reverse pass: end segments, strips of 104 columns, FP64 below 32 cells."""
+    r, steps = (0.3, 0.5, 0.65)[n % 3], 3
+    o = oracle.Oracle2D(n, r, 1.3, closure)
+    lam = workloads.random_fields(n, seed=n + 1)
+    ref = [a.copy() for a in lam]
+    for _ in range(steps):
+        o.step_T(*ref)
+    with pkg.Grid(n, r, z=1.3, precision=pkg.FP32_REFINED, closure=closure) as g:
+        got = g.adjoint_steps(steps, *lam)
+    for a, b in zip(got, ref):
+        assert _rel(a, b) <= 2e-6
