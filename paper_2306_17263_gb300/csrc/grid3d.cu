@@ -210,6 +210,10 @@ __device__ __forceinline__ void ff_add_scaled3_2(float2& hi, float2& lo, float2 
   hi = h2;
 }
 
+__device__ __forceinline__ void cp4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
 // Float-float filter of one component, Eq. "eq:ell" in the units of the FP32 step:
 //   G = 12 beta u + L u,  L = h^2 Delta_h (7 points),
 // with even ghosts on Neumann axes and the stored wall zeros on Dirichlet axes; G = 0 at wall
@@ -689,19 +693,249 @@ __global__ void __launch_bounds__(256, AXIS == 0 ? 4 : 5) k_term3d32(const __gri
   }
 }
 
+// Pade terms along y and z on lines of at least kWalk3Min rows: the walk along y of the 2D step
+// (k_tiled.cu) on the filtered G.  A lane takes one x and walks down its segment of a line, every access
+// coalesced; forward recurrence with the walk, backward over groups of eight rows, the closure's end rows
+// as a rank-one correction.  19 warp instructions per 32 points where the tile form (k_term3d32) issues 115:
+// bound by DRAM.
+constexpr int kWalk3Min = 16, kW3Warps = 4, kEnd3 = 8;
+struct Walk3Term {
+  const float* gh;
+  const float* gl;
+  float* R;
+  int nx, nq;               // lines: x, and the other transverse index
+  unsigned sa, sq, da, dq;  // strides along the line and between the nq, in source and destination
+  int out_len;
+  float sign;
+  int accumulate;
+};
+struct Walk3Args {
+  Walk3Term t[2];
+  int M, off;
+  float g[4], v[kEnd3], sc_hi, sc_lo;
+  int nxt, nq, nseg, chunk, rb;  // x tiles, lines along q (largest), segments as in k_tiled.cu
+};
+
+// Group of eight differences m0 .. m0 + 7 along a line from the filtered points after them: the forward
+// values z, and the rows m0 - 7 .. m0 of the result (in the units of the scaled recurrences) by the backward
+// recurrence.  `first`, `final`: the result rows are the first or last eight of the line.
+template <bool EDGE>
+__device__ __forceinline__ void walk3_group(const Walk3Args& A, const float (&ch)[8], const float (&cl)[8], float& h0,
+                                            float& l0, float& z, float (&zp)[7], float (&y)[8], int m0, bool first,
+                                            bool final) {
+  float zc[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    float d = (ch[t] - h0) + (cl[t] - l0);
+    if (EDGE) d = (m0 + t >= 0 && m0 + t < A.M) ? d : 0.0f;
+    h0 = ch[t];
+    l0 = cl[t];
+    zc[t] = z = fmaf(c_rec3[0], z, d);
+  }
+  float acc = zc[7];
+#pragma unroll
+  for (int t = 6; t >= 1; --t) acc = fmaf(c_rec3[0], acc, zc[t]);
+  y[7] = acc = fmaf(c_rec3[0], acc, zc[0]);
+#pragma unroll
+  for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(c_rec3[0], acc, zp[t]);
+#pragma unroll
+  for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
+  if (EDGE && first) {
+    const float phi = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
+#pragma unroll
+    for (int t = 0; t < kEnd3; ++t) y[t] = fmaf(A.v[t], phi, y[t]);
+  }
+  if (EDGE && final) {
+    const float phi = fmaf(A.g[0], y[7], fmaf(A.g[1], y[6], fmaf(A.g[2], y[5], A.g[3] * y[4])));
+#pragma unroll
+    for (int t = 0; t < kEnd3; ++t) y[7 - t] = fmaf(A.v[t], phi, y[7 - t]);
+  }
+}
+
+template <bool EDGE>
+__device__ __forceinline__ void walk3_segment(const Walk3Args& A, const Walk3Term& T, int x, int q, int seg) {
+  const bool live = x < T.nx, last = seg == A.nseg - 1;
+  const int M = A.M, r0 = last ? A.rb : seg * A.chunk, r1 = last ? M : min(r0 + A.chunk, A.rb);
+  const float* __restrict__ ph = T.gh + (size_t)q * T.sq + min(x, T.nx - 1);
+  const float* __restrict__ pl = T.gl + (size_t)q * T.sq + min(x, T.nx - 1);
+  float* __restrict__ Rq = T.R + (size_t)q * T.dq + min(x, T.nx - 1);
+  auto row = [&](int r) { return (unsigned)(EDGE ? min(max(r, 0), M) : r) * T.sa; };
+  const int ms = r0 - 9;
+  float h0 = ph[row(ms)], l0 = pl[row(ms)];
+  float nh[8], nl[8], old[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    nh[t] = ph[row(ms + 1 + t)];
+    nl[t] = pl[row(ms + 1 + t)];
+  }
+  float z = 0.0f, zp[7] = {};
+  const int ngrp = 2 + (r1 - r0 + 7) / 8;
+  float* bp = Rq + (unsigned)(r0 + A.off) * T.da;
+  for (int gi = 0; gi < ngrp; ++gi) {
+    const int m0 = ms + 8 * gi;
+    float ch[8], cl[8], y[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      ch[t] = nh[t];
+      cl[t] = nl[t];
+    }
+    if (gi + 1 < ngrp) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        nh[t] = ph[row(m0 + 9 + t)];
+        nl[t] = pl[row(m0 + 9 + t)];
+      }
+    }
+    const int left = gi < 2 ? 0 : min(8, r1 - (r0 + 8 * (gi - 2)));
+    if (T.accumulate) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t) old[t] = t < left ? bp[(unsigned)t * T.da] : 0.0f;
+    }
+    walk3_group<EDGE>(A, ch, cl, h0, l0, z, zp, y, m0, seg == 0 && gi == 2, last && gi == ngrp - 1);
+    if (gi < 2) continue;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const float v = fmaf(A.sc_hi, y[t], A.sc_lo * y[t]);
+      if (live && t < left) bp[(unsigned)t * T.da] = T.accumulate ? fmaf(T.sign, v, old[t]) : T.sign * v;
+    }
+    bp += 8u * T.da;
+  }
+  if (live && !T.accumulate) {  // wall points of the line
+    if (seg == 0)
+      for (int r = 0; r < A.off; ++r) Rq[(unsigned)r * T.da] = 0.0f;
+    if (last)
+      for (int r = M + A.off; r < T.out_len; ++r) Rq[(unsigned)r * T.da] = 0.0f;
+  }
+}
+
+__global__ void __launch_bounds__(32 * kW3Warps) k_walk3d32(const __grid_constant__ Walk3Args A) {
+  pdl_wait();
+  int item = blockIdx.x * kW3Warps + (threadIdx.x >> 5);
+  const int xt = item % A.nxt;
+  item /= A.nxt;
+  const int seg = item % A.nseg;
+  item /= A.nseg;
+  const int which = item / A.nq, q = item - which * A.nq;
+  if (which > 1) return;
+  const Walk3Term& T = A.t[which];
+  if (q >= T.nq || 32 * xt >= T.nx) return;
+  const int x = 32 * xt + (threadIdx.x & 31);
+  const int r0 = seg == A.nseg - 1 ? A.rb : seg * A.chunk, r1 = seg == A.nseg - 1 ? A.M : min(r0 + A.chunk, A.rb);
+  if (r0 >= 10 && r1 + 18 <= A.M) walk3_segment<false>(A, T, x, q, seg);
+  else walk3_segment<true>(A, T, x, q, seg);
+}
+
+// The same walk for the terms along x: a lane takes a row of the component (x, all rows of a plane stack
+// being equally long), 32 rows per warp, and sixteen points of every row at a time come through tiles in
+// shared memory, filled by cp.async along x kAX tiles ahead; the results go back through the tile just read and
+// leave along x.  In Walk3Term, nx counts the rows, sq and dq are their strides.
+constexpr int kAX = 1, kRX = kAX + 1, kXW = 16, kXS = kXW + 1, kWXWarps = 2;  // tile stride odd: no bank conflicts
+template <bool EDGE>
+__device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Term& T, int row0, int seg,
+                                               float (*tile)[2][32 * kXS]) {
+  const int lane = threadIdx.x & 31, xr = lane & (kXW - 1), rs = lane / kXW;
+  const int cap = min(31, T.nx - 1 - row0);  // last row of the warp
+  const bool last = seg == A.nseg - 1;
+  const int M = A.M, r0 = last ? A.rb : seg * A.chunk, r1 = last ? M : min(r0 + A.chunk, A.rb);
+  const float* __restrict__ ph = T.gh + (size_t)row0 * T.sq;
+  const float* __restrict__ pl = T.gl + (size_t)row0 * T.sq;
+  float* __restrict__ R = T.R + (size_t)row0 * T.dq + A.off;
+  const int ms = r0 - 9, ngrp = 2 + (r1 - r0 + 7) / 8, ntile = (ngrp + 1) / 2;
+  auto fetch = [&](int c) {
+    if (c < ntile) {
+      const int x = min(max(ms + 1 + kXW * c + xr, 0), M);
+      float* dh = tile[c % kRX][0] + rs * kXS + xr;
+      float* dl = tile[c % kRX][1] + rs * kXS + xr;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const unsigned o = (unsigned)min(rs + 2 * i, cap) * T.sq + x;
+        cp4(dh + 2 * i * kXS, ph + o);
+        cp4(dl + 2 * i * kXS, pl + o);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < kAX; ++c) fetch(c);
+  const unsigned o0 = (unsigned)min(lane, cap) * T.sq + max(ms, 0);
+  float h0 = ph[o0], l0 = pl[o0];
+  float z = 0.0f, zp[7] = {};
+  for (int c = 0; c < ntile; ++c) {
+    __syncwarp();  // the tile read last is free
+    fetch(c + kAX);
+    const int rw = r0 + kXW * (c - 1) + xr;  // result row of the lane when writing
+    const bool out = c > 0 && rw < r1;
+    float old[16];
+    if (T.accumulate) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        old[i] = out && rs + 2 * i <= cap ? R[(unsigned)(rs + 2 * i) * T.dq + rw] : 0.0f;
+    }
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAX) : "memory");
+    __syncwarp();
+    float* th = tile[c % kRX][0] + lane * kXS;
+    const float* tl = tile[c % kRX][1] + lane * kXS;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int gi = 2 * c + u;
+      if (gi >= ngrp) break;
+      float ch[8], cl[8], y[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        ch[t] = th[8 * u + t];
+        cl[t] = tl[8 * u + t];
+      }
+      walk3_group<EDGE>(A, ch, cl, h0, l0, z, zp, y, ms + 8 * gi, seg == 0 && gi == 2, last && gi == ngrp - 1);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) th[8 * u + t] = T.sign * fmaf(A.sc_hi, y[t], A.sc_lo * y[t]);
+    }
+    if (c == 0) continue;
+    __syncwarp();
+    const float* tw = tile[c % kRX][0] + rs * kXS + xr;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (out && rs + 2 * i <= cap)
+        R[(unsigned)(rs + 2 * i) * T.dq + rw] = T.accumulate ? tw[2 * i * kXS] + old[i] : tw[2 * i * kXS];
+  }
+  if (lane <= cap && !T.accumulate) {  // wall points of the lines
+    float* __restrict__ Rl = T.R + (size_t)(row0 + lane) * T.dq;
+    if (seg == 0)
+      for (int r = 0; r < A.off; ++r) Rl[r] = 0.0f;
+    if (last)
+      for (int r = M + A.off; r < T.out_len; ++r) Rl[r] = 0.0f;
+  }
+}
+
+__global__ void __launch_bounds__(32 * kWXWarps) k_walkx3d32(const __grid_constant__ Walk3Args A) {
+  __shared__ float tiles[kWXWarps][kRX][2][32 * kXS];
+  pdl_wait();
+  int item = blockIdx.x * kWXWarps + (threadIdx.x >> 5);
+  const int seg = item % A.nseg;  // the segments of a line share its sectors in L2
+  item /= A.nseg;
+  const int which = item / A.nxt, row0 = 32 * (item - which * A.nxt);
+  if (which > 1) return;
+  const Walk3Term& T = A.t[which];
+  if (row0 >= T.nx) return;
+  const int r0 = seg == A.nseg - 1 ? A.rb : seg * A.chunk, r1 = seg == A.nseg - 1 ? A.M : min(r0 + A.chunk, A.rb);
+  if (r0 >= 10 && r1 + 18 <= A.M) walk3x_segment<false>(A, T, row0, seg, tiles[threadIdx.x >> 5]);
+  else walk3x_segment<true>(A, T, row0, seg, tiles[threadIdx.x >> 5]);
+}
+
 // The solve of a half-step: 6 h^2 P1 = D - T with D = 6 c1 h^2 + 24 and, from the 19-point stencil,
 // T y = 2 e + c + (2 y + e)_{z-1} + (2 y + e)_{z+1}, e and c the sums over the four edge and the four
 // corner neighbours in the plane, spectrum [-8, 24].  The Chebyshev polynomial of k_rec64.cu in Horner
 // form, y <- b + q T y, to a relative error of 1e-10, one level per launch for the three components; T y
 // is 2e-3 of D y at most, so a level rounds the increment at 1e-9 of itself, and the last level's q T y
-// enters the state apart from b.  A thread takes two rows of one column and marches L3Z planes along z
-// with e, c and q = 2 y + e of the planes in registers, the next plane's twelve values fetched ahead: ten
-// operations and six loads (from L1 but for the halo) per point and level, no test in the march, where a Richardson sweep with
-// its residual took 84 instructions on shared-memory tiles.  256^3, three levels of one component: 215 us
-// by the sweeps.
-constexpr int L3Y = 4, L3Z = 16;  // warps (pairs of rows) per block, planes per march
-constexpr int kPre3 = 3;           // planes ahead of the loads that a march asks L2 for
-__device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches L3Z planes along z;
+// the planes come through a ring in shared memory filled by cp.async kA3 planes ahead (loads straight
+// into registers, one plane ahead, left the march waiting for them: 180 to 225 us per level of three
+// components at 256^3), and a thread keeps e, c and q = 2 y + e of its two rows in registers: ten
+// operations and six shared loads per point and level, where a Richardson sweep with its residual issued
+// 84 instructions.
+constexpr int L3Y = 8, L3Z = 16;  // warps (pairs of rows) per block, planes per march
+constexpr int kA3 = 3, kR3 = kA3 + 1;
+constexpr int S3W = 34, S3N = S3W * (2 * L3Y + 2);  // a staged plane: the tile and one point around it
+static_assert(S3N <= 3 * 32 * L3Y, "three staged points per thread");
 struct Lev3d32Args {
   const float* b[3];
   const float* y[3];
@@ -728,126 +962,121 @@ __device__ __forceinline__ void ff_add_scaled_bc(float& hi, float& lo, float b, 
   hi = h2;
 }
 
-template <bool LAST>
-__global__ void __launch_bounds__(32 * L3Y, LAST ? 6 : 8) k_lev3d32(const __grid_constant__ Lev3d32Args A) {
+// FIRST: y is b itself.
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(32 * L3Y, LAST ? 4 : 5) k_lev3d32(const __grid_constant__ Lev3d32Args A) {
+  __shared__ float ring[kR3][S3N];
   pdl_wait();
   const int which = blockIdx.z / A.nz, kz = blockIdx.z - which * A.nz;
   const Shape3& s = A.s[which];
   const int n0 = s.n[0], n1 = s.n[1], n2 = s.n[2];
   const int d0 = s.bc[0] == DIR, d1 = s.bc[1] == DIR, d2 = s.bc[2] == DIR;
-  const int i = d0 + blockIdx.x * 32 + threadIdx.x, j = d1 + 2 * (blockIdx.y * L3Y + threadIdx.y);
+  const int i0 = d0 + blockIdx.x * 32, j0 = d1 + blockIdx.y * 2 * L3Y;
   const int k0 = d2 + kz * L3Z, k1 = min(k0 + L3Z, n2 - d2);
-  if (i >= n0 - d0 || j >= n1 - d1 || k0 >= k1) return;
-  const bool two = j + 1 < n1 - d1;
+  if (i0 >= n0 - d0 || j0 >= n1 - d1 || k0 >= k1) return;  // block-uniform
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
+  const int i = i0 + tx, j = j0 + 2 * ty;
+  const bool in0 = i < n0 - d0 && j < n1 - d1, in1 = in0 && j + 1 < n1 - d1;
   const unsigned sz = n0 * n1;  // points per component fit 31 bits (n <= 512)
   const float* __restrict__ y = A.y[which];
   const float* __restrict__ b = A.b[which];
   float* __restrict__ out = A.out[which];
   float* __restrict__ shi = A.hi[which];
   float* __restrict__ slo = A.lo[which];
-  // offsets in a plane of the rows j - 1 .. j + 2, and of the columns left and right: ghosts of a Neumann
-  // axis mirror, walls of a Dirichlet axis hold zeros (b: the terms write them; y: the level before)
-  unsigned om[4], ol[4], orr[4];
+  // staged points of the thread: ghosts of a Neumann axis mirror (clamped), walls of a Dirichlet axis hold
+  // zeros (b: the terms write them; y: the level before)
+  auto place = [&](int e) {
+    const int r = e / S3W, c = e - r * S3W;
+    return (unsigned)(clampi(j0 - 1 + r, n1) * n0 + clampi(i0 - 1 + c, n0));
+  };
+  const bool has3 = tid + 512 < S3N;
+  const unsigned o1 = place(tid), o2 = place(tid + 256), o3 = has3 ? place(tid + 512) : 0;
+  const int S = k1 - k0 + 2;  // planes k0 - 1 .. k1
+  auto fetch = [&](int st, int slot) {
+    if (st < S) {
+      const float* __restrict__ p = y + (size_t)clampi(k0 - 1 + st, n2) * sz;
+      float* d = ring[slot] + tid;
+      cp4(d, p + o1);
+      cp4(d + 256, p + o2);
+      if (has3) cp4(d + 512, p + o3);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int row = clampi(j - 1 + r, n1) * n0;
-    om[r] = row + i;
-    ol[r] = row + clampi(i - 1, n0);
-    orr[r] = row + clampi(i + 1, n0);
-  }
-  float m[4], l[4], r[4];  // one plane's values
-  auto fetch = [&](int k) {
-    const float* __restrict__ p = y + (size_t)clampi(k, n2) * sz;
+  for (int t = 0; t < kA3; ++t) fetch(t, t);
+  // per-point operands two planes ahead
+  const unsigned own = j * n0 + i;
+  unsigned g = k0 * sz + own;
+  float b1[2] = {}, b2[2] = {}, h1[2] = {}, h2[2] = {}, l1[2] = {}, l2[2] = {};
+  auto operands = [&](int k, float(&bq)[2], float(&hq)[2], float(&lq)[2]) {
+    if (k >= k1) return;
+    const unsigned p = k * sz + own;
+    if (in0) {
+      if (!FIRST) bq[0] = b[p];
+      if (LAST) {
+        hq[0] = shi[p];
+        lq[0] = slo[p];
+      }
+    }
+    if (in1) {
+      if (!FIRST) bq[1] = b[p + n0];
+      if (LAST) {
+        hq[1] = shi[p + n0];
+        lq[1] = slo[p + n0];
+      }
+    }
+  };
+  float qm[2] = {}, q0[2] = {}, u0[2] = {}, m0[2] = {};  // q of planes k - 1, k; 2 e + c and y of plane k
+  int rd = 0, wr = kA3;
+  for (int st = 0; st < S; ++st) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kA3 - 1) : "memory");
+    __syncthreads();  // plane st is there for every thread, and the slot read last is free
+    fetch(st + kA3, wr);
+    const float* r = ring[rd] + (2 * ty) * S3W + tx;
+    rd = rd == kR3 - 1 ? 0 : rd + 1;
+    wr = wr == kR3 - 1 ? 0 : wr + 1;
+    float bc[2], hc[2], lc[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      bc[t] = FIRST ? m0[t] : b1[t];
+      b1[t] = b2[t];
+      hc[t] = h1[t];
+      h1[t] = h2[t];
+      lc[t] = l1[t];
+      l1[t] = l2[t];
+    }
+    operands(k0 + st, b2, h2, l2);  // used two planes on
+    float m[4], x[4], qn[2];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      m[t] = p[om[t]];
-      l[t] = p[ol[t]];
-      r[t] = p[orr[t]];
+      m[t] = r[t * S3W + 1];
+      x[t] = r[t * S3W] + r[t * S3W + 2];
     }
-  };
-  float qm[2], q0[2], e0[2], c0[2], qn[2], en[2], cn[2];
-  auto sums = [&](float(&q)[2], float(&e)[2], float(&c)[2]) {
-    float x[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) x[t] = l[t] + r[t];
+    const bool live = st >= 2;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-      e[t] = x[t + 1] + (m[t] + m[t + 2]);
-      c[t] = x[t] + x[t + 2];
-      q[t] = fmaf(2.0f, m[t + 1], e[t]);
-    }
-  };
-  fetch(k0 - 1);
-  sums(qm, e0, c0);
-  fetch(k0);
-  sums(q0, e0, c0);
-  fetch(k0 + 1);
-  unsigned g[2] = {k0 * sz + om[1], k0 * sz + (two ? om[2] : om[1])};
-  float bn[2] = {b[g[0]], b[g[1]]}, hn[2], ln[2];
-  if (LAST) {
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      hn[t] = shi[g[t]];
-      ln[t] = slo[g[t]];
-    }
-  }
-#pragma unroll 1
-  for (int k = k0; k < k1; ++k) {
-    sums(qn, en, cn);
-    const float bc[2] = {bn[0], bn[1]};
-    float hc[2], lc[2];
-    if (LAST) {
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        hc[t] = hn[t];
-        lc[t] = ln[t];
-      }
-    }
-    const unsigned go[2] = {g[0], g[1]};
-    if (k + 1 < k1) {
-      fetch(k + 2);
-      if (k + 2 + kPre3 <= k1) {
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          prefetch_l2(y + g[t] + (2 + kPre3) * sz);
-          if (y != b) prefetch_l2(b + g[t] + (1 + kPre3) * sz);
-          if (LAST) {
-            prefetch_l2(shi + g[t] + (1 + kPre3) * sz);
-            prefetch_l2(slo + g[t] + (1 + kPre3) * sz);
-          }
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        g[t] += sz;
-        bn[t] = b[g[t]];
+      const float e = x[t + 1] + (m[t] + m[t + 2]);
+      qn[t] = fmaf(2.0f, m[t + 1], e);
+      const float T = u0[t] + (qm[t] + qn[t]);
+      if (live && (t ? in1 : in0)) {
         if (LAST) {
-          hn[t] = shi[g[t]];
-          ln[t] = slo[g[t]];
+          ff_add_scaled_bc(hc[t], lc[t], bc[t], A.q * T, A.s_hi, A.s_lo);
+          shi[g + t * n0] = hc[t];
+          slo[g + t * n0] = lc[t];
+        } else {
+          out[g + t * n0] = fmaf(A.q, T, bc[t]);
         }
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const float T = fmaf(2.0f, e0[t], c0[t]) + (qm[t] + qn[t]);
-      if (LAST) {
-        ff_add_scaled_bc(hc[t], lc[t], bc[t], A.q * T, A.s_hi, A.s_lo);
-        if (t == 0 || two) {
-          shi[go[t]] = hc[t];
-          slo[go[t]] = lc[t];
-        }
-      } else if (t == 0 || two) {
-        out[go[t]] = fmaf(A.q, T, bc[t]);
       }
       qm[t] = q0[t];
       q0[t] = qn[t];
-      e0[t] = en[t];
-      c0[t] = cn[t];
+      u0[t] = fmaf(2.0f, e, x[t] + x[t + 2]);
+      m0[t] = m[t + 1];
     }
+    if (live) g += sz;
   }
-  if (!LAST) {
+  if (!LAST && in0) {
     // zeros on the walls the next level reads: those next to the thread's points, corners included
-    const int jl = two ? j + 1 : j;
+    const int jl = in1 ? j + 1 : j;
     const int di0 = d0 && i == 1 ? -1 : 0, di1 = d0 && i == n0 - 2 ? 1 : 0;
     const int dj0 = d1 && j == 1 ? -1 : 0, dj1 = d1 && jl == n1 - 2 ? 1 : 0;
     const int dk0 = d2 && k0 == 1 ? -1 : 0, dk1 = d2 && k1 == n2 - 1 ? 1 : 0;
@@ -1249,6 +1478,49 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
   const PadeTable& t = g->pade32[kind];
   const int off = (kind == HALF_TO_NODE) ? 1 : 0;
   const Term3* q[2] = {&q0, &q1};
+  if (t.M >= kWalk3Min) {
+    const int Q = axis == 2 ? 1 : 2;
+    auto stride = [](const Shape3& s, int a) { return a == 0 ? 1u : (a == 1 ? (unsigned)s.n[0] : (unsigned)(s.n[0] * s.n[1])); };
+    Walk3Args A;
+    A.M = t.M;
+    A.off = off;
+    const LineEnds& e = g->walk.ends[kind];
+    for (int k = 0; k < 4; ++k) A.g[k] = (float)e.g[k];
+    for (int k = 0; k < kEnd3; ++k) A.v[k] = (float)e.v[k];
+    const double sc = walk_rhs_scale();  // (1 - rho)^2, rho the FP32 root
+    A.sc_hi = (float)sc;
+    A.sc_lo = (float)(sc - (double)A.sc_hi);
+    A.nxt = A.nq = 0;
+    double bytes = 0.0;
+    for (int k = 0; k < 2; ++k) {
+      Walk3Term& a = A.t[k];
+      const Shape3& ss = G3->sh[q[k]->cs];
+      const Shape3& sd = G3->sh[q[k]->cd];
+      a.gh = G3->gh[q[k]->cs % 3];
+      a.gl = G3->gl[q[k]->cs % 3];
+      a.R = G3->s32[1 + q[k]->cd % 3];
+      a.nx = axis ? sd.n[0] : sd.n[1] * sd.n[2];
+      a.nq = axis ? sd.n[Q] : 1;
+      a.sa = stride(ss, axis);
+      a.sq = stride(ss, axis ? Q : 1);
+      a.da = stride(sd, axis);
+      a.dq = stride(sd, axis ? Q : 1);
+      a.out_len = sd.n[axis];
+      a.sign = q[k]->sign;
+      a.accumulate = q[k]->accumulate;
+      A.nxt = std::max(A.nxt, (a.nx + 31) / 32);
+      A.nq = std::max(A.nq, a.nq);
+      bytes += 4.0 * (2.0 * (double)ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)sd.size());
+    }
+    // segments of about 64 rows (16 more warm up each), shorter where that leaves SMs idle
+    const int rows = 2 * A.nxt * A.nq * (t.M / 64) >= 4000 ? 64 : 32;
+    line_segments(t.M, rows, &A.nseg, &A.chunk, &A.rb);
+    const int items = 2 * A.nxt * A.nq * A.nseg;
+    if (axis) launch_pdl(k_walk3d32, dim3((items + kW3Warps - 1) / kW3Warps), dim3(32 * kW3Warps), 0, g->stream, A);
+    else launch_pdl(k_walkx3d32, dim3((items + kWXWarps - 1) / kWXWarps), dim3(32 * kWXWarps), 0, g->stream, A);
+    prof_mark(g, KK_TERM3D32, bytes);
+    return 1;
+  }
   if (t.K + 1 <= K3H) {
     const int P = axis == 0 ? 1 : 0, Q = axis == 2 ? 1 : 2;
     TermArgs2 A;
@@ -1369,8 +1641,11 @@ void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
       A.y[c] = step == 0 ? A.b[c] : buf[(step + 1) & 1];
       A.out[c] = buf[step & 1];
     }
-    if (l == 1) launch_pdl(k_lev3d32<true>, grd, blk, 0, g->stream, A);
-    else launch_pdl(k_lev3d32<false>, grd, blk, 0, g->stream, A);
+    const bool first = step == 0, last = l == 1;
+    if (first && last) launch_pdl(k_lev3d32<true, true>, grd, blk, 0, g->stream, A);
+    else if (first) launch_pdl(k_lev3d32<true, false>, grd, blk, 0, g->stream, A);
+    else if (last) launch_pdl(k_lev3d32<false, true>, grd, blk, 0, g->stream, A);
+    else launch_pdl(k_lev3d32<false, false>, grd, blk, 0, g->stream, A);
     prof_mark(g, KK_SWEEP3D32, 4.0 * pts * ((step == 0 ? 1.0 : 2.0) + (l == 1 ? 4.0 : 1.0)));
   }
   *nl += p.m - 1;
@@ -1704,6 +1979,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
         s = fail3(MS_ECUDA, "copy of FP32 Pade tables failed");
     }
     if (s == MS_OK && upload_band_row() != 0) s = fail3(MS_ECUDA, "cannot upload the interior band row");
+    for (int kind = 0; kind < 2; ++kind) line_ends(d->closure, kind, false, &g->walk.ends[kind]);
     // the solve polynomial to 1e-10 (below the FP32 rounding noise, which is not coherent)
     if (s == MS_OK && !cheb_coefs(6.0 * g->c1 * g->h * g->h + 24.0, 8.0, 16.0, 1e-10, &g->walk.cheb))
       s = fail3(MS_ENOTCONV, "the FP32 solve polynomial needs too high a degree");

@@ -495,18 +495,6 @@ Split split(double v) {
   return s;
 }
 
-// Segments of the y lines: about `rows` rows each, the last one a multiple of 8 rows that ends with the
-// line, every other one ending at least 8 rows before the line's end.
-void y_segments(YArgs* a, int rows) {
-  const int M = a->M;
-  int K = (M + rows - 1) / rows;
-  if (K < 2) K = 2;
-  const int lastr = std::max(8, M / (8 * K) * 8);
-  a->rb = M - lastr;
-  a->chunk = std::max(8, ((a->rb + K - 2) / (K - 1) + 7) / 8 * 8);
-  a->nseg = (a->rb + a->chunk - 1) / a->chunk + 1;
-}
-
 YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const float* src_hi, const float* src_lo) {
   YArgs a{};
   const int N = g->N;
@@ -528,7 +516,7 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
   // Rows per segment: 16 more warm up its recurrences, so long segments do less work, but a grid wants
   // about ten warps per SM, and small grids short walks.  The choice depends on N alone: a cavity of a batch takes the segments of a
   // single grid, and with them its rounding.
-  y_segments(&a, a.nstrip * (a.M / 64) >= 1500 ? 64 : (N > 320 ? 32 : 16));
+  line_segments(a.M, a.nstrip * (a.M / 64) >= 1500 ? 64 : (N > 320 ? 32 : 16), &a.nseg, &a.chunk, &a.rb);
   a.tiny = N <= kTinyN;
   a.step = step;
   a.N = N;
@@ -613,6 +601,15 @@ namespace {
 int blocks_of(int items) { return (items + WPB - 1) / WPB; }
 
 }  // namespace
+
+void line_segments(int M, int rows, int* nseg, int* chunk, int* rb) {
+  int K = (M + rows - 1) / rows;
+  if (K < 2) K = 2;
+  const int lastr = std::max(8, M / (8 * K) * 8);
+  *rb = M - lastr;
+  *chunk = std::max(8, ((*rb + K - 2) / (K - 1) + 7) / 8 * 8);
+  *nseg = (*rb + *chunk - 1) / *chunk + 1;
+}
 
 double walk_rhs_scale() { return (1.0 - (double)kRhoF) * (1.0 - (double)kRhoF); }
 

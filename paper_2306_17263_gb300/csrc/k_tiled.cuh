@@ -22,6 +22,11 @@ MixedConsts mixed_consts(const ms_grid* g);
 // with rho the FP32 root: the recurrences give A^{-1} d up to it, and the increment scales carry it.
 double walk_rhs_scale();
 
+// Segments of a line of M >= 16 rows that warps walk along: about `rows` rows each, `chunk` rows (a multiple
+// of 8) but for the last one, which is [rb, M), a multiple of 8 rows; every other one ends at least 8
+// rows before the line's end, and the first holds the first 8 rows.
+void line_segments(int M, int rows, int* nseg, int* chunk, int* rb);
+
 // FP32 planes of 2D grids: rows of ld floats (a multiple of 32), with the first unknown column of every
 // field on a 16-byte boundary.  plane_floats: floats of one plane; plane_origin: offset of point (0, 0)
 // of field f in it.
