@@ -222,16 +222,16 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
 // accuracy), joins the low word, and two-sum renormalises the pair.  The Pade terms below then
 // difference G: D1 G = (12 beta + L') D1 u, the filter commuting with the difference under the
 // ghost rules (zero differences beyond the ends of a Neumann line, even ones on a Dirichlet line).
-// A thread takes two rows of one column and marches FZ3 planes along z with the planes below and above in
+// A thread takes two rows of one column and marches along z with the planes below and above in
 // registers, the next plane fetched ahead (no shared memory; the neighbour rows and columns come from L1).
 // The tile form before it, 32 x 16 tiles of three planes in shared memory, issued 112 instructions per 32
 // points, 70 us per component at 256^3.
-constexpr int FZ3 = 16, FY3 = 8;
+constexpr int FY3 = 8;
 struct Filter3d32Args {  // the three components of a half-step
   const float *hi[3], *lo[3];
   float *gh[3], *gl[3];
   Shape3 s[3];
-  int nz;  // blocks along z of the largest component
+  int nz, zc;  // marches along z of the largest component, planes per march
 };
 __global__ void __launch_bounds__(32 * FY3, 4) k_ffilt3d32(const __grid_constant__ Filter3d32Args A, float cb_hi,
                                                           float cb_lo) {
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(32 * FY3, 4) k_ffilt3d32(const __grid_constant
   const Shape3& s = A.s[which];
   const int n0 = s.n[0], n1 = s.n[1], n2 = s.n[2];
   const int i = blockIdx.x * 32 + threadIdx.x, j = 2 * (blockIdx.y * FY3 + threadIdx.y);
-  const int k0 = kz * FZ3, k1 = min(k0 + FZ3, n2);
+  const int k0 = kz * A.zc, k1 = min(k0 + A.zc, n2);
   if (i >= n0 || j >= n1 || k0 >= k1) return;
   const bool two = j + 1 < n1, ux = interior(s.bc[0], i, n0);
   const bool u[2] = {ux && interior(s.bc[1], j, n1), ux && interior(s.bc[1], j + 1, n1)};
@@ -332,6 +332,14 @@ __global__ void __launch_bounds__(32 * FY3, 4) k_ffilt3d32(const __grid_constant
       g[t] += sz;
     }
   }
+}
+
+// Planes per march along z for nz planes of `cols` tiles: 16 (two more come in), fewer where that leaves SMs
+// idle (75^3: levels of three components 28 to 31 us with 16, 17 us with 4).
+int march_planes(int cols, int nz) {
+  int zc = 16;
+  while (zc > 4 && cols * ((nz + zc - 1) / zc) < 4 * 152) zc /= 2;
+  return zc;
 }
 
 // First differences of G along AXIS at the destination points (fallback for Pade tables wider
@@ -833,7 +841,7 @@ constexpr int kAX = 1, kRX = kAX + 1, kXW = 16, kXS = kXW + 1, kWXWarps = 2;  //
 template <bool EDGE>
 __device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Term& T, int row0, int seg,
                                                float (*tile)[2][32 * kXS]) {
-  const int lane = threadIdx.x & 31, xr = lane & (kXW - 1), rs = lane / kXW;
+  const int lane = threadIdx.x & 31, xr = lane & (kXW - 1), rs = lane / kXW * 16;  // rows rs .. rs + 15
   const int cap = min(31, T.nx - 1 - row0);  // last row of the warp
   const bool last = seg == A.nseg - 1;
   const int M = A.M, r0 = last ? A.rb : seg * A.chunk, r1 = last ? M : min(r0 + A.chunk, A.rb);
@@ -848,9 +856,9 @@ __device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Te
       float* dl = tile[c % kRX][1] + rs * kXS + xr;
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        const unsigned o = (unsigned)min(rs + 2 * i, cap) * T.sq + x;
-        cp4(dh + 2 * i * kXS, ph + o);
-        cp4(dl + 2 * i * kXS, pl + o);
+        const unsigned o = (unsigned)min(rs + i, cap) * T.sq + x;
+        cp4(dh + i * kXS, ph + o);
+        cp4(dl + i * kXS, pl + o);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -869,7 +877,7 @@ __device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Te
     if (T.accumulate) {
 #pragma unroll
       for (int i = 0; i < 16; ++i)
-        old[i] = out && rs + 2 * i <= cap ? R[(unsigned)(rs + 2 * i) * T.dq + rw] : 0.0f;
+        old[i] = out && rs + i <= cap ? R[(unsigned)(rs + i) * T.dq + rw] : 0.0f;
     }
     asm volatile("cp.async.wait_group %0;" ::"n"(kAX) : "memory");
     __syncwarp();
@@ -894,8 +902,8 @@ __device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Te
     const float* tw = tile[c % kRX][0] + rs * kXS + xr;
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (out && rs + 2 * i <= cap)
-        R[(unsigned)(rs + 2 * i) * T.dq + rw] = T.accumulate ? tw[2 * i * kXS] + old[i] : tw[2 * i * kXS];
+      if (out && rs + i <= cap)
+        R[(unsigned)(rs + i) * T.dq + rw] = T.accumulate ? tw[i * kXS] + old[i] : tw[i * kXS];
   }
   if (lane <= cap && !T.accumulate) {  // wall points of the lines
     float* __restrict__ Rl = T.R + (size_t)(row0 + lane) * T.dq;
@@ -926,16 +934,15 @@ __global__ void __launch_bounds__(32 * kWXWarps) k_walkx3d32(const __grid_consta
 // corner neighbours in the plane, spectrum [-8, 24].  The Chebyshev polynomial of k_rec64.cu in Horner
 // form, y <- b + q T y, to a relative error of 1e-10, one level per launch for the three components; T y
 // is 2e-3 of D y at most, so a level rounds the increment at 1e-9 of itself, and the last level's q T y
-// enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches L3Z planes along z;
-// the planes come through a ring in shared memory filled by cp.async kA3 planes ahead (loads straight
+// enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches along z; the
+// planes come through a ring in shared memory filled by cp.async kA3 planes ahead (loads straight
 // into registers, one plane ahead, left the march waiting for them: 180 to 225 us per level of three
 // components at 256^3), and a thread keeps e, c and q = 2 y + e of its two rows in registers: ten
 // operations and six shared loads per point and level, where a Richardson sweep with its residual issued
 // 84 instructions.
-constexpr int L3Y = 8, L3Z = 16;  // warps (pairs of rows) per block, planes per march
-constexpr int kA3 = 3, kR3 = kA3 + 1;
-constexpr int S3W = 34, S3N = S3W * (2 * L3Y + 2);  // a staged plane: the tile and one point around it
-static_assert(S3N <= 3 * 32 * L3Y, "three staged points per thread");
+constexpr int L3Y = 4, L3T = 32 * L3Y;  // warps (of four rows) and threads per block
+constexpr int kA3 = 3, kR3 = kA3 + 1;   // a power of two of slots
+constexpr int S3W = 34, S3N = S3W * (4 * L3Y + 2), S3P = (S3N + L3T - 1) / L3T;  // a staged plane, per thread
 struct Lev3d32Args {
   const float* b[3];
   const float* y[3];
@@ -943,40 +950,40 @@ struct Lev3d32Args {
   float *hi[3], *lo[3];  // state (LAST)
   Shape3 s[3];
   float q, s_hi, s_lo;
-  int nz;  // marches along z of the largest component
+  int nz, zc;  // marches along z of the largest component, planes per march
 };
 
 // (hi, lo) += (s_hi + s_lo)(b + c): an exact two-product of s_hi b with the other products in its error
-// term, and a two-sum into the pair.
-__device__ __forceinline__ void ff_add_scaled_bc(float& hi, float& lo, float b, float c, float s_hi, float s_lo) {
-  const float p = __fmul_rn(s_hi, b);
-  float e = fmaf(s_hi, b, -p);
-  e = fmaf(s_lo, b, e);
-  e = fmaf(s_hi, c, e);
-  const float u = __fadd_rn(hi, p);
-  const float bb = __fsub_rn(u, hi);
-  const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(u, bb)), __fsub_rn(p, bb));
-  const float l = __fadd_rn(lo, __fadd_rn(err, e));
-  const float h2 = __fadd_rn(u, l);
-  lo = __fsub_rn(l, __fsub_rn(h2, u));
+// term, and a two-sum into the pair; two points at once.
+__device__ __forceinline__ void ff_add_scaled_bc(float2& hi, float2& lo, float2 b, float2 c, float2 s_hi, float2 s_lo) {
+  const float2 p = mul2(s_hi, b);
+  float2 e = fma2(s_hi, b, neg2(p));
+  e = fma2(s_lo, b, e);
+  e = fma2(s_hi, c, e);
+  const float2 u = add2(hi, p);
+  const float2 bb = sub2(u, hi);
+  const float2 err = add2(sub2(hi, sub2(u, bb)), sub2(p, bb));
+  const float2 l = add2(lo, add2(err, e));
+  const float2 h2 = add2(u, l);
+  lo = sub2(l, sub2(h2, u));
   hi = h2;
 }
 
 // FIRST: y is b itself.
 template <bool FIRST, bool LAST>
-__global__ void __launch_bounds__(32 * L3Y, LAST ? 4 : 5) k_lev3d32(const __grid_constant__ Lev3d32Args A) {
+__global__ void __launch_bounds__(L3T, LAST ? 5 : 7) k_lev3d32(const __grid_constant__ Lev3d32Args A) {
   __shared__ float ring[kR3][S3N];
   pdl_wait();
   const int which = blockIdx.z / A.nz, kz = blockIdx.z - which * A.nz;
   const Shape3& s = A.s[which];
   const int n0 = s.n[0], n1 = s.n[1], n2 = s.n[2];
   const int d0 = s.bc[0] == DIR, d1 = s.bc[1] == DIR, d2 = s.bc[2] == DIR;
-  const int i0 = d0 + blockIdx.x * 32, j0 = d1 + blockIdx.y * 2 * L3Y;
-  const int k0 = d2 + kz * L3Z, k1 = min(k0 + L3Z, n2 - d2);
+  const int i0 = d0 + blockIdx.x * 32, j0 = d1 + blockIdx.y * 4 * L3Y;
+  const int k0 = d2 + kz * A.zc, k1 = min(k0 + A.zc, n2 - d2);
   if (i0 >= n0 - d0 || j0 >= n1 - d1 || k0 >= k1) return;  // block-uniform
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
-  const int i = i0 + tx, j = j0 + 2 * ty;
-  const bool in0 = i < n0 - d0 && j < n1 - d1, in1 = in0 && j + 1 < n1 - d1;
+  const int i = i0 + tx, j = j0 + 4 * ty;
+  const int rows = i < n0 - d0 ? min(4, n1 - d1 - j) : 0;  // the thread's unknowns
   const unsigned sz = n0 * n1;  // points per component fit 31 bits (n <= 512)
   const float* __restrict__ y = A.y[which];
   const float* __restrict__ b = A.b[which];
@@ -985,57 +992,51 @@ __global__ void __launch_bounds__(32 * L3Y, LAST ? 4 : 5) k_lev3d32(const __grid
   float* __restrict__ slo = A.lo[which];
   // staged points of the thread: ghosts of a Neumann axis mirror (clamped), walls of a Dirichlet axis hold
   // zeros (b: the terms write them; y: the level before)
-  auto place = [&](int e) {
-    const int r = e / S3W, c = e - r * S3W;
-    return (unsigned)(clampi(j0 - 1 + r, n1) * n0 + clampi(i0 - 1 + c, n0));
-  };
-  const bool has3 = tid + 512 < S3N;
-  const unsigned o1 = place(tid), o2 = place(tid + 256), o3 = has3 ? place(tid + 512) : 0;
+  unsigned po[S3P];
+#pragma unroll
+  for (int q = 0; q < S3P; ++q) {
+    const int e = min(tid + q * L3T, S3N - 1), r = e / S3W, c = e - r * S3W;
+    po[q] = clampi(j0 - 1 + r, n1) * n0 + clampi(i0 - 1 + c, n0);
+  }
+  const bool tail = tid + (S3P - 1) * L3T < S3N;
   const int S = k1 - k0 + 2;  // planes k0 - 1 .. k1
-  auto fetch = [&](int st, int slot) {
+  auto fetch = [&](int st) {
     if (st < S) {
       const float* __restrict__ p = y + (size_t)clampi(k0 - 1 + st, n2) * sz;
-      float* d = ring[slot] + tid;
-      cp4(d, p + o1);
-      cp4(d + 256, p + o2);
-      if (has3) cp4(d + 512, p + o3);
+      float* d = ring[st % kR3] + tid;
+#pragma unroll
+      for (int q = 0; q < S3P; ++q)
+        if (q < S3P - 1 || tail) cp4(d + q * L3T, p + po[q]);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
 #pragma unroll
-  for (int t = 0; t < kA3; ++t) fetch(t, t);
-  // per-point operands two planes ahead
+  for (int t = 0; t < kA3; ++t) fetch(t);
+  // per-point operands two planes ahead; point rows t and t + 2 of the thread are halves of a pair
   const unsigned own = j * n0 + i;
-  unsigned g = k0 * sz + own;
-  float b1[2] = {}, b2[2] = {}, h1[2] = {}, h2[2] = {}, l1[2] = {}, l2[2] = {};
-  auto operands = [&](int k, float(&bq)[2], float(&hq)[2], float(&lq)[2]) {
-    if (k >= k1) return;
-    const unsigned p = k * sz + own;
-    if (in0) {
-      if (!FIRST) bq[0] = b[p];
-      if (LAST) {
-        hq[0] = shi[p];
-        lq[0] = slo[p];
-      }
-    }
-    if (in1) {
-      if (!FIRST) bq[1] = b[p + n0];
-      if (LAST) {
-        hq[1] = shi[p + n0];
-        lq[1] = slo[p + n0];
-      }
-    }
+  float2 b1[2] = {}, b2[2] = {}, h1[2] = {}, h2[2] = {}, l1[2] = {}, l2[2] = {};
+  auto load = [&](const float* __restrict__ p, float2(&v)[2]) {
+    if (rows > 0) v[0].x = p[0];
+    if (rows > 1) v[1].x = p[n0];
+    if (rows > 2) v[0].y = p[2 * n0];
+    if (rows > 3) v[1].y = p[3 * n0];
   };
-  float qm[2] = {}, q0[2] = {}, u0[2] = {}, m0[2] = {};  // q of planes k - 1, k; 2 e + c and y of plane k
-  int rd = 0, wr = kA3;
+  auto store = [&](float* __restrict__ p, const float2(&v)[2]) {
+    if (rows > 0) p[0] = v[0].x;
+    if (rows > 1) p[n0] = v[1].x;
+    if (rows > 2) p[2 * n0] = v[0].y;
+    if (rows > 3) p[3 * n0] = v[1].y;
+  };
+  float2 qm[2] = {}, q0[2] = {}, u0[2] = {}, m0[2] = {};  // q of planes k - 1, k; 2 e + c and y of plane k
+  const float2 two = bc2(2.0f), q = bc2(A.q);
+  unsigned g = k0 * sz + own;
+#pragma unroll 4
   for (int st = 0; st < S; ++st) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kA3 - 1) : "memory");
     __syncthreads();  // plane st is there for every thread, and the slot read last is free
-    fetch(st + kA3, wr);
-    const float* r = ring[rd] + (2 * ty) * S3W + tx;
-    rd = rd == kR3 - 1 ? 0 : rd + 1;
-    wr = wr == kR3 - 1 ? 0 : wr + 1;
-    float bc[2], hc[2], lc[2];
+    fetch(st + kA3);
+    const float* r = ring[st % kR3] + (4 * ty) * S3W + tx;
+    float2 bc[2], hc[2], lc[2];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       bc[t] = FIRST ? m0[t] : b1[t];
@@ -1045,38 +1046,51 @@ __global__ void __launch_bounds__(32 * L3Y, LAST ? 4 : 5) k_lev3d32(const __grid
       lc[t] = l1[t];
       l1[t] = l2[t];
     }
-    operands(k0 + st, b2, h2, l2);  // used two planes on
-    float m[4], x[4], qn[2];
+    if (k0 + st < k1) {  // used two planes on
+      const unsigned p = (k0 + st) * sz + own;
+      if (!FIRST) load(b + p, b2);
+      if (LAST) {
+        load(shi + p, h2);
+        load(slo + p, l2);
+      }
+    }
+    float ms[6], xs[6];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      ms[t] = r[t * S3W + 1];
+      xs[t] = r[t * S3W] + r[t * S3W + 2];
+    }
+    float2 m[4], x[4], v[2];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      m[t] = r[t * S3W + 1];
-      x[t] = r[t * S3W] + r[t * S3W + 2];
+      m[t] = make_float2(ms[t], ms[t + 2]);
+      x[t] = make_float2(xs[t], xs[t + 2]);
     }
-    const bool live = st >= 2;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-      const float e = x[t + 1] + (m[t] + m[t + 2]);
-      qn[t] = fmaf(2.0f, m[t + 1], e);
-      const float T = u0[t] + (qm[t] + qn[t]);
-      if (live && (t ? in1 : in0)) {
-        if (LAST) {
-          ff_add_scaled_bc(hc[t], lc[t], bc[t], A.q * T, A.s_hi, A.s_lo);
-          shi[g + t * n0] = hc[t];
-          slo[g + t * n0] = lc[t];
-        } else {
-          out[g + t * n0] = fmaf(A.q, T, bc[t]);
-        }
-      }
+      const float2 e = add2(x[t + 1], add2(m[t], m[t + 2]));
+      const float2 qn = fma2(two, m[t + 1], e);
+      const float2 T = add2(u0[t], add2(qm[t], qn));
+      if (LAST) ff_add_scaled_bc(hc[t], lc[t], bc[t], mul2(q, T), bc2(A.s_hi), bc2(A.s_lo));
+      else v[t] = fma2(q, T, bc[t]);
       qm[t] = q0[t];
-      q0[t] = qn[t];
-      u0[t] = fmaf(2.0f, e, x[t] + x[t + 2]);
+      q0[t] = qn;
+      u0[t] = fma2(two, e, add2(x[t], x[t + 2]));
       m0[t] = m[t + 1];
     }
-    if (live) g += sz;
+    if (st >= 2) {
+      if (LAST) {
+        store(shi + g, hc);
+        store(slo + g, lc);
+      } else {
+        store(out + g, v);
+      }
+      g += sz;
+    }
   }
-  if (!LAST && in0) {
+  if (!LAST && rows > 0) {
     // zeros on the walls the next level reads: those next to the thread's points, corners included
-    const int jl = in1 ? j + 1 : j;
+    const int jl = j + rows - 1;
     const int di0 = d0 && i == 1 ? -1 : 0, di1 = d0 && i == n0 - 2 ? 1 : 0;
     const int dj0 = d1 && j == 1 ? -1 : 0, dj1 = d1 && jl == n1 - 2 ? 1 : 0;
     const int dk0 = d2 && k0 == 1 ? -1 : 0, dk1 = d2 && k1 == n2 - 1 ? 1 : 0;
@@ -1442,7 +1456,7 @@ void filter3d32(ms_grid* g, int c0, float cb_hi, float cb_lo) {
   Grid3D* G3 = g->g3;
   Filter3d32Args A;
   int nx = 0, ny = 0;
-  A.nz = 0;
+  int nz = 0;
   double pts = 0.0;
   for (int c = 0; c < 3; ++c) {
     const Shape3& s = G3->sh[c0 + c];
@@ -1453,12 +1467,13 @@ void filter3d32(ms_grid* g, int c0, float cb_hi, float cb_lo) {
     A.s[c] = s;
     nx = s.n[0] > nx ? s.n[0] : nx;
     ny = s.n[1] > ny ? s.n[1] : ny;
-    const int nz = (s.n[2] + FZ3 - 1) / FZ3;
-    A.nz = nz > A.nz ? nz : A.nz;
+    nz = s.n[2] > nz ? s.n[2] : nz;
     pts += (double)s.size();
   }
-  launch_pdl(k_ffilt3d32, dim3((nx + 31) / 32, (ny + 2 * FY3 - 1) / (2 * FY3), 3 * A.nz), dim3(32, FY3), 0, g->stream, A,
-             cb_hi, cb_lo);
+  const int tx = (nx + 31) / 32, ty = (ny + 2 * FY3 - 1) / (2 * FY3);
+  A.zc = march_planes(3 * tx * ty, nz);
+  A.nz = (nz + A.zc - 1) / A.zc;
+  launch_pdl(k_ffilt3d32, dim3(tx, ty, 3 * A.nz), dim3(32, FY3), 0, g->stream, A, cb_hi, cb_lo);
   prof_mark(g, KK_FILT3D32, 16.0 * pts);  // state hi + lo in, G hi + lo out
 }
 
@@ -1512,8 +1527,9 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
       A.nq = std::max(A.nq, a.nq);
       bytes += 4.0 * (2.0 * (double)ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)sd.size());
     }
-    // segments of about 64 rows (16 more warm up each), shorter where that leaves SMs idle
-    const int rows = 2 * A.nxt * A.nq * (t.M / 64) >= 4000 ? 64 : 32;
+    // segments of about 64 rows (16 more warm up each), shorter where that leaves SMs idle (75^3: 135 us per
+    // step with 32 rows, 130 us with 24)
+    const int rows = 2 * A.nxt * A.nq * (t.M / 64) >= 4000 ? 64 : 24;
     line_segments(t.M, rows, &A.nseg, &A.chunk, &A.rb);
     const int items = 2 * A.nxt * A.nq * A.nseg;
     if (axis) launch_pdl(k_walk3d32, dim3((items + kW3Warps - 1) / kW3Warps), dim3(32 * kW3Warps), 0, g->stream, A);
@@ -1613,8 +1629,7 @@ void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
   }
   const Cheb& p = g->walk.cheb;
   Lev3d32Args A;
-  int tx = 0, ty = 0;
-  A.nz = 0;
+  int tx = 0, ty = 0, nz = 0;
   double pts = 0.0;
   for (int c = 0; c < 3; ++c) {
     const Shape3& s = G3->sh[c0 + c];
@@ -1625,13 +1640,15 @@ void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
     int u[3];
     for (int a = 0; a < 3; ++a) u[a] = s.n[a] - 2 * (s.bc[a] == DIR);
     tx = std::max(tx, (u[0] + 31) / 32);
-    ty = std::max(ty, (u[1] + 2 * L3Y - 1) / (2 * L3Y));
-    A.nz = std::max(A.nz, (u[2] + L3Z - 1) / L3Z);
+    ty = std::max(ty, (u[1] + 4 * L3Y - 1) / (4 * L3Y));
+    nz = std::max(nz, u[2]);
     pts += (double)s.size();
   }
   const double s = (e ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0;
   A.s_hi = (float)s;
   A.s_lo = (float)(s - (double)A.s_hi);
+  A.zc = march_planes(3 * tx * ty, nz);
+  A.nz = (nz + A.zc - 1) / A.zc;
   const dim3 grd(tx, ty, 3 * A.nz), blk(32, L3Y);
   for (int l = p.m - 1; l >= 1; --l) {
     const int step = p.m - 1 - l;
