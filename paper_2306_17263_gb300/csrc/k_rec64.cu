@@ -7,8 +7,8 @@
 // line ends, so A^{-1} d is a forward and a backward first-order recurrence (one FMA per row each)
 // instead of a band of 34 taps; a segment of L rows starts its recurrences kRecWarm rows outside itself
 // (rho^14 < 1.6e-19).  The closure's end rows change the solution by a multiple of a decaying vector
-// (LineEnds), so a line end costs 18 FMAs, not 16 explicit band rows.  1024 x 1024, one derivative:
-// 62 us by the band.
+// (LineEnds), so a line end costs 18 FMAs, not 16 explicit band rows.  A step at 1024 x 1024 takes 399 us with
+// these kernels, 1023 us with the band and Richardson sweeps; 3D, 96^3: 1.09 and 2.97 ms.
 //
 // P1 solve.  6 h^2 P1 = D - T with T = (L_x + 6)(L_y + 6), D = 6 c1 h^2 + 36, and T has its spectrum in
 // [4, 36] on every field, Dirichlet or Neumann.  The Chebyshev polynomial p(T) ~ 1 / (D - T) in Horner
@@ -176,14 +176,15 @@ struct LineBatch {
   int n1;  // largest n1 of the batch
 };
 
-constexpr int LW = 4;  // warps per block: segments (walk) or segments of a tile (rows)
+constexpr int LW = 4;  // warps per block of the row form (LS <= LW segments per tile)
+constexpr int kShortLS = 1;  // segments of 16 rows per block
 constexpr double kOneMinusRhoSq = 1.093172397520265540654504;  // (1 - rho)^2 = -24 rho
 
 // Lines across a strided axis, lanes across the contiguous one: a thread walks its segment of a line,
 // every load coalesced.  The last segment of a line is aligned to its end and writes all its rows (the
 // one before it stops there), so both ends and the rows they correct sit at fixed places of a segment.
-template <int L, bool TRANS>
-__global__ void __launch_bounds__(32 * LW) k_line_walk64(LineBatch b) {
+template <int L, int LS, bool TRANS>
+__global__ void __launch_bounds__(32 * LS) k_line_walk64(LineBatch b) {
   pdl_wait();
   const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
   const LineArgs& a = b.a[which];
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(32 * LW) k_line_walk64(LineBatch b) {
   const int l0 = blockIdx.x * 32 + threadIdx.x;
   const int R = TRANS ? a.M + 1 : a.M;
   const int nseg = (R + L - 1) / L;
-  const int seg = blockIdx.y * LW + threadIdx.y;
+  const int seg = blockIdx.y * LS + threadIdx.y;
   if (l0 >= a.n0 || seg >= nseg) return;
   double* o = a.out + l0 * a.out_s0 + l1 * a.out_s1;
   const bool live = l0 >= a.lo && l0 < a.hi;
@@ -213,19 +214,30 @@ __global__ void __launch_bounds__(32 * LW) k_line_walk64(LineBatch b) {
   const double* ip = a.in + l0 * a.in_s0 + l1 * a.in_s1;
   const double scale = a.scale * kOneMinusRhoSq;
   const int n_in = TRANS ? a.M : a.M + 1;
+  double ys[L];
   line_segment64<L, TRANS>(
       s, a.M, b.e, [&](int m) { return (m >= 0 && m < n_in) ? ip[m * (ptrdiff_t)a.in_sa] : 0.0; },
-      [&](int t, double v) {
-        if (t < cnt) op[t * a.out_sa] = a.accumulate ? fma(scale, v, op[t * a.out_sa]) : scale * v;
-      });
+      [&](int t, double v) { ys[t] = v; });
+#pragma unroll
+  for (int t0 = 0; t0 < L; t0 += 8) {  // eight loads in flight
+    double old[8] = {};
+    if (a.accumulate) {
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t0 + t < cnt) old[t] = op[(t0 + t) * a.out_sa];
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (t0 + t < cnt) op[(t0 + t) * a.out_sa] = a.accumulate ? fma(scale, ys[t0 + t], old[t]) : scale * ys[t0 + t];
+  }
 }
 
-// Lines along the contiguous axis: a block takes LW segments of 32 lines.  Whole warps read the lines
+// Lines along the contiguous axis: a block takes LS segments of 32 lines.  Whole warps read the lines
 // into shared memory (odd pitch: lanes across the lines are conflict-free), a thread takes one
 // segment of one line, and the results go back through shared memory.
-template <int L, bool TRANS>
+template <int L, int LS, bool TRANS>
 __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
-  constexpr int OUTS = LW * L, PW = OUTS + 2 * kRecWarm + 3;  // odd
+  constexpr int OUTS = LS * L, PW = OUTS + 2 * kRecWarm + 3;  // odd
   static_assert(PW % 2 == 1, "odd row pitch");
   __shared__ double sm[32 * PW];
   pdl_wait();
@@ -242,6 +254,7 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
   const int la = blockIdx.y * 32;
   const double* in = a.in + l1 * a.in_s1;
   double* out = a.out + l1 * a.out_s1;
+#pragma unroll 4
   for (int q = warp; q < 32; q += LW) {
     const int l0 = la + q;
     const bool live = l0 >= a.lo && l0 < a.hi;
@@ -253,8 +266,8 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
     }
   }
   __syncthreads();
-  const int seg = blockIdx.x * LW + warp;
-  const bool lastseg = seg == nseg - 1, has = seg < nseg;
+  const int seg = blockIdx.x * LS + warp;
+  const bool lastseg = seg == nseg - 1, has = warp < LS && seg < nseg;
   const int s = lastseg ? R - L : seg * L;
   double ys[L];
   if (has) {
@@ -270,25 +283,42 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
       if (t < cnt) sm[lane * PW + s - b0 + t] = ys[t];
   }
   __syncthreads();
-  const bool last_tile = (blockIdx.x + 1) * LW >= nseg;
+  const bool last_tile = (blockIdx.x + 1) * LS >= nseg;
   const double scale = a.scale * kOneMinusRhoSq;
   const int nout = (last_tile ? R : min(t0 + OUTS, R - L)) - b0;
-  for (int q = warp; q < 32; q += LW) {
-    const int l0 = la + q;
-    if (l0 >= a.n0) break;
-    const bool live = l0 >= a.lo && l0 < a.hi;
-    double* o = out + l0 * a.out_s0;
-    double* op = o + b0 + a.out_off;
-    for (int c = lane; c < nout; c += 32) {
-      if (a.accumulate) {
-        if (live) op[c] = fma(scale, sm[q * PW + c], op[c]);
-      } else {
-        op[c] = live ? scale * sm[q * PW + c] : 0.0;
+  constexpr int NC = (OUTS + 31) / 32;  // nout <= OUTS: the last tile, aligned to the end, starts earlier
+#pragma unroll
+  for (int q0 = 0; q0 < 32; q0 += 4 * LW) {
+    double old[4][NC] = {};
+    if (a.accumulate) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int l0 = la + q0 + u * LW + warp;
+        const double* op = out + l0 * a.out_s0 + b0 + a.out_off;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+          if (l0 >= a.lo && l0 < a.hi && 32 * c + lane < nout) old[u][c] = op[32 * c + lane];
       }
     }
-    if (!a.accumulate) {
-      if (t0 == 0 && lane < a.out_off) o[lane] = 0.0;
-      if (last_tile && R + a.out_off + lane < a.out_len) o[R + a.out_off + lane] = 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + u * LW + warp, l0 = la + q;
+      if (l0 >= a.n0) continue;
+      const bool live = l0 >= a.lo && l0 < a.hi;
+      double* o = out + l0 * a.out_s0;
+      double* op = o + b0 + a.out_off;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const int col = 32 * c + lane;
+        if (col < nout) {
+          if (live) op[col] = a.accumulate ? fma(scale, sm[q * PW + col], old[u][c]) : scale * sm[q * PW + col];
+          else if (!a.accumulate) op[col] = 0.0;
+        }
+      }
+      if (!a.accumulate) {
+        if (t0 == 0 && lane < a.out_off) o[lane] = 0.0;
+        if (last_tile && R + a.out_off + lane < a.out_len) o[R + a.out_off + lane] = 0.0;
+      }
     }
   }
 }
@@ -308,20 +338,21 @@ void launch_line64(const LineArgs* args, int count, const LineEnds& e, bool tran
   }
   const bool rows = args[0].in_sa == 1;
   // Segments of 32 rows do 3.3 FMAs per output, of 16 rows 4.6; the shorter ones win while the longer
-  // ones would leave FP64 pipes (4 per SM) without a warp.
+  // ones would leave FP64 pipes (4 per SM) without a warp.  A block takes one short segment: warps of one
+  // SM share its FP64 rate (64^2: 64.0 us per step with four, 56.7 us with one; 321^2: 110.4 and 102.1 us).
   const double warps32 = (double)((n0 + 31) / 32) * ((R + 31) / 32) * b.n1 * count;
   const bool l32 = R >= 64 && warps32 >= 600.0;
-  const int L = l32 ? 32 : 16;
+  const int L = l32 ? 32 : 16, LS = l32 ? 4 : kShortLS;
   const int nseg = (R + L - 1) / L;
-  const dim3 blk(32, LW);
-  const dim3 grd = rows ? dim3((nseg + LW - 1) / LW, (n0 + 31) / 32, b.n1 * count)
-                        : dim3((n0 + 31) / 32, (nseg + LW - 1) / LW, b.n1 * count);
-#define MS_LINE(K)                                                       \
-  do {                                                                   \
-    if (l32 && transposed) launch_pdl(K<32, true>, grd, blk, 0, st, b);  \
-    else if (l32) launch_pdl(K<32, false>, grd, blk, 0, st, b);          \
-    else if (transposed) launch_pdl(K<16, true>, grd, blk, 0, st, b);    \
-    else launch_pdl(K<16, false>, grd, blk, 0, st, b);                   \
+  const dim3 blk(32, rows ? LW : LS);
+  const dim3 grd = rows ? dim3((nseg + LS - 1) / LS, (n0 + 31) / 32, b.n1 * count)
+                        : dim3((n0 + 31) / 32, (nseg + LS - 1) / LS, b.n1 * count);
+#define MS_LINE(K)                                                                 \
+  do {                                                                             \
+    if (l32 && transposed) launch_pdl(K<32, 4, true>, grd, blk, 0, st, b);         \
+    else if (l32) launch_pdl(K<32, 4, false>, grd, blk, 0, st, b);                 \
+    else if (transposed) launch_pdl(K<16, kShortLS, true>, grd, blk, 0, st, b);    \
+    else launch_pdl(K<16, kShortLS, false>, grd, blk, 0, st, b);                   \
   } while (0)
   if (rows) MS_LINE(k_line_rows64);
   else MS_LINE(k_line_walk64);
