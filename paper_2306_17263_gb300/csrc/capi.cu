@@ -79,12 +79,19 @@ void curl_he64(ms_grid* g, const double* Gx, const double* Gy, double* R, int* n
 void curl_eh64(ms_grid* g, const double* GE, double* Rx, double* Ry, int* nl) {
   const int N = g->N;
   const double s = g->kappa2 / (g->Z * g->h);
+  const PadeTable& t = g->pade[NODE_TO_HALF];
+  const double bytes = 8.0 * ((double)(N - 1) * (N + 1) + (double)N * (N + 1));
   // delta_y G_E: columns i = 1..N-1 of E_z (N+1 node values) -> H_x rows 0..N-1
-  launch_pade64(1, GE, Rx, N + 1, N + 1, N, N + 1, 0, 1, N, g->pade[NODE_TO_HALF], -s, 0, g->stream);
-  prof_mark(g, KK_PADE64, 8.0 * ((double)(N - 1) * (N + 1) + (double)N * (N + 1)));
   // delta_x G_E: rows j = 1..N-1 of E_z -> H_y columns 0..N-1
-  launch_pade64(0, GE, Ry, N + 1, N + 1, N, N, 0, 1, N, g->pade[NODE_TO_HALF], s, 0, g->stream);
-  prof_mark(g, KK_PADE64, 8.0 * ((double)(N - 1) * (N + 1) + (double)N * (N + 1)));
+  if (launch_pade64_xy(GE, Ry, N, s, GE, Rx, N + 1, -s, N + 1, N + 1, N, 0, 1, N, t, g->stream)) {
+    prof_mark(g, KK_PADE64, 2.0 * bytes);
+    *nl += 1;
+    return;
+  }
+  launch_pade64(1, GE, Rx, N + 1, N + 1, N, N + 1, 0, 1, N, t, -s, 0, g->stream);
+  prof_mark(g, KK_PADE64, bytes);
+  launch_pade64(0, GE, Ry, N + 1, N + 1, N, N, 0, 1, N, t, s, 0, g->stream);
+  prof_mark(g, KK_PADE64, bytes);
   *nl += 2;
 }
 

@@ -10,11 +10,10 @@
 // components per launch.
 // MS_FP32_REFINED: the arithmetic of the 2D FP32 path (k_mixed.cu) carried to 3D: float-float
 // state; each half-step first filters its three source components once into float-float
-// G = 12 beta u + L u (k_ffilt3d32), then per Pade term one tile kernel (k_term3d32) forms the
-// first differences of G along the line (the filter commutes with the difference under the ghost
-// rules) and applies A^{-1} (interior rows by two first-order recurrences, rows near a wall by the
-// explicit band rows, farthest taps first), accumulating the right-hand side (a difference kernel
-// and a band kernel take over for tables wider than the tile holds); the solve (k_lev3d32) is a Chebyshev
+// G = 12 beta u + L u (k_ffilt3d32), then per axis the two Pade terms by walking warps (k_walk3d32,
+// k_walkx3d32): first differences of G along the line (the filter commutes with the difference under the
+// ghost rules) and A^{-1} by two first-order recurrences, accumulating the right-hand side (short lines
+// by explicit table rows, k_short3d32); the solve (k_lev3d32) is a Chebyshev
 // polynomial in Horner form, one level per launch.  The three components of a half-step share launches
 // (14 per step).  The transform solver (k_transform.cu) is followed by Richardson sweeps (k_sweep3d32).
 #include <algorithm>
@@ -49,7 +48,7 @@ struct Grid3D {
   float* hi[6] = {};
   float* lo[6] = {};
   double* s64[9] = {};  // FP64: G[3], R[3], and, with G again, the work planes of the solves; FP32 grids use [0], [1]
-  float* s32[4] = {};   // FP32: differences, R[3]
+  float* s32[3] = {};   // FP32: R
   float* gh[3] = {};    // FP32: filtered components G~ (hi, lo) of one half-step, slot c % 3
   float* gl[3] = {};
   double* dview[6] = {};  // FP32_REFINED grids: FP64 copy of the state for the diagnostics
@@ -177,14 +176,7 @@ __global__ void k_mode_field3(double* __restrict__ out, Shape3 s, const double* 
 // ---------------------------------------------------------------------------------------
 // FP32_REFINED kernels
 
-// Interior row of A^{-1} at offsets -KB3 .. KB3+1 (hi) and the lo parts of offsets -1, 0, 1: the
-// same Toeplitz row for every grid, 24 (-rho) rho^|d| / (1 - rho^2), rho = -11 + sqrt(120).
-constexpr int KB3 = 7;
-__constant__ float c_w3[2 * KB3 + 2];
-__constant__ float c_wl3[3];
-// The interior rows as the recurrences A factors into: rho (FP32), 1 / (1 - rho), and the scale
-// (1 - rho_f) / (1 + rho_f) (hi, lo) that gives them a DC gain of exactly 1.
-__constant__ float c_rec3[4];
+constexpr float kRho3 = -0.045548850f;  // -11 + sqrt(120), the ratio of the recurrences A factors into, in FP32
 
 // Paired FP32 arithmetic (two correctly rounded operations per instruction, sm_100 and later):
 // bitwise the same as the scalar operations on each half.
@@ -223,7 +215,9 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
 // difference G: D1 G = (12 beta + L') D1 u, the filter commuting with the difference under the
 // ghost rules (zero differences beyond the ends of a Neumann line, even ones on a Dirichlet line).
 // A thread takes two rows of one column and marches along z with the planes below and above in
-// registers, the next plane fetched ahead (no shared memory; the neighbour rows and columns come from L1).
+// registers, the next plane fetched ahead (no shared memory; the neighbour rows and columns come from L1):
+// three components at 256^3 in 205 us, 75^3 in 13; planes through a ring in shared memory took 182 to 213 us
+// and 21.
 // The tile form before it, 32 x 16 tiles of three planes in shared memory, issued 112 instructions per 32
 // points, 70 us per component at 256^3.
 constexpr int FY3 = 8;
@@ -342,171 +336,6 @@ int march_planes(int cols, int nz) {
   return zc;
 }
 
-// First differences of G along AXIS at the destination points (fallback for Pade tables wider
-// than the term tile holds): d = (gh_{m+1} - gh_m) + (gl_{m+1} - gl_m) at o = m + out_off, 0 at
-// the other points.  Indices are 32-bit (n <= 512: at most 513^3 points per component).
-template <int AXIS>
-__global__ void k_diff3d32(const float* __restrict__ gh, const float* __restrict__ gl, Shape3 ss, float* __restrict__ d,
-                           Shape3 sd, int out_off, int M) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-  if (x >= sd.n[0] || y >= sd.n[1]) return;
-  const int pd = (z * sd.n[1] + y) * sd.n[0] + x;
-  const int m = (AXIS == 0 ? x : (AXIS == 1 ? y : z)) - out_off;
-  if (m < 0 || m >= M) {
-    d[pd] = 0.0f;
-    return;
-  }
-  const int st[3] = {1, ss.n[0], ss.n[0] * ss.n[1]};
-  const int cx = AXIS == 0 ? m : x, cy = AXIS == 1 ? m : y, cz = AXIS == 2 ? m : z;
-  const int ps = (cz * ss.n[1] + cy) * ss.n[0] + cx;
-  d[pd] = (gh[ps + st[AXIS]] - gh[ps]) + (gl[ps + st[AXIS]] - gl[ps]);
-}
-
-// y = A^{-1} d along AXIS, then R (+)= sign * y at the unknowns of the destination component.
-// Rows away from the line ends use the interior row from constant memory (taps -KB3 .. KB3+1);
-// the end rows use the explicit FP32 hi + lo table rows.  Taps are summed farthest first (see
-// the 2D curl tile for why the order matters).
-template <int AXIS>
-__global__ void k_band3d32(const float* __restrict__ d, float* __restrict__ R, Shape3 sd, int out_off, int M,
-                           const float* __restrict__ whi, const float* __restrict__ wlo, int K, int B,
-                           int all_explicit, float sign, int accumulate) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-  if (x >= sd.n[0] || y >= sd.n[1]) return;
-  const int pd = (z * sd.n[1] + y) * sd.n[0] + x;
-  const int r = (AXIS == 0 ? x : (AXIS == 1 ? y : z)) - out_off;
-  if (!unk3(sd, x, y, z) || r < 0 || r >= M) {
-    if (!accumulate) R[pd] = 0.0f;
-    return;
-  }
-  const int stride = AXIS == 0 ? 1 : (AXIS == 1 ? sd.n[0] : sd.n[0] * sd.n[1]);
-  const float* dc = d + pd;  // dc[t * stride] = d_{r + t}
-  float acc;
-  if (!all_explicit && r >= B && r < M - B && r >= KB3 && r + KB3 + 1 < M) {
-    acc = c_w3[2 * KB3 + 1] * dc[(KB3 + 1) * stride];
-#pragma unroll
-    for (int dist = KB3; dist >= 1; --dist) {
-      acc = fmaf(c_w3[KB3 + dist], dc[dist * stride], acc);
-      acc = fmaf(c_w3[KB3 - dist], dc[-dist * stride], acc);
-    }
-    acc = fmaf(c_wl3[0], dc[-stride], acc);
-    acc = fmaf(c_wl3[2], dc[stride], acc);
-    acc = fmaf(c_wl3[1], dc[0], acc);
-    acc = fmaf(c_w3[KB3], dc[0], acc);
-  } else {
-    const float* wh = pade_row_ptr(whi, r, M, K, B, all_explicit);
-    const float* wl = pade_row_ptr(wlo, r, M, K, B, all_explicit);
-    float lo = 0.0f;
-    acc = 0.0f;
-    for (int dist = K + 1; dist >= 1; --dist) {
-      for (int side = 1; side >= -1; side -= 2) {
-        const int mm = r + side * dist, t = mm - r + K;
-        if (t < 0 || t > 2 * K + 1 || mm < 0 || mm >= M) continue;
-        const float dm = dc[(mm - r) * stride];
-        acc = fmaf(__ldg(wh + t), dm, acc);
-        lo = fmaf(__ldg(wl + t), dm, lo);
-      }
-    }
-    lo = fmaf(__ldg(wl + K), dc[0], lo);
-    acc = fmaf(__ldg(wh + K), dc[0], acc + lo);
-  }
-  R[pd] = accumulate ? R[pd] + sign * acc : sign * acc;
-}
-
-constexpr int T3O = 64;             // band rows per tile
-constexpr int K3H = 13;             // reach held in shared memory (table half-width <= 12)
-constexpr int D3L = T3O + 2 * K3H;  // differences per line
-
-// Interior row of the band at row r, d[t] = delta_{r - KB3 + t} (t = 0 .. 2 KB3 + 1), taps summed
-// farthest first, the lo parts of the three central taps before the central hi tap (rows of a
-// run that also holds end rows; whole interior runs take rec_rows3).
-__device__ __forceinline__ float band_fast3(const float* d) {
-  float acc = c_w3[2 * KB3 + 1] * d[2 * KB3 + 1];
-#pragma unroll
-  for (int dist = KB3; dist >= 1; --dist) {
-    acc = fmaf(c_w3[KB3 + dist], d[KB3 + dist], acc);
-    acc = fmaf(c_w3[KB3 - dist], d[KB3 - dist], acc);
-  }
-  acc = fmaf(c_wl3[0], d[KB3 - 1], acc);
-  acc = fmaf(c_wl3[2], d[KB3 + 1], acc);
-  acc = fmaf(c_wl3[1], d[KB3], acc);
-  return fmaf(c_w3[KB3], d[KB3], acc);
-}
-
-// Eight interior rows rb .. rb + 7 of A^{-1} d (v[t] = d_{rb + t}, t = -KR3 - 1 .. 8 + KR3).
-// A = (1/24) tridiag(1, 22, 1) = (1 - rho E^-1)(1 - rho E) / (1 - rho)^2 with rho^2 + 22 rho + 1 = 0,
-// and by partial fractions 1 / ((1 - rho E^-1)(1 - rho E)) = (F + G - 1) / (1 - rho^2) with
-// F = (1 - rho E^-1)^-1, G = (1 - rho E)^-1: A^{-1} d = (1 - rho) / (1 + rho) (f + g - d) for
-// the forward recurrence f_i = d_i + rho f_{i-1} and the backward one g_i = d_i + rho g_{i+1}.
-// The two are independent chains over d (half the dependent depth of running one after the
-// other).  Each starts KR3 + 1 rows outside the eight from the steady state d / (1 - rho), an
-// error damped by |rho|^(KR3+1) ~ 4e-10 times the change of d over those rows; every product
-// enters through one FMA.
-constexpr int KR3 = 6;
-template <typename Emit>
-__device__ __forceinline__ void rec_rows3(const float* v, Emit emit) {
-  const float rho = c_rec3[0], inv1mr = c_rec3[1];
-  float fs[8];
-  float f = v[-KR3 - 1] * inv1mr;
-#pragma unroll
-  for (int t = -KR3; t < 8; ++t) {
-    f = fmaf(rho, f, v[t]);
-    if (t >= 0) fs[t] = f;
-  }
-  float g = v[8 + KR3] * inv1mr;
-#pragma unroll
-  for (int t = 7 + KR3; t >= 0; --t) {
-    g = fmaf(rho, g, v[t]);
-    if (t < 8) {
-      const float u = (fs[t] + g) - v[t];
-      emit(t, fmaf(c_rec3[2], u, c_rec3[3] * u));
-    }
-  }
-}
-
-// Explicit table row r (hi + lo), dc[t] = delta_{r + t}, taps farthest first as in the interior
-// row, hi and lo products summed apart.  The loop is unrolled to the largest half-width the tile
-// holds, the taps beyond K predicated off; taps outside the line read the zeros stored there.
-__device__ __forceinline__ float band_gen3(const float* dc, int r, int M, const float* __restrict__ whi,
-                                           const float* __restrict__ wlo, int K, int B, int all_explicit) {
-  const float* wh = pade_row_ptr(whi, r, M, K, B, all_explicit) + K;  // wh[d]: tap of delta_{r + d}
-  const float* wl = pade_row_ptr(wlo, r, M, K, B, all_explicit) + K;
-  float acc = 0.0f, lo2 = 0.0f;
-#pragma unroll
-  for (int dist = K3H; dist >= 1; --dist) {
-    if (dist <= K + 1) {
-      const float d = dc[dist];
-      acc = fmaf(__ldg(wh + dist), d, acc);
-      lo2 = fmaf(__ldg(wl + dist), d, lo2);
-    }
-    if (dist <= K) {
-      const float d = dc[-dist];
-      acc = fmaf(__ldg(wh - dist), d, acc);
-      lo2 = fmaf(__ldg(wl - dist), d, lo2);
-    }
-  }
-  lo2 = fmaf(__ldg(wl), dc[0], lo2);
-  return fmaf(__ldg(wh), dc[0], acc + lo2);
-}
-
-// One Pade term y = A^{-1} D1 G along AXIS, R (+)= sign y, on a tile of T3O band rows r0 ..
-// r0 + T3O - 1 of 32 lines along the transverse axis P (y for x lines, x otherwise), at one
-// coordinate q of the other transverse axis Q.  The first differences of G over the rows' reach
-// (K3H on each side) go to shared memory, a row per line; a thread then takes eight consecutive
-// rows of one line (lanes across the lines, so every lane of a warp is at the same rows and the
-// end rows of the table take their path together).  x lines are read and written along x by whole
-// warps, the results passing through shared memory; y and z lines are read and written with the
-// lanes across x.  Runs of rows away from the line ends take the recurrences (rec_rows3); runs
-// that hold end rows take the explicit FP32 hi + lo table rows there and the interior band row
-// from constant memory elsewhere.  Wall lines
-// need no test: G is 0 on them, so y is 0 there.  Without accumulation the first and last tiles of
-// a line also write the wall points beyond the band rows (0).
-template <int AXIS>
-struct TermGeo {
-  static constexpr int P = AXIS == 0 ? 1 : 0;  // in-tile transverse axis
-  static constexpr int Q = AXIS == 2 ? 1 : 2;  // the other transverse axis
-};
-constexpr int DP3 = D3L | 1;  // odd row pitch: lanes across the rows are conflict-free
-
 struct TermArgs {
   const float* gh;
   const float* gl;
@@ -517,195 +346,57 @@ struct TermArgs {
 };
 struct TermArgs2 {  // the two terms of a half-step along one axis
   TermArgs t[2];
-  int nq;  // lines along Q of the larger component
+  int nz;  // planes of the larger component
 };
-template <int AXIS>
-__global__ void __launch_bounds__(256, AXIS == 0 ? 4 : 5) k_term3d32(const __grid_constant__ TermArgs2 A, int out_off, int M,
-                                                     const float* __restrict__ whi, const float* __restrict__ wlo, int K,
-                                                     int B, int all_explicit) {
-  constexpr int P = TermGeo<AXIS>::P, Q = TermGeo<AXIS>::Q;
-  __shared__ float dd[32 * DP3];
+
+// Pade terms y = A^{-1} D1 G, R (+)= sign y, on lines shorter than kWalk3Min rows (grids of up to 16 cells, all
+// end rows): a thread sums its explicit table row over the differences of G, hi and lo parts apart, taps
+// farthest first.  Without accumulation points that no band row reaches get 0.  Indices are 32-bit.
+__global__ void k_short3d32(const __grid_constant__ TermArgs2 A, int axis, int out_off, int M,
+                            const float* __restrict__ whi, const float* __restrict__ wlo, int K, int B,
+                            int all_explicit) {
   pdl_wait();
-  const int which = blockIdx.z / A.nq, q = blockIdx.z - which * A.nq;
+  const int which = blockIdx.z / A.nz;
   const TermArgs& T = A.t[which];
-  const float* __restrict__ gh = T.gh;
-  const float* __restrict__ gl = T.gl;
-  float* __restrict__ R = T.R;
   const Shape3 &ss = T.ss, &sd = T.sd;
-  const float sign = T.sign;
-  const int accumulate = T.accumulate;
-  if (q >= sd.n[Q]) return;
-  const int tr = AXIS == 0 ? blockIdx.x : blockIdx.y, p0 = 32 * (AXIS == 0 ? blockIdx.y : blockIdx.x);
-  const int r0 = tr * T3O;  // first band row of the tile
-  const int st[3] = {1, ss.n[0], ss.n[0] * ss.n[1]};
-  const int sdt[3] = {1, sd.n[0], sd.n[0] * sd.n[1]};
-  const int nA = sd.n[AXIS], nP = sd.n[P];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool last_tile = r0 + T3O >= M;
-  const int mb = r0 - K3H;  // m of difference column 0
-  auto fast = [&](int r) { return !all_explicit && r >= B && r < M - B && r >= KB3 && r + KB3 + 1 < M; };
-  // x lines: warp w reads and writes lines 4 w .. 4 w + 3 of the tile along x
-  float racc[8];  // R at this thread's outputs when accumulating, fetched first
-  if (AXIS == 0) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int p = p0 + 4 * warp + i, ld = p * sdt[P] + q * sdt[Q];
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int r = r0 + lane + 32 * c;
-        racc[2 * i + c] = (accumulate && p < nP && r < M) ? R[ld + r + out_off] : 0.0f;
-      }
-    }
-    // G at source points mb + lane + 32 c of the warp's four lines, every load issued first
-    // (lines past the grid read the last line, unused)
-    const int ns = ss.n[0];
-    const bool inner = mb >= 0 && mb + 96 <= ns;  // block-uniform: no tests along the line
-    float h[4][3], l[4][3];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int pl = min(p0 + 4 * warp + i, nP - 1);
-      const float* hr = gh + pl * st[P] + q * st[Q] + mb + lane;
-      const float* lr = gl + pl * st[P] + q * st[Q] + mb + lane;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int sidx = mb + lane + 32 * c;
-        const bool ok = inner || (sidx >= 0 && sidx < ns);
-        h[i][c] = ok ? hr[32 * c] : 0.0f;
-        l[i][c] = ok ? lr[32 * c] : 0.0f;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int ll = 4 * warp + i;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float h1 = __shfl_down_sync(0xffffffffu, h[i][c], 1), l1 = __shfl_down_sync(0xffffffffu, l[i][c], 1);
-        const float hn = __shfl_sync(0xffffffffu, c < 2 ? h[i][c < 2 ? c + 1 : 0] : 0.0f, 0);
-        const float ln = __shfl_sync(0xffffffffu, c < 2 ? l[i][c < 2 ? c + 1 : 0] : 0.0f, 0);
-        if (lane == 31) {
-          h1 = hn;
-          l1 = ln;
-        }
-        const int j = lane + 32 * c, m = mb + j;
-        if (j < D3L) dd[ll * DP3 + j] = (m >= 0 && m < M) ? (h1 - h[i][c]) + (l1 - l[i][c]) : 0.0f;
-      }
-    }
-  }
-  const int p = p0 + lane;  // the line of this thread in the band phase
-  const bool live = p < nP;
-  const int ob = 8 * warp, rb = r0 + ob;
-  const int sA = sdt[AXIS];
-  const int ld = p * sdt[P] + q * sdt[Q];
-  if (AXIS != 0) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) racc[u] = (accumulate && live && rb + u < M) ? R[ld + (rb + u + out_off) * sA] : 0.0f;
-    // differences j in [w RJ, (w + 1) RJ) of the lane's line, all loads issued first
-    constexpr int RJ = (D3L + 7) / 8;
-    const int sa = st[AXIS];
-    const int ja = warp * RJ;
-    const int pc = live ? p : nP - 1;  // lanes past the tile's lines read the last line, unused
-    const float* gph = gh + pc * st[P] + q * st[Q];
-    const float* gpl = gl + pc * st[P] + q * st[Q];
-    float hv[RJ + 1], lv[RJ + 1];
-    float* row = dd + lane * DP3;
-    if (mb + ja >= 0 && mb + ja + RJ < M) {
-      // the warp's run lies inside the line: no tests (warp-uniform)
-      const float* hr = gph + (mb + ja) * sa;
-      const float* lr = gpl + (mb + ja) * sa;
-#pragma unroll
-      for (int i = 0; i <= RJ; ++i) {
-        hv[i] = hr[i * sa];
-        lv[i] = lr[i * sa];
-      }
-#pragma unroll
-      for (int i = 0; i < RJ; ++i)
-        if (ja + i < D3L) row[ja + i] = (hv[i + 1] - hv[i]) + (lv[i + 1] - lv[i]);
-    } else {
-#pragma unroll
-      for (int i = 0; i <= RJ; ++i) {
-        const int sidx = mb + ja + i;  // source point
-        const bool ok = sidx >= 0 && sidx <= M;
-        hv[i] = ok ? gph[sidx * sa] : 0.0f;
-        lv[i] = ok ? gpl[sidx * sa] : 0.0f;
-      }
-#pragma unroll
-      for (int i = 0; i < RJ; ++i) {
-        const int j = ja + i, m = mb + j;
-        if (j < D3L) row[j] = (m >= 0 && m < M) ? (hv[i + 1] - hv[i]) + (lv[i + 1] - lv[i]) : 0.0f;
-      }
-    }
-  }
-  __syncthreads();
-  if (AXIS != 0) {
-    // y and z lines: each result goes straight to R
-    if (!live) return;
-    const float* row = dd + lane * DP3;
-    float* Rp = R + ld + (rb + out_off) * sA;
-    auto put = [&](int u, float v) { Rp[u * sA] = accumulate ? racc[u] + sign * v : sign * v; };
-    if (rb + 7 < M && fast(rb) && fast(rb + 7)) {
-      rec_rows3(row + ob + K3H, put);
-    } else {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int rr = rb + u;
-        const float* dc = row + rr - r0 + K3H;
-        if (rr < M) put(u, fast(rr) ? band_fast3(dc - KB3) : band_gen3(dc, rr, M, whi, wlo, K, B, all_explicit));
-      }
-    }
-    if (!accumulate && warp == 0) {
-      if (tr == 0)
-        for (int od = 0; od < out_off; ++od) R[ld + od * sA] = 0.0f;
-      if (last_tile)
-        for (int od = M + out_off; od < nA; ++od) R[ld + od * sA] = 0.0f;
-    }
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z - which * A.nz;
+  if (x >= sd.n[0] || y >= sd.n[1] || z >= sd.n[2]) return;
+  const size_t pd = at3(sd, x, y, z);
+  const int r = (axis == 0 ? x : (axis == 1 ? y : z)) - out_off;
+  if (!unk3(sd, x, y, z) || r < 0 || r >= M) {
+    if (!T.accumulate) T.R[pd] = 0.0f;
     return;
   }
-  float y[8];
-  if (live) {
-    const float* row = dd + lane * DP3;
-    if (rb + 7 < M && fast(rb) && fast(rb + 7)) {
-      rec_rows3(row + ob + K3H, [&](int u, float v) { y[u] = v; });
-    } else {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int rr = rb + u;
-        const float* dc = row + rr - r0 + K3H;
-        y[u] = rr >= M ? 0.0f : (fast(rr) ? band_fast3(dc - KB3) : band_gen3(dc, rr, M, whi, wlo, K, B, all_explicit));
-      }
+  const int sa = axis == 0 ? 1 : (axis == 1 ? ss.n[0] : ss.n[0] * ss.n[1]);
+  const size_t ps = at3(ss, axis == 0 ? 0 : x, axis == 1 ? 0 : y, axis == 2 ? 0 : z);
+  const float* __restrict__ h = T.gh + ps;
+  const float* __restrict__ l = T.gl + ps;
+  auto diff = [&](int m) { return (h[(m + 1) * sa] - h[m * sa]) + (l[(m + 1) * sa] - l[m * sa]); };
+  const float* wh = pade_row_ptr(whi, r, M, K, B, all_explicit);
+  const float* wl = pade_row_ptr(wlo, r, M, K, B, all_explicit);
+  float acc = 0.0f, lo = 0.0f;
+  for (int dist = K + 1; dist >= 1; --dist) {
+    for (int side = 1; side >= -1; side -= 2) {
+      const int m = r + side * dist, t = m - r + K;
+      if (t < 0 || t > 2 * K + 1 || m < 0 || m >= M) continue;
+      const float d = diff(m);
+      acc = fmaf(__ldg(wh + t), d, acc);
+      lo = fmaf(__ldg(wl + t), d, lo);
     }
   }
-  // x lines: y through shared memory (row = line, column = band row), written along x
-  __syncthreads();
-  if (live) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) dd[lane * DP3 + ob + u] = y[u];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int ll = 4 * warp + i, pl = p0 + ll;
-    if (pl >= nP) break;
-    const int ldl = pl * sdt[P] + q * sdt[Q];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int o = lane + 32 * c, r = r0 + o;
-      if (r < M) {
-        const float yv = dd[ll * DP3 + o];
-        R[ldl + r + out_off] = accumulate ? racc[2 * i + c] + sign * yv : sign * yv;
-      }
-    }
-    if (!accumulate) {
-      if (tr == 0 && lane < out_off) R[ldl + lane] = 0.0f;
-      if (last_tile && M + out_off + lane < nA) R[ldl + M + out_off + lane] = 0.0f;
-    }
-  }
+  const float d = diff(r);
+  lo = fmaf(__ldg(wl + K), d, lo);
+  acc = fmaf(__ldg(wh + K), d, acc + lo);
+  T.R[pd] = T.accumulate ? T.R[pd] + T.sign * acc : T.sign * acc;
 }
 
 // Pade terms along y and z on lines of at least kWalk3Min rows: the walk along y of the 2D step
 // (k_tiled.cu) on the filtered G.  A lane takes one x and walks down its segment of a line, every access
 // coalesced; forward recurrence with the walk, backward over groups of eight rows, the closure's end rows
-// as a rank-one correction.  19 warp instructions per 32 points where the tile form (k_term3d32) issues 115:
-// bound by DRAM.
+// as a rank-one correction.  45 warp instructions per 32 points, where a tile form with the differences in
+// shared memory issued 115: two terms at 256^3 take 88 us (3.0 to 4.6 TB/s), bound by the loads a warp has in
+// flight, and took 130 to 185 us.  Shorter lines are all end rows (k_short3d32).
 constexpr int kWalk3Min = 16, kW3Warps = 4, kEnd3 = 8;
 struct Walk3Term {
   const float* gh;
@@ -738,14 +429,14 @@ __device__ __forceinline__ void walk3_group(const Walk3Args& A, const float (&ch
     if (EDGE) d = (m0 + t >= 0 && m0 + t < A.M) ? d : 0.0f;
     h0 = ch[t];
     l0 = cl[t];
-    zc[t] = z = fmaf(c_rec3[0], z, d);
+    zc[t] = z = fmaf(kRho3, z, d);
   }
   float acc = zc[7];
 #pragma unroll
-  for (int t = 6; t >= 1; --t) acc = fmaf(c_rec3[0], acc, zc[t]);
-  y[7] = acc = fmaf(c_rec3[0], acc, zc[0]);
+  for (int t = 6; t >= 1; --t) acc = fmaf(kRho3, acc, zc[t]);
+  y[7] = acc = fmaf(kRho3, acc, zc[0]);
 #pragma unroll
-  for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(c_rec3[0], acc, zp[t]);
+  for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRho3, acc, zp[t]);
 #pragma unroll
   for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
   if (EDGE && first) {
@@ -836,7 +527,9 @@ __global__ void __launch_bounds__(32 * kW3Warps) k_walk3d32(const __grid_constan
 // The same walk for the terms along x: a lane takes a row of the component (x, all rows of a plane stack
 // being equally long), 32 rows per warp, and sixteen points of every row at a time come through tiles in
 // shared memory, filled by cp.async along x kAX tiles ahead; the results go back through the tile just read and
-// leave along x.  In Walk3Term, nx counts the rows, sq and dq are their strides.
+// leave along x.  Two accumulating terms at 256^3: 142 and 121 us (200 and 180 us with two tiles ahead, for the
+// warps their shared memory leaves out; 166 us by tiles of 64 x 32).  In Walk3Term, nx counts the rows, sq and
+// dq are their strides.
 constexpr int kAX = 1, kRX = kAX + 1, kXW = 16, kXS = kXW + 1, kWXWarps = 2;  // tile stride odd: no bank conflicts
 template <bool EDGE>
 __device__ __forceinline__ void walk3x_segment(const Walk3Args& A, const Walk3Term& T, int row0, int seg,
@@ -937,9 +630,10 @@ __global__ void __launch_bounds__(32 * kWXWarps) k_walkx3d32(const __grid_consta
 // enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches along z; the
 // planes come through a ring in shared memory filled by cp.async kA3 planes ahead (loads straight
 // into registers, one plane ahead, left the march waiting for them: 180 to 225 us per level of three
-// components at 256^3), and a thread keeps e, c and q = 2 y + e of its two rows in registers: ten
-// operations and six shared loads per point and level, where a Richardson sweep with its residual issued
-// 84 instructions.
+// components at 256^3), and a thread keeps e, c and q = 2 y + e of its four rows in registers as two pairs:
+// 32 instructions per 32 points, 75 with two rows and scalar operations, 84 in a Richardson sweep with its
+// residual.  Three components at 256^3: 107 us for the first level, 147 a middle one, 213 the last one
+// (127, 170, 240 with two rows; 195 to 280 per sweep), 3.8, 4.1 and 4.7 TB/s: bound by loads in flight.
 constexpr int L3Y = 4, L3T = 32 * L3Y;  // warps (of four rows) and threads per block
 constexpr int kA3 = 3, kR3 = kA3 + 1;   // a power of two of slots
 constexpr int S3W = 34, S3N = S3W * (4 * L3Y + 2), S3P = (S3N + L3T - 1) / L3T;  // a staged plane, per thread
@@ -1485,8 +1179,7 @@ struct Term3 {
   int accumulate;
 };
 
-// The two terms of a half-step along one axis in one launch (tables wider than the tile holds: two
-// launches per term).  Returns the number of launches issued.
+// The two terms of a half-step along one axis in one launch.  Returns the number of launches issued.
 int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
   Grid3D* G3 = g->g3;
   const int kind = (G3->sh[q0.cs].bc[axis] == NEU) ? HALF_TO_NODE : NODE_TO_HALF;
@@ -1513,7 +1206,7 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
       const Shape3& sd = G3->sh[q[k]->cd];
       a.gh = G3->gh[q[k]->cs % 3];
       a.gl = G3->gl[q[k]->cs % 3];
-      a.R = G3->s32[1 + q[k]->cd % 3];
+      a.R = G3->s32[q[k]->cd % 3];
       a.nx = axis ? sd.n[0] : sd.n[1] * sd.n[2];
       a.nq = axis ? sd.n[Q] : 1;
       a.sa = stride(ss, axis);
@@ -1537,60 +1230,29 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
     prof_mark(g, KK_TERM3D32, bytes);
     return 1;
   }
-  if (t.K + 1 <= K3H) {
-    const int P = axis == 0 ? 1 : 0, Q = axis == 2 ? 1 : 2;
-    TermArgs2 A;
-    int np = 0;
-    A.nq = 0;
-    double bytes = 0.0;
-    for (int k = 0; k < 2; ++k) {
-      TermArgs& a = A.t[k];
-      a.gh = G3->gh[q[k]->cs % 3];
-      a.gl = G3->gl[q[k]->cs % 3];
-      a.R = G3->s32[1 + q[k]->cd % 3];
-      a.ss = G3->sh[q[k]->cs];
-      a.sd = G3->sh[q[k]->cd];
-      a.sign = q[k]->sign;
-      a.accumulate = q[k]->accumulate;
-      np = a.sd.n[P] > np ? a.sd.n[P] : np;
-      A.nq = a.sd.n[Q] > A.nq ? a.sd.n[Q] : A.nq;
-      // G hi + lo in, R out (read too when accumulating)
-      bytes += 4.0 * (2.0 * (double)a.ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)a.sd.size());
-    }
-    const int nt = (t.M + T3O - 1) / T3O;
-    const dim3 grd = axis == 0 ? dim3(nt, (np + 31) / 32, 2 * A.nq) : dim3((np + 31) / 32, nt, 2 * A.nq), blk(256);
-    auto go = [&](auto kernel) {
-      launch_pdl(kernel, grd, blk, 0, g->stream, A, off, t.M, (const float*)t.d_whi, (const float*)t.d_wlo, t.K, t.B,
-                 (int)t.all_explicit);
-    };
-    if (axis == 0) go(k_term3d32<0>);
-    else if (axis == 1) go(k_term3d32<1>);
-    else go(k_term3d32<2>);
-    prof_mark(g, KK_TERM3D32, bytes);
-    return 1;
-  }
+  TermArgs2 A;
+  int nx = 0, ny = 0;
+  A.nz = 0;
+  double bytes = 0.0;
   for (int k = 0; k < 2; ++k) {
-    const Shape3& ss = G3->sh[q[k]->cs];
-    const Shape3& sd = G3->sh[q[k]->cd];
-    const float* gh = G3->gh[q[k]->cs % 3];
-    const float* gl = G3->gl[q[k]->cs % 3];
-    float* R = G3->s32[1 + q[k]->cd % 3];
-    const float sign = q[k]->sign;
-    const int accumulate = q[k]->accumulate;
-    float* d = G3->s32[0];
-    const dim3 grd = grid3(sd, kBlk);
-    auto go = [&](auto diff, auto band) {
-      diff<<<grd, kBlk, 0, g->stream>>>(gh, gl, ss, d, sd, off, t.M);
-      band<<<grd, kBlk, 0, g->stream>>>(d, R, sd, off, t.M, t.d_whi, t.d_wlo, t.K, t.B, t.all_explicit, sign, accumulate);
-    };
-    if (axis == 0) go(k_diff3d32<0>, k_band3d32<0>);
-    else if (axis == 1) go(k_diff3d32<1>, k_band3d32<1>);
-    else go(k_diff3d32<2>, k_band3d32<2>);
-    // G hi + lo in, d out; d in, R out (read too when accumulating)
-    prof_mark(g, KK_BAND3D32,
-              4.0 * (2.0 * (double)ss.size() + (double)sd.size()) + 4.0 * (double)sd.size() * (accumulate ? 3.0 : 2.0));
+    TermArgs& a = A.t[k];
+    a.gh = G3->gh[q[k]->cs % 3];
+    a.gl = G3->gl[q[k]->cs % 3];
+    a.R = G3->s32[q[k]->cd % 3];
+    a.ss = G3->sh[q[k]->cs];
+    a.sd = G3->sh[q[k]->cd];
+    a.sign = q[k]->sign;
+    a.accumulate = q[k]->accumulate;
+    nx = std::max(nx, a.sd.n[0]);
+    ny = std::max(ny, a.sd.n[1]);
+    A.nz = std::max(A.nz, a.sd.n[2]);
+    // G hi + lo in, R out (read too when accumulating)
+    bytes += 4.0 * (2.0 * (double)a.ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)a.sd.size());
   }
-  return 4;
+  launch_pdl(k_short3d32, dim3((nx + 31) / 32, (ny + 3) / 4, 2 * A.nz), dim3(32, 4), 0, g->stream, A, axis, off, t.M,
+             (const float*)t.d_whi, (const float*)t.d_wlo, t.K, t.B, (int)t.all_explicit);
+  prof_mark(g, KK_TERM3D32, bytes);
+  return 1;
 }
 
 // Transform solve (tensor cores) of component c followed by ts_sweeps Richardson sweeps with the
@@ -1598,7 +1260,7 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
 void solve3d32_ts(ms_grid* g, int c, float d_hi, float d_lo, float omega, float s_hi, float s_lo, int* nl) {
   Grid3D* G3 = g->g3;
   const Shape3& s = G3->sh[c];
-  const float* b = G3->s32[1 + c % 3];
+  const float* b = G3->s32[c % 3];
   float* buf[2] = {G3->gh[c % 3], G3->gl[c % 3]};  // the filter's planes are free by now
   *nl += ts_solve(*G3->ts, s, b, buf[0], 6.0f * (float)(g->c1 * g->h * g->h), g->stream, g);
   const dim3 grd = sweep_grid3(s), blk(SWX, SWT, 1);
@@ -1617,7 +1279,7 @@ void solve3d32_ts(ms_grid* g, int c, float d_hi, float d_lo, float omega, float 
   *nl += R;
 }
 
-// The solves and updates of the components c0 .. c0 + 2 from s32[1..3]; the filter buffers, free by now,
+// The solves and updates of the components c0 .. c0 + 2 from s32; the filter buffers, free by now,
 // hold the iterates.
 void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
   Grid3D* G3 = g->g3;
@@ -1634,7 +1296,7 @@ void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
   for (int c = 0; c < 3; ++c) {
     const Shape3& s = G3->sh[c0 + c];
     A.s[c] = s;
-    A.b[c] = G3->s32[1 + c];
+    A.b[c] = G3->s32[c];
     A.hi[c] = G3->hi[c0 + c];
     A.lo[c] = G3->lo[c0 + c];
     int u[3];
@@ -1687,7 +1349,7 @@ ms_status step3d32(ms_grid* g) {
     nl += terms3d32(g, 0, Term3{cs + 2, c0 + 1, -sign, 1}, Term3{cs + 1, c0 + 2, sign, 1});
     if (g->src3)
       for (int c = 0; c < 3; ++c) {
-        src3_add(g, c0 + c, G3->s32[1 + c]);
+        src3_add(g, c0 + c, G3->s32[c]);
         prof_mark(g, KK_SRC, 8.0 * (double)G3->sh[c0 + c].size());
         nl += 1;
       }
@@ -1727,32 +1389,6 @@ double max_amp2_3d(double r) {
         if (v > worst) worst = v;
       }
   return worst;
-}
-
-// Interior row of A^{-1} in closed form (long double), split hi + lo, and the constants of its
-// recurrences, into constant memory.
-int upload_band_row() {
-  const long double rho = -11.0L + std::sqrt(120.0L);
-  float w[2 * KB3 + 2], wl[3];
-  for (int t = 0; t < 2 * KB3 + 2; ++t) {
-    const int dd = t - KB3;
-    long double v = 24.0L * (-rho) / (1.0L - rho * rho);
-    for (int q = 0; q < (dd < 0 ? -dd : dd); ++q) v *= rho;
-    w[t] = (float)v;
-    if (dd >= -1 && dd <= 1) wl[dd + 1] = (float)(v - (long double)w[t]);
-  }
-  if (cudaMemcpyToSymbol(c_w3, w, sizeof w) != cudaSuccess || cudaMemcpyToSymbol(c_wl3, wl, sizeof wl) != cudaSuccess)
-    return -1;
-  const float rho_f = (float)rho;
-  const long double one_m = 1.0L - (long double)rho_f;
-  const long double scale = one_m / (1.0L + (long double)rho_f);
-  float rec[4];
-  rec[0] = rho_f;
-  rec[1] = (float)(1.0L / one_m);
-  rec[2] = (float)scale;
-  rec[3] = (float)(scale - (long double)rec[2]);
-  if (cudaMemcpyToSymbol(c_rec3, rec, sizeof rec) != cudaSuccess) return -1;
-  return 0;
 }
 
 // The polynomial of the FP64 solves: 6 h^2 P1 = D - T, T in [-8, 24] (k_rec64.cu).
@@ -1995,14 +1631,13 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
                          cudaMemcpy(t.d_wlo, wlo.data(), wlo.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess))
         s = fail3(MS_ECUDA, "copy of FP32 Pade tables failed");
     }
-    if (s == MS_OK && upload_band_row() != 0) s = fail3(MS_ECUDA, "cannot upload the interior band row");
     for (int kind = 0; kind < 2; ++kind) line_ends(d->closure, kind, false, &g->walk.ends[kind]);
     // the solve polynomial to 1e-10 (below the FP32 rounding noise, which is not coherent)
     if (s == MS_OK && !cheb_coefs(6.0 * g->c1 * g->h * g->h + 24.0, 8.0, 16.0, 1e-10, &g->walk.cheb))
       s = fail3(MS_ENOTCONV, "the FP32 solve polynomial needs too high a degree");
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->hi[c], G3->sh[c].size());
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->lo[c], G3->sh[c].size());
-    for (int k = 0; k < 4 && s == MS_OK; ++k) s = alloc3(&G3->s32[k], G3->nmax);
+    for (int k = 0; k < 3 && s == MS_OK; ++k) s = alloc3(&G3->s32[k], G3->nmax);
     for (int k = 0; k < 3 && s == MS_OK; ++k) s = alloc3(&G3->gh[k], G3->nmax);
     for (int k = 0; k < 3 && s == MS_OK; ++k) s = alloc3(&G3->gl[k], G3->nmax);
     for (int k = 0; k < 2 && s == MS_OK; ++k) s = alloc3(&G3->s64[k], G3->nmax);
@@ -2022,7 +1657,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
   }
   for (int k = 0; k < 9; ++k)
     if (G3->s64[k]) cudaMemsetAsync(G3->s64[k], 0, G3->nmax * sizeof(double), g->stream);
-  for (int k = 0; k < 4; ++k)
+  for (int k = 0; k < 3; ++k)
     if (G3->s32[k]) cudaMemsetAsync(G3->s32[k], 0, G3->nmax * sizeof(float), g->stream);
   cudaError_t e = cudaStreamSynchronize(g->stream);
   if (e != cudaSuccess) return cleanup(fail3(MS_ECUDA, std::string("create: ") + cudaGetErrorString(e)));
@@ -2101,7 +1736,7 @@ void destroy_grid3d(ms_grid* g) {
     dev_free(G3->dview[c]);
   }
   for (int k = 0; k < 9; ++k) dev_free(G3->s64[k]);
-  for (int k = 0; k < 4; ++k) dev_free(G3->s32[k]);
+  for (int k = 0; k < 3; ++k) dev_free(G3->s32[k]);
   for (int k = 0; k < 3; ++k) {
     dev_free(G3->gh[k]);
     dev_free(G3->gl[k]);

@@ -183,26 +183,43 @@ void launch_filter64(const double* u, double* G, const Shape& s, double beta, cu
   launch_pdl(k_filter64, grid2(s.nx, s.ny, blk), blk, 0, st, A, beta - 4.0 / 12.0);
 }
 
+static LineArgs line_args64(int axis, const double* in, double* out, int n_lines, int in_ld, int out_len, int out_ld,
+                            int out_off, int line_lo, int line_hi, const PadeTable& t, double scale, int accumulate) {
+  LineArgs a{};
+  a.in = in;
+  a.out = out;
+  a.M = t.M;
+  a.out_len = out_len;
+  a.out_off = out_off;
+  a.n0 = n_lines;
+  a.n1 = 1;
+  a.lo = line_lo;
+  a.hi = line_hi;
+  a.in_sa = axis == 0 ? 1 : in_ld;
+  a.in_s0 = axis == 0 ? in_ld : 1;
+  a.out_sa = axis == 0 ? 1 : out_ld;
+  a.out_s0 = axis == 0 ? out_ld : 1;
+  a.scale = scale;
+  a.accumulate = accumulate;
+  return a;
+}
+
+bool launch_pade64_xy(const double* in_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
+                      double* out_y, int out_ld_y, double scale_y, int n_lines, int in_ld, int out_len, int out_off,
+                      int line_lo, int line_hi, const PadeTable& t, cudaStream_t st) {
+  return t.M >= kRecMinLine &&
+         launch_line64_pair(
+             line_args64(0, in_x, out_x, n_lines, in_ld, out_len, out_ld_x, out_off, line_lo, line_hi, t, scale_x, 0),
+             line_args64(1, in_y, out_y, n_lines, in_ld, out_len, out_ld_y, out_off, line_lo, line_hi, t, scale_y, 0),
+             t.ends, t.transposed, st);
+}
+
 void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_ld, int out_len, int out_ld,
                    int out_off, int line_lo, int line_hi, const PadeTable& t, double scale, int accumulate,
                    cudaStream_t st) {
   if (t.M >= kRecMinLine) {
-    LineArgs a{};
-    a.in = in;
-    a.out = out;
-    a.M = t.M;
-    a.out_len = out_len;
-    a.out_off = out_off;
-    a.n0 = n_lines;
-    a.n1 = 1;
-    a.lo = line_lo;
-    a.hi = line_hi;
-    a.in_sa = axis == 0 ? 1 : in_ld;
-    a.in_s0 = axis == 0 ? in_ld : 1;
-    a.out_sa = axis == 0 ? 1 : out_ld;
-    a.out_s0 = axis == 0 ? out_ld : 1;
-    a.scale = scale;
-    a.accumulate = accumulate;
+    const LineArgs a = line_args64(axis, in, out, n_lines, in_ld, out_len, out_ld, out_off, line_lo, line_hi, t, scale,
+                                   accumulate);
     launch_line64(&a, 1, t.ends, t.transposed, st);
     return;
   }

@@ -29,6 +29,11 @@ void launch_filter64x2(const double* u0, double* G0, const Shape& s0, const doub
 void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_ld, int out_len, int out_ld,
                    int out_off, int line_lo, int line_hi, const PadeTable& t, double scale, int accumulate,
                    cudaStream_t st);
+// Derivatives along x and along y into two planes, neither accumulated, in one launch where the lines are cut
+// into short segments; false (nothing launched) elsewhere.
+bool launch_pade64_xy(const double* in_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
+                      double* out_y, int out_ld_y, double scale_y, int n_lines, int in_ld, int out_len, int out_off,
+                      int line_lo, int line_hi, const PadeTable& t, cudaStream_t st);
 void launch_p1_sweep64(const double* b, const double* xin, double* xout, const Shape& s, double c1h2, double omega,
                        double bscale, int first, cudaStream_t st);
 void launch_p1_apply64(const double* x, double* out, const Shape& s, double c1h2, double out_scale, cudaStream_t st);

@@ -183,16 +183,10 @@ constexpr double kOneMinusRhoSq = 1.093172397520265540654504;  // (1 - rho)^2 = 
 // Lines across a strided axis, lanes across the contiguous one: a thread walks its segment of a line,
 // every load coalesced.  The last segment of a line is aligned to its end and writes all its rows (the
 // one before it stops there), so both ends and the rows they correct sit at fixed places of a segment.
-template <int L, int LS, bool TRANS>
-__global__ void __launch_bounds__(32 * LS) k_line_walk64(LineBatch b) {
-  pdl_wait();
-  const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
-  const LineArgs& a = b.a[which];
-  if (l1 >= a.n1) return;
-  const int l0 = blockIdx.x * 32 + threadIdx.x;
+template <int L, bool TRANS>
+__device__ __forceinline__ void line_walk64(const LineArgs& a, const LineEnds& e, int l0, int l1, int seg) {
   const int R = TRANS ? a.M + 1 : a.M;
   const int nseg = (R + L - 1) / L;
-  const int seg = blockIdx.y * LS + threadIdx.y;
   if (l0 >= a.n0 || seg >= nseg) return;
   double* o = a.out + l0 * a.out_s0 + l1 * a.out_s1;
   const bool live = l0 >= a.lo && l0 < a.hi;
@@ -216,7 +210,7 @@ __global__ void __launch_bounds__(32 * LS) k_line_walk64(LineBatch b) {
   const int n_in = TRANS ? a.M : a.M + 1;
   double ys[L];
   line_segment64<L, TRANS>(
-      s, a.M, b.e, [&](int m) { return (m >= 0 && m < n_in) ? ip[m * (ptrdiff_t)a.in_sa] : 0.0; },
+      s, a.M, e, [&](int m) { return (m >= 0 && m < n_in) ? ip[m * (ptrdiff_t)a.in_sa] : 0.0; },
       [&](int t, double v) { ys[t] = v; });
 #pragma unroll
   for (int t0 = 0; t0 < L; t0 += 8) {  // eight loads in flight
@@ -232,26 +226,33 @@ __global__ void __launch_bounds__(32 * LS) k_line_walk64(LineBatch b) {
   }
 }
 
+template <int L, int LS, bool TRANS>
+__global__ void __launch_bounds__(32 * LS) k_line_walk64(LineBatch b) {
+  pdl_wait();
+  const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
+  if (l1 >= b.a[which].n1) return;
+  line_walk64<L, TRANS>(b.a[which], b.e, blockIdx.x * 32 + threadIdx.x, l1, blockIdx.y * LS + threadIdx.y);
+}
+
 // Lines along the contiguous axis: a block takes LS segments of 32 lines.  Whole warps read the lines
 // into shared memory (odd pitch: lanes across the lines are conflict-free), a thread takes one
 // segment of one line, and the results go back through shared memory.
-template <int L, int LS, bool TRANS>
-__global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
-  constexpr int OUTS = LS * L, PW = OUTS + 2 * kRecWarm + 3;  // odd
+template <int L, int LS>
+struct RowsTile {
+  static constexpr int OUTS = LS * L, PW = OUTS + 2 * kRecWarm + 3;  // odd
   static_assert(PW % 2 == 1, "odd row pitch");
-  __shared__ double sm[32 * PW];
-  pdl_wait();
-  const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
-  const LineArgs& a = b.a[which];
-  if (l1 >= a.n1) return;
+};
+template <int L, int LS, bool TRANS>
+__device__ __forceinline__ void line_rows64(const LineArgs& a, const LineEnds& e, int bx, int by, int l1, double* sm) {
+  constexpr int OUTS = RowsTile<L, LS>::OUTS, PW = RowsTile<L, LS>::PW;
   const int lane = threadIdx.x, warp = threadIdx.y;
   const int R = TRANS ? a.M + 1 : a.M;
   const int nseg = (R + L - 1) / L;
-  const int t0 = blockIdx.x * OUTS;
+  const int t0 = bx * OUTS;
   const int b0 = min(t0, R - L);           // first output of the tile
   const int base = b0 - kRecWarm - 1;      // input index of column 0
   const int n_in = TRANS ? a.M : a.M + 1;
-  const int la = blockIdx.y * 32;
+  const int la = by * 32;
   const double* in = a.in + l1 * a.in_s1;
   double* out = a.out + l1 * a.out_s1;
 #pragma unroll 4
@@ -266,13 +267,13 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
     }
   }
   __syncthreads();
-  const int seg = blockIdx.x * LS + warp;
+  const int seg = bx * LS + warp;
   const bool lastseg = seg == nseg - 1, has = warp < LS && seg < nseg;
   const int s = lastseg ? R - L : seg * L;
   double ys[L];
   if (has) {
     const double* row = sm + lane * PW - base;  // row[m]: input m of the line
-    line_segment64<L, TRANS>(s, a.M, b.e, [&](int m) { return row[m]; },
+    line_segment64<L, TRANS>(s, a.M, e, [&](int m) { return row[m]; },
                              [&](int t, double v) { ys[t] = v; });
   }
   __syncthreads();
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
       if (t < cnt) sm[lane * PW + s - b0 + t] = ys[t];
   }
   __syncthreads();
-  const bool last_tile = (blockIdx.x + 1) * LS >= nseg;
+  const bool last_tile = (bx + 1) * LS >= nseg;
   const double scale = a.scale * kOneMinusRhoSq;
   const int nout = (last_tile ? R : min(t0 + OUTS, R - L)) - b0;
   constexpr int NC = (OUTS + 31) / 32;  // nout <= OUTS: the last tile, aligned to the end, starts earlier
@@ -323,7 +324,34 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
   }
 }
 
+template <int L, int LS, bool TRANS>
+__global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
+  __shared__ double sm[32 * RowsTile<L, LS>::PW];
+  pdl_wait();
+  const int which = blockIdx.z / b.n1, l1 = blockIdx.z - which * b.n1;
+  if (l1 >= b.a[which].n1) return;
+  line_rows64<L, LS, TRANS>(b.a[which], b.e, blockIdx.x, blockIdx.y, l1, sm);
+}
+
+// One derivative along each axis (a[0] along the contiguous one), independent of one another, in one
+// launch: on small grids a launch takes the latency of one chain of recurrences whatever it holds.
+template <int L, bool TRANS>
+__global__ void __launch_bounds__(32 * LW) k_line_pair64(LineBatch b, int rows_x, int rows_n, int walk_x) {
+  __shared__ double sm[32 * RowsTile<L, 1>::PW];
+  pdl_wait();
+  const int q = blockIdx.x - rows_n;
+  if (q < 0) line_rows64<L, 1, TRANS>(b.a[0], b.e, blockIdx.x % rows_x, blockIdx.x / rows_x, 0, sm);
+  else if (threadIdx.y == 0) line_walk64<L, TRANS>(b.a[1], b.e, (q % walk_x) * 32 + threadIdx.x, 0, q / walk_x);
+}
+
 }  // namespace
+
+// Segments of 32 rows do 3.3 FMAs per output, of 16 rows 4.6; the shorter ones win while the longer
+// ones would leave FP64 pipes (4 per SM) without a warp.  A block takes one short segment: warps of one
+// SM share its FP64 rate (64^2: 64.0 us per step with four, 56.7 us with one; 321^2: 110.4 and 102.1 us).
+static bool lines64_short(int n0, int R, int n1) {
+  return R < 64 || (double)((n0 + 31) / 32) * ((R + 31) / 32) * n1 < 600.0;
+}
 
 void launch_line64(const LineArgs* args, int count, const LineEnds& e, bool transposed, cudaStream_t st) {
   LineBatch b;
@@ -337,11 +365,7 @@ void launch_line64(const LineArgs* args, int count, const LineEnds& e, bool tran
     n0 = b.a[k].n0 > n0 ? b.a[k].n0 : n0;
   }
   const bool rows = args[0].in_sa == 1;
-  // Segments of 32 rows do 3.3 FMAs per output, of 16 rows 4.6; the shorter ones win while the longer
-  // ones would leave FP64 pipes (4 per SM) without a warp.  A block takes one short segment: warps of one
-  // SM share its FP64 rate (64^2: 64.0 us per step with four, 56.7 us with one; 321^2: 110.4 and 102.1 us).
-  const double warps32 = (double)((n0 + 31) / 32) * ((R + 31) / 32) * b.n1 * count;
-  const bool l32 = R >= 64 && warps32 >= 600.0;
+  const bool l32 = !lines64_short(n0, R, b.n1 * count);
   const int L = l32 ? 32 : 16, LS = l32 ? 4 : kShortLS;
   const int nseg = (R + L - 1) / L;
   const dim3 blk(32, rows ? LW : LS);
@@ -357,6 +381,20 @@ void launch_line64(const LineArgs* args, int count, const LineEnds& e, bool tran
   if (rows) MS_LINE(k_line_rows64);
   else MS_LINE(k_line_walk64);
 #undef MS_LINE
+}
+
+bool launch_line64_pair(const LineArgs& x, const LineArgs& y, const LineEnds& e, bool transposed, cudaStream_t st) {
+  const int R = transposed ? x.M + 1 : x.M;
+  if (!lines64_short(x.n0, R, 1)) return false;
+  LineBatch b;
+  b.e = e;
+  b.n1 = 1;
+  for (int k = 0; k < kLineBatch; ++k) b.a[k] = k == 1 ? y : x;
+  const int nseg = (R + 15) / 16, nl = (x.n0 + 31) / 32, nw = (y.n0 + 31) / 32;
+  const dim3 grd(nseg * (nl + nw)), blk(32, LW);
+  if (transposed) launch_pdl(k_line_pair64<16, true>, grd, blk, 0, st, b, nseg, nseg * nl, nw);
+  else launch_pdl(k_line_pair64<16, false>, grd, blk, 0, st, b, nseg, nseg * nl, nw);
+  return true;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -36,6 +36,9 @@ struct LineArgs {
 // contiguous axis (in_sa == 1) or all across it.
 constexpr int kLineBatch = 3;
 void launch_line64(const LineArgs* a, int count, const LineEnds& e, bool transposed, cudaStream_t st);
+// Derivatives along x (contiguous) and y of one half-step that do not depend on one another, with equal M:
+// one launch where the lines are cut into short segments; false (nothing launched) otherwise.
+bool launch_line64_pair(const LineArgs& x, const LineArgs& y, const LineEnds& e, bool transposed, cudaStream_t st);
 
 // P1 x = b for one or two 2D fields in one launch; upd (if not NULL) gains upd_scale x, out (if not
 // NULL) receives x (0 on the walls).  b may not be out.
