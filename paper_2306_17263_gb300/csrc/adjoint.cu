@@ -163,7 +163,8 @@ void adjoint_step64(ms_grid* g) {
   // interior nodes of u_E; l_H += h_tau F_H v
   p1_solve64(g, EZ, lE, e, nullptr, 0.0, &nl);
   const PadeTable& th = g->padeT[HALF_TO_NODE];
-  if (!launch_pade64_xy(e + 1, y, N, s_he, e + (N + 1), x, N + 1, -s_he, N + 1, N + 1, N, 0, 1, N, th, g->stream)) {
+  if (!launch_pade64_xy(e + 1, N + 1, y, N, s_he, e + (N + 1), N + 1, x, N + 1, -s_he, N + 1, N, 0, 1, N, th,
+                        g->stream)) {
     launch_pade64(0, e + 1, y, N + 1, N + 1, N, N, 0, 1, N, th, s_he, 0, g->stream);
     launch_pade64(1, e + (N + 1), x, N + 1, N + 1, N, N + 1, 0, 1, N, th, -s_he, 0, g->stream);
   }

@@ -62,10 +62,18 @@ ms_status dalloc(T** p, size_t n) {
 // ---------------------------------------------------------------------------------------
 // FP64 operator building blocks on arbitrary device arrays.
 
-// R = kappa^2 Z (delta_x G_y - delta_y G_x) on E_z (Step 1, third row of curl_h).
-void curl_he64(ms_grid* g, const double* Gx, const double* Gy, double* R, int* nl) {
+// R = kappa^2 Z (delta_x G_y - delta_y G_x) on E_z (Step 1, third row of curl_h).  With R2, on grids whose
+// solve can add two right-hand sides, the second term goes there, both in one launch, and true is returned.
+bool curl_he64(ms_grid* g, const double* Gx, const double* Gy, double* R, int* nl, double* R2 = nullptr) {
   const int N = g->N;
   const double s = g->kappa2 * g->Z / g->h;
+  if (R2 && cheb2d64_tiles((long)g->sh[EZ].size()) &&
+      launch_pade64_xy(Gy, N, R, N + 1, s, Gx, N + 1, R2, N + 1, -s, N + 1, N + 1, 1, 1, N, g->pade[HALF_TO_NODE],
+                       g->stream)) {
+    prof_mark(g, KK_PADE64, 16.0 * ((double)(N - 1) * N + (double)(N + 1) * (N + 1)));
+    *nl += 1;
+    return true;
+  }
   // delta_x G_y: rows j = 1..N-1 of H_y (N half-node values) -> E_z columns 1..N-1
   launch_pade64(0, Gy, R, N + 1, N, N + 1, N + 1, 1, 1, N, g->pade[HALF_TO_NODE], s, 0, g->stream);
   prof_mark(g, KK_PADE64, 8.0 * ((double)(N - 1) * N + (double)(N + 1) * (N + 1)));
@@ -73,6 +81,7 @@ void curl_he64(ms_grid* g, const double* Gx, const double* Gy, double* R, int* n
   launch_pade64(1, Gx, R, N + 1, N + 1, N + 1, N + 1, 1, 1, N, g->pade[HALF_TO_NODE], -s, 1, g->stream);
   prof_mark(g, KK_PADE64, 8.0 * ((double)(N - 1) * N + 2.0 * (N + 1) * (N + 1)));
   *nl += 2;
+  return false;
 }
 
 // (R_x, R_y) = (kappa^2/Z) (-delta_y G_E, delta_x G_E) (Step 2).
@@ -83,7 +92,7 @@ void curl_eh64(ms_grid* g, const double* GE, double* Rx, double* Ry, int* nl) {
   const double bytes = 8.0 * ((double)(N - 1) * (N + 1) + (double)N * (N + 1));
   // delta_y G_E: columns i = 1..N-1 of E_z (N+1 node values) -> H_x rows 0..N-1
   // delta_x G_E: rows j = 1..N-1 of E_z -> H_y columns 0..N-1
-  if (launch_pade64_xy(GE, Ry, N, s, GE, Rx, N + 1, -s, N + 1, N + 1, N, 0, 1, N, t, g->stream)) {
+  if (launch_pade64_xy(GE, N + 1, Ry, N, s, GE, N + 1, Rx, N + 1, -s, N + 1, N, 0, 1, N, t, g->stream)) {
     prof_mark(g, KK_PADE64, 2.0 * bytes);
     *nl += 1;
     return;
@@ -98,13 +107,14 @@ void curl_eh64(ms_grid* g, const double* GE, double* Rx, double* Ry, int* nl) {
 }  // namespace
 
 namespace ms {
-void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl) {
+void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl,
+                const double* b2) {
   const Shape& s = g->sh[f];
   if (b == out) {  // a block's halo would read points that another block has overwritten
     cudaMemcpyAsync(g->s64[5], b, s.size() * sizeof(double), cudaMemcpyDeviceToDevice, g->stream);
     b = g->s64[5];
   }
-  const Cheb2dField F{b, out, upd, s};
+  const Cheb2dField F{b, out, upd, s, b2};
   double* const buf[1][2] = {{g->s64[3], g->s64[4]}};
   launch_cheb2d64(&F, 1, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
   prof_mark(g, KK_P1SWEEP64, 8.0 * (double)s.size() * (1.0 + (out ? 1.0 : 0.0) + (upd ? 2.0 : 0.0)));
@@ -162,8 +172,8 @@ ms_status step64_tracked(ms_grid* g) {
   launch_filter64x2(hx, Gx, g->sh[HX], hy, Gy, g->sh[HY], g->beta, g->stream);
   prof_mark(g, KK_FILTER64, 32.0 * (double)g->sh[HX].size());
   nl += 1;
-  curl_he64(g, Gx, Gy, R, &nl);
-  p1_solve64(g, EZ, R, g->s64[5], ez, g->ht, &nl);  // E* in s64[5], E += h_tau E*
+  double* const R2 = curl_he64(g, Gx, Gy, R, &nl, g->s64[3]) ? g->s64[3] : nullptr;
+  p1_solve64(g, EZ, R, g->s64[5], ez, g->ht, &nl, R2);  // E* in s64[5], E += h_tau E*
   curl_he64(g, hx, hy, g->s64[0], &nl);              // kappa^2 Z curl_h H (unfiltered)
   double* GE = g->s64[1];
   launch_de_update64(g->de64, g->s64[5], g->s64[0], ez, GE, g->N, g->ht, g->kappa2, g->beta, g->h, g->stream);
@@ -212,7 +222,7 @@ ms_status step64(ms_grid* g) {
     prof_mark(g, KK_SRC, 8.0 * 8.0 * g->N);
     nl += 1;
   }
-  curl_he64(g, Gx, Gy, R, &nl);
+  double* const R2 = curl_he64(g, Gx, Gy, R, &nl, g->s64[3]) ? g->s64[3] : nullptr;
   if (g->nsrc) {
     launch_src_time(g, 1.0, 1.0);
     prof_mark(g, KK_SRC, 0.0);
@@ -220,7 +230,7 @@ ms_status step64(ms_grid* g) {
     prof_mark(g, KK_SRC, 16.0 * (double)g->sh[EZ].size());
     nl += 2;
   }
-  p1_solve64(g, EZ, R, nullptr, ez, g->ht, &nl);  // E += h_tau E*
+  p1_solve64(g, EZ, R, nullptr, ez, g->ht, &nl, R2);  // E += h_tau E*
   // Step 2 on E^{n+1}
   h_increment64(g, ez, nullptr, nullptr, hx, hy, &nl, true);
   if (g->nsrc) {

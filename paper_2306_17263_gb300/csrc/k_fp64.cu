@@ -204,13 +204,13 @@ static LineArgs line_args64(int axis, const double* in, double* out, int n_lines
   return a;
 }
 
-bool launch_pade64_xy(const double* in_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
-                      double* out_y, int out_ld_y, double scale_y, int n_lines, int in_ld, int out_len, int out_off,
+bool launch_pade64_xy(const double* in_x, int in_ld_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
+                      int in_ld_y, double* out_y, int out_ld_y, double scale_y, int n_lines, int out_len, int out_off,
                       int line_lo, int line_hi, const PadeTable& t, cudaStream_t st) {
   return t.M >= kRecMinLine &&
          launch_line64_pair(
-             line_args64(0, in_x, out_x, n_lines, in_ld, out_len, out_ld_x, out_off, line_lo, line_hi, t, scale_x, 0),
-             line_args64(1, in_y, out_y, n_lines, in_ld, out_len, out_ld_y, out_off, line_lo, line_hi, t, scale_y, 0),
+             line_args64(0, in_x, out_x, n_lines, in_ld_x, out_len, out_ld_x, out_off, line_lo, line_hi, t, scale_x, 0),
+             line_args64(1, in_y, out_y, n_lines, in_ld_y, out_len, out_ld_y, out_off, line_lo, line_hi, t, scale_y, 0),
              t.ends, t.transposed, st);
 }
 

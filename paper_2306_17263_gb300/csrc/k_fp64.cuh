@@ -31,8 +31,8 @@ void launch_pade64(int axis, const double* in, double* out, int n_lines, int in_
                    cudaStream_t st);
 // Derivatives along x and along y into two planes, neither accumulated, in one launch where the lines are cut
 // into short segments; false (nothing launched) elsewhere.
-bool launch_pade64_xy(const double* in_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
-                      double* out_y, int out_ld_y, double scale_y, int n_lines, int in_ld, int out_len, int out_off,
+bool launch_pade64_xy(const double* in_x, int in_ld_x, double* out_x, int out_ld_x, double scale_x, const double* in_y,
+                      int in_ld_y, double* out_y, int out_ld_y, double scale_y, int n_lines, int out_len, int out_off,
                       int line_lo, int line_hi, const PadeTable& t, cudaStream_t st);
 void launch_p1_sweep64(const double* b, const double* xin, double* xout, const Shape& s, double c1h2, double omega,
                        double bscale, int first, cudaStream_t st);
@@ -80,7 +80,9 @@ void launch_nc_h64(const double* ez, double* hx, double* hy, int N, double c_h, 
 // x = P1^{-1} b for field f (k_rec64.cu): writes `out` (if not nullptr; it may be b, then s64[5] is
 // scratch) and, when upd != nullptr, adds upd_scale * x to upd; work planes s64[3], s64[4].  The second
 // form solves both H fields with the work planes given (capi.cu).
-void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl);
+// b2, if any, is added to b (where cheb2d64_tiles holds for the field).
+void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, double upd_scale, int* nl,
+                const double* b2 = nullptr);
 void p1_solve64_h(ms_grid* g, const double* bx, const double* by, double* outx, double* outy, double* updx, double* updy,
                   double upd_scale, double* const (*buf)[2], int* nl);
 // Reverse pass (adjoint.cu): releases the transposed tables, adjoint planes and graphs.

@@ -334,7 +334,8 @@ __global__ void __launch_bounds__(32 * LW) k_line_rows64(LineBatch b) {
 }
 
 // One derivative along each axis (a[0] along the contiguous one), independent of one another, in one
-// launch: on small grids a launch takes the latency of one chain of recurrences whatever it holds.
+// launch: on small grids a launch takes the latency of one chain of recurrences whatever it holds.  With both
+// half-steps' pairs joined, 64^2 went 58.3 -> 39.9 us per step, 321^2 101 -> 83 us.
 template <int L, bool TRANS>
 __global__ void __launch_bounds__(32 * LW) k_line_pair64(LineBatch b, int rows_x, int rows_n, int walk_x) {
   __shared__ double sm[32 * RowsTile<L, 1>::PW];
@@ -435,7 +436,11 @@ __global__ void __launch_bounds__(C2T) k_cheb2d64(Cheb2dArgs A) {
   for (int t = threadIdx.x; t < W * W; t += C2T) {
     const int r = t / W, c = t - r * W;
     const int gx = gx0 + c, gy = gy0 + r;
-    const double v = unknown(gx, gy) ? F.b[(size_t)gy * nx + gx] : 0.0;
+    double v = 0.0;
+    if (unknown(gx, gy)) {
+      v = F.b[(size_t)gy * nx + gx];
+      if (F.b2) v += F.b2[(size_t)gy * nx + gx];
+    }
     bs[t] = v;
     ys[t] = v;
   }
@@ -546,7 +551,7 @@ void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], cons
   const int nx = f[0].s.nx > f[nf - 1].s.nx ? f[0].s.nx : f[nf - 1].s.nx;
   const int ny = f[0].s.ny > f[nf - 1].s.ny ? f[0].s.ny : f[nf - 1].s.ny;
   const long pts = (long)nx * ny * nf;
-  if (pts > 300000) {
+  if (!cheb2d64_tiles(pts)) {
     // the tiles' halo would cost 1.4 to 1.9 times the operations; a launch per level costs about 1 us
     const dim3 grd((nx + 31) / 32, (ny + 4 * C2R - 1) / (4 * C2R), nf);
     for (int k = p.m - 1; k >= 1; --k) {

@@ -47,7 +47,10 @@ struct Cheb2dField {
   double* out;
   double* upd;
   Shape s;
+  const double* b2 = nullptr;  // with cheb2d64_tiles only: b + b2 is the right-hand side
 };
+// Whether the solve of `pts` points runs all its levels in one launch (k_cheb2d64).
+inline bool cheb2d64_tiles(long pts) { return pts <= 300000; }
 // buf: two work planes per field, all distinct from each other and from b and out.
 void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], const Cheb& p, double bscale,
                      double upd_scale, cudaStream_t st);

@@ -78,3 +78,21 @@ def test_3d_step(n, closure):
         got = g.get_fields()
     for a, b in zip(got, ref):
         assert np.linalg.norm(a - b) <= 1e-12 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n", [31, 32, 33, 64, 546, 547, 764, 800])
+def test_2d_steps_at_launch_limits(n):
+    """Both derivatives of a half-step in one launch, and the two terms of Step 1 summed by the solve, up to
+    the sizes where the solve's levels (547) and then the derivatives (about 780) take launches of their own."""
+    r, steps = 0.5, 2
+    o = oracle.Oracle2D(n, r)
+    init = workloads.random_fields(n, seed=n)
+    ref = [a.copy() for a in init]
+    o.run(*ref, steps)
+    with pkg.Grid(n, r) as g:
+        g.set_fields(*init)
+        g.run(steps)
+        got = g.get_fields()
+    for a, b in zip(got, ref):
+        assert np.linalg.norm(a - b) <= 1e-12 * np.linalg.norm(b)
+        assert np.all(a[b == 0.0] == 0.0)
