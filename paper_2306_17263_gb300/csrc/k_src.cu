@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "k_fp64.cuh"
+#include "k_pdl.cuh"
 
 namespace ms {
 namespace {
@@ -52,6 +53,7 @@ struct SrcFac {
 // t_H = (n + 1) h_tau; the float copies scaled by scale_e and scale_h.
 __global__ void k_src_time(const SrcDev* __restrict__ s, int nsrc, const long* __restrict__ d_step, double ht,
                            double scale_e, double scale_h, SrcFac* __restrict__ fac) {
+  pdl_wait();
   const int q = threadIdx.x;
   if (q >= nsrc) return;
   const double te = ((double)*d_step + 0.5) * ht, th = ((double)*d_step + 1.0) * ht;
@@ -87,10 +89,11 @@ __host__ __device__ inline WallView wall_view(const double* wd, const float* wr,
 }
 
 // Point kernels: a block is 32 columns by kSrcBy rows, and each thread takes kSrcRows rows kSrcBy
-// apart, all loads of a thread issued before its first update (one point per thread left the kernel
-// waiting on one memory round trip per wave).  Per point the arithmetic is that of the plain sum.
+// apart, all loads of a thread issued before its first update.  Two rows leave enough blocks for the last
+// wave and small grids (a driven FP32 step in replay: 43.9 us at 1024^2 and 111.5 at 2048^2, with eight rows
+// 47.0 and 126.8).  Per point the arithmetic is that of the plain sum.
 constexpr int kSrcBy = 8;
-constexpr int kSrcRows = 8;
+constexpr int kSrcRows = 2;
 
 // R += sum_q e_q X_q(i) Y_q(j) at the interior E_z nodes.  FP32 with wall data: plus, in the units of
 // R scaled by cE / (kappa^2 Z / h), the Pade responses to the filter's ghost terms of Step 1,
@@ -100,6 +103,7 @@ template <typename T>
 __global__ void __launch_bounds__(32 * kSrcBy) k_src_e(T* __restrict__ R, int ld, int N, int nsrc, const double* __restrict__ tab,
                                                        const float* __restrict__ tab32, const SrcFac* __restrict__ fac,
                                                        WallView wv, float cE) {
+  pdl_wait();
   const int i = blockIdx.x * 32 + threadIdx.x;
   const int j0 = blockIdx.y * (kSrcBy * kSrcRows) + threadIdx.y;
   if (i < 1 || i >= N) return;
@@ -163,6 +167,7 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __
                                                        int N, int nsrc,
                                                        const double* __restrict__ tab, const float* __restrict__ tab32,
                                                        const SrcFac* __restrict__ fac, WallView wv, float cH, double sP) {
+  pdl_wait();
   const int i = blockIdx.x * 32 + threadIdx.x;
   const int j0 = blockIdx.y * (kSrcBy * kSrcRows) + threadIdx.y;
   if (i > N) return;
@@ -230,7 +235,10 @@ __global__ void __launch_bounds__(32 * kSrcBy) k_src_h(T* __restrict__ Rx, T* __
   }
 }
 
-__global__ void k_tick(long* d_step) { *d_step += 1; }
+__global__ void k_tick(long* d_step) {
+  pdl_wait();
+  *d_step += 1;
+}
 
 // Table layout per source (4 (N + 1) doubles): X at nodes i = 0..N, Y at nodes j = 0..N,
 // X'/(pi m) at half-nodes i = 0..N-1, Y'/(pi n) at half-nodes j = 0..N-1.
@@ -402,33 +410,33 @@ int build_sources(ms_grid* g, const SrcSpec* src, int nsrc, std::vector<unsigned
 size_t src_factor_bytes() { return sizeof(SrcFac); }
 
 void launch_src_time(ms_grid* g, double scale_e, double scale_h) {
-  k_src_time<<<1, kMaxSrc, 0, g->stream>>>((const SrcDev*)g->d_src, g->nsrc, g->d_step, g->ht, scale_e, scale_h,
-                                           (SrcFac*)g->d_srcfac);
+  launch_pdl(k_src_time, dim3(1), dim3(kMaxSrc), 0, g->stream, (const SrcDev*)g->d_src, g->nsrc, g->d_step, g->ht, scale_e,
+             scale_h, (SrcFac*)g->d_srcfac);
 }
 static dim3 src_grid(int N) { return dim3((N + 1 + 31) / 32, (N + 1 + kSrcBy * kSrcRows - 1) / (kSrcBy * kSrcRows)); }
 
 void launch_src_e64(ms_grid* g, double* R) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
-  k_src_e<double><<<grd, blk, 0, g->stream>>>(R, g->N + 1, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  launch_pdl(k_src_e<double>, grd, blk, 0, g->stream, R, g->N + 1, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                                (const SrcFac*)g->d_srcfac, WallView{}, 0.0f);
 }
 void launch_src_h64(ms_grid* g, double* Rx, double* Ry) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
-  k_src_h<double><<<grd, blk, 0, g->stream>>>(Rx, Ry, g->N + 1, g->N, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  launch_pdl(k_src_h<double>, grd, blk, 0, g->stream, Rx, Ry, g->N + 1, g->N, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                                (const SrcFac*)g->d_srcfac, WallView{}, 0.0f, 0.0);
 }
 void launch_src_e32(ms_grid* g, float* R, int ld, double scale_e) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
   const WallView wv = g->d_walldata ? wall_view(g->d_walldata, g->d_wresp, g->N) : WallView{};
   const float cE = (float)(scale_e * g->kappa2 * g->Z / g->h);
-  k_src_e<float><<<grd, blk, 0, g->stream>>>(R, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  launch_pdl(k_src_e<float>, grd, blk, 0, g->stream, R, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                               (const SrcFac*)g->d_srcfac, wv, cE);
 }
 void launch_src_h32(ms_grid* g, float* Rx, float* Ry, int ld, double scale_h) {
   dim3 blk(32, kSrcBy), grd = src_grid(g->N);
   const WallView wv = g->d_walldata ? wall_view(g->d_walldata, g->d_wresp, g->N) : WallView{};
   const float cH = (float)(scale_h * g->kappa2 / (g->Z * g->h));
-  k_src_h<float><<<grd, blk, 0, g->stream>>>(Rx, Ry, ld, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
+  launch_pdl(k_src_h<float>, grd, blk, 0, g->stream, Rx, Ry, ld, ld, g->N, g->nsrc, g->d_srctab, g->d_srctab32,
                                               (const SrcFac*)g->d_srcfac, wv, cH, scale_h / (g->h * g->h));
 }
 void launch_wall_data(ms_grid* g) {
@@ -455,7 +463,7 @@ void wall_responses(int N, std::vector<float>* wr) {
     }
   }
 }
-void launch_tick(ms_grid* g) { k_tick<<<1, 1, 0, g->stream>>>(g->d_step); }
+void launch_tick(ms_grid* g) { launch_pdl(k_tick, dim3(1), dim3(1), 0, g->stream, g->d_step); }
 
 void launch_wall_hfilter64(ms_grid* g, double* Gx, double* Gy) {
   k_wall_hfilter64<<<(g->N + 127) / 128, 128, 0, g->stream>>>(Gx, Gy, g->N, (const SrcDev*)g->d_src, g->nsrc,

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "k_fp64.cuh"
+#include "k_pdl.cuh"
 #include "k_src3.cuh"
 
 namespace ms {
@@ -31,6 +32,7 @@ ms_status sfail(ms_status s, const std::string& m) {
 __global__ void k_src3_time(const double* __restrict__ coef, const double* __restrict__ omega, int nsrc,
                             const long* __restrict__ d_step, double ht, double kappa2, double unit_e, double unit_h,
                             double* __restrict__ fac, float* __restrict__ fac32) {
+  pdl_wait();
   const int q = threadIdx.x;
   if (q >= nsrc) return;
   const double w = omega[q];
@@ -48,6 +50,7 @@ __global__ void k_src3_time(const double* __restrict__ coef, const double* __res
 template <typename T>
 __global__ void k_src3_add(T* __restrict__ R, Shape3 s, const T* __restrict__ tab, const T* __restrict__ fac,
                            int nsrc) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
   if (i >= s.n[0] || j >= s.n[1]) return;
   if (!(interior(s.bc[0], i, s.n[0]) && interior(s.bc[1], j, s.n[1]) && interior(s.bc[2], k, s.n[2]))) return;
@@ -149,7 +152,7 @@ void src3_time(ms_grid* g) {
   const Src3* S = g->src3;
   // units of the FP32 right-hand side b: 6 h^2 P1 x = b with E += (12 Z / r) x, H += (12 / (r Z)) x
   const double hr2 = g->h * g->h * g->h * g->desc.r * g->desc.r;
-  k_src3_time<<<1, kMaxSrc3, 0, g->stream>>>(S->coef, S->omega, S->nsrc, g->d_step, g->ht, g->kappa2,
+  launch_pdl(k_src3_time, dim3(1), dim3(kMaxSrc3), 0, g->stream, S->coef, S->omega, S->nsrc, g->d_step, g->ht, g->kappa2,
                                              hr2 / (2.0 * g->Z), hr2 * g->Z / 2.0, S->fac, S->fac32);
 }
 
@@ -158,10 +161,10 @@ void src3_add(ms_grid* g, int c, void* R) {
   const Shape3 s = field_shape3(g->N, c);
   const dim3 grd((s.n[0] + kSrcBlk.x - 1) / kSrcBlk.x, (s.n[1] + kSrcBlk.y - 1) / kSrcBlk.y, s.n[2]);
   if (g->desc.precision == MS_FP64)
-    k_src3_add<double><<<grd, kSrcBlk, 0, g->stream>>>((double*)R, s, S->tab + S->tab_off[c], S->fac + c * S->nsrc,
+    launch_pdl(k_src3_add<double>, grd, kSrcBlk, 0, g->stream, (double*)R, s, S->tab + S->tab_off[c], S->fac + c * S->nsrc,
                                                        S->nsrc);
   else
-    k_src3_add<float><<<grd, kSrcBlk, 0, g->stream>>>((float*)R, s, S->tab32 + S->tab_off[c], S->fac32 + c * S->nsrc,
+    launch_pdl(k_src3_add<float>, grd, kSrcBlk, 0, g->stream, (float*)R, s, S->tab32 + S->tab_off[c], S->fac32 + c * S->nsrc,
                                                       S->nsrc);
 }
 
