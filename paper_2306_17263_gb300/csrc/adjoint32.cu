@@ -17,7 +17,10 @@
 // so the difference is taken first, of the float-float u, and A^{-1} is applied to it in FP32: with
 // e_j = u_{j-1} - u_j (u_{-1} = u_M = 0, zero beyond the line) and w the infinite-line solution for e,
 // (Y^T u)_j = w_j + k_j w_0 near the first end and its mirror image at the last (the end rows of A^{-T}
-// change v by a multiple of its first value, and w_0 = (rho - 1) v_0).  u = p_0 (l + c), c the last level
+// change v by a multiple of its first value, and w_0 = (rho - 1) v_0).  The difference of the high parts is
+// kept apart from that of the low parts and the recurrences' rho z, both a twentieth of it or less, until w
+// itself is rounded: one rounding of w's size per value, as in a float-float A^{-1} whose result is differenced.
+// u = p_0 (l + c), c the last level
 // of the solve's polynomial applied to l_hi: the pair (l_hi, l_lo + c) holds it to about 31 bits without
 // a new high part.  The filter and the scaling act on the difference, a well-conditioned FP32 value, and
 // the result is added to l with error-free transformations.  The step is the transpose of the
@@ -128,11 +131,11 @@ __device__ __forceinline__ void yt_segment(const YTArgs& A, int strip, int seg) 
     nh[t] = get(ph, ms + t);
     nl[t] = get(pl, ms + t);
   }
-  float z = 0.0f, zp[7] = {}, w0 = 0.0f;
+  float z = 0.0f, ep[7] = {}, gp[7] = {}, w0 = 0.0f;
   const int ngrp = 2 + (r1 - r0 + 7) / 8;
   for (int gi = 0; gi < ngrp; ++gi) {
     const int m0 = ms + 8 * gi;
-    float ch[8], cl[8], zc[8], y[8];
+    float ch[8], cl[8], ec[8], gc[8], zc[8], y[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       ch[t] = nh[t];
@@ -147,19 +150,23 @@ __device__ __forceinline__ void yt_segment(const YTArgs& A, int strip, int seg) 
     }
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      const float e = (h0 - ch[t]) + (l0 - cl[t]);
+      ec[t] = h0 - ch[t];
+      gc[t] = fmaf(kRhoF, z, l0 - cl[t]);
       h0 = ch[t];
       l0 = cl[t];
-      zc[t] = z = fmaf(kRhoF, z, e);
+      zc[t] = z = ec[t] + gc[t];
     }
     float acc = zc[7];
 #pragma unroll
     for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
-    y[7] = acc = fmaf(kRhoF, acc, zc[0]);
+    y[7] = acc = ec[0] + fmaf(kRhoF, acc, gc[0]);
 #pragma unroll
-    for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRhoF, acc, zp[t]);
+    for (int t = 6; t >= 0; --t) y[t] = acc = ep[t] + fmaf(kRhoF, acc, gp[t]);
 #pragma unroll
-    for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
+    for (int t = 0; t < 7; ++t) {
+      ep[t] = ec[t + 1];
+      gp[t] = gc[t + 1];
+    }
     if (gi < 2) continue;
     if (EDGE && seg < 2) {  // the first end's rows
       if (gi == 2) w0 = y[0];
@@ -241,7 +248,7 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
     fetch(wr);
     rd = rd == kRing - 1 ? 0 : rd + 1;
     wr = wr == kRing - 1 ? 0 : wr + 1;
-    float h[4] = {H.x, H.y, H.z, H.w}, l[4] = {L.x, L.y, L.z, L.w}, d[4], y[4];
+    float h[4] = {H.x, H.y, H.z, H.w}, l[4] = {L.x, L.y, L.z, L.w}, e[4], d[4], y[4];
     if (EDGE) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -252,20 +259,28 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
     // e of output j = u_{j-1} - u_j
     if (FROM_H) {  // j = column + 1
       const float hn = __shfl_down_sync(kFull, h[0], 1), ln = __shfl_down_sync(kFull, l[0], 1);
-      d[0] = (h[0] - h[1]) + (l[0] - l[1]);
-      d[1] = (h[1] - h[2]) + (l[1] - l[2]);
-      d[2] = (h[2] - h[3]) + (l[2] - l[3]);
-      d[3] = (h[3] - hn) + (l[3] - ln);
+      const float hq[5] = {h[0], h[1], h[2], h[3], hn}, lq[5] = {l[0], l[1], l[2], l[3], ln};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        e[q] = hq[q] - hq[q + 1];
+        l[q] = lq[q] - lq[q + 1];
+      }
     } else {  // j = column
       const float hp = __shfl_up_sync(kFull, h[3], 1), lp = __shfl_up_sync(kFull, l[3], 1);
-      d[0] = (hp - h[0]) + (lp - l[0]);
-      d[1] = (h[0] - h[1]) + (l[0] - l[1]);
-      d[2] = (h[1] - h[2]) + (l[1] - l[2]);
-      d[3] = (h[2] - h[3]) + (l[2] - l[3]);
-    }
-    if (EDGE) {
+      const float hq[5] = {hp, h[0], h[1], h[2], h[3]}, lq[5] = {lp, l[0], l[1], l[2], l[3]};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) d[q] = ine[q] ? d[q] : 0.0f;
+      for (int q = 0; q < 4; ++q) {
+        e[q] = hq[q] - hq[q + 1];
+        l[q] = lq[q] - lq[q + 1];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (EDGE) {
+        e[q] = ine[q] ? e[q] : 0.0f;
+        l[q] = ine[q] ? l[q] : 0.0f;
+      }
+      d[q] = e[q] + l[q];
     }
     float t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[0], d[1]), d[2]), d[3]);
     float c1 = __shfl_up_sync(kFull, t, 1), c2 = __shfl_up_sync(kFull, t, 2);
@@ -275,7 +290,10 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
     }
     float c = fmaf(kR4, c2, c1);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) c = d[q] = fmaf(kRhoF, c, d[q]);
+    for (int q = 0; q < 4; ++q) {
+      l[q] = fmaf(kRhoF, c, l[q]);
+      c = d[q] = e[q] + l[q];
+    }
     t = fmaf(kRhoF, fmaf(kRhoF, fmaf(kRhoF, d[3], d[2]), d[1]), d[0]);
     c1 = __shfl_down_sync(kFull, t, 1);
     c2 = __shfl_down_sync(kFull, t, 2);
@@ -285,7 +303,7 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
     }
     c = fmaf(kR4, c2, c1);
 #pragma unroll
-    for (int q = 3; q >= 0; --q) c = y[q] = fmaf(kRhoF, c, d[q]);
+    for (int q = 3; q >= 0; --q) c = y[q] = e[q] + fmaf(kRhoF, c, l[q]);
     if (EDGE) {
       auto pick = [&](int e) { return e == 0 ? y[0] : (e == 1 ? y[1] : (e == 2 ? y[2] : y[3])); };
       float wl = 0.0f, wrt = 0.0f;
