@@ -166,7 +166,8 @@ def bf16_peak():
 
 # source files that define each kernel kind reported by ms_step_profiled
 KIND_SOURCES = {
-    "curl32": ["k_tiled.cu", "k_tiled.cuh"], "solve32": ["k_tiled.cu", "k_tiled.cuh"],
+    "curl32": ["k_tiled.cu", "k_tiled.cuh", "k_walk_dev.cuh"],
+    "solve32": ["k_tiled.cu", "k_tiled.cuh", "k_walk_dev.cuh"],
     "filter64": ["k_fp64.cu", "k_fp64.cuh"], "pade64": ["k_rec64.cu", "k_rec64.cuh"],
     "filt3d32": ["grid3d.cu", "grid3d.cuh"], "band3d32": ["grid3d.cu", "grid3d.cuh"],
     "term3d32": ["grid3d.cu", "grid3d.cuh"], "tsgemm": ["k_transform.cu", "k_transform.cuh"],
@@ -187,6 +188,8 @@ def kernel_sources_hash(kind: str):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2306_17263_gb300", "csrc")
     for f in KIND_SOURCES.get(kind, []):
+        if not os.path.exists(os.path.join(csrc, f)):
+            continue
         with open(os.path.join(csrc, f), encoding="utf-8") as fh:
             h.update(f.encode() + _code_only(fh.read()).encode())
     return h.hexdigest()[:16]
