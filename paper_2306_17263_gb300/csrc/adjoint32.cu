@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(32 * WPB) k_walk_dT(const __grid_constant__ YT
 
 // ---- filter and update ---------------------------------------------------------------------
 
-// l (hi, lo) += (s_hi + s_lo)(12 beta y + L y) at the unknowns of a field, y = p1 + p2 (or p1) there, 0 on
+// l (hi, lo) += s (12 beta y + L y) at the unknowns of a field, y = p1 + p2 (or p1) there, 0 on
 // Dirichlet walls, mirrored across Neumann ones.  Bound by memory: a lane takes four columns of a row.
 struct FArgs {
   const float* p1;  // at column m = 0 of row 0
@@ -344,7 +344,7 @@ struct FArgs {
   float* lh;
   float* ll;
   int ld, M, u0, u1, neu_x, neu_y;
-  float cb_hi, cb_lo, s_hi, s_lo;  // 12 beta - 4
+  float c_hi, c_lo, s;  // 12 beta s, s
 };
 struct FArgs2 {
   FArgs f[2];
@@ -393,10 +393,12 @@ __global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (m0 + q >= M) continue;  // the pads keep their zeros
-    const float f = fmaf(A.cb_hi, y[q], fmaf(A.cb_lo, y[q], (l[q] + r[q]) + (a[q] + b[q])));
-    const float p = __fmul_rn(A.s_hi, f);
-    float e = fmaf(A.s_hi, f, -p);
-    e = fmaf(A.s_lo, f, e);
+    // an exact two-product of 12 beta s y; s L y, first differences, joins its error term
+    const float lap = ((l[q] - y[q]) + (r[q] - y[q])) + ((a[q] - y[q]) + (b[q] - y[q]));
+    const float p = __fmul_rn(A.c_hi, y[q]);
+    float e = fmaf(A.c_hi, y[q], -p);
+    e = fmaf(A.c_lo, y[q], e);
+    e = fmaf(A.s, lap, e);
     const float u = __fadd_rn(h[q], p);
     const float bb = __fsub_rn(u, h[q]);
     const float err = __fadd_rn(__fsub_rn(h[q], __fsub_rn(u, bb)), __fsub_rn(p, bb));
@@ -504,12 +506,11 @@ FArgs filter_args(ms_grid* g, int f) {
   a.u1 = N;
   a.neu_x = f == HY;
   a.neu_y = f == HX;
-  const double cb = 12.0 * g->beta - 4.0;
-  a.cb_hi = (float)cb;
-  a.cb_lo = (float)(cb - (double)a.cb_hi);
-  const double s = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * g->walk.cheb.p0 * walk_rhs_scale();
-  a.s_hi = (float)s;
-  a.s_lo = (float)(s - (double)a.s_hi);
+  const double sc = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * g->walk.cheb.p0 * walk_rhs_scale();
+  const double c = 12.0 * g->beta * sc;
+  a.c_hi = (float)c;
+  a.c_lo = (float)(c - (double)a.c_hi);
+  a.s = (float)sc;
   return a;
 }
 
