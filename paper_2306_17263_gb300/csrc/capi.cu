@@ -1198,13 +1198,23 @@ ms_status batch_step_launch(ms_batch* b) {
   return check_launch("batch step");
 }
 
-// Apply a plan: rebuild the work lists when the order changes, drop the captured graphs.
+// Apply a plan: rebuild the work lists when the order changes, drop the captured graphs.  The lists in use, which
+// the graphs hold too, go only once the new ones are there: a failed build leaves the batch as it was.
 ms_status batch_apply_plan(ms_batch* b, const int* plan) {
   if (plan[0] != b->plan[0]) {
-    MS_CUDA(cudaStreamSynchronize(b->stream));
-    walk_batch_free(&b->tb);
+    WalkBatch tb;
     std::string err;
-    if (walk_batch_build(b->cav.data(), (int)b->cav.size(), plan[0], &b->tb, &err) != 0) return fail(MS_ENOMEM, err);
+    if (walk_batch_build(b->cav.data(), (int)b->cav.size(), plan[0], &tb, &err) != 0) {
+      walk_batch_free(&tb);
+      return fail(MS_ENOMEM, err);
+    }
+    const cudaError_t e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) {
+      walk_batch_free(&tb);
+      return fail(MS_ECUDA, std::string("cudaStreamSynchronize: ") + cudaGetErrorString(e));
+    }
+    walk_batch_free(&b->tb);
+    b->tb = tb;
   }
   free_graph(&b->graph1);
   free_graph(&b->graphk);
