@@ -116,17 +116,13 @@ void p1_solve64(ms_grid* g, int f, const double* b, double* out, double* upd, do
   }
   const Cheb2dField F{b, out, upd, s, b2};
   double* const buf[1][2] = {{g->s64[3], g->s64[4]}};
-  launch_cheb2d64(&F, 1, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
-  prof_mark(g, KK_P1SWEEP64, 8.0 * (double)s.size() * (1.0 + (out ? 1.0 : 0.0) + (upd ? 2.0 : 0.0)));
-  *nl += 1;
+  *nl += launch_cheb2d64(g, KK_P1SWEEP64, &F, 1, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale);
 }
 
 void p1_solve64_h(ms_grid* g, const double* bx, const double* by, double* outx, double* outy, double* updx, double* updy,
                   double upd_scale, double* const (*buf)[2], int* nl) {
   const Cheb2dField F[2] = {{bx, outx, updx, g->sh[HX]}, {by, outy, updy, g->sh[HY]}};
-  launch_cheb2d64(F, 2, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
-  prof_mark(g, KK_P1SWEEP64, 16.0 * (double)g->sh[HX].size() * (1.0 + (outx ? 1.0 : 0.0) + (updx ? 2.0 : 0.0)));
-  *nl += 1;
+  *nl += launch_cheb2d64(g, KK_P1SWEEP64, F, 2, buf, g->cheb64, 6.0 * g->h * g->h, upd_scale);
 }
 }  // namespace ms
 

@@ -1081,7 +1081,6 @@ void solve3d64(ms_grid* g, int c0, double* const* b, double* const* upd, double 
   Grid3D* G3 = g->g3;
   Cheb3dField f[3];
   double* buf[3][2];
-  double pts = 0.0;
   const int m = g->cheb64.m;
   for (int c = 0; c < 3; ++c) {
     const Shape3& s = G3->sh[c0 + c];
@@ -1098,11 +1097,8 @@ void solve3d64(ms_grid* g, int c0, double* const* b, double* const* upd, double 
       f[c].n[a] = s.n[a];
       f[c].bc[a] = s.bc[a];
     }
-    pts += (double)s.size();
   }
-  launch_cheb3d64(f, buf, 3, g->cheb64, 6.0 * g->h * g->h, upd_scale, g->stream);
-  prof_mark(g, KK_SWEEP3D64, 8.0 * pts * (3.0 * (m - 1) + (upd ? 1.0 : 0.0)));
-  *nl += m - 1;
+  *nl += launch_cheb3d64(g, KK_SWEEP3D64, f, buf, 3, g->cheb64, 6.0 * g->h * g->h, upd_scale);
 }
 
 ms_status step3d64(ms_grid* g) {

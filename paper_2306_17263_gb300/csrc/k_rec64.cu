@@ -545,8 +545,21 @@ __global__ void __launch_bounds__(128) k_cheb2d64_level(Cheb2dLevel A) {
 
 }  // namespace
 
-void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], const Cheb& p, double bscale,
-                     double upd_scale, cudaStream_t st) {
+// Planes a launch of the solve must touch: b, and y apart from it after the first level, read; the iterate, or
+// the solution and the updated field (read and written), written.
+static double level_planes(bool first, bool last, bool b2, bool out, bool upd) {
+  return 1.0 + !first + b2 + (last ? (out ? 1.0 : 0.0) + (upd ? 2.0 : 0.0) : 1.0);
+}
+
+int launch_cheb2d64(ms_grid* g, int kind, const Cheb2dField* f, int nf, double* const (*buf)[2], const Cheb& p,
+                    double bscale, double upd_scale) {
+  const cudaStream_t st = g->stream;
+  auto mark = [&](bool first, bool last) {
+    double bytes = 0.0;
+    for (int q = 0; q < nf; ++q)
+      bytes += 8.0 * (double)f[q].s.size() * level_planes(first, last, f[q].b2, f[q].out, f[q].upd);
+    prof_mark(g, kind, bytes);
+  };
   const double out_scale = p.p0 * bscale;
   const int nx = f[0].s.nx > f[nf - 1].s.nx ? f[0].s.nx : f[nf - 1].s.nx;
   const int ny = f[0].s.ny > f[nf - 1].s.ny ? f[0].s.ny : f[nf - 1].s.ny;
@@ -569,8 +582,9 @@ void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], cons
       A.upd_scale = upd_scale * out_scale;
       if (k == 1) launch_pdl(k_cheb2d64_level<true>, grd, dim3(32, 4), 0, st, A);
       else launch_pdl(k_cheb2d64_level<false>, grd, dim3(32, 4), 0, st, A);
+      mark(step == 0, k == 1);
     }
-    return;
+    return p.m - 1;
   }
   Cheb2dArgs A;
   A.f[0] = f[0];
@@ -583,6 +597,8 @@ void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], cons
   const int W = A.TS + 2 * (p.m - 1);
   const size_t smem = 3 * sizeof(double) * (size_t)W * W;  // at most 35 KB
   launch_pdl(k_cheb2d64, dim3((nx + A.TS - 1) / A.TS, (ny + A.TS - 1) / A.TS, nf), dim3(C2T), smem, st, A);
+  mark(true, true);
+  return 1;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -665,8 +681,9 @@ __global__ void __launch_bounds__(C3T) k_cheb3d64(Cheb3dArgs A) {
 
 }  // namespace
 
-void launch_cheb3d64(const Cheb3dField* f, double* const (*buf)[2], int count, const Cheb& p, double bscale,
-                     double upd_scale, cudaStream_t st) {
+int launch_cheb3d64(ms_grid* g, int kind, const Cheb3dField* f, double* const (*buf)[2], int count, const Cheb& p,
+                    double bscale, double upd_scale) {
+  const cudaStream_t st = g->stream;
   Cheb3dArgs A;
   size_t plane = 0;
   int nz = 0;
@@ -692,7 +709,12 @@ void launch_cheb3d64(const Cheb3dField* f, double* const (*buf)[2], int count, c
     }
     if (k == 1) launch_pdl(k_cheb3d64<true>, grd, dim3(C3T), 0, st, A);
     else launch_pdl(k_cheb3d64<false>, grd, dim3(C3T), 0, st, A);
+    double bytes = 0.0;
+    for (int c = 0; c < count; ++c)
+      bytes += 8.0 * (double)f[c].n[0] * f[c].n[1] * f[c].n[2] * level_planes(step == 0, k == 1, false, f[c].out, f[c].upd);
+    prof_mark(g, kind, bytes);
   }
+  return p.m - 1;
 }
 
 }  // namespace ms

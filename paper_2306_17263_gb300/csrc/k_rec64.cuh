@@ -51,9 +51,10 @@ struct Cheb2dField {
 };
 // Whether the solve of `pts` points runs all its levels in one launch (k_cheb2d64).
 inline bool cheb2d64_tiles(long pts) { return pts <= 300000; }
-// buf: two work planes per field, all distinct from each other and from b and out.
-void launch_cheb2d64(const Cheb2dField* f, int nf, double* const (*buf)[2], const Cheb& p, double bscale,
-                     double upd_scale, cudaStream_t st);
+// buf: two work planes per field, all distinct from each other and from b and out.  On the grid's stream; every
+// launch is marked for the profiler as `kind`.  Returns the number of launches.
+int launch_cheb2d64(ms_grid* g, int kind, const Cheb2dField* f, int nf, double* const (*buf)[2], const Cheb& p,
+                    double bscale, double upd_scale);
 
 // The same for up to three 3D components; buf: two work arrays per component, in which every wall point
 // of a Dirichlet axis may hold anything (they are not read).
@@ -65,7 +66,7 @@ struct Cheb3dField {
   double* upd;
   int n[3], bc[3];
 };
-void launch_cheb3d64(const Cheb3dField* f, double* const (*buf)[2], int count, const Cheb& p, double bscale,
-                     double upd_scale, cudaStream_t st);
+int launch_cheb3d64(ms_grid* g, int kind, const Cheb3dField* f, double* const (*buf)[2], int count, const Cheb& p,
+                    double bscale, double upd_scale);
 
 }  // namespace ms
