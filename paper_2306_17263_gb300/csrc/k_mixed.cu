@@ -77,9 +77,9 @@ ms_status step_mixed(ms_grid* g, int* nl) {
   // write), the algorithmic bytes of a step being 48 B per cell (each component read and written
   // once); the right-hand-side planes are intermediates and are not counted
   prof_mark(g, KK_CURL32, 16.0 * nh);                        // H_x, H_y (hi, lo) read
-  // sources in the units of b: 6 h^2 P1 x = (1 - rho)^2 b with E += (12 Z / r) x, so
-  // b = (h^3 r^2 / (2 Z)) R / (1 - rho)^2; H += (12 / (r Z)) x, b = (h^3 r^2 Z / 2) R / (1 - rho)^2
-  const double hr2 = g->h * g->h * g->h * g->desc.r * g->desc.r / walk_rhs_scale();
+  // sources in the units of b: 6 h^2 P1 x = s b, s the planes' factor, with E += (12 Z / r) x, so
+  // b = (h^3 r^2 / (2 Z)) R / s; H += (12 / (r Z)) x, b = (h^3 r^2 Z / 2) R / s
+  const double hr2 = g->h * g->h * g->h * g->desc.r * g->desc.r / plane_rhs_scale(g);
   const double scale_e = hr2 / (2.0 * g->Z), scale_h = hr2 * g->Z / 2.0;
   if (g->nsrc) {
     launch_src_time(g, scale_e, scale_h);

@@ -221,18 +221,16 @@ __device__ __forceinline__ void tiny_curl(const YArgs& A) {
     }
     return hi + lo;
   };
-  // the planes hold right-hand sides over (1 - rho)^2
-  constexpr float inv = 1.0f / ((1.0f - kRhoF) * (1.0f - kRhoF));
   if (A.step == 0) {
     for (int p = lane; p < (N - 1) * (N - 1); p += 32) {
       const int j = 1 + p / (N - 1), i = 1 + p % (N - 1);
-      A.tb[0][(size_t)j * A.ld + i] = inv * (term(0, 0, j, i - 1) - term(1, 1, i, j - 1));
+      A.tb[0][(size_t)j * A.ld + i] = term(0, 0, j, i - 1) - term(1, 1, i, j - 1);
     }
   } else {
     for (int p = lane; p < N * (N - 1); p += 32) {
       const int j = p / (N - 1), i = 1 + p % (N - 1);
-      A.tb[0][(size_t)j * A.ld + i] = -inv * term(0, 1, i, j);
-      A.tb[1][(size_t)i * A.ld + j] = inv * term(0, 0, i, j);
+      A.tb[0][(size_t)j * A.ld + i] = -term(0, 1, i, j);
+      A.tb[1][(size_t)i * A.ld + j] = term(0, 0, i, j);
     }
   }
 }
@@ -581,7 +579,7 @@ SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfie
   a.kind = f == EZ ? KIND_E : (f == HX ? KIND_HX : KIND_HY);
   const Cheb& p = g->walk.cheb;
   for (int l = 0; l < p.m - 1; ++l) a.q[l] = (float)p.q[p.m - 1 - l];
-  const Split sp = split((f == EZ ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0 * walk_rhs_scale());
+  const Split sp = split((f == EZ ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0 * plane_rhs_scale(g));
   a.s_hi = sp.hi;
   a.s_lo = sp.lo;
   a.nstrip = (a.M + SOUT - 1) / SOUT;
@@ -612,6 +610,7 @@ void line_segments(int M, int rows, int* nseg, int* chunk, int* rb) {
 }
 
 double walk_rhs_scale() { return (1.0 - (double)kRhoF) * (1.0 - (double)kRhoF); }
+double plane_rhs_scale(const ms_grid* g) { return g->N <= kTinyN ? 1.0 : walk_rhs_scale(); }
 
 int walk_ld(int N) { return (N + 8 + 31) / 32 * 32; }
 size_t plane_floats(int N) { return (size_t)(N + 1) * walk_ld(N) + 64; }

@@ -21,6 +21,9 @@ MixedConsts mixed_consts(const ms_grid* g);
 // The right-hand sides of the walk kernels are those of 6 h^2 P1 x = b over this factor, (1 - rho)^2
 // with rho the FP32 root: the recurrences give A^{-1} d up to it, and the increment scales carry it.
 double walk_rhs_scale();
+// The factor of a 2D grid's planes: that one, or 1 on grids of at most kTinyN cells (explicit rows of A^{-1}).
+// One FP32 number 1 / (1 - rho)^2 on every right-hand side would shift every frequency of those grids by 8e-8.
+double plane_rhs_scale(const ms_grid* g);
 
 // Segments of a line of M >= 16 rows that warps walk along: about `rows` rows each, `chunk` rows (a multiple
 // of 8) but for the last one, which is [rb, M), a multiple of 8 rows; every other one ends at least 8

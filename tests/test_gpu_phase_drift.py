@@ -1,0 +1,47 @@
+"""Coefficients of the FP32_REFINED step over long runs: the phase of one cavity mode after tens of thousands of
+steps against the FP64 step.  A coefficient that is off by a relative eps shifts the frequency by about eps, the
+same way in every step, where rounding averages out."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2306_17263_gb300 as pkg  # noqa: E402
+
+
+def _phase(fields, n, k, z):
+    x = np.pi * k * np.arange(n + 1) / n
+    s, c = np.sin(x), np.cos(np.pi * k * (np.arange(n) + 0.5) / n)
+    ez, hx, hy = fields
+    e = np.sum(ez * np.outer(s, s)) / np.sum(np.outer(s, s) ** 2)
+    b = np.sum(np.outer(c, s) ** 2)
+    h = (np.sum(hy * np.outer(s, c)) - np.sum(hx * np.outer(c, s))) / b
+    return math.atan2(h * z / math.sqrt(2.0), e)
+
+
+def _shift(n, r, k, steps, closure, z=1.3):
+    ph = []
+    for precision in (pkg.FP64, pkg.FP32_REFINED):
+        with pkg.Grid(n, r, z=z, precision=precision, closure=closure) as g:
+            g.init_modes([(k, k, 1.0)])
+            g.run(steps)
+            ph.append(_phase(g.get_fields(), n, k, z))
+    d = (ph[1] - ph[0] + math.pi) % (2.0 * math.pi) - math.pi
+    return abs(d) / (math.pi * k * math.sqrt(2.0) * steps * r / n)
+
+
+CLOSURES = [pkg.CLOSURE_PAPER, pkg.CLOSURE_REFLECT]
+
+
+@pytest.mark.parametrize("closure", CLOSURES)
+@pytest.mark.parametrize("n, r, k", [(8, 0.5, 2), (16, 0.5, 3), (16, 0.65, 2)])
+def test_smallest_grids_scale(n, r, k, closure):
+    """Grids of at most 16 cells, whose derivatives come from explicit rows: no factor common to all of them is off
+    by half an FP32 ulp."""
+    assert _shift(n, r, k, 8000, closure) <= 2.0 ** -25
