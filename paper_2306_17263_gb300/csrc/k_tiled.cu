@@ -206,9 +206,10 @@ __device__ __forceinline__ void tiny_curl(const YArgs& A) {
       }
       return axis == 0 ? u(h, l, cc, m, cc, m + 1) : u(h, l, m, cc, m + 1, cc);
     };
+    // farthest taps first: added after the nearest ones, those beyond the sixth would round away in every sum
     float hi = 0.0f, lo = 0.0f;
-    for (int t = 0; t < rs; ++t) {
-      const int m = r - K + t;
+    for (int q = 2 * K + 1; q >= 0; --q) {
+      const int m = r + ((q & 1) ? (q + 1) / 2 : -(q / 2)), t = m - r + K;
       if (m < 0 || m >= M) continue;
       const float x = delta(c, m);
       float d = x;
@@ -216,10 +217,10 @@ __device__ __forceinline__ void tiny_curl(const YArgs& A) {
         const float lap = ((delta(c, m - 1) - x) + (delta(c, m + 1) - x)) + ((delta(c - 1, m) - x) + (delta(c + 1, m) - x));
         d = fmaf(A.tcb_hi, x, fmaf(A.tcb_lo, x, lap));
       }
-      hi = fmaf(A.whi[r * rs + t], d, hi);
       lo = fmaf(A.wlo[r * rs + t], d, lo);
+      hi = fmaf(A.whi[r * rs + t], d, q ? hi : hi + lo);
     }
-    return hi + lo;
+    return hi;
   };
   if (A.step == 0) {
     for (int p = lane; p < (N - 1) * (N - 1); p += 32) {
