@@ -59,10 +59,10 @@ struct YArgs {
   float cb_hi, cb_lo;  // 12 beta - 4: coefficient of delta beside the sum of its four neighbours
   float g[4], v[kEnd];
   int nstrip, nseg, chunk, rb;  // column strips; segments of `chunk` rows, the last one [rb, M)
-  // grids of at most kTinyN cells: explicit rows of A^{-1}, every derivative of the half-step
+  // grids of at most kTinyN cells: explicit rows of A^{-1}, both derivatives of the half-step
   int tiny, step, N;
-  const float *th[2], *tl[2];  // sources: Step 1 H_y, H_x; Step 2 E_z
-  float* tb[2];
+  const float *th[2], *tl[2];  // sources of the derivatives along x and y: Step 1 H_y, H_x; Step 2 E_z
+  float* tb[2];                // destinations of those along y and x
   const float *whi, *wlo;
   int K;
   float tcb_hi, tcb_lo;  // 12 beta
@@ -189,57 +189,51 @@ __device__ __forceinline__ void y_segment(const YArgs& A, int strip, int seg) {
   }
 }
 
-// Lines of fewer than 16 rows: every output from the explicit rows of A^{-1}, a point per lane.
-__device__ __forceinline__ void tiny_curl(const YArgs& A) {
-  const int lane = threadIdx.x & 31, N = A.N, K = A.K, rs = 2 * K + 2;
-  auto u = [&](const float* h, const float* l, int j, int i, int j2, int i2) {
-    return (h[(size_t)j2 * A.ld + i2] - h[(size_t)j * A.ld + i]) + (l[(size_t)j2 * A.ld + i2] - l[(size_t)j * A.ld + i]);
+// Lines of at most 16 rows (grids of up to kTinyN cells): outputs from the explicit rows of A^{-1}.  A warp
+// takes two lines of one axis, a lane one difference and one output; the differences of a line come from the
+// lanes of its half.  A step is bound by the latency of its launches, so the lines go over as many warps as
+// there are (8^2 and 16^2: 14 and 17 us per step; 49 and 212 with one warp for a whole half-step).
+__device__ __forceinline__ void tiny_item(const YArgs& A, int item) {
+  const int N = A.N, M = A.M, K = A.K, rs = 2 * K + 2, per = N / 2;  // items per axis
+  if (item >= 2 * per) return;
+  const int axis = item >= per, r = threadIdx.x & 15;  // axis 0: lines are rows of the source, 1 columns
+  const int c = 1 + 2 * (item - axis * per) + ((threadIdx.x >> 4) & 1), cc = min(c, N - 1);
+  const float *h = A.th[axis], *l = A.tl[axis];
+  const size_t sm = axis == 0 ? 1 : A.ld, sc = axis == 0 ? A.ld : 1;
+  auto delta = [&](int line) {
+    const size_t p = line * sc + r * sm;
+    return r < M ? (h[p + sm] - h[p]) + (l[p + sm] - l[p]) : 0.0f;
   };
-  // y of line c at row r: axis 0 lines are rows of the source, 1 columns
-  auto term = [&](int s, int axis, int c, int r) {
-    const int M = A.M;
-    const float *h = A.th[s], *l = A.tl[s];
-    auto delta = [&](int cc, int m) -> float {
-      if (m < 0 || m >= M) {
-        if (!A.even || m < -1 || m > M) return 0.0f;
-        m = m < 0 ? 0 : M - 1;
-      }
-      return axis == 0 ? u(h, l, cc, m, cc, m + 1) : u(h, l, m, cc, m + 1, cc);
-    };
-    // farthest taps first: added after the nearest ones, those beyond the sixth would round away in every sum
-    float hi = 0.0f, lo = 0.0f;
-    for (int q = 2 * K + 1; q >= 0; --q) {
-      const int m = r + ((q & 1) ? (q + 1) / 2 : -(q / 2)), t = m - r + K;
-      if (m < 0 || m >= M) continue;
-      const float x = delta(c, m);
-      float d = x;
-      if (A.filter) {
-        const float lap = ((delta(c, m - 1) - x) + (delta(c, m + 1) - x)) + ((delta(c - 1, m) - x) + (delta(c + 1, m) - x));
-        d = fmaf(A.tcb_hi, x, fmaf(A.tcb_lo, x, lap));
-      }
-      lo = fmaf(A.wlo[r * rs + t], d, lo);
-      hi = fmaf(A.whi[r * rs + t], d, q ? hi : hi + lo);
-    }
-    return hi;
-  };
-  if (A.step == 0) {
-    for (int p = lane; p < (N - 1) * (N - 1); p += 32) {
-      const int j = 1 + p / (N - 1), i = 1 + p % (N - 1);
-      A.tb[0][(size_t)j * A.ld + i] = term(0, 0, j, i - 1) - term(1, 1, i, j - 1);
-    }
-  } else {
-    for (int p = lane; p < N * (N - 1); p += 32) {
-      const int j = p / (N - 1), i = 1 + p % (N - 1);
-      A.tb[0][(size_t)j * A.ld + i] = -term(0, 1, i, j);
-      A.tb[1][(size_t)i * A.ld + j] = term(0, 0, i, j);
-    }
+  float d = delta(cc);
+  if (A.filter) {
+    const float x = d, up = delta(cc - 1), dn = delta(cc + 1);
+    float a = __shfl_up_sync(kFull, x, 1, 16), b = __shfl_down_sync(kFull, x, 1, 16);
+    if (r == 0) a = A.even ? x : 0.0f;
+    if (r == M - 1) b = A.even ? x : 0.0f;
+    const float lap = ((a - x) + (b - x)) + ((up - x) + (dn - x));
+    d = fmaf(A.tcb_hi, x, fmaf(A.tcb_lo, x, lap));
   }
+  // farthest taps first: added after the nearest ones, those beyond the sixth would round away in every sum
+  const float *wh = A.whi + r * rs, *wl = A.wlo + r * rs;
+  float hi = 0.0f, lo = 0.0f;
+#pragma unroll 8
+  for (int q = 2 * K + 1; q >= 0; --q) {
+    const int m = r + ((q & 1) ? (q + 1) / 2 : -(q / 2)), t = m - r + K;
+    const float x = __shfl_sync(kFull, d, m & 15, 16);
+    if (r >= M || m < 0 || m >= M) continue;
+    lo = fmaf(wl[t], x, lo);
+    hi = fmaf(wh[t], x, q ? hi : hi + lo);
+  }
+  if (r >= M || c >= N) return;
+  const int o = r + (A.step == 0);
+  if (axis == 0) A.tb[1][(size_t)c * A.ld + o] = hi;
+  else A.tb[0][(size_t)o * A.ld + c] = -hi;
 }
 
 template <bool FILTER>
 __device__ __forceinline__ void y_item(const YArgs& A, int item) {
   if (A.tiny) {
-    if (item == 0) tiny_curl(A);
+    tiny_item(A, item);
     return;
   }
   if (item >= A.nstrip * A.nseg) return;
@@ -531,7 +525,8 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
     a.K = g->pade32[kind].K;
     a.tcb_hi = t.hi;
     a.tcb_lo = t.lo;
-    a.nstrip = a.nseg = 1;
+    a.nstrip = 1;
+    a.nseg = 2 * (N / 2);  // two lines of one axis per item
   }
   a.filter = src_hi == nullptr;
   return a;
@@ -629,7 +624,7 @@ ms_status walk_setup(ms_grid* g) {
 
 void walk_d(ms_grid* g, int step, const float* src_hi, const float* src_lo) {
   // Step 1: along y into s32[4], along x into s32[1]; Step 2: s32[2] (H_x), s32[3] (H_y)
-  const YArgs y = make_y(g, step, step == 0 ? g->s32[4] : g->s32[2], step == 0 ? nullptr : g->s32[3], src_hi, src_lo);
+  const YArgs y = make_y(g, step, step == 0 ? g->s32[4] : g->s32[2], step == 0 ? g->s32[1] : g->s32[3], src_hi, src_lo);
   const XArgs x = make_x(g, step, step == 0 ? g->s32[1] : g->s32[3], src_hi, src_lo);
   const int nyb = blocks_of(y.nstrip * y.nseg);
   const dim3 grd(nyb + blocks_of(x.nstrip * x.nblk)), blk(32 * WPB);
@@ -668,7 +663,7 @@ int walk_batch_build(ms_grid* const* cav, int count, int order, WalkBatch* wb, s
   wb->ny = 2 * count;
   for (int c = 0; c < count; ++c) {
     const ms_grid* g = cav[c];
-    ya[c] = make_y(g, 0, g->s32[4], nullptr, nullptr, nullptr);
+    ya[c] = make_y(g, 0, g->s32[4], g->s32[1], nullptr, nullptr);
     ya[count + c] = make_y(g, 1, g->s32[2], g->s32[3], nullptr, nullptr);
     xa[c] = make_x(g, 0, g->s32[1], nullptr, nullptr);
     xa[count + c] = make_x(g, 1, g->s32[3], nullptr, nullptr);

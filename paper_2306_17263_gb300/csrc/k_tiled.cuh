@@ -41,8 +41,8 @@ size_t plane_origin(int f);
 ms_status walk_setup(ms_grid* g);
 
 // step 0 (Step 1): the derivatives into the E_z planes s32[4] (along y) and s32[1] (along x); step 1
-// (Step 2): into s32[2] (H_x, along y) and s32[3] (H_y, along x).  Grids of at most kTinyN cells put all
-// of Step 1 into s32[4].  src_hi, src_lo != NULL: Step 2 from that already filtered E_z-shaped field.
+// (Step 2): into s32[2] (H_x, along y) and s32[3] (H_y, along x).  src_hi, src_lo != NULL: Step 2 from that
+// already filtered E_z-shaped field.
 void walk_d(ms_grid* g, int step, const float* src_hi = nullptr, const float* src_lo = nullptr);
 // The solve and the state update of the half-step's fields from those planes.
 void walk_s(ms_grid* g, int step);
