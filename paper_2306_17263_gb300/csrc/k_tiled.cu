@@ -57,7 +57,7 @@ struct YArgs {
   float* b;         // destination plane, row of output 0, column 0
   int ld, ncol, M, even;
   float cb_hi, cb_lo;  // 12 beta - 4: coefficient of delta beside the sum of its four neighbours
-  float g[4], v[kEnd];
+  float g[4], gl[4], v[kEnd];  // end correction, g in pairs
   int nstrip, nseg, chunk, rb;  // column strips; segments of `chunk` rows, the last one [rb, M)
   // grids of at most kTinyN cells: explicit rows of A^{-1}, both derivatives of the half-step
   int tiny, step, N;
@@ -77,11 +77,29 @@ struct XArgs {
   int ld, M;        // outputs 0 .. M-1 of every row
   int u0, u1;       // rows u0 .. u1-1
   float cb_hi, cb_lo;
-  float g[4], v[kEnd];
+  float g[4], gl[4], v[kEnd];
   int nstrip, nblk, rows;
 };
 
 namespace {
+
+// phi = g_0 y_0 + .. + g_3 y_3 of the end correction (y counted from the line's end).
+template <typename Args>
+__device__ __forceinline__ float end_phi(const Args& A, float y0, float y1, float y2, float y3) {
+  const float lo = fmaf(A.gl[0], y0, fmaf(A.gl[1], y1, fmaf(A.gl[2], y2, A.gl[3] * y3)));
+  return fmaf(A.g[0], y0, fmaf(A.g[1], y1, fmaf(A.g[2], y2, fmaf(A.g[3], y3, lo))));
+}
+
+// The eight rows at an end of a line with their correction, y_t = z_t + (rho y_{t+1} + v phi).  It joins rho y, a
+// twentieth of y: added to y itself it would round away from the fifth row on, always the same way (frequencies of
+// small grids off by 1e-9 to 3e-9; 1e-10 to 4e-10 this way).  v is one FP32 number each, an error of 6e-11 y.
+template <bool LAST>
+__device__ __forceinline__ void end_rows(float (&y)[8], const float (&z)[8], float ynext, float phi,
+                                         const float (&v)[kEnd]) {
+#pragma unroll
+  for (int t = 0; t < kEnd; ++t)
+    y[t] = z[t] + fmaf(v[LAST ? kEnd - 1 - t : t], phi, kRhoF * (t < kEnd - 1 ? y[t + 1 < kEnd ? t + 1 : t] : ynext));
+}
 
 // ---- derivative along y --------------------------------------------------------------------------------
 
@@ -161,24 +179,18 @@ __device__ __forceinline__ void y_segment(const YArgs& A, int strip, int seg) {
     float acc = zc[7];
 #pragma unroll
     for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
+    const float ynext = acc;  // of the row after the group
     y[7] = acc = fmaf(kRhoF, acc, zc[0]);
 #pragma unroll
     for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRhoF, acc, zp[t]);
+    if (EDGE && gidx >= 2) {
+      const float zr[8] = {zp[0], zp[1], zp[2], zp[3], zp[4], zp[5], zp[6], zc[0]};
+      if (seg == 0 && gidx == 2) end_rows<false>(y, zr, ynext, end_phi(A, y[0], y[1], y[2], y[3]), A.v);
+      if (last && gidx == ngrp - 1) end_rows<true>(y, zr, ynext, end_phi(A, y[7], y[6], y[5], y[4]), A.v);
+    }
 #pragma unroll
     for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
     if (gidx < 2) continue;
-    if (EDGE) {
-      if (seg == 0 && gidx == 2) {
-        const float phi = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
-#pragma unroll
-        for (int t = 0; t < kEnd; ++t) y[t] = fmaf(A.v[t], phi, y[t]);
-      }
-      if (last && gidx == ngrp - 1) {
-        const float phi = fmaf(A.g[0], y[7], fmaf(A.g[1], y[6], fmaf(A.g[2], y[5], A.g[3] * y[4])));
-#pragma unroll
-        for (int t = 0; t < kEnd; ++t) y[7 - t] = fmaf(A.v[t], phi, y[7 - t]);
-      }
-    }
     if (live) {
       const int left = r1 - (r0 + 8 * (gidx - 2));
 #pragma unroll
@@ -262,7 +274,7 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
   auto load = [&](const float* p, int row) { return ok ? ld4(p + (size_t)row * ld + m0) : zero4; };
   // edge strips: masks, and the end corrections' coefficients at the lane's columns
   bool in[4] = {true, true, true, true}, first[4] = {}, lastc[4] = {};
-  float vl[4] = {}, vr[4] = {}, gr[4] = {};
+  float vl[4] = {}, vr[4] = {}, gr[4] = {}, grl[4] = {};
   int la = 0, lb = 0;
   bool right = false;
   if (EDGE) {
@@ -278,6 +290,7 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
       vl[k] = (strip == 0 && m >= 0 && m < kEnd) ? A.v[m & 7] : 0.0f;
       vr[k] = (right && e >= 0 && e < kEnd) ? A.v[e & 7] : 0.0f;
       gr[k] = (right && e >= 0 && e < 4) ? A.g[e & 3] : 0.0f;
+      grl[k] = (right && e >= 0 && e < 4) ? A.gl[e & 3] : 0.0f;
     }
   }
   // differences of one source row
@@ -377,22 +390,26 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
       c2 = lane > 29 ? 0.0f : c2;
     }
     c = fmaf(kR4, c2, c1);
+    const float ynext = c;
 #pragma unroll
     for (int k = 3; k >= 0; --k) c = y[k] = fmaf(kRhoF, c, d[k]);
-    if (EDGE) {
+    if (EDGE) {  // as end_rows
+      float n[4] = {kRhoF * y[1], kRhoF * y[2], kRhoF * y[3], kRhoF * ynext};
       if (strip == 0) {  // columns 0 .. 3 are lane 2's
-        const float part = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
-        const float phi = __shfl_sync(kFull, part, XHALO / 4);
+        const float phi = __shfl_sync(kFull, end_phi(A, y[0], y[1], y[2], y[3]), XHALO / 4);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) y[k] = fmaf(vl[k], phi, y[k]);
+        for (int k = 0; k < 4; ++k) n[k] = fmaf(vl[k], phi, n[k]);
       }
       if (right) {
-        const float part = fmaf(gr[0], y[0], fmaf(gr[1], y[1], fmaf(gr[2], y[2], gr[3] * y[3])));
+        const float lo = fmaf(grl[0], y[0], fmaf(grl[1], y[1], fmaf(grl[2], y[2], grl[3] * y[3])));
+        const float part = fmaf(gr[0], y[0], fmaf(gr[1], y[1], fmaf(gr[2], y[2], fmaf(gr[3], y[3], lo))));
         const float pa = __shfl_sync(kFull, part, la), pb = __shfl_sync(kFull, part, lb);
         const float phi = la == lb ? pa : pa + pb;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) y[k] = fmaf(vr[k], phi, y[k]);
+        for (int k = 0; k < 4; ++k) n[k] = fmaf(vr[k], phi, n[k]);
       }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) y[k] = d[k] + n[k];
     }
     if (out) *reinterpret_cast<float4*>(bp) = make_float4(y[0], y[1], y[2], y[3]);  // (pads: never read unmasked)
   }
@@ -488,6 +505,16 @@ Split split(double v) {
   return s;
 }
 
+template <typename Args>
+void set_ends(const LineEnds& e, Args* a) {
+  for (int k = 0; k < 4; ++k) {
+    const Split g = split(e.g[k]);
+    a->g[k] = g.hi;
+    a->gl[k] = g.lo;
+  }
+  for (int k = 0; k < kEnd; ++k) a->v[k] = (float)e.v[k];
+}
+
 YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const float* src_hi, const float* src_lo) {
   YArgs a{};
   const int N = g->N;
@@ -503,8 +530,7 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
   const Split c = split(12.0 * g->beta - 4.0), t = split(12.0 * g->beta);
   a.cb_hi = c.hi;
   a.cb_lo = c.lo;
-  for (int k = 0; k < 4; ++k) a.g[k] = (float)g->walk.ends[kind].g[k];
-  for (int k = 0; k < kEnd; ++k) a.v[k] = (float)g->walk.ends[kind].v[k];
+  set_ends(g->walk.ends[kind], &a);
   a.nstrip = (N - 1 + YOUT - 1) / YOUT;
   // Rows per segment: 16 more warm up its recurrences, so long segments do less work, but a grid wants
   // about ten warps per SM, and small grids short walks.  The choice depends on N alone: a cavity of a batch takes the segments of a
@@ -548,9 +574,7 @@ XArgs make_x(const ms_grid* g, int step, float* plane, const float* src_hi, cons
   const Split c = split(12.0 * g->beta - 4.0);
   a.cb_hi = c.hi;
   a.cb_lo = c.lo;
-  const LineEnds& e = g->walk.ends[step == 0 ? HALF_TO_NODE : NODE_TO_HALF];
-  for (int k = 0; k < 4; ++k) a.g[k] = (float)e.g[k];
-  for (int k = 0; k < kEnd; ++k) a.v[k] = (float)e.v[k];
+  set_ends(g->walk.ends[step == 0 ? HALF_TO_NODE : NODE_TO_HALF], &a);
   a.nstrip = N <= kTinyN ? 0 : (a.M + XOUT - 1) / XOUT;
   const int rows = a.nstrip * (N / 8) < 1216 ? 4 : 8;  // as in make_s
   a.nblk = (N - 1 + rows - 1) / rows;

@@ -62,3 +62,10 @@ def test_smallest_grids_scale(n, r, k, closure):
 def test_smallest_grids(n, r, k, closure):
     """The same grids: the rows' sums lose none of their small terms."""
     assert _shift(n, r, k, 20000, closure) <= _bound(n, k, 20000)
+
+
+@pytest.mark.parametrize("closure", CLOSURES)
+@pytest.mark.parametrize("n, r, k", [(17, 0.5, 2), (20, 0.5, 2), (32, 0.5, 3)])
+def test_line_ends(n, r, k, closure):
+    """Short lines of the walks: the closure's end rows."""
+    assert _shift(n, r, k, 40000, closure) <= _bound(n, k, 40000)
