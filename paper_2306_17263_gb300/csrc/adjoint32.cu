@@ -480,6 +480,9 @@ void solve_pair(ms_grid* g, bool of_h) {
     const int f = of_h ? (k ? HY : HX) : EZ, mc = f == HY ? 0 : 1;
     a[k] = make_s(g, f, A->lh[f], nullptr, nf);
     a[k].hi = nullptr;
+    const double q = g->walk.cheb.q[1];
+    a[k].l_hi = (float)q;
+    a[k].l_lo = (float)(q - (double)a[k].l_hi);
     a[k].lo = A->ll[f] + mc;
     a[k].out = A->uc[f] + mc;
     nb[k] = blocks_of(a[k].nstrip * a[k].nblk);

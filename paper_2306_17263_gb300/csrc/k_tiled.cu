@@ -28,8 +28,8 @@
 //
 // The solve is the Chebyshev polynomial of k_rec64.cu, 6 h^2 P1 = D - T with T = (L_x + 6)(L_y + 6), in
 // Horner form y <- b + q T y to a relative error of 1e-10: five operations per point and level.  T y is
-// 7e-3 of D y at most, so an FP32 level rounds the increment at 1e-9 of itself, and the last level's
-// q T y enters the state apart from b, never rounded into it.
+// 36 / D of D y at most (7e-3 at r = 0.5, 2.2e-2 at the stability limit), so an FP32 level rounds the increment at
+// 4e-10 to 1.3e-9 of itself, and the last level's q T y enters the state apart from b, never rounded into it.
 //
 // Why walks: both kernels of the tile form this replaces (64 x 64 tiles in shared memory) were bound by
 // instruction issue, 140-150 warp instructions per 32 points and field.  Derivative along x and solve in
@@ -598,10 +598,13 @@ SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfie
   a.u1 = N;
   a.kind = f == EZ ? KIND_E : (f == HX ? KIND_HX : KIND_HY);
   const Cheb& p = g->walk.cheb;
-  for (int l = 0; l < p.m - 1; ++l) a.q[l] = (float)p.q[p.m - 1 - l];
-  const Split sp = split((f == EZ ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0 * plane_rhs_scale(g));
+  for (int l = 0; l < p.m - 2; ++l) a.q[l] = (float)p.q[p.m - 1 - l];
+  const double s = (f == EZ ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0 * plane_rhs_scale(g);
+  const Split sp = split(s), lp = split(s * p.q[1]);
   a.s_hi = sp.hi;
   a.s_lo = sp.lo;
+  a.l_hi = lp.hi;
+  a.l_lo = lp.lo;
   a.nstrip = (a.M + SOUT - 1) / SOUT;
   // Rows per block: P rows above and below are computed twice, but a grid wants about thirteen warps per
   // SM; small grids are bound by the length of one walk.

@@ -17,8 +17,9 @@ struct SArgs {
   int ld, M;        // unknown columns 0 .. M-1
   int u0, u1;       // unknown rows u0 .. u1-1
   int kind;         // KIND_*
-  float q[4];          // level l + 1 of the solve
-  float s_hi, s_lo;    // increment scale
+  float q[4];          // levels of the solve but for the last
+  float s_hi, s_lo;    // increment scale s
+  float l_hi, l_lo;    // last level: s q (reverse pass: q)
   int nstrip, nblk, rows;
 };
 
@@ -61,14 +62,17 @@ __device__ __forceinline__ void cp_wait() {
 
 // ---- solve and update ----------------------------------------------------------------------
 
-// (hi, lo) += (s_hi + s_lo)(b + c), |c| <= 8e-3 |b|: an exact two-product of s_hi b with the other
-// products in its error term, and a two-sum into the pair.
-__device__ __forceinline__ void ff_add_scaled(float2& hi, float2& lo, float2 b, float2 c, float2 s_hi, float2 n_hi,
-                                              float2 s_lo) {
+// (hi, lo) += s b + l t, s and l hi + lo pairs, |l t| <= 36 / D |s b| over a field (2.2e-2 at the stability
+// limit): an exact two-product of s_hi b with the other products in its error term, and a two-sum into the
+// pair.  One FP32 number each for the last level's q and for s on it were coherent errors of up to 1e-9 of the
+// increment; an earlier level's q is off by (36 / D)^2 2^-25 of it, 1.4e-11 at most.
+__device__ __forceinline__ void ff_add_scaled(float2& hi, float2& lo, float2 b, float2 t, float2 s_hi, float2 n_hi,
+                                              float2 s_lo, float2 l_hi, float2 l_lo) {
   const float2 np = mul2(n_hi, b);  // -p, p = fl(s_hi b)
   float2 e = fma2(s_hi, b, np);
   e = fma2(s_lo, b, e);
-  e = fma2(s_hi, c, e);
+  e = fma2(l_lo, t, e);
+  e = fma2(l_hi, t, e);
   const float2 u = sub2(hi, np);
   const float2 bb = sub2(u, hi);
   const float2 err = sub2(sub2(hi, sub2(u, bb)), add2(np, bb));
@@ -161,7 +165,7 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
   for (int l = 0; l <= P; ++l) b[l][0] = b[l][1] = z2;
 #pragma unroll
   for (int l = 0; l < P; ++l) w[l][0][0] = w[l][0][1] = w[l][1][0] = w[l][1][1] = z2;
-  const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo);
+  const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo), l_hi = bc2(A.l_hi), l_lo = bc2(A.l_lo);
   float* ph = (PAIR ? A.out : A.hi) + off + (size_t)j0 * ld;
   float* pl = A.lo + off + (size_t)j0 * ld;
   const int jend = j1 + P;
@@ -221,7 +225,7 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
           float2 o[2] = {make_float2(sl.x, sl.y), make_float2(sl.z, sl.w)};
           if (PAIR) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) o[k] = fma2(bc2(A.q[P - 1]), tt[k], o[k]);
+            for (int k = 0; k < 2; ++k) o[k] = fma2(l_hi, tt[k], fma2(l_lo, tt[k], o[k]));
             if (!EDGE || m0 + 4 <= M) {
               *reinterpret_cast<float4*>(ph) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
             } else {
@@ -234,7 +238,7 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
             const float4 sh = r[64];
             float2 h[2] = {make_float2(sh.x, sh.y), make_float2(sh.z, sh.w)};
 #pragma unroll
-            for (int k = 0; k < 2; ++k) ff_add_scaled(h[k], o[k], b[P][k], mul2(bc2(A.q[P - 1]), tt[k]), s_hi, n_hi, s_lo);
+            for (int k = 0; k < 2; ++k) ff_add_scaled(h[k], o[k], b[P][k], tt[k], s_hi, n_hi, s_lo, l_hi, l_lo);
             if (!EDGE || m0 + 4 <= M) {
               *reinterpret_cast<float4*>(ph) = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
               *reinterpret_cast<float4*>(pl) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);

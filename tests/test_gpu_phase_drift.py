@@ -69,3 +69,11 @@ def test_smallest_grids(n, r, k, closure):
 def test_line_ends(n, r, k, closure):
     """Short lines of the walks: the closure's end rows."""
     assert _shift(n, r, k, 40000, closure) <= _bound(n, k, 40000)
+
+
+@pytest.mark.parametrize("n, q, k, z", [(64, 96, 4, 1.0), (64, 52, 4, 1.0), (128, 52, 4, 1.3), (256, 57, 8, 1.0),
+                                        (256, 57, 8, 1.3)])
+def test_level_coefficients(n, q, k, z):
+    """The solve's levels at r = sqrt(24 / q), where the filter's coefficient 12 + 24 / r^2 is a whole number; they
+    weigh most near the stability limit."""
+    assert _shift(n, math.sqrt(24.0 / q), k, 40000, pkg.CLOSURE_REFLECT, z) <= _bound(n, k, 40000)
