@@ -13,13 +13,15 @@
 //
 // Differences are taken on the float-float state, delta_m = (hi_{m+1} - hi_m) + (lo_{m+1} - lo_m), and
 // filtered, d = 12 beta delta + L delta (the filter of Eq. "eq:ell" commutes with the difference: D1
-// (12 beta + L) u = (12 beta + L') D1 u with the ghost rules below).  A^{-1} d is the two first-order
+// (12 beta + L) u = (12 beta + L') D1 u with the ghost rules below); L delta, the sum of the four neighbours less 4
+// delta, is formed on its own, small as it is, before the low part of 12 beta joins it: that part is about an ulp of
+// the neighbours' sum and would be rounded the same way everywhere (1e-9 of the filter at r = 0.68).  A^{-1} d is the two first-order
 // recurrences A factors into, z_i = d_i + rho z_{i-1} and y_i = z_i + rho y_{i+1}, up to the factor (1 -
 // rho)^2 that the increment scales carry, each z and y rounded once.  Along y the forward one follows the
 // walk and the backward one runs over groups of eight rows from seven rows beyond (|rho|^8 = 2e-11);
-// along x a lane runs both over its four columns and takes the carries of two lanes on either side.  The closure's end rows
-// change the solution by a multiple of the decaying vector rho^i (LineEnds), added to the first and the
-// last eight rows of a line.
+// along x a lane runs both over its four columns and takes the carries of two lanes on either side.  The closure's
+// end rows change the solution by a multiple of the decaying vector rho^i (LineEnds) in the first and the last
+// eight rows of a line (end_rows).
 //
 // Ghost rules of the difference along a line: a source that is Neumann along it (H_y along x, H_x along
 // y; even ghost u(-1) = u(0), Cor. "cor:ghost_cor") has zero differences beyond the ends; one that is
@@ -56,7 +58,7 @@ struct YArgs {
   const float* sl;
   float* b;         // destination plane, row of output 0, column 0
   int ld, ncol, M, even;
-  float cb_hi, cb_lo;  // 12 beta - 4: coefficient of delta beside the sum of its four neighbours
+  float cb_hi, cb_lo;  // 12 beta
   float g[4], gl[4], v[kEnd];  // end correction, g in pairs
   int nstrip, nseg, chunk, rb;  // column strips; segments of `chunk` rows, the last one [rb, M)
   // grids of at most kTinyN cells: explicit rows of A^{-1}, both derivatives of the half-step
@@ -65,7 +67,6 @@ struct YArgs {
   float* tb[2];                // destinations of those along y and x
   const float *whi, *wlo;
   int K;
-  float tcb_hi, tcb_lo;  // 12 beta
   int filter;
 };
 
@@ -165,7 +166,7 @@ __device__ __forceinline__ void y_segment(const YArgs& A, int strip, int seg) {
           um = m == 0 ? d0 : um;
           up = m == A.M - 1 ? d0 : up;
         }
-        d = fmaf(A.cb_hi, d0, fmaf(A.cb_lo, d0, (a + b) + (um + up)));
+        d = fmaf(A.cb_hi, d0, fmaf(A.cb_lo, d0, fmaf(-4.0f, d0, (a + b) + (um + up))));
       } else {
         d = d0;
       }
@@ -223,7 +224,7 @@ __device__ __forceinline__ void tiny_item(const YArgs& A, int item) {
     if (r == 0) a = A.even ? x : 0.0f;
     if (r == M - 1) b = A.even ? x : 0.0f;
     const float lap = ((a - x) + (b - x)) + ((up - x) + (dn - x));
-    d = fmaf(A.tcb_hi, x, fmaf(A.tcb_lo, x, lap));
+    d = fmaf(A.cb_hi, x, fmaf(A.cb_lo, x, lap));
   }
   // farthest taps first: added after the nearest ones, those beyond the sixth would round away in every sum
   const float *wh = A.whi + r * rs, *wl = A.wlo + r * rs;
@@ -357,7 +358,7 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
         const float2 x = make_float2(d0[k], d0[k + 1]);
         const float2 nb = add2(make_float2(l[k] + r[k], l[k + 1] + r[k + 1]),
                                add2(make_float2(dm[k], dm[k + 1]), make_float2(dp[k], dp[k + 1])));
-        const float2 v = fma2(bc2(A.cb_hi), x, fma2(bc2(A.cb_lo), x, nb));
+        const float2 v = fma2(bc2(A.cb_hi), x, fma2(bc2(A.cb_lo), x, fma2(bc2(-4.0f), x, nb)));
         d[k] = v.x;
         d[k + 1] = v.y;
       }
@@ -527,7 +528,7 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
   a.ncol = N + 1;
   a.M = step == 0 ? N - 1 : N;
   a.even = step == 1;
-  const Split c = split(12.0 * g->beta - 4.0), t = split(12.0 * g->beta);
+  const Split c = split(12.0 * g->beta);
   a.cb_hi = c.hi;
   a.cb_lo = c.lo;
   set_ends(g->walk.ends[kind], &a);
@@ -549,8 +550,6 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
     a.whi = g->pade32[kind].d_whi;
     a.wlo = g->pade32[kind].d_wlo;
     a.K = g->pade32[kind].K;
-    a.tcb_hi = t.hi;
-    a.tcb_lo = t.lo;
     a.nstrip = 1;
     a.nseg = 2 * (N / 2);  // two lines of one axis per item
   }
@@ -571,7 +570,7 @@ XArgs make_x(const ms_grid* g, int step, float* plane, const float* src_hi, cons
   a.M = step == 0 ? N - 1 : N;
   a.u0 = 1;
   a.u1 = N;
-  const Split c = split(12.0 * g->beta - 4.0);
+  const Split c = split(12.0 * g->beta);
   a.cb_hi = c.hi;
   a.cb_lo = c.lo;
   set_ends(g->walk.ends[step == 0 ? HALF_TO_NODE : NODE_TO_HALF], &a);

@@ -77,3 +77,11 @@ def test_level_coefficients(n, q, k, z):
     """The solve's levels at r = sqrt(24 / q), where the filter's coefficient 12 + 24 / r^2 is a whole number; they
     weigh most near the stability limit."""
     assert _shift(n, math.sqrt(24.0 / q), k, 40000, pkg.CLOSURE_REFLECT, z) <= _bound(n, k, 40000)
+
+
+@pytest.mark.parametrize("n, r, k, z", [(17, 0.65, 2, 1.3), (32, 0.68, 3, 1.0), (64, 0.68, 4, 1.3), (128, 0.68, 4, 1.0),
+                                        (256, 0.65, 8, 1.0), (256, 0.65, 8, 1.3)])
+@pytest.mark.parametrize("closure", CLOSURES)
+def test_filter_coefficient(n, r, k, z, closure):
+    """12 beta not exact in FP32."""
+    assert _shift(n, r, k, 40000, closure, z) <= _bound(n, k, 40000)
