@@ -29,6 +29,7 @@
 #include "k_tiled.cuh"
 #include "k_src3.cuh"
 #include "k_transform.cuh"
+#include "k_walk_dev.cuh"
 
 namespace ms {
 
@@ -176,16 +177,7 @@ __global__ void k_mode_field3(double* __restrict__ out, Shape3 s, const double* 
 // ---------------------------------------------------------------------------------------
 // FP32_REFINED kernels
 
-constexpr float kRho3 = -0.045548850f;  // -11 + sqrt(120), the ratio of the recurrences A factors into, in FP32
-
-// Paired FP32 arithmetic (two correctly rounded operations per instruction, sm_100 and later):
-// bitwise the same as the scalar operations on each half.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
 
 // (hi, lo) += (s_hi + s_lo) x with error-free transformations (two-product by FMA, Knuth two-sum), on two
 // independent pairs at once.
@@ -397,7 +389,7 @@ __global__ void k_short3d32(const __grid_constant__ TermArgs2 A, int axis, int o
 // as a rank-one correction.  45 warp instructions per 32 points, where a tile form with the differences in
 // shared memory issued 115: two terms at 256^3 take 88 us (3.0 to 4.6 TB/s), bound by the loads a warp has in
 // flight, and took 130 to 185 us.  Shorter lines are all end rows (k_short3d32).
-constexpr int kWalk3Min = 16, kW3Warps = 4, kEnd3 = 8;
+constexpr int kWalk3Min = 16, kW3Warps = 4;
 struct Walk3Term {
   const float* gh;
   const float* gl;
@@ -411,7 +403,7 @@ struct Walk3Term {
 struct Walk3Args {
   Walk3Term t[2];
   int M, off;
-  float g[4], v[kEnd3], sc_hi, sc_lo;
+  float g[4], gl[4], v[kEnd], sc_hi, sc_lo;
   int nxt, nq, nseg, chunk, rb;  // x tiles, lines along q (largest), segments as in k_tiled.cu
 };
 
@@ -429,26 +421,22 @@ __device__ __forceinline__ void walk3_group(const Walk3Args& A, const float (&ch
     if (EDGE) d = (m0 + t >= 0 && m0 + t < A.M) ? d : 0.0f;
     h0 = ch[t];
     l0 = cl[t];
-    zc[t] = z = fmaf(kRho3, z, d);
+    zc[t] = z = fmaf(kRhoF, z, d);
   }
   float acc = zc[7];
 #pragma unroll
-  for (int t = 6; t >= 1; --t) acc = fmaf(kRho3, acc, zc[t]);
-  y[7] = acc = fmaf(kRho3, acc, zc[0]);
+  for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
+  const float ynext = acc;  // of the row after the group
+  y[7] = acc = fmaf(kRhoF, acc, zc[0]);
 #pragma unroll
-  for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRho3, acc, zp[t]);
+  for (int t = 6; t >= 0; --t) y[t] = acc = fmaf(kRhoF, acc, zp[t]);
+  if (EDGE && (first || final)) {
+    const float zr[8] = {zp[0], zp[1], zp[2], zp[3], zp[4], zp[5], zp[6], zc[0]};
+    if (first) end_rows<false>(y, zr, ynext, end_phi(A, y[0], y[1], y[2], y[3]), A.v);
+    if (final) end_rows<true>(y, zr, ynext, end_phi(A, y[7], y[6], y[5], y[4]), A.v);
+  }
 #pragma unroll
   for (int t = 0; t < 7; ++t) zp[t] = zc[t + 1];
-  if (EDGE && first) {
-    const float phi = fmaf(A.g[0], y[0], fmaf(A.g[1], y[1], fmaf(A.g[2], y[2], A.g[3] * y[3])));
-#pragma unroll
-    for (int t = 0; t < kEnd3; ++t) y[t] = fmaf(A.v[t], phi, y[t]);
-  }
-  if (EDGE && final) {
-    const float phi = fmaf(A.g[0], y[7], fmaf(A.g[1], y[6], fmaf(A.g[2], y[5], A.g[3] * y[4])));
-#pragma unroll
-    for (int t = 0; t < kEnd3; ++t) y[7 - t] = fmaf(A.v[t], phi, y[7 - t]);
-  }
 }
 
 template <bool EDGE>
@@ -507,7 +495,7 @@ __device__ __forceinline__ void walk3_segment(const Walk3Args& A, const Walk3Ter
   }
 }
 
-__global__ void __launch_bounds__(32 * kW3Warps) k_walk3d32(const __grid_constant__ Walk3Args A) {
+__global__ void __launch_bounds__(32 * kW3Warps, 7) k_walk3d32(const __grid_constant__ Walk3Args A) {
   pdl_wait();
   int item = blockIdx.x * kW3Warps + (threadIdx.x >> 5);
   const int xt = item % A.nxt;
@@ -1188,9 +1176,7 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
     Walk3Args A;
     A.M = t.M;
     A.off = off;
-    const LineEnds& e = g->walk.ends[kind];
-    for (int k = 0; k < 4; ++k) A.g[k] = (float)e.g[k];
-    for (int k = 0; k < kEnd3; ++k) A.v[k] = (float)e.v[k];
+    set_ends(g->walk.ends[kind], &A);
     const double sc = walk_rhs_scale();  // (1 - rho)^2, rho the FP32 root
     A.sc_hi = (float)sc;
     A.sc_lo = (float)(sc - (double)A.sc_hi);

@@ -50,8 +50,6 @@
 
 namespace ms {
 
-constexpr int kEnd = 8;  // rows of a line the end correction reaches
-
 // Arguments of a derivative along y: lines are the columns 1 .. ncol-2 of the source.
 struct YArgs {
   const float* sh;  // source, point (0, 0)
@@ -83,24 +81,6 @@ struct XArgs {
 };
 
 namespace {
-
-// phi = g_0 y_0 + .. + g_3 y_3 of the end correction (y counted from the line's end).
-template <typename Args>
-__device__ __forceinline__ float end_phi(const Args& A, float y0, float y1, float y2, float y3) {
-  const float lo = fmaf(A.gl[0], y0, fmaf(A.gl[1], y1, fmaf(A.gl[2], y2, A.gl[3] * y3)));
-  return fmaf(A.g[0], y0, fmaf(A.g[1], y1, fmaf(A.g[2], y2, fmaf(A.g[3], y3, lo))));
-}
-
-// The eight rows at an end of a line with their correction, y_t = z_t + (rho y_{t+1} + v phi).  It joins rho y, a
-// twentieth of y: added to y itself it would round away from the fifth row on, always the same way (frequencies of
-// small grids off by 1e-9 to 3e-9; 1e-10 to 4e-10 this way).  v is one FP32 number each, an error of 6e-11 y.
-template <bool LAST>
-__device__ __forceinline__ void end_rows(float (&y)[8], const float (&z)[8], float ynext, float phi,
-                                         const float (&v)[kEnd]) {
-#pragma unroll
-  for (int t = 0; t < kEnd; ++t)
-    y[t] = z[t] + fmaf(v[LAST ? kEnd - 1 - t : t], phi, kRhoF * (t < kEnd - 1 ? y[t + 1 < kEnd ? t + 1 : t] : ynext));
-}
 
 // ---- derivative along y --------------------------------------------------------------------------------
 
@@ -495,26 +475,6 @@ __global__ void __launch_bounds__(32 * WPB, P <= 3 ? 5 : 4) k_batch_s(const SArg
 }
 
 // ---- host ----------------------------------------------------------------------------------
-
-struct Split {
-  float hi, lo;
-};
-Split split(double v) {
-  Split s;
-  s.hi = (float)v;
-  s.lo = (float)(v - (double)s.hi);
-  return s;
-}
-
-template <typename Args>
-void set_ends(const LineEnds& e, Args* a) {
-  for (int k = 0; k < 4; ++k) {
-    const Split g = split(e.g[k]);
-    a->g[k] = g.hi;
-    a->gl[k] = g.lo;
-  }
-  for (int k = 0; k < kEnd; ++k) a->v[k] = (float)e.v[k];
-}
 
 YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const float* src_hi, const float* src_lo) {
   YArgs a{};

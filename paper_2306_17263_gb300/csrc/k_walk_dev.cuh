@@ -1,5 +1,5 @@
-// Device code shared by the FP32 walks of the step (k_tiled.cu) and of the reverse pass (adjoint32.cu):
-// constants, paired arithmetic, the row ring and the solve.
+// Device code shared by the FP32 walks of the 2D step (k_tiled.cu), of the reverse pass (adjoint32.cu) and of the
+// 3D step (grid3d.cu): constants, paired arithmetic, line ends, the row ring and the 2D solve.
 #pragma once
 
 #include "k_fp64.cuh"
@@ -34,6 +34,7 @@ constexpr int XHALO = 8;
 constexpr int SOUT = 120;   // columns a walk_s warp writes
 constexpr int SHALO = 4;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kEnd = 8;     // rows of a line the end correction reaches
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
@@ -44,6 +45,44 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
+
+// phi = g_0 y_0 + .. + g_3 y_3 of the end correction (y counted from the line's end).
+template <typename Args>
+__device__ __forceinline__ float end_phi(const Args& A, float y0, float y1, float y2, float y3) {
+  const float lo = fmaf(A.gl[0], y0, fmaf(A.gl[1], y1, fmaf(A.gl[2], y2, A.gl[3] * y3)));
+  return fmaf(A.g[0], y0, fmaf(A.g[1], y1, fmaf(A.g[2], y2, fmaf(A.g[3], y3, lo))));
+}
+
+// The eight rows at an end of a line with their correction, y_t = z_t + (rho y_{t+1} + v phi).  It joins rho y, a
+// twentieth of y: added to y itself it would round away from the fifth row on, always the same way (frequencies of
+// small grids off by 1e-9 to 3e-9; 1e-10 to 4e-10 this way).  v is one FP32 number each, an error of 6e-11 y.
+template <bool LAST>
+__device__ __forceinline__ void end_rows(float (&y)[8], const float (&z)[8], float ynext, float phi,
+                                         const float (&v)[kEnd]) {
+#pragma unroll
+  for (int t = 0; t < kEnd; ++t)
+    y[t] = z[t] + fmaf(v[LAST ? kEnd - 1 - t : t], phi, kRhoF * (t < kEnd - 1 ? y[t + 1 < kEnd ? t + 1 : t] : ynext));
+}
+
+// Host: a coefficient as a pair, and the end corrections of a kind of line.
+struct Split {
+  float hi, lo;
+};
+inline Split split(double v) {
+  Split s;
+  s.hi = (float)v;
+  s.lo = (float)(v - (double)s.hi);
+  return s;
+}
+template <typename Args>
+void set_ends(const LineEnds& e, Args* a) {
+  for (int k = 0; k < 4; ++k) {
+    const Split g = split(e.g[k]);
+    a->g[k] = g.hi;
+    a->gl[k] = g.lo;
+  }
+  for (int k = 0; k < kEnd; ++k) a->v[k] = (float)e.v[k];
+}
 
 // Rows come through a ring in shared memory that each warp fills for itself with cp.async, kAhead rows
 // ahead: the walk of a row is shorter than a memory round trip, and the registers are taken.  A slot is

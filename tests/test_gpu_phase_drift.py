@@ -85,3 +85,30 @@ def test_level_coefficients(n, q, k, z):
 def test_filter_coefficient(n, r, k, z, closure):
     """12 beta not exact in FP32."""
     assert _shift(n, r, k, 40000, closure, z) <= _bound(n, k, 40000)
+
+
+def _shift3(n, r, steps, closure, z=1.3):
+    """The same in 3D for the mode (2, 1, 2): E and H projected on their own shapes at the start."""
+    w = 3.0 * math.pi
+    ph = []
+    for precision in (pkg.FP64, pkg.FP32_REFINED):
+        with pkg.Grid(n, r, z=z, precision=precision, closure=closure, dim=3) as g:
+            g.init_modes([(2, 1, 2, 1.0, 0.0, -1.0)])
+            s = g.get_fields()
+            g.run(steps)
+            f = g.get_fields()
+        e, h = (sum(np.sum(a * b) for a, b in zip(f[q], s[q])) / sum(np.sum(b * b) for b in s[q])
+                for q in (slice(0, 3), slice(3, 6)))
+        ph.append(math.atan2(h * math.sin(0.5 * w * r / n), e))
+    d = (ph[1] - ph[0] + math.pi) % (2.0 * math.pi) - math.pi
+    return abs(d) / (w * steps * r / n)
+
+
+def _bound3(n, steps):
+    return 1e-10 + 2e-9 * (2.0 * math.pi / n) ** 2 + 16.0 * 2.0 ** -24 / ((n - 1) ** 1.5 * math.sqrt(steps))
+
+
+@pytest.mark.parametrize("closure", CLOSURES)
+@pytest.mark.parametrize("n, r", [(17, 0.4), (20, 0.3), (24, 0.4)])
+def test_line_ends_3d(n, r, closure):
+    assert _shift3(n, r, 10000, closure) <= _bound3(n, 10000)
