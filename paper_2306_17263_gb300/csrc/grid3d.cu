@@ -614,8 +614,8 @@ __global__ void __launch_bounds__(32 * kWXWarps) k_walkx3d32(const __grid_consta
 // T y = 2 e + c + (2 y + e)_{z-1} + (2 y + e)_{z+1}, e and c the sums over the four edge and the four
 // corner neighbours in the plane, spectrum [-8, 24].  The Chebyshev polynomial of k_rec64.cu in Horner
 // form, y <- b + q T y, to a relative error of 1e-10, one level per launch for the three components; T y
-// is 2e-3 of D y at most, so a level rounds the increment at 1e-9 of itself, and the last level's q T y
-// enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches along z; the
+// is 24 / D of D y at most (2e-3 at r = 0.4, 7e-3 at the stability limit), so a level rounds the increment at 1e-10
+// to 4e-10 of itself, and the last level's q T y enters the state apart from b.  A block takes a tile of 32 x 16 columns and marches along z; the
 // planes come through a ring in shared memory filled by cp.async kA3 planes ahead (loads straight
 // into registers, one plane ahead, left the march waiting for them: 180 to 225 us per level of three
 // components at 256^3), and a thread keeps e, c and q = 2 y + e of its four rows in registers as two pairs:
@@ -631,25 +631,10 @@ struct Lev3d32Args {
   float* out[3];         // iterate (not LAST)
   float *hi[3], *lo[3];  // state (LAST)
   Shape3 s[3];
-  float q, s_hi, s_lo;
+  float q;                       // of this level (not LAST)
+  float s_hi, s_lo, l_hi, l_lo;  // increment scale s, s q (LAST)
   int nz, zc;  // marches along z of the largest component, planes per march
 };
-
-// (hi, lo) += (s_hi + s_lo)(b + c): an exact two-product of s_hi b with the other products in its error
-// term, and a two-sum into the pair; two points at once.
-__device__ __forceinline__ void ff_add_scaled_bc(float2& hi, float2& lo, float2 b, float2 c, float2 s_hi, float2 s_lo) {
-  const float2 p = mul2(s_hi, b);
-  float2 e = fma2(s_hi, b, neg2(p));
-  e = fma2(s_lo, b, e);
-  e = fma2(s_hi, c, e);
-  const float2 u = add2(hi, p);
-  const float2 bb = sub2(u, hi);
-  const float2 err = add2(sub2(hi, sub2(u, bb)), sub2(p, bb));
-  const float2 l = add2(lo, add2(err, e));
-  const float2 h2 = add2(u, l);
-  lo = sub2(l, sub2(h2, u));
-  hi = h2;
-}
 
 // FIRST: y is b itself.
 template <bool FIRST, bool LAST>
@@ -711,6 +696,7 @@ __global__ void __launch_bounds__(L3T, LAST ? 5 : 7) k_lev3d32(const __grid_cons
   };
   float2 qm[2] = {}, q0[2] = {}, u0[2] = {}, m0[2] = {};  // q of planes k - 1, k; 2 e + c and y of plane k
   const float2 two = bc2(2.0f), q = bc2(A.q);
+  const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo), l_hi = bc2(A.l_hi), l_lo = bc2(A.l_lo);
   unsigned g = k0 * sz + own;
 #pragma unroll 4
   for (int st = 0; st < S; ++st) {
@@ -753,7 +739,7 @@ __global__ void __launch_bounds__(L3T, LAST ? 5 : 7) k_lev3d32(const __grid_cons
       const float2 e = add2(x[t + 1], add2(m[t], m[t + 2]));
       const float2 qn = fma2(two, m[t + 1], e);
       const float2 T = add2(u0[t], add2(qm[t], qn));
-      if (LAST) ff_add_scaled_bc(hc[t], lc[t], bc[t], mul2(q, T), bc2(A.s_hi), bc2(A.s_lo));
+      if (LAST) ff_add_scaled(hc[t], lc[t], bc[t], T, s_hi, n_hi, s_lo, l_hi, l_lo);
       else v[t] = fma2(q, T, bc[t]);
       qm[t] = q0[t];
       q0[t] = qn;
@@ -1289,8 +1275,11 @@ void solve3d32(ms_grid* g, int c0, const MixedConsts& k, int* nl) {
     pts += (double)s.size();
   }
   const double s = (e ? 12.0 * g->Z / g->desc.r : 12.0 / (g->desc.r * g->Z)) * p.p0;
-  A.s_hi = (float)s;
-  A.s_lo = (float)(s - (double)A.s_hi);
+  const Split sp = split(s), lp = split(s * p.q[1]);
+  A.s_hi = sp.hi;
+  A.s_lo = sp.lo;
+  A.l_hi = lp.hi;
+  A.l_lo = lp.lo;
   A.zc = march_planes(3 * tx * ty, nz);
   A.nz = (nz + A.zc - 1) / A.zc;
   const dim3 grd(tx, ty, 3 * A.nz), blk(32, L3Y);

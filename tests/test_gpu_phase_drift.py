@@ -112,3 +112,9 @@ def _bound3(n, steps):
 @pytest.mark.parametrize("n, r", [(17, 0.4), (20, 0.3), (24, 0.4)])
 def test_line_ends_3d(n, r, closure):
     assert _shift3(n, r, 10000, closure) <= _bound3(n, 10000)
+
+
+@pytest.mark.parametrize("r, z", [(0.515, 2.0), (0.54, 1.0), (0.55, 1.0)])
+def test_level_coefficients_3d(r, z):
+    """Where the last level's coefficient and the increment scale are farthest from FP32 numbers."""
+    assert _shift3(64, r, 4000, pkg.CLOSURE_REFLECT, z) <= _bound3(64, 4000)
