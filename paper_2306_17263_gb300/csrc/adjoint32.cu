@@ -88,7 +88,7 @@ struct YTArgs {
   const float* ul;
   float* b;         // row of output 0
   int ld, ncol, M;
-  float k[kEndT];
+  float k[kEndT], kl[kEndT];  // end correction, in pairs
   int nstrip, nseg, chunk, end;  // segments: 0 down from the first end, 1 up from the last (`end` rows
                                  // each), the others `chunk` rows down between them
 };
@@ -101,7 +101,7 @@ struct XTArgs {
   int ld, M;     // inputs per line
   int from_h;    // input u_i at column i of H_y, output j at column j - 1 of E_z; else u_i at column i of
                  // E_z, output j at column j of H_y
-  float k[kEndT];
+  float k[kEndT], kl[kEndT];
   int nrows, nstrip, nblk, rows;
 };
 
@@ -131,7 +131,7 @@ __device__ __forceinline__ void yt_segment(const YTArgs& A, int strip, int seg) 
     nh[t] = get(ph, ms + t);
     nl[t] = get(pl, ms + t);
   }
-  float z = 0.0f, ep[7] = {}, gp[7] = {}, w0 = 0.0f;
+  float z = 0.0f, ep[7] = {}, gp[7] = {}, w0 = 0.0f, w0l = 0.0f;
   const int ngrp = 2 + (r1 - r0 + 7) / 8;
   for (int gi = 0; gi < ngrp; ++gi) {
     const int m0 = ms + 8 * gi;
@@ -159,22 +159,30 @@ __device__ __forceinline__ void yt_segment(const YTArgs& A, int strip, int seg) 
     float acc = zc[7];
 #pragma unroll
     for (int t = 6; t >= 1; --t) acc = fmaf(kRhoF, acc, zc[t]);
+    const float ynext = acc;
     y[7] = acc = ec[0] + fmaf(kRhoF, acc, gc[0]);
 #pragma unroll
     for (int t = 6; t >= 0; --t) y[t] = acc = ep[t] + fmaf(kRhoF, acc, gp[t]);
+    if (EDGE && seg < 2 && gi >= 2 && gi < 2 + kEndT / 8) {  // the first end's rows
+      float n[8];                                             // y less e
+#pragma unroll
+      for (int t = 0; t < 8; ++t) n[t] = fmaf(kRhoF, t < 7 ? y[t < 7 ? t + 1 : t] : ynext, t < 7 ? gp[t < 7 ? t : 0] : gc[0]);
+      if (gi == 2) {
+        w0 = y[0];
+        w0l = n[0] - (w0 - ep[0]);
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int j = 8 * (gi - 2) + t;
+        y[t] = (t < 7 ? ep[t < 7 ? t : 0] : ec[0]) + fmaf(A.k[j], w0, fmaf(A.kl[j], w0, fmaf(A.k[j], w0l, n[t])));
+      }
+    }
 #pragma unroll
     for (int t = 0; t < 7; ++t) {
       ep[t] = ec[t + 1];
       gp[t] = gc[t + 1];
     }
     if (gi < 2) continue;
-    if (EDGE && seg < 2) {  // the first end's rows
-      if (gi == 2) w0 = y[0];
-      if (gi < 2 + kEndT / 8) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) y[t] = fmaf(A.k[8 * (gi - 2) + t], w0, y[t]);
-      }
-    }
     if (live) {
       const int left = r1 - (r0 + 8 * (gi - 2));
 #pragma unroll
@@ -205,7 +213,7 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
   const bool ok = !EDGE || (m0 >= -4 && m0 + 8 <= A.ld);
   const bool out = lane >= THALO / 4 && lane < (THALO + TOUT) / 4 && (!EDGE || (m0 >= 0 && m0 < Mo));
   bool inu[4] = {true, true, true, true}, ine[4] = {true, true, true, true};
-  float kl[4] = {}, kr[4] = {};
+  float kl[4] = {}, kr[4] = {}, kll[4] = {}, krl[4] = {};
   bool left = false, right = false;
   int ll = 0, el = 0, lr = 0, er = 0;  // lane and element of output 0 and of output M
   if (EDGE) {
@@ -222,6 +230,8 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
       ine[q] = j >= 0 && j <= M;
       kl[q] = (left && j >= 0 && j < kEndT) ? A.k[j & (kEndT - 1)] : 0.0f;
       kr[q] = (right && r >= 0 && r < kEndT) ? A.k[r & (kEndT - 1)] : 0.0f;
+      kll[q] = (left && j >= 0 && j < kEndT) ? A.kl[j & (kEndT - 1)] : 0.0f;
+      krl[q] = (right && r >= 0 && r < kEndT) ? A.kl[r & (kEndT - 1)] : 0.0f;
     }
   }
   const size_t off = ok ? m0 : 0;
@@ -302,15 +312,27 @@ __device__ __forceinline__ void xt_block(const XTArgs& A, float4* ring, int stri
       c2 = lane > 29 ? 0.0f : c2;
     }
     c = fmaf(kR4, c2, c1);
+    float n[4];  // y less e
 #pragma unroll
-    for (int q = 3; q >= 0; --q) c = y[q] = e[q] + fmaf(kRhoF, c, l[q]);
+    for (int q = 3; q >= 0; --q) {
+      n[q] = fmaf(kRhoF, c, l[q]);
+      c = y[q] = e[q] + n[q];
+    }
     if (EDGE) {
-      auto pick = [&](int e) { return e == 0 ? y[0] : (e == 1 ? y[1] : (e == 2 ? y[2] : y[3])); };
-      float wl = 0.0f, wrt = 0.0f;
-      if (left) wl = __shfl_sync(kFull, pick(el), ll);
-      if (right) wrt = __shfl_sync(kFull, pick(er), lr);
+      auto pick = [&](const float(&v)[4], int e) { return e == 0 ? v[0] : (e == 1 ? v[1] : (e == 2 ? v[2] : v[3])); };
+      // c += (k + kl) (w + wl), w + wl = output 0 (or M) of the infinite line
+      auto end = [&](const float(&k)[4], const float(&kl)[4], float(&c)[4], int lane0, int el0) {
+        const float pe = pick(e, el0), pn = pick(n, el0);
+        const float w = pe + pn;
+        const float wh = __shfl_sync(kFull, w, lane0), wl = __shfl_sync(kFull, pn - (w - pe), lane0);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) y[q] = fmaf(kr[q], wrt, fmaf(kl[q], wl, y[q]));
+        for (int q = 0; q < 4; ++q) c[q] = fmaf(k[q], wh, fmaf(kl[q], wh, fmaf(k[q], wl, c[q])));
+      };
+      float c4[4] = {n[0], n[1], n[2], n[3]};
+      if (left) end(kl, kll, c4, ll, el);
+      if (right) end(kr, krl, c4, lr, er);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] = e[q] + c4[q];
     }
     if (out) *reinterpret_cast<float4*>(bp) = make_float4(y[0], y[1], y[2], y[3]);  // (pads: never read unmasked)
   }
@@ -417,14 +439,16 @@ int blocks_of(int items) { return (items + WPB - 1) / WPB; }
 
 // The end correction of the transposed derivative: v = y + t (y_0) with t the vector of the closure's
 // A^{-T} (LineEnds), t_{-1} = -rho, so k_j = (t_{j-1} - t_j) / (rho - 1) on w_0 = (rho - 1) y_0.
-void end_rows_T(int closure, int kind, float* k) {
+void end_rows_T(int closure, int kind, float* k, float* kl) {
   LineEnds e;
   line_ends(closure, kind, true, &e);
   const double rho = (double)kRhoF;
   double prev = -rho;
   for (int j = 0; j < kEndT; ++j) {
     const double t = j < kRecWarm ? e.v[j] : 0.0;
-    k[j] = (float)((prev - t) / (rho - 1.0));
+    const Split p = split((prev - t) / (rho - 1.0));
+    k[j] = p.hi;
+    kl[j] = p.lo;
     prev = t;
   }
 }
@@ -444,8 +468,11 @@ void derivatives_T(ms_grid* g, bool from_h) {
   y.ul = A->uc[ys] + row1;
   y.b = A->py[yd];
   y.ncol = N + 1;
-  end_rows_T(g->desc.closure, kind, y.k);
-  for (int j = 0; j < kEndT; ++j) x.k[j] = y.k[j];
+  end_rows_T(g->desc.closure, kind, y.k, y.kl);
+  for (int j = 0; j < kEndT; ++j) {
+    x.k[j] = y.k[j];
+    x.kl[j] = y.kl[j];
+  }
   y.nstrip = (N - 1 + 31) / 32;
   const int R = y.M + 1;
   const int rows = y.nstrip * (R / 64) >= 1500 ? 64 : 32;
@@ -480,9 +507,9 @@ void solve_pair(ms_grid* g, bool of_h) {
     const int f = of_h ? (k ? HY : HX) : EZ, mc = f == HY ? 0 : 1;
     a[k] = make_s(g, f, A->lh[f], nullptr, nf);
     a[k].hi = nullptr;
-    const double q = g->walk.cheb.q[1];
-    a[k].l_hi = (float)q;
-    a[k].l_lo = (float)(q - (double)a[k].l_hi);
+    const Split q = split(g->walk.cheb.q[1]);
+    a[k].l_hi = q.hi;
+    a[k].l_lo = q.lo;
     a[k].lo = A->ll[f] + mc;
     a[k].out = A->uc[f] + mc;
     nb[k] = blocks_of(a[k].nstrip * a[k].nblk);
