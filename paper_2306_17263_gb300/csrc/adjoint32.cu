@@ -358,56 +358,53 @@ __global__ void __launch_bounds__(32 * WPB) k_walk_dT(const __grid_constant__ YT
 
 // ---- filter and update ---------------------------------------------------------------------
 
-// l (hi, lo) += s (12 beta y + L y) at the unknowns of a field, y = p1 + p2 (or p1) there, 0 on
-// Dirichlet walls, mirrored across Neumann ones.  Bound by memory: a lane takes four columns of a row.
+// l (hi, lo) += s (12 beta y + L y) at the unknowns of a field, y = px + py there (E_z; the H fields have one of
+// them), 0 on Dirichlet walls, mirrored across Neumann ones.  Bound by memory: a lane takes four columns of a row.
+// rho of the recurrences is an FP32 number, off by d = 1.1e-9, which multiplies a derivative's symbol along its line
+// by 1 + kRhoErr L to first order (its gain at theta = 0 is exact); 12 beta y takes that back: without it the
+// gradient after 2000 steps at 32^2 was off by 2.3e-6, 1.1e-6 of it rounding.
+constexpr double kRho = -0.045548849896677730860604;  // -11 + sqrt(120)
+constexpr double kRhoErr = ((double)kRhoF - kRho) * (1.0 + kRho) / ((1.0 - kRho) * (1.0 - kRho) * (1.0 - kRho));
 struct FArgs {
-  const float* p1;  // at column m = 0 of row 0
-  const float* p2;
+  const float* px;  // derivative along x, at column m = 0 of row 0 (E_z, H_y)
+  const float* py;  // along y (E_z, H_x)
   float* lh;
   float* ll;
-  int ld, M, u0, u1, neu_x, neu_y;
-  float c_hi, c_lo, s;  // 12 beta s, s
+  int ld, M, u0, u1;
+  float c_hi, c_lo, s_hi, s_lo;  // 12 beta s, s
+  float r;                       // -12 beta s kRhoErr
 };
 struct FArgs2 {
   FArgs f[2];
 };
 constexpr int FY = 8;
-__global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant__ FArgs2 A2) {
-  pdl_wait();
-  const FArgs& A = A2.f[blockIdx.z];
+// F: the field (E_z has both parts, H_x the one along y, H_y the one along x).
+template <int F>
+__device__ __forceinline__ void filter_update4(const FArgs& A) {
+  constexpr bool PX = F != HX, PY = F != HY;
   const int m0 = 4 * (blockIdx.x * 32 + threadIdx.x), j = A.u0 + blockIdx.y * FY + threadIdx.y;
   if (m0 >= A.M || j >= A.u1) return;
   const size_t ld = A.ld;
   const int M = A.M;
   // rows above and below: 0 beyond a Dirichlet wall, the row itself across a Neumann one
+  constexpr bool neu_x = F == HY, neu_y = F == HX;
   const int ja = j > A.u0 ? j - 1 : j, jb = j + 1 < A.u1 ? j + 1 : j;
-  const bool oka = j > A.u0 || A.neu_y, okb = j + 1 < A.u1 || A.neu_y;
-  auto row = [&](int r, bool ok, float(&y)[4]) {
-    if (!ok) {
-      y[0] = y[1] = y[2] = y[3] = 0.0f;
-      return;
-    }
-    float4 a = ld4(A.p1 + r * ld + m0);
-    if (A.p2) {
-      const float4 b = ld4(A.p2 + r * ld + m0);
-      a = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-    }
-    y[0] = a.x;
-    y[1] = a.y;
-    y[2] = a.z;
-    y[3] = a.w;
+  const bool oka = j > A.u0 || neu_y, okb = j + 1 < A.u1 || neu_y;
+  struct Row {
+    float v[4];
   };
-  auto one = [&](int m) { return A.p1[j * ld + m] + (A.p2 ? A.p2[j * ld + m] : 0.0f); };
-  float y[4], a[4], b[4];
-  row(j, true, y);
-  row(ja, oka, a);
-  row(jb, okb, b);
+  auto row = [&](bool part, const float* p, int r, bool ok) {
+    const float4 a = part && ok ? ld4(p + r * ld + m0) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    return Row{{a.x, a.y, a.z, a.w}};
+  };
+  auto one = [&](bool part, const float* p, int m) { return part ? p[j * ld + m] : 0.0f; };
+  const Row x = row(PX, A.px, j, true), xa = row(PX, A.px, ja, oka), xb = row(PX, A.px, jb, okb);
+  const Row z = row(PY, A.py, j, true), za = row(PY, A.py, ja, oka), zb = row(PY, A.py, jb, okb);
+  auto sum = [&](float a, float b) { return PX && PY ? a + b : (PX ? a : b); };
   // columns beside the four, and those past the field
-  const float yl = m0 > 0 ? one(m0 - 1) : (A.neu_x ? y[0] : 0.0f);
-  float l[4] = {yl, y[0], y[1], y[2]}, r[4] = {y[1], y[2], y[3], m0 + 4 < M ? one(m0 + 4) : 0.0f};
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (m0 + q == M - 1) r[q] = A.neu_x ? y[q] : 0.0f;
+  const bool in0 = m0 > 0, in1 = m0 + 4 < M;
+  const float xl = in0 ? one(PX, A.px, m0 - 1) : (neu_x ? x.v[0] : 0.0f), xr = in1 ? one(PX, A.px, m0 + 4) : 0.0f;
+  const float zl = in0 ? one(PY, A.py, m0 - 1) : 0.0f, zr = in1 ? one(PY, A.py, m0 + 4) : 0.0f;
   float* ph = A.lh + j * ld + m0;
   float* pl = A.ll + j * ld + m0;
   const float4 H = ld4(ph), L = ld4(pl);
@@ -415,12 +412,24 @@ __global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (m0 + q >= M) continue;  // the pads keep their zeros
+    const bool wall = m0 + q == M - 1;
+    const float xq = x.v[q], zq = z.v[q], y = sum(xq, zq);
+    const float lx = q ? x.v[q ? q - 1 : 0] : xl, lz = q ? z.v[q ? q - 1 : 0] : zl;
+    const float rx = wall ? (neu_x ? xq : 0.0f) : (q < 3 ? x.v[q < 3 ? q + 1 : 0] : xr);
+    const float rz = wall ? 0.0f : (q < 3 ? z.v[q < 3 ? q + 1 : 0] : zr);
     // an exact two-product of 12 beta s y; s L y, first differences, joins its error term
-    const float lap = ((l[q] - y[q]) + (r[q] - y[q])) + ((a[q] - y[q]) + (b[q] - y[q]));
-    const float p = __fmul_rn(A.c_hi, y[q]);
-    float e = fmaf(A.c_hi, y[q], -p);
-    e = fmaf(A.c_lo, y[q], e);
-    e = fmaf(A.s, lap, e);
+    const float ly = (sum(xa.v[q], za.v[q]) - y) + (sum(xb.v[q], zb.v[q]) - y);
+    const float lap = ((sum(lx, lz) - y) + (sum(rx, rz) - y)) + ly;
+    float along = PX ? (lx - xq) + (rx - xq) : ly;
+    if (PX && PY) along += (za.v[q] - zq) + (zb.v[q] - zq);
+    const float p = __fmul_rn(A.c_hi, y);
+    float e = fmaf(A.c_hi, y, -p);
+    e = fmaf(A.c_lo, y, e);
+    if (PX && PY) {  // what px + py rounds away
+      const float yb = __fsub_rn(y, xq);
+      e = fmaf(A.c_hi, __fadd_rn(__fsub_rn(xq, __fsub_rn(y, yb)), __fsub_rn(zq, yb)), e);
+    }
+    e = fmaf(A.s_hi, lap, fmaf(A.s_lo, lap, fmaf(A.r, along, e)));
     const float u = __fadd_rn(h[q], p);
     const float bb = __fsub_rn(u, h[q]);
     const float err = __fadd_rn(__fsub_rn(h[q], __fsub_rn(u, bb)), __fsub_rn(p, bb));
@@ -431,6 +440,14 @@ __global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant
   }
   *reinterpret_cast<float4*>(ph) = make_float4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<float4*>(pl) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+template <bool OF_H>
+__global__ void __launch_bounds__(32 * FY) k_filter_update(const __grid_constant__ FArgs2 A) {
+  pdl_wait();
+  if (!OF_H) filter_update4<EZ>(A.f[0]);
+  else if (blockIdx.z == 0) filter_update4<HX>(A.f[0]);
+  else filter_update4<HY>(A.f[1]);
 }
 
 // ---- host ----------------------------------------------------------------------------------
@@ -526,21 +543,22 @@ FArgs filter_args(ms_grid* g, int f) {
   Adj32* A = g->adj32;
   const int N = g->N, mc = f == HY ? 0 : 1;
   FArgs a{};
-  a.p1 = (f == HX ? A->py[HX] : A->px[f]) + mc;
-  a.p2 = f == EZ ? A->py[EZ] + mc : nullptr;
+  a.px = f == HX ? nullptr : A->px[f] + mc;
+  a.py = f == HY ? nullptr : A->py[f] + mc;
   a.lh = A->lh[f] + mc;
   a.ll = A->ll[f] + mc;
   a.ld = g->ld32;
   a.M = f == HY ? N : N - 1;
   a.u0 = f == HX ? 0 : 1;
   a.u1 = N;
-  a.neu_x = f == HY;
-  a.neu_y = f == HX;
   const double sc = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * g->walk.cheb.p0 * walk_rhs_scale();
   const double c = 12.0 * g->beta * sc;
-  a.c_hi = (float)c;
-  a.c_lo = (float)(c - (double)a.c_hi);
-  a.s = (float)sc;
+  const Split cp = split(c), sp = split(sc);
+  a.c_hi = cp.hi;
+  a.c_lo = cp.lo;
+  a.s_hi = sp.hi;
+  a.s_lo = sp.lo;
+  a.r = (float)(-c * kRhoErr);
   return a;
 }
 
@@ -549,7 +567,8 @@ void filter_update(ms_grid* g, bool of_h) {
   A.f[0] = filter_args(g, of_h ? HX : EZ);
   A.f[1] = filter_args(g, of_h ? HY : EZ);
   const dim3 grd((g->N + 127) / 128, (g->N + FY - 1) / FY, of_h ? 2 : 1), blk(32, FY);
-  launch_pdl(k_filter_update, grd, blk, 0, g->stream, A);
+  if (of_h) launch_pdl(k_filter_update<true>, grd, blk, 0, g->stream, A);
+  else launch_pdl(k_filter_update<false>, grd, blk, 0, g->stream, A);
 }
 
 // One transposed step on the float-float adjoint state.

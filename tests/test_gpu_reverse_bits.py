@@ -50,3 +50,9 @@ CLOSURES = [pkg.CLOSURE_PAPER, pkg.CLOSURE_REFLECT]
 @pytest.mark.parametrize("n, r, k, steps", [(33, 0.65, 3, 40000), (128, 0.65, 4, 20000)])
 def test_line_ends(n, r, k, steps, closure):
     assert _shift(n, r, k, steps, closure, 1.0) <= _bound(n, k, steps, with_rho=True)
+
+
+@pytest.mark.parametrize("n, r, k, z", [(32, 0.5, 10, 1.0), (32, 0.5, 10, 1.3), (64, 0.68, 20, 1.0), (64, 0.65, 12, 1.3)])
+def test_filter_coefficients(n, r, k, z):
+    """Short waves: rho of the recurrences, s and 12 beta s of the filter."""
+    assert _shift(n, r, k, 40000, pkg.CLOSURE_REFLECT, z) <= _bound(n, k, 40000)
