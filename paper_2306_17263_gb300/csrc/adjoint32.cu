@@ -18,18 +18,21 @@
 // e_j = u_{j-1} - u_j (u_{-1} = u_M = 0, zero beyond the line) and w the infinite-line solution for e,
 // (Y^T u)_j = w_j + k_j w_0 near the first end and its mirror image at the last (the end rows of A^{-T}
 // change v by a multiple of its first value, and w_0 = (rho - 1) v_0).  The difference of the high parts is
-// kept apart from that of the low parts and the recurrences' rho z, both a twentieth of it or less, until w
+// kept apart from that of the low parts, the recurrences' rho z and the end correction, all small beside it, until w
 // itself is rounded: one rounding of w's size per value, as in a float-float A^{-1} whose result is differenced.
-// u = p_0 (l + c), c the last level
-// of the solve's polynomial applied to l_hi: the pair (l_hi, l_lo + c) holds it to about 31 bits without
-// a new high part.  The filter and the scaling act on the difference, a well-conditioned FP32 value, and
-// the result is added to l with error-free transformations.  The step is the transpose of the
-// FP32_REFINED forward operator up to this rounding.
+//   u is a pair (l_hi, uc) over the value of the solve's polynomial at t = 36, where smooth fields sit, so that
+// uc, the rest, holds only what (T - 36) makes of them: its rounding, which the difference amplifies too, is that of
+// a second difference.  As p_0 (l_hi, l_lo + q T y) before, uc was 36 / D of l_hi (1.8e-2 at r = 0.65) and a step's
+// derivatives at 2048^2 were off by 1.3e-7 of themselves, 5.3e-8 by the Richardson solve before that, 3.2e-8 now
+// (1024^2, r = 0.5: 3.5e-8, 3.6e-8, 2.6e-8).
+//   The filter and the scaling act on the difference, a well-conditioned FP32 value, and the result is added to l
+// with error-free transformations.  The step is the transpose of the FP64 operator up to this rounding.  Gradients
+// after 2000 steps at 1024^2 stand 1.9e-8 from the FP64 reverse pass (bands and sweeps: 2.2e-8).
 //
 // Kernels, six launches per reverse step, the walks of k_tiled.cu turned round: solve (k_solve_pair),
 // both transposed derivatives into planes (k_walk_dT), filter and update (k_filter_update), for the H
-// fields and then for E_z.  The band form before it (separate sweeps, transposed bands in float-float, one
-// kernel per operator, 18 launches) took 165 us per reverse step at 1024^2.
+// fields and then for E_z: 43 us per step at 1024^2, 124 at 2048^2.  The band form before it (separate sweeps,
+// transposed bands in float-float, one kernel per operator, 18 launches) took 165 and 506 us.
 #include <string>
 #include <vector>
 
@@ -45,7 +48,7 @@ struct Adj32 {
   float* slab = nullptr;
   float* lh[3] = {};  // adjoint state (l_E, l_Hx, l_Hy), hi parts
   float* ll[3] = {};  // lo parts
-  float* uc[3] = {};  // low parts of the solutions u = p_0 (l_hi + uc)
+  float* uc[3] = {};  // low parts of the solutions, u = gain (l_hi + uc)
   float* py[3] = {};  // transposed derivatives along y (E_z, H_x) and ...
   float* px[3] = {};  // ... along x (E_z, H_y)
   Graph g1, gk;
@@ -70,8 +73,10 @@ constexpr int THALO = 12;
 
 // ---- solve ---------------------------------------------------------------------------------
 
+// (Four blocks per SM with three levels: with five, 124 bytes of spills.)
+
 template <int P>
-__global__ void __launch_bounds__(32 * WPB, P <= 3 ? 5 : 4) k_solve_pair(const __grid_constant__ SArgs A,
+__global__ void __launch_bounds__(32 * WPB, P <= 2 ? 5 : 4) k_solve_pair(const __grid_constant__ SArgs A,
                                                                          const __grid_constant__ SArgs B, int na) {
   __shared__ float4 ring[WPB][4 * kRing * 32];
   pdl_wait();
@@ -514,19 +519,42 @@ void derivatives_T(ms_grid* g, bool from_h) {
   else launch_pdl(k_walk_dT<false>, grd, blk, 0, g->stream, y, x, nyb);
 }
 
-// u = P~^{-1} l over p_0 for the H fields or E_z: uc.
+// The solve's polynomial p about t = 36, where the smoothest fields sit: p(t) = gain (1 + q (t - 36) r(t)), with r in
+// the Horner form of the levels, coefficients r[l] of level l + 1.
+struct PairPoly {
+  double gain, q, r[kChebMax];
+};
+PairPoly pair_poly(const Cheb& c) {
+  long double p[kChebMax + 1] = {c.p0}, gain = 0.0L, h = 0.0L;
+  for (int k = 1; k < c.m; ++k) p[k] = p[k - 1] * (long double)c.q[k];
+  for (int k = c.m - 1; k >= 0; --k) gain = 36.0L * gain + p[k];
+  PairPoly out{};
+  out.gain = (double)gain;
+  // 1 - p / gain = (36 - t) h(t), q r = h, by synthetic division from the constant term
+  for (int k = 0; k < c.m - 1; ++k) {
+    const long double n = ((k ? 0.0L : 1.0L) - p[k] / gain + h) / 36.0L;
+    if (k == 0) out.q = (double)n;
+    else out.r[c.m - 2 - k] = (double)(n / h);
+    h = n;
+  }
+  return out;
+}
+
+// u = P~^{-1} l over the gain of its polynomial for the H fields or E_z: uc.
 void solve_pair(ms_grid* g, bool of_h) {
   Adj32* A = g->adj32;
   SArgs a[2];
   int nb[2] = {0, 0};
   const int nf = of_h ? 2 : 1;
+  const PairPoly poly = pair_poly(g->walk.cheb);
   for (int k = 0; k < nf; ++k) {
     const int f = of_h ? (k ? HY : HX) : EZ, mc = f == HY ? 0 : 1;
     a[k] = make_s(g, f, A->lh[f], nullptr, nf);
     a[k].hi = nullptr;
-    const Split q = split(g->walk.cheb.q[1]);
+    const Split q = split(poly.q);
     a[k].l_hi = q.hi;
     a[k].l_lo = q.lo;
+    for (int l = 0; l < g->walk.cheb.m - 2; ++l) a[k].q[l] = (float)poly.r[l];
     a[k].lo = A->ll[f] + mc;
     a[k].out = A->uc[f] + mc;
     nb[k] = blocks_of(a[k].nstrip * a[k].nblk);
@@ -551,7 +579,8 @@ FArgs filter_args(ms_grid* g, int f) {
   a.M = f == HY ? N : N - 1;
   a.u0 = f == HX ? 0 : 1;
   a.u1 = N;
-  const double sc = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * g->walk.cheb.p0 * walk_rhs_scale();
+  const double sc = (f == EZ ? 12.0 / (g->desc.r * g->Z) : 12.0 * g->Z / g->desc.r) * pair_poly(g->walk.cheb).gain *
+                    walk_rhs_scale();
   const double c = 12.0 * g->beta * sc;
   const Split cp = split(c), sp = split(sc);
   a.c_hi = cp.hi;

@@ -19,7 +19,7 @@ struct SArgs {
   int kind;         // KIND_*
   float q[4];          // levels of the solve but for the last
   float s_hi, s_lo;    // increment scale s
-  float l_hi, l_lo;    // last level: s q (reverse pass: q)
+  float l_hi, l_lo;    // last level: s q (reverse pass: its coefficient alone)
   int nstrip, nblk, rows;
 };
 
@@ -125,8 +125,8 @@ __device__ __forceinline__ void ff_add_scaled(float2& hi, float2& lo, float2 b, 
 enum { KIND_E = 0, KIND_HX = 1, KIND_HY = 2 };
 
 // One block of rows of one 128-column strip; P levels.  EDGE: lanes beyond the field hold zeros.  PAIR (the
-// reverse pass): the right-hand side is the float-float field (p1, lo) and the solution over p_0 is left as
-// the pair (p1, out), out = lo + q T y.
+// reverse pass): the right-hand side is the float-float field (p1, lo) and the solution over its value at T = 36 is
+// left as the pair (p1, out), out = lo + l (T - 36) y (adjoint32.cu), the last level on first differences of y.
 template <int P, int KIND, bool EDGE, bool PAIR>
 __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip, int blk) {
   constexpr bool TWO = KIND == KIND_E && !PAIR;
@@ -169,6 +169,20 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
     w[0] = fma2(four, y[0], make_float2(a + r0, y[0].x + r1));
     w[1] = fma2(four, y[1], make_float2(y[0].y + r2, y[1].x + b));
   };
+  // l = (left - y) + (right - y)
+  auto lapx = [&](const float2(&y)[2], float2(&l)[2]) {
+    float a = __shfl_up_sync(kFull, y[1].y, 1), b = __shfl_down_sync(kFull, y[0].x, 1);
+    float r0 = y[0].y, r1 = y[1].x, r2 = y[1].y;
+    if (EDGE && KIND == KIND_HY) {
+      a = first ? y[0].x : a;
+      r0 = lastc[0] ? y[0].x : r0;
+      r1 = lastc[1] ? y[0].y : r1;
+      r2 = lastc[2] ? y[1].x : r2;
+      b = lastc[3] ? y[1].y : b;
+    }
+    l[0] = add2(sub2(make_float2(a, y[0].x), y[0]), sub2(make_float2(r0, r1), y[0]));
+    l[1] = add2(sub2(make_float2(y[0].y, y[1].x), y[1]), sub2(make_float2(r2, b), y[1]));
+  };
   const int js = max(j0 - P, u0);
   // ring: [slot][p1, p2 of row jj, hi, lo of row jj - P][lane]
   const size_t off = ok ? m0 : 0;
@@ -204,6 +218,8 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
   for (int l = 0; l <= P; ++l) b[l][0] = b[l][1] = z2;
 #pragma unroll
   for (int l = 0; l < P; ++l) w[l][0][0] = w[l][0][1] = w[l][1][0] = w[l][1][1] = z2;
+  float2 x[2][2], yn[2], xr[2], rn[2];  // PAIR: w[P - 1] holds l of the last level's y, x that y, xr what it rounded away
+  x[0][0] = x[0][1] = x[1][0] = x[1][1] = yn[0] = yn[1] = xr[0] = xr[1] = rn[0] = rn[1] = z2;
   const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo), l_hi = bc2(A.l_hi), l_lo = bc2(A.l_lo);
   float* ph = (PAIR ? A.out : A.hi) + off + (size_t)j0 * ld;
   float* pl = A.lo + off + (size_t)j0 * ld;
@@ -241,10 +257,24 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
       float2 tt[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        float2 ud = add2(w[l][0][k], wn[k]);
-        if (KIND == KIND_HX && (t == u0 || t == u1 - 1))  // the ghost row equals the wall row
-          ud = add2(w[l][1][k], t == u0 ? wn[k] : w[l][0][k]);
-        tt[k] = fma2(four, w[l][1][k], ud);
+        if (PAIR && l == P - 1) {  // (T - 36) y = 6 (L_x + L_y) y + L_y L_x y
+          float2 yu = x[0][k], yd = yn[k], lu = w[l][0][k], ld = wn[k];
+          if (KIND == KIND_HX && (t == u0 || t == u1 - 1)) {  // the ghost row equals the wall row
+            yu = t == u0 ? x[1][k] : yu;
+            lu = t == u0 ? w[l][1][k] : lu;
+            yd = t == u1 - 1 ? x[1][k] : yd;
+            ld = t == u1 - 1 ? w[l][1][k] : ld;
+          }
+          const float2 ly = add2(sub2(yu, x[1][k]), sub2(yd, x[1][k]));
+          tt[k] = fma2(bc2(6.0f), add2(w[l][1][k], ly), add2(sub2(lu, w[l][1][k]), sub2(ld, w[l][1][k])));
+          x[0][k] = x[1][k];
+          x[1][k] = yn[k];
+        } else {
+          float2 ud = add2(w[l][0][k], wn[k]);
+          if (KIND == KIND_HX && (t == u0 || t == u1 - 1))  // the ghost row equals the wall row
+            ud = add2(w[l][1][k], t == u0 ? wn[k] : w[l][0][k]);
+          tt[k] = fma2(four, w[l][1][k], ud);
+        }
         w[l][0][k] = w[l][1][k];
         w[l][1][k] = wn[k];
       }
@@ -252,11 +282,20 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
         if ((unsigned)(t - u0) < (unsigned)(u1 - u0)) {
           float2 y[2];
 #pragma unroll
-          for (int k = 0; k < 2; ++k) y[k] = fma2(bc2(A.q[l]), tt[k], b[l + 1][k]);
+          for (int k = 0; k < 2; ++k) {
+            y[k] = fma2(bc2(A.q[l]), tt[k], b[l + 1][k]);
+            if (PAIR && l == P - 2) rn[k] = fma2(bc2(A.q[l]), tt[k], sub2(b[l + 1][k], y[k]));
+          }
           mask(y);
-          wsum(y, wn);
+          if (PAIR && l == P - 2) {
+            yn[0] = y[0];
+            yn[1] = y[1];
+            lapx(y, wn);
+          } else {
+            wsum(y, wn);
+          }
         } else {
-          wn[0] = wn[1] = z2;
+          wn[0] = wn[1] = yn[0] = yn[1] = rn[0] = rn[1] = z2;
         }
       } else if (t >= j0) {
         if (out) {
@@ -264,7 +303,11 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
           float2 o[2] = {make_float2(sl.x, sl.y), make_float2(sl.z, sl.w)};
           if (PAIR) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) o[k] = fma2(l_hi, tt[k], fma2(l_lo, tt[k], o[k]));
+            for (int k = 0; k < 2; ++k) {
+              // with what y rounded away and the field's low part, of which the point itself is most of the sum
+              const float2 T = fma2(bc2(-20.0f), add2(xr[k], o[k]), tt[k]);
+              o[k] = fma2(l_hi, T, fma2(l_lo, T, o[k]));
+            }
             if (!EDGE || m0 + 4 <= M) {
               *reinterpret_cast<float4*>(ph) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
             } else {
@@ -296,6 +339,8 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
         pl += ld;
       }
     }
+    xr[0] = rn[0];
+    xr[1] = rn[1];
   }
 }
 
