@@ -541,6 +541,16 @@ XArgs make_x(const ms_grid* g, int step, float* plane, const float* src_hi, cons
   return a;
 }
 
+// Rows per block of a solve launch, warps(rows) in all: P rows above and below are computed twice, but a launch
+// wants `most` warps, about thirteen per SM, and small ones are bound by the length of one walk.
+template <typename Warps>
+int solve_rows(Warps warps, int most) {
+  int rows = 32;
+  while (rows > 8 && warps(rows) < most) rows /= 2;
+  if (rows == 8 && warps(8) < 608) rows = 4;
+  return rows;
+}
+
 }  // namespace
 
 SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfields) {
@@ -565,12 +575,8 @@ SArgs make_s(const ms_grid* g, int f, const float* p1, const float* p2, int nfie
   a.l_hi = lp.hi;
   a.l_lo = lp.lo;
   a.nstrip = (a.M + SOUT - 1) / SOUT;
-  // Rows per block: P rows above and below are computed twice, but a grid wants about thirteen warps per
-  // SM; small grids are bound by the length of one walk.
   const int nr = a.u1 - a.u0;
-  int rows = 32;
-  while (rows > 8 && nfields * a.nstrip * ((nr + rows - 1) / rows) < 2000) rows /= 2;
-  if (rows == 8 && nfields * a.nstrip * ((nr + 7) / 8) < 608) rows = 4;
+  const int rows = solve_rows([&](int q) { return nfields * a.nstrip * ((nr + q - 1) / q); }, 2000);
   a.nblk = (nr + rows - 1) / rows;
   a.rows = (nr + a.nblk - 1) / a.nblk;
   return a;
@@ -656,11 +662,20 @@ int walk_batch_build(ms_grid* const* cav, int count, int order, WalkBatch* wb, s
     sa[c] = make_s(g, EZ, g->s32[4], g->s32[1], 1);
     sa[count + c] = make_s(g, HX, g->s32[2], nullptr, 2);
     sa[2 * count + c] = make_s(g, HY, g->s32[3], nullptr, 2);
-    for (int k = 0; k < 3; ++k) {  // the batch fills the GPU, whatever its cavities' sizes: long blocks
-      SArgs& a = sa[(size_t)k * count + c];
-      const int nr = a.u1 - a.u0;
-      a.nblk = (nr + 31) / 32;
-      a.rows = (nr + a.nblk - 1) / a.nblk;
+  }
+  // row blocks by the warps of a whole launch, all cavities together (us per step, chosen so and with 32 rows
+  // whatever the cavities: four of 64 to 256 cells 21 and 46, a hundred of 32 cells 24 and 44, 16 of 256 cells 45 and 60)
+  for (int l = 0; l < 2; ++l) {
+    SArgs *first = sa.data() + (size_t)l * count, *last = sa.data() + (size_t)(l ? 3 : 1) * count;
+    const int rows = solve_rows([&](int q) {
+      int n = 0;
+      for (const SArgs* a = first; a != last; ++a) n += a->nstrip * ((a->u1 - a->u0 + q - 1) / q);
+      return n;
+    }, 1216);
+    for (SArgs* a = first; a != last; ++a) {
+      const int nr = a->u1 - a->u0;
+      a->nblk = (nr + rows - 1) / rows;
+      a->rows = (nr + a->nblk - 1) / a->nblk;
     }
   }
   std::vector<int> list[4];
@@ -705,7 +720,8 @@ int walk_batch_build(ms_grid* const* cav, int count, int order, WalkBatch* wb, s
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pd, k_batch_d<true>, 32 * WPB, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_batch_s<4>, 32 * WPB, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, wb->P == 2 ? k_batch_s<2> : (wb->P == 3 ? k_batch_s<3> : k_batch_s<4>),
+                                                32 * WPB, 0);
   wb->resident_d = sms * pd;
   wb->resident_s = sms * ps;
   return 0;
