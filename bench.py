@@ -165,14 +165,15 @@ def bf16_peak():
 
 
 # source files that define each kernel kind reported by ms_step_profiled
+_WALK = ["k_tiled.cu", "k_tiled.cuh", "k_walk_dev.cuh", "k_pdl.cuh", "k_rec64.cu", "k_rec64.cuh"]
+_REC64 = ["k_rec64.cu", "k_rec64.cuh", "k_pdl.cuh"]
+_GRID3D = ["grid3d.cu", "grid3d.cuh", "k_walk_dev.cuh", "k_pdl.cuh", "k_rec64.cu", "k_rec64.cuh"]
 KIND_SOURCES = {
-    "curl32": ["k_tiled.cu", "k_tiled.cuh", "k_walk_dev.cuh"],
-    "solve32": ["k_tiled.cu", "k_tiled.cuh", "k_walk_dev.cuh"],
-    "filter64": ["k_fp64.cu", "k_fp64.cuh"], "pade64": ["k_rec64.cu", "k_rec64.cuh"],
-    "filt3d32": ["grid3d.cu", "grid3d.cuh"], "band3d32": ["grid3d.cu", "grid3d.cuh"],
-    "term3d32": ["grid3d.cu", "grid3d.cuh"], "tsgemm": ["k_transform.cu", "k_transform.cuh"],
-    "sweep3d32": ["grid3d.cu", "grid3d.cuh"],
-    "p1sweep64": ["k_rec64.cu", "k_rec64.cuh"], "yee64": ["k_fp64.cu", "k_fp64.cuh"],
+    "curl32": _WALK, "solve32": _WALK,
+    "filter64": ["k_fp64.cu", "k_fp64.cuh", "k_pdl.cuh"], "pade64": _REC64, "p1sweep64": _REC64,
+    "yee64": ["k_fp64.cu", "k_fp64.cuh"],
+    "filt3d32": _GRID3D, "band3d32": _GRID3D, "term3d32": _GRID3D, "sweep3d32": _GRID3D,
+    "tsgemm": ["k_transform.cu", "k_transform.cuh"],
 }
 
 
@@ -188,9 +189,11 @@ def kernel_sources_hash(kind: str):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2306_17263_gb300", "csrc")
     for f in KIND_SOURCES.get(kind, []):
-        if not os.path.exists(os.path.join(csrc, f)):
+        path = os.path.join(csrc, f)
+        if not os.path.exists(path):  # not the hash of any tree that has the file, nor of a list without it
+            h.update(f.encode() + b" is missing")
             continue
-        with open(os.path.join(csrc, f), encoding="utf-8") as fh:
+        with open(path, encoding="utf-8") as fh:
             h.update(f.encode() + _code_only(fh.read()).encode())
     return h.hexdigest()[:16]
 
