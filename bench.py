@@ -172,7 +172,7 @@ KIND_SOURCES = {
     "curl32": _WALK, "solve32": _WALK,
     "filter64": ["k_fp64.cu", "k_fp64.cuh", "k_pdl.cuh"], "pade64": _REC64, "p1sweep64": _REC64,
     "yee64": ["k_fp64.cu", "k_fp64.cuh"],
-    "filt3d32": _GRID3D, "band3d32": _GRID3D, "term3d32": _GRID3D, "sweep3d32": _GRID3D,
+    "filt3d32": _GRID3D, "term3d32": _GRID3D, "sweep3d32": _GRID3D,
     "tsgemm": ["k_transform.cu", "k_transform.cuh"],
 }
 

@@ -14,6 +14,7 @@
 
 #include "k_fp64.cuh"
 #include "k_mixed.cuh"
+#include "k_rec64.cuh"
 
 namespace ms {
 
@@ -89,6 +90,7 @@ ms_status adjoint_setup(ms_grid* g) {
   for (int kind = 0; kind < 2; ++kind) {
     PadeTable& t = g->padeT[kind];
     build_pade_table_T(g->pade[kind], &t);
+    if (t.M >= kRecMinLine) continue;  // longer lines take the recurrences
     const cudaError_t e = dev_malloc((void**)&t.d_w, t.w.size() * sizeof(double));
     if (e != cudaSuccess) {
       release();

@@ -432,7 +432,7 @@ void prof_mark(ms_grid* g, int kind, double bytes) {
 
 const char* kernel_kind_name(int k) {
   static const char* names[KK_COUNT] = {"filter64", "pade64", "p1sweep64", "yee64", "curl32", "solve32",
-                                        "filter3d64", "pade3d64", "sweep3d64", "filt3d32", "band3d32",
+                                        "filter3d64", "pade3d64", "sweep3d64", "filt3d32", "",
                                         "sweep3d32", "nc64", "source", "term3d32", "tsgemm", "tspack", "tracked32"};
   return (k >= 0 && k < KK_COUNT) ? names[k] : "";
 }
@@ -587,18 +587,10 @@ static ms_status create_grid_impl(const ms_grid_desc* d, double* const* shared64
     const int M = (kind == HALF_TO_NODE) ? g->N - 1 : g->N;
     if (build_pade_table(M, d->closure, kind, 1e-18, &g->pade[kind], &err) != 0) return cleanup(fail(MS_EINVAL, err));
     PadeTable& t = g->pade[kind];
-    std::vector<float> whi(t.w.size()), wlo(t.w.size());
-    for (size_t k = 0; k < t.w.size(); ++k) {
-      whi[k] = (float)t.w[k];
-      wlo[k] = (float)(t.w[k] - (double)whi[k]);
-    }
-    ms_status s = dalloc(&t.d_w, t.w.size());
-    if (s == MS_OK) s = dalloc(&t.d_whi, t.w.size());
-    if (s == MS_OK) s = dalloc(&t.d_wlo, t.w.size());
+    if (M >= kRecMinLine) continue;  // longer lines take the recurrences
+    const ms_status s = dalloc(&t.d_w, t.w.size());
     if (s != MS_OK) return cleanup(s);
-    if (cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t.d_whi, whi.data(), whi.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t.d_wlo, wlo.data(), wlo.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
       return cleanup(fail(MS_ECUDA, "copy of Pade tables failed"));
   }
   if (compact) {
@@ -655,8 +647,6 @@ ms_status ms_destroy(ms_grid* g) {
   for (cudaEvent_t e : g->prof.pool) cudaEventDestroy(e);
   for (int k = 0; k < 2; ++k) {
     dev_free(g->pade[k].d_w);
-    dev_free(g->pade[k].d_whi);
-    dev_free(g->pade[k].d_wlo);
   }
   for (int f = 0; f < 3; ++f) {
     dev_free(g->f64[f]);

@@ -1578,6 +1578,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
       const int M = (kind == HALF_TO_NODE) ? g->N - 1 : g->N;
       PadeTable& t = g->pade[kind];
       if (build_pade_table(M, d->closure, kind, 1e-18, &t, &err) != 0) return cleanup(fail3(MS_EINVAL, err));
+      if (M >= kRecMinLine) continue;  // longer lines take the recurrences
       s = alloc3(&t.d_w, t.w.size());
       if (s == MS_OK && cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
         s = fail3(MS_ECUDA, "copy of Pade tables failed");
@@ -1591,6 +1592,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
       PadeTable& t = g->pade32[kind];
       if (build_pade_table(M, d->closure, kind, 1e-12, &t, &err, /*of_differences=*/true) != 0)
         return cleanup(fail3(MS_EINVAL, err));
+      if (M >= kWalk3Min) continue;  // longer lines take the walks
       std::vector<float> whi(t.w.size()), wlo(t.w.size());
       for (size_t q = 0; q < t.w.size(); ++q) {
         whi[q] = (float)t.w[q];
@@ -1786,9 +1788,10 @@ ms_status diag_view3d(ms_grid* g, double** f) {
   std::string err;
   for (int kind = 0; kind < 2; ++kind) {
     PadeTable& t = g->pade[kind];
-    if (t.d_w) continue;
+    if (t.d_w || t.M >= kRecMinLine) continue;
     const int M = (kind == HALF_TO_NODE) ? g->N - 1 : g->N;
     if (build_pade_table(M, g->desc.closure, kind, 1e-18, &t, &err) != 0) return fail3(MS_EINVAL, err);
+    if (M >= kRecMinLine) continue;
     MS3_TRY(alloc3(&t.d_w, t.w.size()));
     if (cudaMemcpy(t.d_w, t.w.data(), t.w.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
       return fail3(MS_ECUDA, "copy of Pade tables failed");

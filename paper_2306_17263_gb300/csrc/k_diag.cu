@@ -112,30 +112,8 @@ void launch_dot(const double* a, const double* b, size_t n, double* partial, int
   k_dot_final<<<1, kRedThreads, 0, st>>>(partial, blocks, results, slot, accumulate);
 }
 
-// v = hi + lo with hi = fl32(v), lo = fl32(v - hi): the FP32 pair represents v to ~2^-48.
-__global__ void k_split(const double* __restrict__ v, float* __restrict__ hi, float* __restrict__ lo, size_t n) {
-  for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
-    const double x = v[p];
-    const float h = (float)x;
-    hi[p] = h;
-    lo[p] = (float)(x - (double)h);
-  }
-}
-
-__global__ void k_join(const float* __restrict__ hi, const float* __restrict__ lo, double* __restrict__ v, size_t n) {
-  for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x)
-    v[p] = (double)hi[p] + (double)lo[p];
-}
-
-void launch_split(const double* v, float* hi, float* lo, size_t n, cudaStream_t st) {
-  k_split<<<reduce_blocks(n), kRedThreads, 0, st>>>(v, hi, lo, n);
-}
-
-void launch_join(const float* hi, const float* lo, double* v, size_t n, cudaStream_t st) {
-  k_join<<<reduce_blocks(n), kRedThreads, 0, st>>>(hi, lo, v, n);
-}
-
-// The same between a dense FP64 field and pitched FP32 planes; the split stores 0 on Dirichlet walls.
+// v = hi + lo with hi = fl32(v), lo = fl32(v - hi), between a dense FP64 field and pitched FP32 planes: the FP32
+// pair represents v to ~2^-48; the split stores 0 on Dirichlet walls.
 __global__ void k_split2d(const double* __restrict__ v, float* __restrict__ hi, float* __restrict__ lo, int ld, int nx,
                           int ny, int bcx, int bcy) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;

@@ -99,8 +99,6 @@ void launch_err_reduce(const double* a, const double* b, size_t n, double* parti
 void launch_dot(const double* a, const double* b, size_t n, double* partial, int blocks, double* results, int slot,
                 int accumulate, cudaStream_t st);
 // FP32 hi/lo <-> FP64 conversion
-void launch_split(const double* v, float* hi, float* lo, size_t n, cudaStream_t st);
-void launch_join(const float* hi, const float* lo, double* v, size_t n, cudaStream_t st);
 void launch_split2d(const double* v, float* hi, float* lo, int ld, const Shape& s, cudaStream_t st);
 void launch_join2d(const float* hi, const float* lo, int ld, double* v, const Shape& s, cudaStream_t st);
 void launch_zero_dirichlet64(double* u, const Shape& s, cudaStream_t st);

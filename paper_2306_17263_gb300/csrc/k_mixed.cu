@@ -64,7 +64,6 @@ MixedConsts mixed_consts(const ms_grid* g) {
   k.sE_lo = sE.lo;
   k.sH_hi = sH.hi;
   k.sH_lo = sH.lo;
-  k.S = g->p1_sweeps32;
   return k;
 }
 
@@ -124,11 +123,12 @@ ms_status mixed_setup(ms_grid* g) {
       g_mixed_err = err;
       return MS_EINVAL;
     }
-    // the band kernels (tracked form, reverse pass) hold half-widths up to kBand32Max
+    // the band kernels (tracked form) hold half-widths up to kBand32Max
     if (t.K > kBand32Max) {
       g_mixed_err = "FP32 Pade band half-width outside the range the kernels hold";
       return MS_EUNSUPPORTED;
     }
+    if (g->N > kTinyN && g->desc.scheme != MS_SCHEME_C4_DE) continue;  // the walks take the recurrences
     std::vector<float> whi(t.w.size()), wlo(t.w.size());
     for (size_t k = 0; k < t.w.size(); ++k) {
       Split s = split(t.w[k]);
@@ -145,12 +145,6 @@ ms_status mixed_setup(ms_grid* g) {
       g_mixed_err = "copy of FP32 Pade tables failed";
       return MS_ECUDA;
     }
-  }
-  // Richardson sweeps of the reverse pass to 1e-10 (below the FP32 rounding noise, which is not coherent)
-  const ms_status sw = ms_solver_sweeps(2, g->desc.r, MS_FP32_REFINED, 1e-10, &g->p1_sweeps32);
-  if (sw != MS_OK) {
-    g_mixed_err = "too many Richardson sweeps for the FP32 solve";
-    return sw;
   }
   const ms_status wk = walk_setup(g);
   if (wk != MS_OK) {

@@ -7,14 +7,13 @@
 
 namespace ms {
 
-constexpr int kBand32Max = 12;   // largest half-width of the FP32 band tables (reverse pass, 3D, tracked form)
+constexpr int kBand32Max = 12;   // largest half-width of the FP32 band tables
 constexpr int kMaxSweeps32 = 6;  // largest Richardson sweep count ms_solver_sweeps grants in 2D
 
 // Coefficients of the FP32 step of a grid (k_mixed.cu), split hi + lo: 12 beta, 6 c1 h^2, the Richardson
-// relaxation and sweep count (3D, reverse pass), and the increment scales 12 Z / r and 12 / (r Z).
+// relaxation of the sweeps after a transform solve, and the increment scales 12 Z / r and 12 / (r Z).
 struct MixedConsts {
   float cb_hi, cb_lo, d_hi, d_lo, omega, sE_hi, sE_lo, sH_hi, sH_lo;
-  int S;
 };
 MixedConsts mixed_consts(const ms_grid* g);
 

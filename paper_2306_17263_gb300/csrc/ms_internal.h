@@ -53,7 +53,7 @@ struct PadeTable {
   bool transposed = false;
   LineEnds ends, ends_T;             // end corrections of the recurrences of this table, of its transpose
   std::vector<double> w;             // (2B + 1) rows x (2K + 2)
-  double* d_w = nullptr;             // device copy (FP64)
+  double* d_w = nullptr;             // device copy (FP64), of lines shorter than kRecMinLine
   float* d_whi = nullptr;            // device FP32 split: w = whi + wlo exactly to ~2^-48
   float* d_wlo = nullptr;
   int row_stride() const { return 2 * K + 2; }
@@ -79,7 +79,7 @@ struct Graph {
 // Kernel kinds reported by ms_step_profiled.
 enum KernelKind {
   KK_FILTER64 = 0, KK_PADE64 = 1, KK_P1SWEEP64 = 2, KK_YEE64 = 3, KK_CURL32 = 4, KK_SOLVE32 = 5,
-  KK_FILTER3D64 = 6, KK_PADE3D64 = 7, KK_SWEEP3D64 = 8, KK_FILT3D32 = 9, KK_BAND3D32 = 10, KK_SWEEP3D32 = 11,
+  KK_FILTER3D64 = 6, KK_PADE3D64 = 7, KK_SWEEP3D64 = 8, KK_FILT3D32 = 9, KK_SWEEP3D32 = 11,
   KK_NC64 = 12, KK_SRC = 13, KK_TERM3D32 = 14, KK_TSGEMM = 15, KK_TSPACK = 16, KK_TRACKED32 = 17,
   KK_COUNT
 };
@@ -127,9 +127,8 @@ struct ms_grid {
   // Pade tables: [0] half->node (M = N-1), [1] node->half (M = N)
   ms::PadeTable pade[2];
   ms::Cheb cheb64;  // polynomial of the FP64 solve
-  // FP32 path: tables truncated for FP32 and split hi/lo; Richardson sweeps for FP32
+  // FP32 path: tables truncated for FP32 and split hi/lo (on the device where lines are short, and for the tracked form)
   ms::PadeTable pade32[2];
-  int p1_sweeps32 = 0;
   int ld32 = 0;            // row pitch of the 2D FP32 planes
   float* slab32 = nullptr;  // their storage: hi[3], lo[3], s32[1..4]
   struct {
