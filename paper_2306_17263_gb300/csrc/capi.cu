@@ -933,11 +933,16 @@ ms_status ms_divergence(ms_grid* g, double* norm) {
   double* div = g->s64[0];
   const PadeTable& t = g->pade[NODE_TO_HALF];
   // delta_x H_x: rows j = 0..N-1 of H_x (N+1 nodes) -> N cell centres
-  launch_pade64(0, view[HX], div, N, N + 1, N, N, 0, 0, N, t, 1.0 / g->h, 0, g->stream);
   // delta_y H_y: columns i = 0..N-1 of H_y (N+1 nodes) -> N cell centres
-  launch_pade64(1, view[HY], div, N, N, N, N, 0, 0, N, t, 1.0 / g->h, 1, g->stream);
   const size_t n = (size_t)N * N;
-  launch_dot(div, div, n, g->d_partial, reduce_blocks(n), g->d_result, 0, 0, g->stream);
+  if (launch_pade64_xy(view[HX], N + 1, div, N, 1.0 / g->h, view[HY], N, g->s64[1], N, 1.0 / g->h, N, N, 0, 0, N, t,
+                       g->stream)) {  // both at once on small grids, which the length of a line's recurrences bounds
+    launch_square_sum(div, g->s64[1], n, g->d_partial, reduce_blocks(n), g->d_result, g->stream);
+  } else {
+    launch_pade64(0, view[HX], div, N, N + 1, N, N, 0, 0, N, t, 1.0 / g->h, 0, g->stream);
+    launch_pade64(1, view[HY], div, N, N, N, N, 0, 0, N, t, 1.0 / g->h, 1, g->stream);
+    launch_dot(div, div, n, g->d_partial, reduce_blocks(n), g->d_result, 0, 0, g->stream);
+  }
   MS_TRY(check_launch("divergence"));
   double r;
   MS_CUDA(cudaMemcpyAsync(&r, g->d_result, sizeof r, cudaMemcpyDeviceToHost, g->stream));

@@ -98,6 +98,17 @@ __global__ void k_dot_partial(const double* __restrict__ a, const double* __rest
   if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
 }
 
+__global__ void k_square_sum_partial(const double* __restrict__ a, const double* __restrict__ b, size_t n,
+                                     double* __restrict__ partial) {
+  double v[1] = {0};
+  for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
+    const double s = a[p] + b[p];
+    v[0] = fma(s, s, v[0]);
+  }
+  block_reduce<1>(v, 0);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
+}
+
 __global__ void k_dot_final(const double* __restrict__ partial, int blocks, double* __restrict__ res, int slot,
                             int acc) {
   double v[1] = {0};
@@ -110,6 +121,12 @@ void launch_dot(const double* a, const double* b, size_t n, double* partial, int
                 int accumulate, cudaStream_t st) {
   k_dot_partial<<<blocks, kRedThreads, 0, st>>>(a, b, n, partial);
   k_dot_final<<<1, kRedThreads, 0, st>>>(partial, blocks, results, slot, accumulate);
+}
+
+void launch_square_sum(const double* a, const double* b, size_t n, double* partial, int blocks, double* results,
+                       cudaStream_t st) {
+  k_square_sum_partial<<<blocks, kRedThreads, 0, st>>>(a, b, n, partial);
+  k_dot_final<<<1, kRedThreads, 0, st>>>(partial, blocks, results, 0, 0);
 }
 
 // v = hi + lo with hi = fl32(v), lo = fl32(v - hi), between a dense FP64 field and pitched FP32 planes: the FP32

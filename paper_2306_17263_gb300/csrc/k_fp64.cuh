@@ -95,6 +95,9 @@ void launch_mode_field(double* out, const Shape& s, const double* tab_x, const d
 // over calls when accumulate != 0).  partial must hold 4 * blocks doubles.
 void launch_err_reduce(const double* a, const double* b, size_t n, double* partial, int blocks, double* results,
                        int accumulate, cudaStream_t st);
+// results[0] = sum (a + b)^2
+void launch_square_sum(const double* a, const double* b, size_t n, double* partial, int blocks, double* results,
+                       cudaStream_t st);
 // results[slot] (+)= sum a*b
 void launch_dot(const double* a, const double* b, size_t n, double* partial, int blocks, double* results, int slot,
                 int accumulate, cudaStream_t st);
