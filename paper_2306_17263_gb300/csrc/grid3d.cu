@@ -49,6 +49,7 @@ struct Grid3D {
   float* hi[6] = {};
   float* lo[6] = {};
   double* s64[9] = {};  // FP64: G[3], R[3], and, with G again, the work planes of the solves; FP32 grids use [0], [1]
+  double* slab64 = nullptr;  // FP64: storage of s64 (one allocation: each takes as long as many steps of a small grid)
   float* s32[3] = {};   // FP32: R
   float* gh[3] = {};    // FP32: filtered components G~ (hi, lo) of one half-step, slot c % 3
   float* gl[3] = {};
@@ -1585,7 +1586,9 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
     }
     if (s == MS_OK) s = cheb3d64(g);
     for (int c = 0; c < 6 && s == MS_OK; ++c) s = alloc3(&G3->f64[c], G3->sh[c].size());
-    for (int k = 0; k < 9 && s == MS_OK; ++k) s = alloc3(&G3->s64[k], G3->nmax);
+    const size_t pl = (G3->nmax + 31) / 32 * 32;
+    if (s == MS_OK) s = alloc3(&G3->slab64, 9 * pl);
+    for (int k = 0; k < 9 && s == MS_OK; ++k) G3->s64[k] = G3->slab64 + k * pl;
   } else {
     for (int kind = 0; kind < 2 && s == MS_OK; ++kind) {
       const int M = (kind == HALF_TO_NODE) ? g->N - 1 : g->N;
@@ -1708,7 +1711,8 @@ void destroy_grid3d(ms_grid* g) {
     dev_free(G3->lo[c]);
     dev_free(G3->dview[c]);
   }
-  for (int k = 0; k < 9; ++k) dev_free(G3->s64[k]);
+  dev_free(G3->slab64);
+  for (int k = 0; k < 9 && !G3->slab64; ++k) dev_free(G3->s64[k]);
   for (int k = 0; k < 3; ++k) dev_free(G3->s32[k]);
   for (int k = 0; k < 3; ++k) {
     dev_free(G3->gh[k]);
