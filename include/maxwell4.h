@@ -55,10 +55,11 @@ typedef enum {
 
 /* Arithmetic of the time step.
  *   MS_FP64:          every kernel computes in FP64.
- *   MS_FP32_REFINED:  FP32 arithmetic; every scalar coefficient that is not exact in FP32 is
- *                     applied as an error-free hi+lo pair, the elliptic and Pade solves are
- *                     iterated to convergence against residuals with those exact coefficients,
- *                     and the state is kept as an unevaluated FP32 hi+lo sum updated with
+ *   MS_FP32_REFINED:  FP32 arithmetic; scalar coefficients that are not exact in FP32 are applied
+ *                     as hi+lo pairs where one FP32 number would shift a frequency by more than the
+ *                     solve's tolerance of 1e-10 (the recurrences of the Pade derivative take their
+ *                     ratio as one number, 1.1e-9 off, with an exact gain for smooth fields), and
+ *                     the state is kept as an unevaluated FP32 hi+lo sum updated with
  *                     error-free transformations (about 48 significant bits). */
 typedef enum { MS_FP64 = 0, MS_FP32_REFINED = 1 } ms_precision;
 
@@ -247,7 +248,7 @@ ms_status ms_stability_limit(int dim, double* rmax);
 
 /* Advance one step like ms_step, recording a CUDA event on the grid's stream after every
  * kernel launch, then wait for it.  On return count = number of launches (at most cap are
- * written), launch_ms[k] = time between the end of launch k-1 (or the step's start) and the
+ * written; the two device copies of a tracked FP32 step share one entry), launch_ms[k] = time between the end of launch k-1 (or the step's start) and the
  * end of launch k, kinds[k] = kernel kind (see ms_kernel_kind_name), bytes[k] = the launch's
  * algorithmic bytes (each input array element read once, each output element written once).
  * Synchronous. */
@@ -278,28 +279,31 @@ const char* ms_kernel_kind_name(int kind);
 #define MS_STATIC_SCRATCH_BYTES (2u * (MS_STATIC_MAX_N + 1u) * (MS_STATIC_MAX_N + 1u) * 8u)
 ms_status ms_p1_solve_static(int n, double r, int field, const double* b, double* x, void* stream);
 
-/* Richardson sweeps the GPU elliptic solves take to reduce the error of P1 x = b by the factor
- * tol from x = 0, from the spectral bound of App. A.2: h^2 P1 has its spectrum in
+/* Richardson sweeps that reduce the error of P1 x = b by the factor tol from x = 0, from the spectral
+ * bound of App. A.2: h^2 P1 has its spectrum in
  * [c1 h^2, c1 h^2 + 16/3] (2D and 3D), c1 h^2 = (24/r^2)(1 + 2/r^2), so one sweep with the
  * optimal relaxation contracts the error by (16/3) / (2 c1 h^2 + 16/3) (about 0.003 at r = 0.5).
  *   dim: 2 or 3;  r: CFL number, 0 < r < the stability limit (MS_ECFL at or above it);
- *   precision: ms_precision; it fixes the largest sweep count the solve kernels hold (FP64: 64;
- *              FP32_REFINED: 6 in 2D, 8 in 3D);  tol: in (0, 1).
+ *   precision: ms_precision; it fixes the largest sweep count granted (FP64: 64; FP32_REFINED: 6 in
+ *              2D, 8 in 3D);  tol: in (0, 1).
  * *sweeps receives the count (0 on failure).  Returns MS_ENOTCONV, with a message, when tol needs
- * more sweeps than the kernels hold, i.e. when the solve would stop short of tol.  Grid creation
- * runs the same check with tol = 1e-17 (FP64) and 1e-10 (FP32_REFINED) and fails with the same
- * status.  Needs no GPU. */
+ * more sweeps than that.  Sweeps are what ms_p1_solve_static takes (to 1e-17) and what refines a
+ * transform solve (MS_SOLVER_TRANSFORM_TC; this count decides there).  A grid's other solves take a
+ * Chebyshev polynomial in P1 whose degree creation fixes from the same spectral bounds, to 1e-17
+ * (FP64) or 1e-10 (FP32_REFINED); creation fails with MS_ENOTCONV if the kernels hold no such degree,
+ * which no stable r needs.  Needs no GPU. */
 ms_status ms_solver_sweeps(int dim, double r, int precision, double tol, int* sweeps);
 
-/* P1 solver of a grid.  MS_SOLVER_RICHARDSON (every grid's default): Richardson sweeps of the 9- or
- * 19-point operator, their count fixed by the spectral bound of App. A.2 (ms_solver_sweeps).
+/* P1 solver of a grid.  MS_SOLVER_RICHARDSON (every grid's default, named for the iteration it replaced):
+ * a Chebyshev polynomial in the 9- or 19-point operator, one stencil per degree, to 1e-17 (FP64) or
+ * 1e-10 (FP32_REFINED) by the spectral bound of App. A.2.
  * MS_SOLVER_TRANSFORM_TC (3D FP32_REFINED grids only): the separable solve.  Every 1D operator of P1
  * (Def. "def:operatorsP") is a Kronecker lift of D_2 (App. A.1), diagonalised per axis by the
  * orthonormal sine transform (Dirichlet axes) or cosine transform (Neumann axes with even ghosts,
  * Table "tab:bc"), so P1^{-1} is three transforms, a division by the eigenvalues and three inverse
  * transforms.  Each transform is a dense GEMM on the tensor cores (bf16 operands split hi + lo, three
  * products, FP32 accumulation in tensor memory), and the result is refined by Richardson sweeps
- * with the exact residual until the App. A.2 bound reaches the Richardson path's tolerance.
+ * with the exact residual until the App. A.2 bound reaches the default solve's tolerance.
  *   ms_set_solver: MS_EINVAL for an unknown solver, MS_EUNSUPPORTED for the transform solver on
  *     other grids, MS_ENOMEM / MS_ECUDA if its set-up (two padded working copies of a component,
  *     transform matrices) fails.  The first selection allocates; a selection drops the captured
@@ -410,11 +414,11 @@ ms_status ms_taylor_init_T(ms_grid* g, const double* l_hx, const double* l_hy, d
 
 /* Arithmetic of the reverse pass: MS_FP64 (every grid), or MS_FP32_REFINED (FP32_REFINED grids,
  * their default).  The FP32 reverse pass keeps the adjoint state as float-float pairs and is the
- * transpose of the FP32_REFINED forward operator (its truncated Pade tables): the adjoint solve
- * u = P1^{-1} l returns its last Richardson iterate and correction as a pair, the transposed band
- * W^T u is accumulated in float-float, and only the difference D^T W^T u (the transposed Pade
- * derivative) is rounded to FP32, so a smooth adjoint field loses no accuracy to cancellation.
- * ms_adjoint_run / _steps convert at the FP64 interface; the Taylor transpose stays FP64.
+ * transpose of the step up to FP32 rounding: the adjoint solve u = P1^{-1} l leaves u as a pair, the
+ * first difference is taken of that pair, and the recurrences of A^{-T} act on it, so the transposed
+ * Pade derivative is rounded once at its own size and a smooth adjoint field loses no accuracy to
+ * cancellation.  Grids of fewer than 32 cells, whose lines are shorter than its two end segments, run
+ * the reverse pass in FP64 whichever arithmetic is selected.  ms_adjoint_run / _steps convert at the FP64 interface; the Taylor transpose stays FP64.
  * MS_EINVAL for an unknown precision, MS_EUNSUPPORTED for FP32 on an FP64 grid. */
 ms_status ms_set_adjoint_precision(ms_grid* g, int precision);
 
@@ -422,7 +426,7 @@ ms_status ms_set_adjoint_precision(ms_grid* g, int precision);
  * Batches: many independent 2D cavities of uneven sizes advanced together.  Each cavity is the
  * problem of ms_create_grid with n = n[b] cells per side; all share the rest of the descriptor
  * (z_imp, r, precision, closure, scheme, stream).  Every kernel of a step is one launch for the
- * whole batch (its blocks walk a list of (cavity, tile) entries), and ms_batch_run replays a
+ * whole batch (its blocks walk a list of (cavity, item) entries), and ms_batch_run replays a
  * captured CUDA graph.  Requires MS_FP32_REFINED and MS_SCHEME_C4 (MS_EUNSUPPORTED otherwise).
  * Cavity indices are 0 .. count-1; the per-cavity calls behave like their ms_* counterparts. */
 typedef struct ms_batch ms_batch;
@@ -439,13 +443,14 @@ ms_status ms_batch_error_vs_exact(ms_batch* b, int cavity, const ms_mode* modes,
 /* count: cavities; cells: sum of n[b]^2 (Yee cells advanced per step); launches: kernels per step. */
 ms_status ms_batch_info(ms_batch* b, int* count, long long* cells, int* launches);
 
-/* Launch plan of a batch: plan[0] = work-list order (0: cavity by cavity, tiles row by row; 1: the
- * boundary-ring tiles of every cavity first, since they take the general and slower paths; 2:
- * largest cavities first), plan[1] = steps per captured graph in ms_batch_run (1..256), plan[2] = 1
+/* Launch plan of a batch: plan[0] = work-list order (0: cavity by cavity; 1: the cavities one strip of
+ * 120 columns wide first, since all their strips see walls and take the slower paths; 2: largest
+ * cavities first), plan[1] = steps per captured graph in ms_batch_run (1..256), plan[2] = 1
  * for persistent launches (as many blocks as are resident at once, each striding over the work
  * list), 0 for one block per work item.  Every plan runs exactly the same arithmetic per cavity;
  * only the order and the launch shape change.  The default is {0, 16, 0}.  ms_batch_set_plan drops
- * the captured graphs (MS_EINVAL for an invalid plan).
+ * the captured graphs (MS_EINVAL for an invalid plan, MS_ENOMEM if its work lists cannot be allocated;
+ * the plan in use then stays).
  *
  * ms_batch_autotune: chooses the plan by measurement.  Candidates: orders 0..2 x 8 or 32 steps per
  * graph x persistent or not; each is captured and timed with CUDA events over about trial_steps

@@ -236,8 +236,9 @@ def stability_limit(dim: int = 2) -> float:
 
 
 def solver_sweeps(dim: int, r: float, precision: int, tol: float) -> int:
-    """Richardson sweeps of the GPU elliptic solve for error reduction `tol` (App. A.2 bound);
-    raises MaxwellError (MS_ENOTCONV) when the solve kernels cannot hold that many; needs no GPU."""
+    """Richardson sweeps that reduce the error of P1 x = b by `tol` (App. A.2 bound), as the allocation-free
+    solve and the refinement of a transform solve take them; raises MaxwellError (MS_ENOTCONV) above the
+    largest count granted (maxwell4.h, ms_solver_sweeps); needs no GPU."""
     v = ctypes.c_int()
     _check(load().ms_solver_sweeps(int(dim), float(r), int(precision), float(tol), ctypes.byref(v)))
     return v.value
@@ -404,11 +405,13 @@ class Grid:
         _check(load().ms_init_driven3(self._h, arr, n))
 
     def set_adjoint_precision(self, precision: int):
-        """Arithmetic of the reverse pass (FP64, or FP32_REFINED on FP32_REFINED grids, their default)."""
+        """Arithmetic of the reverse pass (FP64, or FP32_REFINED on FP32_REFINED grids, their default; grids of
+        fewer than 32 cells run it in FP64 either way)."""
         _check(load().ms_set_adjoint_precision(self._h, int(precision)))
 
     def set_solver(self, solver: int):
-        """Select the P1 solver (SOLVER_RICHARDSON, or SOLVER_TRANSFORM_TC on 3D FP32_REFINED grids)."""
+        """Select the P1 solver (SOLVER_RICHARDSON, the default polynomial solve, or SOLVER_TRANSFORM_TC on 3D
+        FP32_REFINED grids)."""
         _check(load().ms_set_solver(self._h, int(solver)))
 
     def transform_solve(self, comp: int, b, x):

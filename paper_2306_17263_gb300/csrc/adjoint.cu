@@ -7,9 +7,10 @@
 // with F the right-hand-side filter of Eq. "eq:ell" and P1 of Definition "def:operatorsP".
 // F and P1 are symmetric on the unknowns (Dirichlet zeros, even Neumann ghosts), so
 //   S2^T: l_E += h_tau F_E C_EH^T P1_H^{-1} l_H,   S1^T: l_H += h_tau F_H C_HE^T P1_E^{-1} l_E,
-// and M^T = S1^T S2^T applies S2^T first.  The transposed Pade derivative delta^T is the
-// transpose of the truncated band the forward kernels apply (build_pade_table_T), so the
-// reverse pass is the transpose of the forward FP64 step up to rounding.
+// and M^T = S1^T S2^T applies S2^T first.  The transposed Pade derivative delta^T is the recurrences of
+// A^{-T} (k_rec64.cu) and the difference of their result, on lines shorter than kRecMinLine the transpose of the
+// truncated band the forward kernels apply there (build_pade_table_T), so the reverse pass is the transpose of the
+// forward FP64 step up to rounding.
 #include <string>
 
 #include "k_fp64.cuh"
@@ -233,7 +234,7 @@ ms_status taylor_init_dev(ms_grid* g, const double* ez0) {
 }
 
 // The reverse pass in FP32 (adjoint32.cu) on FP32_REFINED grids unless FP64 was selected.  Grids of fewer
-// cells than the walks' two end segments take (32) run it in FP64: fewer launches' work there.
+// cells than the walks' two end segments take (32) run it in FP64 (16^2: 38 us per step, 40 by the FP32 bands).
 bool use32(const ms_grid* g) {
   const int prec = g->adj_precision < 0 ? g->desc.precision : g->adj_precision;
   return prec == MS_FP32_REFINED && g->N >= 32;

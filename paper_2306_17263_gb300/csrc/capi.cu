@@ -487,7 +487,7 @@ ms_status ms_stability_limit(int dim, double* rmax) {
   return MS_OK;
 }
 
-// Largest Richardson sweep count the solve kernels of a precision hold.
+// Largest Richardson sweep count ms_solver_sweeps grants (the transform solve's refinement holds no more in 3D).
 static int max_sweeps(int dim, int precision) {
   if (precision == MS_FP64) return 64;
   return dim == 2 ? kMaxSweeps32 : kMaxSweeps3d32;

@@ -1643,7 +1643,7 @@ ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out) {
 
 // Accuracy of one transform solve relative to the solution (bf16 three-product split: about 16
 // correct bits per pass over six passes, measured at up to 2e-5 on random data), which fixes the
-// refinement sweeps: ts_accuracy * rho^R <= 1e-10, the target of the Richardson solve.
+// refinement sweeps: ts_accuracy * rho^R <= 1e-10, the target of the polynomial solve.
 constexpr double kTsAccuracy = 5e-5;
 
 ms_status set_solver3d(ms_grid* g, int solver) {
@@ -1782,7 +1782,7 @@ ms_status get_fields3d(ms_grid* g, double* const* comps, int host) {
 
 // FP64 components for the diagnostics.  An FP64 grid gives its state; an FP32_REFINED grid joins
 // its float-float state into FP64 copies, and on the first call builds what the FP64 kernels need
-// (FP64 Pade tables, the FP64 sweep count, FP64 scratch), kept until the grid is destroyed.
+// (FP64 Pade tables, the FP64 polynomial, FP64 scratch), kept until the grid is destroyed.
 ms_status diag_view3d(ms_grid* g, double** f) {
   Grid3D* G3 = g->g3;
   if (g->desc.precision == MS_FP64) {
@@ -1814,7 +1814,7 @@ ms_status diag_view3d(ms_grid* g, double** f) {
 
 // Discrete energy of a 3D grid: W = h^3 [Z^-1 sum E.E + Z (sum H.H - h_tau sum H*.H)], H* the Step 2
 // increment that the current E gives (P1^{-1} of the H right-hand side), computed in FP64 with the
-// step's own filter, Pade and sweep kernels but not added to H.
+// step's own filter, Pade and solve kernels but not added to H.
 ms_status energy3d(ms_grid* g, double* W) {
   Grid3D* G3 = g->g3;
   double* f[6];

@@ -18,7 +18,7 @@ Shape3 field_shape3(int N, int c);
 
 struct Grid3D;
 
-constexpr int kMaxSweeps3d32 = 8;  // largest Richardson sweep count of the FP32 3D solve
+constexpr int kMaxSweeps3d32 = 8;  // largest Richardson sweep count ms_solver_sweeps grants in 3D FP32
 
 // 3D counterparts of the grid life cycle and state access, dispatched from capi.cu.
 ms_status create_grid3d(const ms_grid_desc* d, ms_grid** out);

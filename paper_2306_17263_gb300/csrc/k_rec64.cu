@@ -6,7 +6,7 @@
 // Pade derivative.  A = (1/24) tridiag(1, 22, 1) = (1 - rho E^-1)(1 - rho E) / (1 - rho)^2 away from the
 // line ends, so A^{-1} d is a forward and a backward first-order recurrence (one FMA per row each)
 // instead of a band of 34 taps; a segment of L rows starts its recurrences kRecWarm rows outside itself
-// (rho^14 < 1.6e-19).  The closure's end rows change the solution by a multiple of a decaying vector
+// (rho^14 = 1.65e-19).  The closure's end rows change the solution by a multiple of a decaying vector
 // (LineEnds), so a line end costs 18 FMAs, not 16 explicit band rows.  A step at 1024 x 1024 takes 399 us with
 // these kernels, 1023 us with the band and Richardson sweeps; 3D, 96^3: 1.09 and 2.97 ms.
 //

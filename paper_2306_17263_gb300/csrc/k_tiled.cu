@@ -1,5 +1,5 @@
 // FP32_REFINED step of 2D grids.  Two launches per half-step, both made of warps that walk along y with
-// everything they carry in registers: no shared memory, no barriers.
+// everything they carry in registers and the rows ahead in a ring in shared memory of each warp's own: no barriers.
 //
 //   walk_d : the Pade derivatives (App. A.1, Eq. "eq:lhs") of the filtered source into right-hand-side
 //            planes, one plane per axis.  Along y a lane takes one column (30 of 32 lanes write, the

@@ -1,4 +1,5 @@
-// FP32_REFINED step of 2D grids (k_tiled.cu): warps that walk along y, two launches per half-step.
+// FP32_REFINED step of 2D grids (k_tiled.cu): warps that walk along y, two launches per half-step; and constants
+// shared with the other FP32 paths.
 #pragma once
 
 #include <string>

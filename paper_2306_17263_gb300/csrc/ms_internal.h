@@ -21,7 +21,7 @@ struct Shape {
 };
 Shape field_shape(int N, int f);
 
-// rho^kRecWarm < 1.6e-19: a recurrence started that many rows outside a segment has forgotten its start.
+// rho^kRecWarm = 1.65e-19: a recurrence started that many rows outside a segment has forgotten its start.
 constexpr int kRecWarm = 14;
 // End rows of A^{-1} (or of its transpose) on a line of M rows.  With Y the solution of the infinite
 // Toeplitz line for the zero-extended right-hand side, the solution with the closure's end rows is
