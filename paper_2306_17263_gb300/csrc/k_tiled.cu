@@ -313,6 +313,7 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
     diff(ah, al, dm);
     diff(bh, bl, d0);
   }
+  const float2 cb_hi = bc2(A.cb_hi), cb_lo = bc2(A.cb_lo);
   float* bp = A.b + (size_t)j0 * ld + m0;
   int rd = 0, wr = kAhead;  // slots of rows jj + 1 and jj + 1 + kAhead
   for (int jj = j0; jj < j1; ++jj, bp += ld) {
@@ -338,7 +339,7 @@ __device__ __forceinline__ void x_block(const XArgs& A, float4* ring, int strip,
         const float2 x = make_float2(d0[k], d0[k + 1]);
         const float2 nb = add2(make_float2(l[k] + r[k], l[k + 1] + r[k + 1]),
                                add2(make_float2(dm[k], dm[k + 1]), make_float2(dp[k], dp[k + 1])));
-        const float2 v = fma2(bc2(A.cb_hi), x, fma2(bc2(A.cb_lo), x, fma2(bc2(-4.0f), x, nb)));
+        const float2 v = fma2(cb_hi, x, fma2(cb_lo, x, fma2(bc2(-4.0f), x, nb)));
         d[k] = v.x;
         d[k + 1] = v.y;
       }

@@ -220,6 +220,9 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
   for (int l = 0; l < P; ++l) w[l][0][0] = w[l][0][1] = w[l][1][0] = w[l][1][1] = z2;
   float2 x[2][2], yn[2], xr[2], rn[2];  // PAIR: w[P - 1] holds l of the last level's y, x that y, xr what it rounded away
   x[0][0] = x[0][1] = x[1][0] = x[1][1] = yn[0] = yn[1] = xr[0] = xr[1] = rn[0] = rn[1] = z2;
+  float2 ql[P];  // (a batch's arguments sit in shared memory, read again after every asynchronous copy)
+#pragma unroll
+  for (int l = 0; l < P - 1; ++l) ql[l] = bc2(A.q[l]);
   const float2 s_hi = bc2(A.s_hi), n_hi = bc2(-A.s_hi), s_lo = bc2(A.s_lo), l_hi = bc2(A.l_hi), l_lo = bc2(A.l_lo);
   float* ph = (PAIR ? A.out : A.hi) + off + (size_t)j0 * ld;
   float* pl = A.lo + off + (size_t)j0 * ld;
@@ -283,8 +286,8 @@ __device__ __forceinline__ void s_block(const SArgs& A, float4* ring, int strip,
           float2 y[2];
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
-            y[k] = fma2(bc2(A.q[l]), tt[k], b[l + 1][k]);
-            if (PAIR && l == P - 2) rn[k] = fma2(bc2(A.q[l]), tt[k], sub2(b[l + 1][k], y[k]));
+            y[k] = fma2(ql[l], tt[k], b[l + 1][k]);
+            if (PAIR && l == P - 2) rn[k] = fma2(ql[l], tt[k], sub2(b[l + 1][k], y[k]));
           }
           mask(y);
           if (PAIR && l == P - 2) {
