@@ -1189,8 +1189,8 @@ int terms3d32(ms_grid* g, int axis, const Term3& q0, const Term3& q1) {
       A.nq = std::max(A.nq, a.nq);
       bytes += 4.0 * (2.0 * (double)ss.size() + (a.accumulate ? 2.0 : 1.0) * (double)sd.size());
     }
-    // segments of about 64 rows (16 more warm up each), shorter where that leaves SMs idle (75^3: 135 us per
-    // step with 32 rows, 130 us with 24)
+    // segments of about 64 rows (16 more warm up each), shorter where that leaves SMs idle: steps with 24 and 64
+    // rows, us: 75^3 131, 142; 100^3 273, 275; 128^3 345, 342; 160^3 581, 564; 256^3 1986, 1911
     const int rows = 2 * A.nxt * A.nq * (t.M / 64) >= 4000 ? 64 : 24;
     line_segments(t.M, rows, &A.nseg, &A.chunk, &A.rb);
     const int items = 2 * A.nxt * A.nq * A.nseg;

@@ -495,8 +495,10 @@ YArgs make_y(const ms_grid* g, int step, float* plane0, float* plane1, const flo
   set_ends(g->walk.ends[kind], &a);
   a.nstrip = (N - 1 + YOUT - 1) / YOUT;
   // Rows per segment: 16 more warm up its recurrences, so long segments do less work, but a grid wants
-  // about ten warps per SM, and small grids short walks.  The choice depends on N alone: a cavity of a batch takes the segments of a
-  // single grid, and with them its rounding.
+  // about ten warps per SM, and small grids short walks.  Steps with 16, 32 and 64 rows, us: 256^2 17.5, 19.4, 22.8;
+  // 512^2 22.6, 23.5, 26.8; 777^2 28.4, 28.8, 31.2; 1024^2 34.0, 33.3, 36.0; 1536^2 56.9, 55.1, 55.0; 2048^2 86.9,
+  // 82.8, 81.4.  The choice depends on N alone: a cavity of a batch takes the segments of a single grid, and with
+  // them its rounding.
   line_segments(a.M, a.nstrip * (a.M / 64) >= 1500 ? 64 : (N > 320 ? 32 : 16), &a.nseg, &a.chunk, &a.rb);
   a.tiny = N <= kTinyN;
   a.step = step;
@@ -536,14 +538,20 @@ XArgs make_x(const ms_grid* g, int step, float* plane, const float* src_hi, cons
   a.cb_lo = c.lo;
   set_ends(g->walk.ends[step == 0 ? HALF_TO_NODE : NODE_TO_HALF], &a);
   a.nstrip = N <= kTinyN ? 0 : (a.M + XOUT - 1) / XOUT;
-  const int rows = a.nstrip * (N / 8) < 1216 ? 4 : 8;  // as in make_s
+  // Rows per block, 4 and 8, us per step: 256^2 17.5, 18.0; 512^2 23.5, 22.8; 777^2 28.8, 29.2; 1024^2 33.0, 33.3;
+  // 1280^2 44.4, 43.9; 2048^2 82.3, 81.3.
+  const int rows = a.nstrip * (N / 8) < 1216 ? 4 : 8;
   a.nblk = (N - 1 + rows - 1) / rows;
   a.rows = (N - 1 + a.nblk - 1) / a.nblk;
   return a;
 }
 
 // Rows per block of a solve launch, warps(rows) in all: P rows above and below are computed twice, but a launch
-// wants `most` warps, about thirteen per SM, and small ones are bound by the length of one walk.
+// wants `most` warps, about thirteen per SM, and small ones are bound by the length of one walk.  Steps of one grid
+// with 4, 8, 16 and 32 rows, us: 256^2 17.5, 20.7, 27.3, 40.8; 777^2 27.2, 28.8, 32.6, 42.9; 1024^2 36.2, 33.3, 36.8,
+// 47.6; 1536^2 62.7, 57.2, 56.5, 65.9; 2048^2 99.3, 85.7, 84.1, 84.6, and 81.3 with 16 for E_z and 32 for H.  In a
+// batch the next shorter blocks begin to pay at fewer warps, 1216: 64 cavities of 256 cells, 1536 warps for E_z with 32
+// rows, take 137.8 us per step so and 140.6 with 16 (r = 0.65: 158.7, 163.9).
 template <typename Warps>
 int solve_rows(Warps warps, int most) {
   int rows = 32;
